@@ -1,11 +1,11 @@
-// batch.cu -- planning and histogram / LUT kernels for batches of shards.
+// batch.cu -- planning and histogram kernels for batches of shards.
 //
 // A batch is an array of qlc_desc in device memory (the paper's own workload
 // is 1152 shards per tensor type, Section 3).  plan_kernel turns the shard
-// sizes into work items (histogram: 256 KiB pieces; encode / decode: groups of
-// 32 chunks) with a block-wide prefix sum; the persistent kernels then take
-// items from a device counter, so shards of very different sizes share the
-// GPU evenly and no host round trip is needed.
+// sizes into work items (encode / decode: groups of 32 chunks) with a
+// block-wide prefix sum; the persistent kernels then take items from a device
+// counter, so shards of very different sizes share the GPU evenly and no host
+// round trip is needed.  The histogram kernel scans the sizes itself.
 #define QLC_FILE_ID 4
 #include "hist_cols.cuh"
 
@@ -27,14 +27,6 @@ __device__ __forceinline__ bool al16(const void* p) {
 
 // Work items of one shard; 0 (and a status) for a shard that cannot be run.
 __device__ uint64_t item_count(int kind, const qlc_desc& d, uint32_t cs, uint32_t* status) {
-  if (kind == kPlanHistogram) {
-    if (d.in_bytes == 0) return 0;
-    if (!d.in || !al16(d.in)) {
-      set_status(status, QLC_ERR_ARG);
-      return 0;
-    }
-    return (d.in_bytes + kHistItem - 1) / kHistItem;
-  }
   if (kind == kPlanEncode) {
     const uint64_t n = d.in_bytes;
     const uint64_t n_chunks = (n + cs - 1) / cs;
@@ -108,57 +100,107 @@ plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs 
 
 // ------------------------------------------------------------- histograms
 
-// Each CTA (seven warps, lane-private columns from hist_cols.cuh; two CTAs
-// per SM over the launch, one resident at a time) takes a contiguous run of
+// Histogram work items of shard s: its 64 KiB pieces, and one more without
+// bytes that stands for the flush after it (about as long as a piece), so that
+// a run of small shards is not all one CTA's.  0 for a shard that is empty or
+// cannot be read (its encode reports it: histograms have no status word).
+__device__ __forceinline__ unsigned long long hist_items(const qlc_desc* descs, int n_shards, int s) {
+  if (s >= n_shards) return 0;
+  const qlc_desc* d = descs + s;
+  return d->in && al16(d->in) && d->in_bytes ? (d->in_bytes + kHistItem - 1) / kHistItem + 1 : 0;
+}
+
+// Inclusive prefix sums of the CTA's kHcThreads values v (thread t's at
+// s_incl[t]); returns their total.  Called by every thread; s_warp holds a
+// value per warp.
+__device__ __forceinline__ unsigned long long cta_scan(unsigned long long v, unsigned long long* s_incl,
+                                                       unsigned long long* s_warp, int tid) {
+  static_assert(kHcWarps == 32, "the warps' totals are scanned by one warp");
+  const int lane = tid & 31, warp = tid >> 5;
+  auto warp_scan = [&](unsigned long long x) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long t = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += t;
+    }
+    return x;
+  };
+  const unsigned long long incl = warp_scan(v);
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  const unsigned long long w = warp_scan(s_warp[lane]);  // every warp for itself
+  const unsigned long long before = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+  s_incl[tid] = incl + (warp ? before : 0ull);
+  const unsigned long long total = __shfl_sync(0xffffffffu, w, 31);
+  __syncthreads();
+  return total;
+}
+
+// Each CTA (32 warps, hist_cols.cuh; one per SM) takes a contiguous run of
 // items.  Its items of one shard are one contiguous byte range, counted in a
-// single streaming pass; the columns are flushed into a shard's histogram
-// when the target histogram changes (never, for one shared histogram).  A
-// run is 1 / (2 x SMs) of the batch's items, so a lane's counters stay below
-// 2^32 for any batch smaller than 2^32 x 2 x SMs bytes, far above the
-// device's memory.
+// single streaming pass; the table is flushed into a shard's histogram when
+// the target histogram changes (never, for one shared histogram).  A run is
+// 1 / SMs of the batch's items, so a counter stays below 2^32 for any batch
+// smaller than 2^32 x SMs bytes, far above the device's memory.
+// Every CTA scans the shard sizes itself, kHcThreads at a time (once for a
+// batch of up to 1024 shards, else once for the total and once for its run):
+// a load and two warp scans, where a planning kernel of its own and the search
+// in its prefix cost a launch and a chain of dependent loads.  24 shards of
+// 4 KiB - 64 MiB (139 MB): 30 us, from 4.5 us of planning and 43.5 us; 1152
+// shards (3.2 GB): 517 us (6.2 TB/s), from 600 us.
 __global__ void __launch_bounds__(kHcThreads, 1)
-hist_batch_kernel(const qlc_desc* descs, int n_shards, const unsigned long long* item_base,
-                  unsigned long long* hists, int shared) {
-  extern __shared__ __align__(16) uint32_t hc_sm[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const unsigned long long total = item_base[n_shards];
+hist_batch_kernel(const qlc_desc* descs, int n_shards, unsigned long long* hists, int shared) {
+  __shared__ __align__(16) uint32_t cols[kHcColWords];
+  __shared__ unsigned long long s_incl[kHcThreads], s_warp[kHcWarps];
+  const int tid = threadIdx.x, lane = tid & 31;
+  zero_cols(cols, tid);  // published by the scan's barriers
+  unsigned long long cnt = hist_items(descs, n_shards, tid), total = cta_scan(cnt, s_incl, s_warp, tid);
+  for (int base = kHcThreads; base < n_shards; base += kHcThreads)
+    total += cta_scan(hist_items(descs, n_shards, base + tid), s_incl, s_warp, tid);
   const unsigned long long per = (total + gridDim.x - 1) / gridDim.x;
   const unsigned long long t0 = (unsigned long long)blockIdx.x * per;
   const unsigned long long t1 = min(t0 + per, total);
   if (t0 >= t1) return;
-  zero_cols(hc_sm, warp, lane);
-  __syncwarp();
-  const uint32_t col = lane_col(hc_sm, warp, lane);
-  int s = 0;
-  {
-    int lo = 0, hi = n_shards - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (item_base[mid] <= t0) lo = mid; else hi = mid - 1;
+  const uint32_t col = lane_col(cols, lane);
+  int target = -1;  // the histogram the table's counts belong to
+  unsigned long long first = 0;  // first item of the scanned shards
+  for (int base = 0; base < n_shards && first < t1; base += kHcThreads) {
+    unsigned long long part = s_incl[kHcThreads - 1];
+    if (n_shards > kHcThreads) {
+      __syncthreads();
+      part = cta_scan(hist_items(descs, n_shards, base + tid), s_incl, s_warp, tid);
     }
-    s = lo;
+    if (first + part > t0) {
+      // the first shard here with an item at or after t0: the number of
+      // shards that end at or before it
+      int j = 0;
+      {
+        const unsigned long long rel = t0 > first ? t0 - first : 0;
+        for (int half = kHcThreads / 2; half > 0; half >>= 1)
+          if (s_incl[j + half - 1] <= rel) j += half;
+      }
+      for (; j < kHcThreads && base + j < n_shards; j++) {
+        const unsigned long long sb = first + (j ? s_incl[j - 1] : 0ull), se = first + s_incl[j];  // the shard's items
+        if (sb >= t1) break;
+        if (sb == se) continue;
+        const int tgt = shared ? 0 : base + j;
+        if (target >= 0 && tgt != target)
+          flush_cols(cols, hists + (size_t)(QLC_GUARD(target < n_shards, nullptr) ? target : 0) * 256, tid, true);
+        target = tgt;
+        const uint8_t* in = static_cast<const uint8_t*>(descs[base + j].in);
+        const uint64_t n = descs[base + j].in_bytes;
+        const uint64_t beg = min((uint64_t)((max(t0, sb) - sb) * kHistItem), n);  // a multiple of 16, or the end
+        const uint64_t end = min((uint64_t)((min(t1, se) - sb) * kHistItem), n);
+        const uint64_t vb = beg / 16, ve = end / 16;
+        if (beg < end) {
+          count_span(reinterpret_cast<const uint4*>(in) + vb, ve - vb, col, tid);
+          count_bytes(in + ve * 16, end - ve * 16, col, tid);
+        }
+      }
+    }
+    first += part;
   }
-  int target = shared ? 0 : s;
-  for (unsigned long long t = t0; t < t1;) {
-    while (s + 1 < n_shards && item_base[s + 1] <= t) s++;
-    const int tgt = shared ? 0 : s;
-    if (tgt != target) {
-      flush_cols(hc_sm, hists + (size_t)(QLC_GUARD(target < n_shards, nullptr) ? target : 0) * 256, tid);
-      target = tgt;
-    }
-    const unsigned long long e = min(t1, item_base[s + 1]);  // this CTA's items of shard s end here
-    const qlc_desc d = descs[s];
-    const uint8_t* in = static_cast<const uint8_t*>(d.in);
-    const uint64_t beg = (t - item_base[s]) * kHistItem;      // a multiple of 16
-    const uint64_t end = min((uint64_t)((e - item_base[s]) * kHistItem), (uint64_t)d.in_bytes);
-    const uint64_t vb = beg / 16, ve = end / 16;
-    if (QLC_GUARD(s < n_shards && beg <= end, nullptr)) {
-      count_span(reinterpret_cast<const uint4*>(in) + vb, ve - vb, col, tid);
-      count_bytes(in + ve * 16, end - ve * 16, col, tid);
-    }
-    t = e;
-  }
-  flush_cols(hc_sm, hists + (size_t)target * 256, tid);
+  if (target >= 0) flush_cols(cols, hists + (size_t)target * 256, tid, false);
 }
 
 }  // namespace qlc
@@ -181,16 +223,11 @@ qlc_status qlc_histogram_batch(const qlc_desc* d_descs, int n_shards, uint64_t* 
   if (!aligned(d_ws, 16) || !aligned(d_descs, 16) || !aligned(d_hists, 8)) return QLC_ERR_ARG;
   BatchWs w;
   if (!batch_ws_layout(d_ws, ws_bytes, n_shards, &w)) return QLC_ERR_CAPACITY;
-  static int smem_done[64] = {0};
-  if (!hist_cols_smem_ok(hist_batch_kernel, smem_done)) return QLC_ERR_CUDA;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const size_t hist_bytes = (size_t)(shared ? 1 : n_shards) * 256 * sizeof(uint64_t);
   if (cudaMemsetAsync(d_hists, 0, hist_bytes, st) != cudaSuccess) return QLC_ERR_CUDA;
-  // histogram errors (misaligned shards) have no status word: they are
-  // reported as QLC_ERR_ARG by the encode plan of the same descriptors
-  plan_kernel<<<1, kPlanThreads, 0, st>>>(kPlanHistogram, d_descs, n_shards, 0, w, nullptr);
-  hist_batch_kernel<<<sm_count() * kHcBatchWaves, kHcThreads, kHcSmemBytes, st>>>(
-      d_descs, n_shards, w.item_base, reinterpret_cast<unsigned long long*>(d_hists), shared ? 1 : 0);
+  hist_batch_kernel<<<sm_count(), kHcThreads, 0, st>>>(d_descs, n_shards,
+                                                       reinterpret_cast<unsigned long long*>(d_hists), shared ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
 }
 

@@ -10,24 +10,35 @@
 
 namespace qlc {
 
-// One CTA of seven warps per SM counts a contiguous slice of the tensor into
-// lane-private columns (hist_cols.cuh); the last CTA also counts the bytes
-// after the last whole 16-byte vector.
+// One CTA of 32 warps per SM counts a contiguous slice of the tensor
+// (hist_cols.cuh); the last CTA also counts the bytes after the last whole
+// 16-byte vector.  A single CTA (small tensors) can write the counts itself
+// (overwrite): no memset has to run before it.
 __global__ void __launch_bounds__(kHcThreads, 1)
-hist_kernel(const uint8_t* __restrict__ in, uint64_t n, unsigned long long* __restrict__ hist) {
-  extern __shared__ __align__(16) uint32_t hc_sm[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  zero_cols(hc_sm, warp, lane);
-  __syncwarp();
-  const uint32_t col = lane_col(hc_sm, warp, lane);
+hist_kernel(const uint8_t* __restrict__ in, uint64_t n, unsigned long long* __restrict__ hist, bool overwrite) {
+  __shared__ __align__(16) uint32_t cols[kHcColWords];
+  const int tid = threadIdx.x, lane = tid & 31;
+  zero_cols(cols, tid);
+  __syncthreads();
+  const uint32_t col = lane_col(cols, lane);
   const uint64_t nvec = n / 16;
   const uint64_t per = (nvec + gridDim.x - 1) / gridDim.x;
   const uint64_t beg = (uint64_t)blockIdx.x * per;
   const uint64_t end = min(beg + per, nvec);
   if (beg < end) count_span(reinterpret_cast<const uint4*>(in) + beg, end - beg, col, tid);
   if (blockIdx.x == gridDim.x - 1) count_bytes(in + nvec * 16, n - nvec * 16, col, tid);
-  flush_cols(hc_sm, hist, tid);
+  if (overwrite) {
+    __syncthreads();
+    const uint32_t t = sum_cols(cols, tid);
+    if ((tid & 3) == 0) hist[tid >> 2] = t;
+  } else {
+    flush_cols(cols, hist, tid, false);
+  }
 }
+
+// Fewest vectors per histogram CTA (64 KiB): up to there one CTA counts alone
+// and no memset precedes it.
+constexpr uint64_t kHistCtaVecs = 4096;
 
 // Rank of a symbol (Section 7): symbols with a larger count, or the same
 // count and a smaller value, come first.  With key(t) = count(t) * 256 +
@@ -198,21 +209,21 @@ qlc_status qlc_histogram(const uint8_t* d_in, size_t n, uint64_t* d_hist, int ac
   NvtxRange nvtx_range("qlc_histogram");
   if (!d_hist || (n > 0 && !d_in)) return QLC_ERR_ARG;
   if (!aligned(d_in, 16) || !aligned(d_hist, 8)) return QLC_ERR_ARG;
-  static int smem_done[64] = {0};
-  if (!hist_cols_smem_ok(hist_kernel, smem_done)) return QLC_ERR_CUDA;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (!accumulate && cudaMemsetAsync(d_hist, 0, 256 * sizeof(uint64_t), st) != cudaSuccess)
-    return QLC_ERR_CUDA;
-  if (n == 0) return QLC_OK;
-  // one CTA per SM, at least 48 KiB each; a CTA counts under 2^31 bytes
+  // One CTA per SM, at least kHistCtaVecs vectors each; a CTA counts under
+  // 2^31 bytes.
   const uint64_t nvec = n / 16;
-  uint64_t grid = (nvec + 3071) / 3072;
+  uint64_t grid = (nvec + kHistCtaVecs - 1) / kHistCtaVecs;
   const uint64_t cap = (uint64_t)sm_count();
   if (grid > cap) grid = cap;
   const uint64_t floor_grid = (nvec >> 27) + 1;
   if (grid < floor_grid) grid = floor_grid;
   if (grid > 0x7fffffffu) return QLC_ERR_ARG;
-  hist_kernel<<<(int)grid, kHcThreads, kHcSmemBytes, st>>>(d_in, n, reinterpret_cast<unsigned long long*>(d_hist));
+  const bool overwrite = !accumulate && n > 0 && grid == 1;
+  if (!accumulate && !overwrite && cudaMemsetAsync(d_hist, 0, 256 * sizeof(uint64_t), st) != cudaSuccess)
+    return QLC_ERR_CUDA;
+  if (n == 0) return QLC_OK;
+  hist_kernel<<<(int)grid, kHcThreads, 0, st>>>(d_in, n, reinterpret_cast<unsigned long long*>(d_hist), overwrite);
   return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
 }
 

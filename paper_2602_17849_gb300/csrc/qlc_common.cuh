@@ -180,7 +180,7 @@ struct NvtxRange {
 // item of each shard; the last entry is the total), then one look-back word
 // per encode work item.
 struct BatchWs {
-  unsigned int* ticket;                // shared by encode / decode / histogram
+  unsigned int* ticket;                // shared by encode / decode
   unsigned long long* item_base;
   unsigned long long* gstat;
   unsigned long long gstat_cap;        // look-back words available
@@ -196,12 +196,12 @@ inline bool batch_ws_layout(void* ws, size_t bytes, int n_shards, BatchWs* w) {
   return true;
 }
 
-enum PlanKind { kPlanHistogram = 0, kPlanEncode = 1, kPlanDecode = 2 };
+enum PlanKind { kPlanEncode = 1, kPlanDecode = 2 };
 constexpr int kPlanThreads = 1024;
-constexpr uint64_t kHistItem = 256 * 1024;  // symbols per histogram work item
+constexpr uint64_t kHistItem = 64 * 1024;  // symbols per histogram work item
 
-// One CTA: the number of work items of every shard (histogram: 256 KiB
-// pieces; encode: groups of 32 chunks; decode: the container's groups),
+// One CTA: the number of work items of every shard (encode: groups of 32
+// chunks; decode: the container's groups),
 // their exclusive prefix in item_base, and zeroed counters / look-back words.
 // Shards that cannot be processed get no items and set *status.
 __global__ void plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w,
