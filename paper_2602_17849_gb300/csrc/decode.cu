@@ -20,77 +20,13 @@
 // of its use so that no memory access lies on the round-to-round chain.
 // Output: each lane writes its 32 symbols of a block with one 32-byte
 // streaming store.
-#include <cuda_bf16.h>
-
 #define QLC_FILE_ID 1
-#include "qlc_common.cuh"
+#include "decode_common.cuh"
+#include "decode_span.cuh"
 
 namespace qlc {
 
 constexpr int kDecCtasPerSm = 20;  // 20 x (8.3 KB + 1 KB reserved); at 24 the register cap (80) spills
-
-struct DecHeader {
-  uint64_t n, payload_bytes, P, n_chunks, n_groups;
-  uint64_t in_bytes, out_cap;  // the caller's buffers (bounds of the checked build)
-  uint32_t cs;
-  uint32_t len_lo, len_hi;  // code length of areas 0-3 / 4-7, one byte each
-};
-
-__constant__ uint16_t c_table_n[2][8] = {{8, 8, 8, 8, 8, 16, 32, 168}, {2, 8, 8, 8, 8, 32, 32, 158}};
-__constant__ uint8_t c_table_b[2][8] = {{3, 3, 3, 3, 3, 4, 5, 8}, {1, 3, 3, 3, 3, 5, 5, 8}};
-
-// Parses and validates the header (all lanes, redundantly); same checks, in
-// the same order of kinds, as the container rules: 0 = ok, else a status.
-__device__ uint32_t parse_header(const uint8_t* in, uint64_t in_bytes, uint64_t out_cap,
-                                 DecHeader* h, uint32_t* s_seen, int lane) {
-  if (in_bytes < kIndexOff) return QLC_ERR_CORRUPT;
-  const uint32_t w0 = *reinterpret_cast<const uint32_t*>(in);
-  const uint32_t w1 = *reinterpret_cast<const uint32_t*>(in + 4);
-  const unsigned long long reserved = *reinterpret_cast<const unsigned long long*>(in + 56);
-  bool ok = w0 == 0x31434C51u && (w1 & 0xFFFFu) == QLC_VERSION && (w1 >> 24) == 0 && reserved == 0;
-  const uint32_t id = (w1 >> 16) & 0xFFu;
-  uint16_t an[8];
-  uint8_t ab[8];
-  for (int i = 0; i < 8; i++) {
-    an[i] = *reinterpret_cast<const uint16_t*>(in + 24 + 2 * i);
-    ab[i] = in[40 + i];
-  }
-  ok = ok && scheme_ok(an, ab);
-  if (id == 1 || id == 2) {
-    for (int i = 0; i < 8; i++) ok = ok && an[i] == c_table_n[id - 1][i] && ab[i] == c_table_b[id - 1][i];
-  } else {
-    ok = ok && id == 0;
-  }
-  h->n = *reinterpret_cast<const unsigned long long*>(in + 8);
-  h->cs = *reinterpret_cast<const uint32_t*>(in + 16);
-  h->n_chunks = *reinterpret_cast<const uint32_t*>(in + 20);
-  ok = ok && chunk_symbols_ok(h->cs) && h->n_chunks == (h->n + h->cs - 1) / h->cs;
-  // dec must be a permutation of 0..255
-  if (lane < 8) s_seen[lane] = 0;
-  __syncwarp();
-  for (int i = lane; i < 256; i += 32) {
-    const uint32_t s = in[64 + i];
-    atomicOr(&s_seen[s >> 5], 1u << (s & 31));
-  }
-  __syncwarp();
-  uint32_t seen = 0;
-  for (int i = 0; i < 8; i++) seen += __popc(s_seen[i]);
-  ok = ok && seen == 256;
-  h->n_groups = n_groups_of(h->n_chunks);
-  h->P = payload_start(h->n_chunks);
-  h->payload_bytes = *reinterpret_cast<const unsigned long long*>(in + 48);
-  ok = ok && h->P <= in_bytes && h->payload_bytes <= in_bytes - h->P;
-  if (!ok) return QLC_ERR_CORRUPT;
-  if (out_cap < h->n) return QLC_ERR_CAPACITY;
-  h->in_bytes = in_bytes;
-  h->out_cap = out_cap;
-  h->len_lo = h->len_hi = 0;
-  for (int i = 0; i < 4; i++) {
-    h->len_lo |= (3u + ab[i]) << (8 * i);
-    h->len_hi |= (3u + ab[i + 4]) << (8 * i);
-  }
-  return 0;
-}
 
 // cp.async (global -> shared, 16 bytes, bypassing L1) and its groups.
 __device__ __forceinline__ void cp_async16(uint32_t smem, const void* g) {
@@ -106,31 +42,17 @@ constexpr uint32_t kBlk = 32;       // symbols per lane per block
 constexpr uint32_t kStageVec = 8;   // 16-byte vectors staged per lane (128 B of its stream)
 constexpr uint32_t kColRows = 16;   // words in each lane's column ring
 
-__device__ __forceinline__ uint32_t mad_hi(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-  return d;
-}
-// prmt.b32 in its default mode; a selector nibble with bit 3 set yields the
-// sign of the selected byte replicated (0x00 for bytes below 0x80).
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
-  return d;
-}
-__device__ __forceinline__ uint32_t mad_lo(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-  return d;
-}
-
-// Shared memory of one decoding warp (one CTA): the lanes' staging ring and
-// column ring, and the code table.
-struct DecShared {
+// Shared memory of one warp decoding a group: the lanes' staging ring and
+// column ring.
+struct LaneShared {
   uint32_t col[kColRows][32];  // word k of lane l at col[k % 16][l]
   uint4 stage[kStageVec][32];  // vector v of lane l at stage[v % 8][l]
+};
+// ... of a CTA of one such warp: with its code table and header.
+struct DecShared {
+  LaneShared lanes;
   uint8_t T[2048];                // code -> symbol
-  __align__(16) uint8_t dec[256];
+  __align__(16) uint8_t hdr[kIndexOff];  // the container's header and dec
   uint32_t seen[8];
 };
 
@@ -191,14 +113,14 @@ struct LaneDec {
           : "memory");
     tv += q;
   }
-  __device__ __forceinline__ uint32_t ring(const DecShared& sm, uint32_t k) const {
+  __device__ __forceinline__ uint32_t ring(const LaneShared& sm, uint32_t k) const {
     return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint8_t*>(sm.col) + (((k << 7) & 0x780u) | lane4));
   }
   // Set-up at bit S of the group: fill the staging ring, wait for it, move
   // the words the first block can read, load the buffer, refill.  Words
   // j .. j + 2 (at most two vectors) go to the buffer before the rest is
   // moved: the ring holds 16 words, and word j + 16 shares word j's row.
-  __device__ __forceinline__ void start(const DecShared& sm, uint32_t S) {
+  __device__ __forceinline__ void start(const LaneShared& sm, uint32_t S) {
     p = S;
     tv = fv = min(S >> 7, vend);
     fetch<kStageVec>(min(tv + kStageVec, vend));
@@ -228,15 +150,9 @@ struct LaneDec {
     fetch<3>(min(tv + kStageVec, vend));
     cp_async_commit();
   }
-  // Code length of the codeword at the top of x (Section 7: the area code,
-  // i.e. the top 3 bits, fixes it): a byte permute of two registers; the
-  // selector's sign-mode nibbles make bytes 1-3 zero.
-  __device__ __forceinline__ static uint32_t code_len(uint32_t x, uint32_t len_lo, uint32_t len_hi) {
-    return prmt(len_lo, len_hi, mad_hi(x, 8u, 0x8880u));
-  }
   // Advances the position to pn (less than 32 bits on): when it crosses into
   // the next word the buffer moves up a word and the word after nxt is read.
-  __device__ __forceinline__ void step_to(const DecShared& sm, uint32_t pn) {
+  __device__ __forceinline__ void step_to(const LaneShared& sm, uint32_t pn) {
     if ((pn ^ p) & 32u) {
       hi = lo;
       lo = nxt;
@@ -245,49 +161,28 @@ struct LaneDec {
     p = pn;
   }
   // Two symbols (at most 22 bits) from the window, packed as s0 | s1 << 8.
-  __device__ __forceinline__ uint32_t round2(const DecShared& sm, uint32_t len_lo, uint32_t len_hi) {
+  __device__ __forceinline__ uint32_t round2(const LaneShared& sm, const uint8_t* T, uint32_t len_lo, uint32_t len_hi) {
     const uint32_t x = __funnelshift_l(lo, hi, p);
     const uint32_t la = code_len(x, len_lo, len_hi);
     const uint32_t ia = __funnelshift_l(x, 0u, la);
-    const uint32_t a = QLC_GUARD(ia < 2048u, nullptr) ? sm.T[ia] : 0u;
+    const uint32_t a = QLC_GUARD(ia < 2048u, nullptr) ? (uint32_t)T[ia] : 0u;
     const uint32_t x2 = x << la;
     const uint32_t lb = code_len(x2, len_lo, len_hi);
     const uint32_t ib = __funnelshift_l(x2, 0u, lb);
-    const uint32_t b = QLC_GUARD(ib < 2048u, nullptr) ? sm.T[ib] : 0u;
+    const uint32_t b = QLC_GUARD(ib < 2048u, nullptr) ? (uint32_t)T[ib] : 0u;
     step_to(sm, p + la + lb);
     return mad_lo(b, 256u, a);
   }
   // One symbol (ragged chunk ends only).
-  __device__ __forceinline__ uint32_t round1(const DecShared& sm, uint32_t len_lo, uint32_t len_hi) {
+  __device__ __forceinline__ uint32_t round1(const LaneShared& sm, const uint8_t* T, uint32_t len_lo, uint32_t len_hi) {
     const uint32_t x = __funnelshift_l(lo, hi, p);
     const uint32_t la = code_len(x, len_lo, len_hi);
     const uint32_t ia = __funnelshift_l(x, 0u, la);
-    const uint32_t a = QLC_GUARD(ia < 2048u, nullptr) ? sm.T[ia] : 0u;
+    const uint32_t a = QLC_GUARD(ia < 2048u, nullptr) ? (uint32_t)T[ia] : 0u;
     step_to(sm, p + la);
     return a;
   }
 };
-
-// code -> symbol table: every code (i << bits[i]) | s of every area i maps to
-// dec[offset_i + s] (offset 0 for 8-bit areas); dec is staged in shared.
-__device__ void build_table(const uint8_t* in, DecShared& sm, int lane) {
-  reinterpret_cast<uint32_t*>(sm.dec)[lane] = reinterpret_cast<const uint32_t*>(in + 64)[lane];
-  reinterpret_cast<uint32_t*>(sm.dec)[lane + 32] = reinterpret_cast<const uint32_t*>(in + 64)[lane + 32];
-  __syncwarp();
-  uint32_t base = 0;
-  for (int i = 0; i < 8; i++) {
-    const uint32_t b = in[40 + i];
-    for (uint32_t s = lane; s < (1u << b); s += 32)
-      if (QLC_GUARD(((i << b) | s) < 2048u && (b == 8 ? s : base + s) < 256u, nullptr))
-        sm.T[(i << b) | s] = sm.dec[b == 8 ? s : base + s];
-    base += *reinterpret_cast<const uint16_t*>(in + 24 + 2 * i);
-  }
-  __syncwarp();
-}
-
-// Output of the decoder: the symbols themselves (kOutCodes), or their
-// block-32 dequantised values (value(code) * scale, fp32 or rounded to bf16).
-constexpr int kOutCodes = -1;
 
 // Streaming 32-byte store (dst 32-byte aligned) or two 16-byte stores.
 __device__ __forceinline__ void st_cs_32(uint8_t* dst, const uint32_t w[8], bool aligned32) {
@@ -301,23 +196,6 @@ __device__ __forceinline__ void st_cs_32(uint8_t* dst, const uint32_t w[8], bool
     asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(dst + 16), "r"(w[4]), "r"(w[5]), "r"(w[6]),
                  "r"(w[7])
                  : "memory");
-  }
-}
-
-// Single symbols (ragged chunk ends).
-template <int kOut>
-__device__ __forceinline__ void put_tail(void* out, const float* scales, uint64_t i, const uint8_t* sb,
-                                         uint32_t cnt) {
-  for (uint32_t b = 0; b < cnt; b++) {
-    if (kOut == kOutCodes) {
-      static_cast<uint8_t*>(out)[i + b] = sb[b];
-    } else {
-      const float y = e4m3_to_f32(sb[b]) * scales[(i + b) / 32];
-      if (kOut == QLC_DTYPE_F32)
-        static_cast<float*>(out)[i + b] = y;
-      else
-        static_cast<__nv_bfloat16*>(out)[i + b] = __float2bfloat16_rn(y);
-    }
   }
 }
 
@@ -351,13 +229,6 @@ __device__ __forceinline__ void put32(void* out, float sc, uint64_t i, const uin
   }
 }
 
-// One decoded symbol s at index i of the tensor (ragged chunk ends).
-template <int kOut>
-__device__ __forceinline__ void put1(void* out, const float* scales, uint64_t i, uint32_t s) {
-  const uint8_t b = (uint8_t)s;
-  put_tail<kOut>(out, scales, i, &b, 1);
-}
-
 // Decodes group g of a validated container (one warp; lane = chunk).  With
 // out_slot the output pointer is read from that shared word at each block
 // instead of out: a pointer that is not a kernel parameter would otherwise
@@ -365,7 +236,7 @@ __device__ __forceinline__ void put1(void* out, const float* scales, uint64_t i,
 // more instructions (the batch decoder, 124.3 M against 112.8 M on 256 MiB).
 template <int kOut>
 __device__ __forceinline__ void decode_group(const DecHeader& h, const uint8_t* __restrict__ in, void* __restrict__ out,
-                             const float* __restrict__ scales, uint64_t g, DecShared& sm, LaneDec& d,
+                             const float* __restrict__ scales, uint64_t g, LaneShared& sm, const uint8_t* T, LaneDec& d,
                              uint32_t* status, int lane, bool aligned32, bool sc_vec = false,
                              void* const volatile* out_slot = nullptr) {
   const unsigned long long* group_off = reinterpret_cast<const unsigned long long*>(in + kIndexOff);
@@ -434,14 +305,14 @@ __device__ __forceinline__ void decode_group(const DecHeader& h, const uint8_t* 
       uint32_t w[8];
 #pragma unroll
       for (int j = 0; j < 8; j++) {
-        const uint32_t p0 = d.round2(sm, len_lo, len_hi);
-        const uint32_t p1 = d.round2(sm, len_lo, len_hi);
+        const uint32_t p0 = d.round2(sm, T, len_lo, len_hi);
+        const uint32_t p1 = d.round2(sm, T, len_lo, len_hi);
         w[j] = __byte_perm(p0, p1, 0x5410);
       }
       if (QLC_GUARD(i_chunk + i0 + kBlk <= h.out_cap, status)) put32<kOut>(o, sc, i_chunk + i0, w, aligned32);
     } else {
       for (uint32_t k = 0; k < cnt; k++) {
-        const uint32_t sym = d.round1(sm, len_lo, len_hi);
+        const uint32_t sym = d.round1(sm, T, len_lo, len_hi);
         if (QLC_GUARD(i_chunk + i0 + k < h.out_cap, status)) put1<kOut>(o, scales, i_chunk + i0 + k, sym);
       }
     }
@@ -452,7 +323,7 @@ __device__ __forceinline__ void decode_group(const DecHeader& h, const uint8_t* 
 
 // Lane set-up shared by the kernels; 0 if the ring is not placed as its
 // addressing requires.
-__device__ __forceinline__ bool lane_init(DecShared& sm, LaneDec& d, int lane) {
+__device__ __forceinline__ bool lane_init(LaneShared& sm, LaneDec& d, int lane) {
   d.lane4 = 4u * lane;
   d.col_s = (uint32_t)__cvta_generic_to_shared(&sm.col[0][lane]);
   d.stage_s = (uint32_t)__cvta_generic_to_shared(&sm.stage[0][lane]);
@@ -469,7 +340,9 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
   __shared__ DecShared sm;
   const int lane = threadIdx.x;
   DecHeader h;
-  const uint32_t err = parse_header(in, in_bytes, out_cap, &h, sm.seen, lane);
+  load_header(in, in_bytes, sm.hdr, lane, 32);
+  __syncwarp();
+  const uint32_t err = parse_header(sm.hdr, in_bytes, out_cap, &h, sm.seen, lane);
   if (err) {
     if (blockIdx.x == 0 && lane == 0) {
       if (err == QLC_ERR_CAPACITY) *n_out = h.n;
@@ -480,15 +353,79 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
   if (blockIdx.x == 0 && lane == 0) *n_out = h.n;
   if (blockIdx.x >= h.n_groups) return;
   LaneDec d;
-  if (!lane_init(sm, d, lane)) {
+  if (!lane_init(sm.lanes, d, lane)) {
     if (lane == 0) set_status(status, QLC_ERR_CUDA);
     return;
   }
-  build_table(in, sm, lane);
+  build_table(sm.hdr, sm.T, lane, 32);
+  __syncwarp();
   const bool aligned32 = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
   const bool sc_vec = (reinterpret_cast<uintptr_t>(scales) & 15u) == 0;  // scales read four at a time
   for (uint64_t g = blockIdx.x; g < h.n_groups; g += gridDim.x)
-    decode_group<kOut>(h, in, out, scales, g, sm, d, status, lane, aligned32, sc_vec);
+    decode_group<kOut>(h, in, out, scales, g, sm.lanes, sm.T, d, status, lane, aligned32, sc_vec);
+}
+
+// Shared memory of a split-decoding CTA; its warps decode spans, or groups.
+struct SpanShared {
+  union {
+    SpanWarp span;
+    LaneShared lanes;
+  } w[kSpanWarps];
+  uint8_t T[2048];                          // code -> symbol
+  __align__(16) uint8_t hdr[kIndexOff];     // the container's header and dec
+  uint32_t seen[kSpanWarps][8];
+};
+
+// One container, split: CTAs of kSpanWarps warps validate the header, build
+// the code table once and decode spans (decode_span.cuh), or whole groups
+// with a lane per chunk where that is faster (split_pays).
+template <int kOut>
+__global__ void __launch_bounds__(32 * kSpanWarps, kSpanCtasPerSm)
+decode_span_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restrict__ out,
+                   const float* __restrict__ scales, uint64_t out_cap, unsigned long long* __restrict__ n_out,
+                   uint32_t* __restrict__ status) {
+  __shared__ SpanShared sm;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  load_header(in, in_bytes, sm.hdr, tid, 32 * kSpanWarps);
+  __syncthreads();
+  DecHeader h;
+  const uint32_t err = parse_header(sm.hdr, in_bytes, out_cap, &h, sm.seen[warp], lane);
+  if (blockIdx.x == 0 && tid == 0) {
+    if (!err || err == QLC_ERR_CAPACITY) *n_out = h.n;
+    if (err) set_status(status, err);
+  }
+  if (err) return;
+  build_table(sm.hdr, sm.T, tid, 32 * kSpanWarps);
+  __syncthreads();
+  if (!split_pays(h, h.n)) {
+    LaneDec d;
+    if (!lane_init(sm.w[warp].lanes, d, lane)) {
+      if (lane == 0) set_status(status, QLC_ERR_CUDA);
+      return;
+    }
+    const bool aligned32 = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
+    const bool sc_vec = (reinterpret_cast<uintptr_t>(scales) & 15u) == 0;
+    for (uint64_t g = blockIdx.x + (uint64_t)warp * gridDim.x; g < h.n_groups; g += (uint64_t)gridDim.x * kSpanWarps)
+      decode_group<kOut>(h, in, out, scales, g, sm.w[warp].lanes, sm.T, d, status, lane, aligned32, sc_vec);
+    return;
+  }
+  const SpanShape shape(h.cs);
+  const uint32_t warm = warm_bits(h.len_lo, h.len_hi);
+  const uint32_t k = (uint32_t)lane / shape.lanes, seg = (uint32_t)lane - k * shape.lanes;
+  // span s is span r of group g; the step to the warp's next span is made in both
+  const uint32_t stride = gridDim.x * kSpanWarps, dg = stride / shape.per_group, dr = stride % shape.per_group;
+  const uint32_t s0 = blockIdx.x * kSpanWarps + warp;
+  uint64_t g = s0 / shape.per_group;
+  uint32_t r = s0 % shape.per_group;
+  while (g < h.n_groups) {
+    decode_span<kOut>(h, shape, in, out, scales, g, r * shape.chunks, k, seg, sm.w[warp].span, sm.T, warm, status, lane);
+    g += dg;
+    r += dr;
+    if (r >= shape.per_group) {
+      r -= shape.per_group;
+      g++;
+    }
+  }
 }
 
 // A batch: warps take (shard, group) items from a device counter; a warp
@@ -500,7 +437,7 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
   __shared__ DecShared sm;
   const int lane = threadIdx.x;
   LaneDec d;
-  if (!lane_init(sm, d, lane)) {
+  if (!lane_init(sm.lanes, d, lane)) {
     if (lane == 0) set_status(status, QLC_ERR_CUDA);
     return;
   }
@@ -519,7 +456,10 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
     const uint8_t* in = static_cast<const uint8_t*>(dd.in);
     const uint64_t g = t - item_base[sh];
     if (sh != cur) {
-      const uint32_t err = parse_header(in, dd.in_bytes, dd.out_cap, &h, sm.seen, lane);
+      __syncwarp();  // every lane is done with the previous shard's header
+      load_header(in, dd.in_bytes, sm.hdr, lane, 32);
+      __syncwarp();
+      const uint32_t err = parse_header(sm.hdr, dd.in_bytes, dd.out_cap, &h, sm.seen, lane);
       if (err) {
         if (lane == 0) {
           if (err == QLC_ERR_CAPACITY && dd.out_bytes) *dd.out_bytes = h.n;
@@ -529,7 +469,8 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
         cur = -1;
         continue;
       }
-      build_table(in, sm, lane);
+      build_table(sm.hdr, sm.T, lane, 32);
+      __syncwarp();
       cur = sh;
     }
     if (g == 0 && lane == 0 && dd.out_bytes) *dd.out_bytes = h.n;
@@ -538,7 +479,7 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
     if (lane == 0) s_out = dd.out;
     __syncwarp();
     if (g < h.n_groups)
-      decode_group<kOutCodes>(h, in, nullptr, nullptr, g, sm, d, status, lane, aligned32, false, &s_out);
+      decode_group<kOutCodes>(h, in, nullptr, nullptr, g, sm.lanes, sm.T, d, status, lane, aligned32, false, &s_out);
   }
 }
 
@@ -566,15 +507,32 @@ static int decode_grid(uint64_t out_cap) {
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
+// CTAs of the split decoder: a warp per span.
+static int span_grid(uint64_t out_cap) {
+  const uint64_t want = (out_cap / kSpanSyms + kSpanWarps) / kSpanWarps, cap = (uint64_t)sm_count() * kSpanCtasPerSm;
+  return (int)(want < cap ? want : cap);
+}
+
+template <int kOut>
+static qlc_status launch_decode(const uint8_t* d_in, size_t in_bytes, void* d_out, const float* d_scales,
+                                size_t out_cap, uint64_t* d_n_out, uint32_t* d_status, cudaStream_t st) {
+  unsigned long long* no = reinterpret_cast<unsigned long long*>(d_n_out);
+  if (out_cap <= kSplitMax)
+    decode_span_kernel<kOut><<<span_grid(out_cap), 32 * kSpanWarps, 0, st>>>(d_in, in_bytes, d_out, d_scales, out_cap,
+                                                                             no, d_status);
+  else
+    decode_kernel<kOut><<<decode_grid(out_cap), 32, 0, st>>>(d_in, in_bytes, d_out, d_scales, out_cap, no, d_status);
+  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+}
+
 extern "C" qlc_status qlc_decode(const uint8_t* d_in, size_t in_bytes, uint8_t* d_out, size_t out_cap,
                                  uint64_t* d_n_out, uint32_t* d_status, qlc_stream_t stream) {
   NvtxRange nvtx_range("qlc_decode");
   if (!d_in || !d_n_out || (out_cap > 0 && !d_out)) return QLC_ERR_ARG;
   if (!aligned(d_in, 16) || !aligned(d_out, 16) || !aligned(d_n_out, 8) || !aligned(d_status, 4))
     return QLC_ERR_ARG;
-  decode_kernel<kOutCodes><<<decode_grid(out_cap), 32, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      d_in, in_bytes, d_out, nullptr, out_cap, reinterpret_cast<unsigned long long*>(d_n_out), d_status);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  return launch_decode<kOutCodes>(d_in, in_bytes, d_out, nullptr, out_cap, d_n_out, d_status,
+                                  reinterpret_cast<cudaStream_t>(stream));
 }
 
 extern "C" qlc_status qlc_decode_dequantize(const uint8_t* d_in, size_t in_bytes, const float* d_scales,
@@ -587,14 +545,9 @@ extern "C" qlc_status qlc_decode_dequantize(const uint8_t* d_in, size_t in_bytes
       !aligned(d_status, 4))
     return QLC_ERR_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  unsigned long long* no = reinterpret_cast<unsigned long long*>(d_n_out);
   if (dtype == QLC_DTYPE_F32)
-    decode_kernel<QLC_DTYPE_F32><<<decode_grid(out_cap), 32, 0, st>>>(d_in, in_bytes, d_out, d_scales, out_cap, no,
-                                                                     d_status);
-  else
-    decode_kernel<QLC_DTYPE_BF16><<<decode_grid(out_cap), 32, 0, st>>>(d_in, in_bytes, d_out, d_scales, out_cap,
-                                                                      no, d_status);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+    return launch_decode<QLC_DTYPE_F32>(d_in, in_bytes, d_out, d_scales, out_cap, d_n_out, d_status, st);
+  return launch_decode<QLC_DTYPE_BF16>(d_in, in_bytes, d_out, d_scales, out_cap, d_n_out, d_status, st);
 }
 
 extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, void* d_ws, size_t ws_bytes,

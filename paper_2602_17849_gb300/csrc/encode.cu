@@ -42,13 +42,6 @@ constexpr unsigned long long kFlagError = 3ull << 62;
 constexpr unsigned long long kValMask = (1ull << 62) - 1;
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // 1 s per look-back wait
 
-// Streaming (evict-first) 16-byte store: the container is written once and
-// should not push the input, which pass 2 re-reads, out of L2.
-__device__ __forceinline__ void st_cs_v4(uint4* p, uint4 v) {
-  asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-               : "memory");
-}
-
 // OR v into a shared word.
 __device__ __forceinline__ void red_or(uint32_t saddr, uint32_t v) {
   asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(saddr), "r"(v) : "memory");

@@ -113,6 +113,13 @@ __device__ __forceinline__ uint4 ldg_nc_v4(const uint4* p) {
   return r;
 }
 
+// Streaming (evict-first) 16-byte store: what is written once should not push
+// out of L2 what is read again (the encoder's second pass over its input).
+__device__ __forceinline__ void st_cs_v4(uint4* p, uint4 v) {
+  asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+
 __device__ __forceinline__ uint64_t ld_acquire_u64(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");

@@ -1,0 +1,96 @@
+"""The split decoder against the oracle's containers (bytes: no tolerance), its
+values against the oracle's dequantisation, corrupt containers' statuses, and
+the choice between it and a lane per chunk."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2602_17849_gb300 import inputs
+from tests import _split_cases as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def qlc():
+    from paper_2602_17849_gb300 import _build
+    _build.build()
+    from paper_2602_17849_gb300 import qlc as q
+    return q
+
+
+def _decode(qlc, cont, n):
+    y = torch.full((n + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+    n_out = torch.zeros(1, dtype=torch.int64, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    qlc.qlc_decode(torch.from_numpy(cont).cuda(), y, n_out, st, out_cap=n)
+    assert int(st.item()) == 0 and int(n_out.item()) == n
+    y = y.cpu().numpy()
+    assert np.all(y[n:] == 0xA5)  # nothing written past the symbols
+    return y[:n]
+
+
+def test_containers_of_the_oracle(qlc):
+    for name, x, cont in S.containers():
+        assert np.array_equal(_decode(qlc, cont, x.size), x), name
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_values(qlc, dtype):
+    for i, (n, cs) in enumerate([(33, 128), (4097, 4096), (70_001, 1024), (300_013, 4096)]):
+        codes = S.data(("runs", "t4")[i % 2], n, i)
+        scales = np.random.default_rng(i).uniform(0.01, 3.0, (n + 31) // 32).astype(np.float32)
+        cont = torch.from_numpy(oracle.encode(codes, chunk_symbols=cs)).cuda()
+        y = torch.zeros(n, dtype=dtype, device="cuda")
+        n_out = torch.zeros(1, dtype=torch.int64, device="cuda")
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        qlc.qlc_decode_dequantize(cont, torch.from_numpy(scales).cuda(), y, n_out, st)
+        assert int(st.item()) == 0
+        want = torch.from_numpy(oracle.dequantize_block32(codes, scales)).to(dtype)
+        assert torch.equal(y.cpu().view(torch.int16), want.view(torch.int16)), (n, cs)
+
+
+def test_corrupt_payload_and_index_statuses(qlc):
+    rng = np.random.default_rng(3)
+    for sid, cs in ((1, 4096), (2, 1024), (1, 1280)):
+        x = S.data("t4", 3 * 32 * 1024 + 999, sid)
+        cont = oracle.encode(x, scheme_id=sid, chunk_symbols=cs)
+        for pos in [int(v) for v in rng.integers(320, cont.size, 60)]:
+            c = cont.copy()
+            c[pos] ^= np.uint8(1 << int(rng.integers(0, 8)))
+            ost, oy, _ = oracle.decode(c, cap=x.size)
+            y = torch.zeros(x.size, dtype=torch.uint8, device="cuda")
+            n_out = torch.zeros(1, dtype=torch.int64, device="cuda")
+            st = torch.zeros(1, dtype=torch.int32, device="cuda")
+            qlc.qlc_decode(torch.from_numpy(c).cuda(), y, n_out, st)
+            assert int(st.item()) == ost, (sid, cs, pos)
+            if ost == oracle.OK:
+                assert np.array_equal(y.cpu().numpy(), oy), (sid, cs, pos)
+
+
+@pytest.mark.parametrize("kind,n", [("t4", 64 << 20), ("t4", (64 << 20) + 128), ("relu_t4", 40 << 20),
+                                    ("relu_t4", (40 << 20) + 128)])
+def test_both_sides_of_the_choice(qlc, kind, n):
+    x = inputs.make_e4m3(kind, n, seed=2, device="cuda")
+    codec = qlc.Codec(n)
+    cont = codec.new_container()
+    codec.encode_into(x, cont)
+    y = torch.empty_like(x)
+    codec.decode_into(cont, y)
+    codec.check()
+    assert torch.equal(x, y)
+
+
+def test_checked_build():
+    import os
+    import subprocess
+    import sys
+
+    from paper_2602_17849_gb300 import _build
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, QLC_LIBRARY=_build.build(checked=True))
+    r = subprocess.run([sys.executable, os.path.join(root, "tests", "_checked_split.py")], env=env,
+                       capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    assert "no index check failed" in r.stdout
