@@ -35,6 +35,8 @@ constexpr int kSub = 32 * 16;  // symbols a warp packs per step (16 per lane)
 // per-warp staging buffer: 4 guard words, 4 carry words, one step's words, 4 spare
 constexpr int kWStage = 4 + 4 + (kSub * kMaxCode + 31) / 32 + 4;
 constexpr int kPass1Unroll = 8;
+// Tensors of up to this many chunks are encoded in parts (lengths_kernel, pack_kernel).
+constexpr uint64_t kPartMaxChunks = 1 << 14;
 
 constexpr unsigned long long kFlagAgg = 1ull << 62;
 constexpr unsigned long long kFlagPrefix = 2ull << 62;
@@ -304,14 +306,133 @@ struct Packer {
   }
 };
 
+// A LUT entry as the kernels keep it, codeword << (32 - len) | len, or 0 for
+// one that is not a codeword of 3..11 bits (a LUT not made by qlc_build_lut*),
+// which would overrun the staging window and the output bound.
+__device__ __forceinline__ uint32_t table_entry(uint32_t e) {
+  const uint32_t len = e & 15u, code = e >> 4;
+  return len < 3 || len > kMaxCode || (code >> len) != 0 ? 0u : (code << (32 - len)) | len;
+}
+// Stages entry v of symbol s, one copy per lane.
+__device__ __forceinline__ void stage_entry(uint32_t* s_enc, int s, uint32_t v) {
+  uint4* row = reinterpret_cast<uint4*>(&s_enc[32 * s]);
+#pragma unroll
+  for (int k = 0; k < 8; k++) row[k] = make_uint4(v, v, v, v);
+}
+
+// Bits of m symbols at p (16-byte aligned; m <= 4096, so that a lane's sum
+// stays below 2^21), the same in every lane.
+__device__ __forceinline__ uint32_t chunk_length(const uint32_t* tab, const uint8_t* p, uint32_t m, int lane) {
+  uint32_t bits = 0;
+  const uint32_t nv = m / 16;
+  const uint4* v = reinterpret_cast<const uint4*>(p);
+  uint32_t k = lane;
+  for (; k + (kPass1Unroll - 1) * 32 < nv; k += kPass1Unroll * 32) {
+    uint4 q[kPass1Unroll];
+#pragma unroll
+    for (int u = 0; u < kPass1Unroll; u++) q[u] = ldg_nc_v4(v + k + 32 * u);
+#pragma unroll
+    for (int u = 0; u < kPass1Unroll; u++) bits += entry_sum16(tab, q[u]);
+  }
+  for (; k < nv; k += 32) bits += entry_sum16(tab, ldg_nc_v4(v + k));
+  for (uint32_t t = nv * 16 + lane; t < m; t += 32) bits += enc_entry(tab, p[t]);
+  return warp_sum_u32(bits & ((1u << 21) - 1));
+}
+
+// The 16-byte blocks that chunks share with their neighbours: a chunk's first
+// / last one, and their block index within the group (~0u if none).
+struct Seams {
+  __align__(16) uint4 blk[kGroupChunks][2];
+  uint32_t idx[kGroupChunks][2];
+};
+
+// Packs chunk c of a group (m symbols at src, group-relative bits [S, E)) to
+// the group's payload dst; the blocks it shares with its neighbours wait in
+// seam slot c.
+__device__ __forceinline__ void pack_chunk(const uint32_t* tab, uint32_t* stage, uint32_t stage_s, const uint8_t* p,
+                                           uint32_t m, uint32_t S, uint32_t E, uint4* dst, uint32_t blk_lim,
+                                           Seams& seam, uint32_t c, int lane) {
+  Packer pk;
+  pk.tab = tab;
+  pk.stage = stage;
+  pk.stage_s = stage_s;
+  pk.dst = dst;
+  pk.blk_lim = blk_lim;
+  pk.seam_s = (uint32_t)__cvta_generic_to_shared(&seam.blk[c][0]);
+  pk.seam_idx_s = (uint32_t)__cvta_generic_to_shared(&seam.idx[c][0]);
+  pk.seam_blk = (S & 127u) ? (S >> 7) : ~0u;
+  pk.base_bit = S;
+  pk.win = (S >> 5) & ~3u;
+  pk.cur = 0;
+  pk.lane = lane;
+  // full steps, with the input of the next two steps in flight
+  const uint32_t n_full = m / kSub;
+  const uint4* src = reinterpret_cast<const uint4*>(p) + lane;
+  uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
+  if (n_full > 0) q0 = ldg_nc_v4(src);
+  if (n_full > 1) q1 = ldg_nc_v4(src + 32);
+  for (uint32_t i = 0; i < n_full; i++) {
+    const uint4 q = q0;
+    q0 = q1;
+    if (i + 2 < n_full) q1 = ldg_nc_v4(src + 32 * (i + 2));
+    pk.step<false>(q, 16);
+  }
+  // a ragged end (chunks of a size that kSub does not divide, or a tensor's
+  // last chunk): lane l takes symbols 16 l ...
+  if (m % kSub) {
+    const uint32_t off = n_full * kSub + 16u * lane;
+    const int cnt = off < m ? (int)min(16u, m - off) : 0;
+    uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int j = 0; j < 16; j++)
+      if (j < cnt) w[j >> 2] |= (uint32_t)p[off + j] << (8 * (j & 3));
+    pk.step<true>(make_uint4(w[0], w[1], w[2], w[3]), cnt);
+  }
+  // the chunk's partial last block (shared with the next chunk, or the
+  // group's zero-padded end) goes to the seam; the buffer is left zeroed
+  if (lane == 0) {
+    uint32_t* cb = pk.stage + pk.cur * kWStage + 4;
+    if (E & 127u) {
+      seam.blk[c][1] = make_uint4(bswap32(cb[0]), bswap32(cb[1]), bswap32(cb[2]), bswap32(cb[3]));
+      seam.idx[c][1] = E >> 7;
+    }
+    cb[0] = cb[1] = cb[2] = cb[3] = 0;
+  }
+  __syncwarp();
+}
+
+// Seams of a group's chunks [first, first + 32) that were packed together
+// (warp-wide): the lane of chunk l writes the block holding the chunk's end,
+// OR-ed with the blocks of chunk l + 1 that fall in the same 16 bytes and with
+// more (the bits that follow the last of these chunks).  A chunk shorter than
+// a block (only the last chunk of a tensor) is merged by the lane of the chunk
+// before it.
+__device__ __forceinline__ void merge_seams(const Seams& seam, uint4* dst, uint32_t blk_lim, uint32_t more_idx,
+                                            uint4 more, uint32_t* status, int lane) {
+  const uint32_t i1 = seam.idx[lane][1];
+  const bool mine = i1 != ~0u && !(lane > 0 && seam.idx[lane - 1][1] == i1);
+  if (!mine) return;
+  uint4 v = seam.blk[lane][1];
+  auto merge = [&](uint4 u) {
+    v.x |= u.x;
+    v.y |= u.y;
+    v.z |= u.z;
+    v.w |= u.w;
+  };
+  if (lane + 1 < kGroupChunks)
+    for (int k = 0; k < 2; k++)
+      if (seam.idx[lane + 1][k] == i1) merge(seam.blk[lane + 1][k]);
+  if (i1 == more_idx) merge(more);
+  if (QLC_GUARD(i1 < blk_lim, status)) st_cs_v4(&dst[i1], v);
+}
+
 __global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm)
 encode_kernel(EncArgs A) {
   __shared__ __align__(16) uint32_t s_enc[256 * 32];  // codeword << (32 - len) | len, one copy per lane
   __shared__ __align__(16) uint32_t s_stage[kEncWarps][2][kWStage];  // per-warp ping-pong
   __shared__ uint32_t s_chunk_bits[kGroupChunks];
   __shared__ uint32_t s_chunk_start[kGroupChunks + 1];  // group-relative bit of each chunk
-  __shared__ __align__(16) uint4 s_seam[kGroupChunks][2];  // a chunk's first / last 16-byte block
-  __shared__ uint32_t s_seam_idx[kGroupChunks][2];         // their block index, ~0u if none
+  __shared__ Seams s_seam;
   __shared__ unsigned long long s_item, s_first, s_excl;
   __shared__ const uint8_t* s_in;
   __shared__ uint64_t s_n;
@@ -370,12 +491,8 @@ encode_kernel(EncArgs A) {
     uint8_t* out = s_out;
     const qlc_lut* lut = s_lut;
     if (lut != cur_lut) {
-      // A LUT entry must be a codeword of 3..11 bits; anything else (a LUT
-      // not made by qlc_build_lut*) would overrun the staging window and the
-      // output bound, so the tensor is refused.
-      const uint32_t e = lut->enc[tid];
-      const uint32_t len = e & 15u, code = e >> 4;
-      const bool bad = len < 3 || len > kMaxCode || (code >> len) != 0;
+      const uint32_t e = table_entry(lut->enc[tid]);
+      const bool bad = e == 0;  // the tensor is refused
       if (__syncthreads_or(bad)) {
         if (tid == 0) {
           set_status(A.status, QLC_ERR_ARG);
@@ -384,12 +501,7 @@ encode_kernel(EncArgs A) {
         cur_lut = nullptr;
         continue;
       }
-      {
-        const uint32_t v = (code << (32 - len)) | len;
-        uint4* row = reinterpret_cast<uint4*>(&s_enc[32 * tid]);
-#pragma unroll
-        for (int k = 0; k < 8; k++) row[k] = make_uint4(v, v, v, v);
-      }
+      stage_entry(s_enc, tid, e);
       cur_lut = lut;
       __syncthreads();
     }
@@ -417,20 +529,7 @@ encode_kernel(EncArgs A) {
       uint32_t bits = 0;
       if (cbeg < gend) {
         const uint32_t m = (uint32_t)(min(cbeg + cs, gend) - cbeg);
-        const uint32_t nv = m / 16;
-        const uint4* v = reinterpret_cast<const uint4*>(in + cbeg);
-        uint32_t k = lane;
-        for (; k + (kPass1Unroll - 1) * 32 < nv; k += kPass1Unroll * 32) {
-          uint4 q[kPass1Unroll];
-#pragma unroll
-          for (int u = 0; u < kPass1Unroll; u++) q[u] = ldg_nc_v4(v + k + 32 * u);
-#pragma unroll
-          for (int u = 0; u < kPass1Unroll; u++) bits += entry_sum16(tab, q[u]);
-        }
-        for (; k < nv; k += 32) bits += entry_sum16(tab, ldg_nc_v4(v + k));
-        for (uint32_t t = nv * 16 + lane; t < m; t += 32) bits += enc_entry(tab, in[cbeg + t]);
-        bits &= (1u << 21) - 1;  // a lane sums at most 4096 lengths of <= 11 bits
-        bits = warp_sum_u32(bits);
+        bits = chunk_length(tab, in + cbeg, m, lane);
         if (lane == 0 && QLC_GUARD(g * kGroupChunks + c < n_chunks, A.status))
           chunk_bits[g * kGroupChunks + c] = (uint16_t)bits;
       }
@@ -449,7 +548,7 @@ encode_kernel(EncArgs A) {
       }
       s_chunk_start[lane] = incl - cb;
       if (lane == 31) s_chunk_start[32] = incl;
-      s_seam_idx[lane][0] = s_seam_idx[lane][1] = ~0u;
+      s_seam.idx[lane][0] = s_seam.idx[lane][1] = ~0u;
       const uint32_t gbits = __shfl_sync(0xffffffffu, incl, 31);
       const uint64_t gbytes = align16((gbits + 7) / 8);
       bool err = !QLC_GUARD(item < A.gstat_cap, A.status);
@@ -471,6 +570,7 @@ encode_kernel(EncArgs A) {
     __syncthreads();
     if (s_err) continue;
     uint4* dst = reinterpret_cast<uint4*>(payload + s_excl);
+    const uint32_t blk_lim = (uint32_t)min((uint64_t)((s_cap - P - s_excl) / 16), (uint64_t)0xFFFFFFFEu);
 
     // ---- pass 2: each warp packs its own chunks (w, w+8, w+16, w+24), 512
     // symbols per step, with warp scans only: a chunk's start bit is known
@@ -481,79 +581,156 @@ encode_kernel(EncArgs A) {
       if (cbeg >= gend) break;
       const uint32_t m = (uint32_t)(min(cbeg + cs, gend) - cbeg);
       if (!QLC_GUARD(cbeg + m <= n, A.status)) break;
-      const uint32_t S = s_chunk_start[c];
-      Packer pk;
-      pk.tab = tab;
-      pk.stage = &s_stage[warp][0][0];
-      pk.stage_s = stage_s;
-      pk.dst = dst;
-      pk.blk_lim = (uint32_t)min((uint64_t)((s_cap - P - s_excl) / 16), (uint64_t)0xFFFFFFFFu);
-      pk.seam_s = (uint32_t)__cvta_generic_to_shared(&s_seam[c][0]);
-      pk.seam_idx_s = (uint32_t)__cvta_generic_to_shared(&s_seam_idx[c][0]);
-      pk.seam_blk = (S & 127u) ? (S >> 7) : ~0u;
-      pk.base_bit = S;
-      pk.win = (S >> 5) & ~3u;
-      pk.cur = 0;
-      pk.lane = lane;
-      // full steps, with the input of the next two steps in flight
-      const uint32_t n_full = m / kSub;
-      const uint4* src = reinterpret_cast<const uint4*>(in + cbeg) + lane;
-      uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
-      if (n_full > 0) q0 = ldg_nc_v4(src);
-      if (n_full > 1) q1 = ldg_nc_v4(src + 32);
-      for (uint32_t i = 0; i < n_full; i++) {
-        const uint4 q = q0;
-        q0 = q1;
-        if (i + 2 < n_full) q1 = ldg_nc_v4(src + 32 * (i + 2));
-        pk.step<false>(q, 16);
-      }
-      // the ragged end of a tensor's last chunk: lane l takes symbols 16 l ...
-      if (m % kSub) {
-        const uint32_t off = n_full * kSub + 16u * lane;
-        const int cnt = off < m ? (int)min(16u, m - off) : 0;
-        uint32_t w[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int j = 0; j < 16; j++)
-          if (j < cnt) w[j >> 2] |= (uint32_t)in[cbeg + off + j] << (8 * (j & 3));
-        pk.step<true>(make_uint4(w[0], w[1], w[2], w[3]), cnt);
-      }
-      // the chunk's partial last block (shared with the next chunk, or the
-      // group's zero-padded end) goes to the seam; the buffer is left zeroed
-      if (lane == 0) {
-        const uint32_t E = s_chunk_start[c + 1];
-        uint32_t* cb = pk.stage + pk.cur * kWStage + 4;
-        if (E & 127u) {
-          s_seam[c][1] = make_uint4(bswap32(cb[0]), bswap32(cb[1]), bswap32(cb[2]), bswap32(cb[3]));
-          s_seam_idx[c][1] = E >> 7;
-        }
-        cb[0] = cb[1] = cb[2] = cb[3] = 0;
-      }
-      __syncwarp();
+      pack_chunk(tab, &s_stage[warp][0][0], stage_s, in + cbeg, m, s_chunk_start[c], s_chunk_start[c + 1], dst, blk_lim,
+                 s_seam, c, lane);
     }
     __syncthreads();
-    // Seams: lane l writes the block holding chunk l's end, OR-ed with the
-    // blocks of chunk l+1 that fall in the same 16 bytes.  A chunk shorter
-    // than a block (only the last chunk of a tensor) is merged by the lane of
-    // the chunk before it.
-    if (warp == 0) {
-      const uint32_t i1 = s_seam_idx[lane][1];
-      const bool mine = i1 != ~0u && !(lane > 0 && s_seam_idx[lane - 1][1] == i1);
-      if (mine) {
-        uint4 v = s_seam[lane][1];
-        if (lane + 1 < kGroupChunks) {
-          for (int k = 0; k < 2; k++) {
-            if (s_seam_idx[lane + 1][k] == i1) {
-              const uint4 u = s_seam[lane + 1][k];
-              v.x |= u.x;
-              v.y |= u.y;
-              v.z |= u.z;
-              v.w |= u.w;
-            }
-          }
-        }
-        if (QLC_GUARD((uint64_t)i1 < (s_cap - P - s_excl) / 16, A.status)) st_cs_v4(&dst[i1], v);
+    if (warp == 0) merge_seams(s_seam, dst, blk_lim, ~0u, make_uint4(0, 0, 0, 0), A.status, lane);
+  }
+}
+
+// ------------------------------------------------------- tensors of few groups
+//
+// A CTA per group leaves most of the GPU idle below a few hundred groups, and
+// a CTA takes about 30 us for a group of 32 x 4096 symbols.  Up to
+// kPartMaxChunks chunks the work is cut finer, in two kernels without
+// look-back (and without the memset of its words).  Histogram, LUT and encode
+// of Student-t symbols, us, a CTA per group / parts: 256 Ki symbols in chunks
+// of 4096 48.5 / 31, 1 Mi 48 / 31.8, 4 Mi 49 / 33, 16 Mi 52.6 / 44, 64 Mi
+// 113.6 / 97, 96 Mi 145 / 141, 256 Mi 296 / 320; in chunks of 1024 16 Mi 61 /
+// 54, 64 Mi 131 / 134; in chunks of 128 2 Mi 54 / 49, 8 Mi 102.5 / 105: the
+// line lies at 16384 chunks.
+//   lengths  a warp per chunk: chunk_bits (and the container's header);
+//   pack     a CTA per part of kEncWarps chunks, a chunk per warp. The sizes of
+//            the groups before a part's are summed from chunk_bits (2 bytes per
+//            chunk, from L2), so a CTA needs nothing from the others. A 16-byte
+//            block that two parts share belongs to the part it starts in, whose
+//            CTA also encodes the up to 43 symbols after the part that reach
+//            into it.
+__global__ void __launch_bounds__(kEncThreads)
+lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __restrict__ lut, uint32_t cs, uint8_t* out,
+               uint32_t* status) {
+  __shared__ __align__(16) uint32_t s_enc[256 * 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint64_t n_chunks = (n + cs - 1) / cs;
+  const uint32_t e = table_entry(lut->enc[tid]);
+  stage_entry(s_enc, tid, e);
+  if (__syncthreads_or(e == 0)) {  // not a LUT of this library: refused
+    if (blockIdx.x == 0 && tid == 0) set_status(status, QLC_ERR_ARG);
+    return;
+  }
+  if (blockIdx.x == 0) write_header(out, n, cs, n_chunks, lut, tid);
+  uint16_t* chunk_bits = reinterpret_cast<uint16_t*>(out + kIndexOff + 8 * n_groups_of(n_chunks));
+  for (uint64_t c = (uint64_t)blockIdx.x * kEncWarps + warp; c < n_chunks; c += (uint64_t)gridDim.x * kEncWarps) {
+    const uint64_t beg = c * cs;
+    const uint32_t bits = chunk_length(&s_enc[lane], in + beg, (uint32_t)min((uint64_t)cs, n - beg), lane);
+    if (lane == 0) chunk_bits[c] = (uint16_t)bits;
+  }
+}
+
+constexpr uint32_t kParts = kGroupChunks / kEncWarps;  // parts per group
+
+__global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm)
+pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __restrict__ lut, uint32_t cs, uint8_t* out,
+            uint64_t out_cap, unsigned long long* out_bytes, uint32_t* status) {
+  __shared__ __align__(16) uint32_t s_enc[256 * 32];
+  __shared__ __align__(16) uint32_t s_stage[kEncWarps][2][kWStage];
+  __shared__ Seams s_seam;
+  __shared__ unsigned long long s_sum[kEncWarps];
+  __shared__ uint32_t s_more[4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t e = table_entry(lut->enc[tid]);
+  stage_entry(s_enc, tid, e);
+  for (int i = tid; i < kEncWarps * 2 * kWStage; i += kEncThreads) (&s_stage[0][0][0])[i] = 0;
+  if (__syncthreads_or(e == 0)) return;  // lengths_kernel has set the status
+  const uint32_t* tab = &s_enc[lane];
+  const uint32_t n_chunks = (uint32_t)((n + cs - 1) / cs);  // <= kPartMaxChunks
+  const uint32_t n_groups = (uint32_t)n_groups_of(n_chunks);
+  const uint64_t P = payload_start(n_chunks);
+  unsigned long long* group_off = reinterpret_cast<unsigned long long*>(out + kIndexOff);
+  const uint16_t* chunk_bits = reinterpret_cast<const uint16_t*>(out + kIndexOff + 8 * (uint64_t)n_groups);
+  unsigned long long excl = 0;  // payload offset of group g_at
+  uint32_t g_at = 0;
+  for (uint32_t item = blockIdx.x; item < n_groups * kParts; item += gridDim.x) {
+    const uint32_t g = item / kParts, first = (item % kParts) * kEncWarps;  // the part's first chunk in the group
+    // the sizes of groups g_at .. g - 1 (all of 32 chunks): 8 lanes per group, 4 chunks each
+    unsigned long long sum = 0;
+    for (uint32_t b = 8 * g_at + 32 * warp; b < 8 * g; b += 32 * kEncWarps) {
+      uint32_t bits = 0;
+      if (b + lane < 8 * g) {
+        const uint2 q = *reinterpret_cast<const uint2*>(chunk_bits + 4 * (b + lane));
+        bits = (q.x & 0xFFFFu) + (q.x >> 16) + (q.y & 0xFFFFu) + (q.y >> 16);
+      }
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) bits += __shfl_xor_sync(0xffffffffu, bits, o);
+      if ((lane & 7) == 0) sum += align16((bits + 7) / 8);
+    }
+    sum = warp_sum_u64(sum);
+    // the group's chunks: bit offsets, in every warp
+    const uint32_t cg = g * kGroupChunks + lane;
+    const uint32_t cb = cg < n_chunks ? chunk_bits[cg] : 0u;
+    uint32_t incl = cb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const uint32_t gbits = __shfl_sync(0xffffffffu, incl, 31);
+    __syncthreads();  // the previous part's seams and sums are done with
+    if (lane == 0) s_sum[warp] = sum;
+    if (warp == 0) s_seam.idx[lane][0] = s_seam.idx[lane][1] = ~0u;
+    if (tid < 4) s_more[tid] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kEncWarps; w++) excl += s_sum[w];
+    g_at = g;
+    if (first == 0 && tid == 0) {
+      const unsigned long long gbytes = align16((gbits + 7) / 8);
+      if (QLC_GUARD(g < n_groups, status)) group_off[g] = excl;
+      if (g == n_groups - 1) {
+        *reinterpret_cast<unsigned long long*>(out + 48) = excl + gbytes;
+        *out_bytes = P + excl + gbytes;
       }
     }
+    uint4* dst = reinterpret_cast<uint4*>(out + P + excl);
+    const uint32_t blk_lim = (uint32_t)min((uint64_t)((out_cap - P - excl) / 16), (uint64_t)0xFFFFFFFEu);
+    const uint64_t gbeg = (uint64_t)g * kGroupChunks * cs;
+    const uint64_t gend = min(gbeg + (uint64_t)kGroupChunks * cs, n);
+    const uint32_t c = first + warp;
+    const uint32_t E = __shfl_sync(0xffffffffu, incl, c), S = E - __shfl_sync(0xffffffffu, cb, c);
+    const uint64_t cbeg = gbeg + (uint64_t)c * cs;
+    if (cbeg < gend) {
+      pack_chunk(tab, &s_stage[warp][0][0], (uint32_t)__cvta_generic_to_shared(&s_stage[warp][0][0]), in + cbeg,
+                 (uint32_t)min((uint64_t)cs, gend - cbeg), S, E, dst, blk_lim, s_seam, c, lane);
+      // a tensor's last chunk may lie within one block: the part before has it
+      if (c == first && (S & 127u) && (S >> 7) == (E >> 7) && lane == 0) s_seam.idx[c][1] = ~0u;
+    }
+    // the symbols after the part that fall in its last block, two per lane
+    const uint64_t after = gbeg + (uint64_t)(first + kEncWarps) * cs;
+    const uint32_t end = __shfl_sync(0xffffffffu, incl, first + kEncWarps - 1);
+    const bool shared_end = (end & 127u) != 0 && after < gend;
+    if (warp == 0 && shared_end) {
+      const uint64_t i = after + 2 * lane;
+      const uint32_t e0 = i < gend ? enc_entry(tab, in[i]) : 0u, e1 = i + 1 < gend ? enc_entry(tab, in[i + 1]) : 0u;
+      const uint32_t l0 = e0 & 31u, len = l0 + (e1 & 31u);
+      uint32_t pos = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, pos, o);
+        if (lane >= o) pos += t;
+      }
+      pos += (end & 127u) - len;
+      auto put = [&](uint32_t code, uint32_t at) {  // an MSB-aligned codeword at bit `at` of the block
+        if (at < 128) atomicOr(&s_more[at >> 5], code >> (at & 31u));
+        if (at < 96 && (at & 31u)) atomicOr(&s_more[(at >> 5) + 1], code << (32u - (at & 31u)));
+      };
+      put(e0 & ~31u, pos);
+      put(e1 & ~31u, pos + l0);
+    }
+    __syncthreads();
+    if (warp == 0)
+      merge_seams(s_seam, dst, blk_lim, shared_end ? end >> 7 : ~0u,
+                  make_uint4(bswap32(s_more[0]), bswap32(s_more[1]), bswap32(s_more[2]), bswap32(s_more[3])), status, lane);
   }
 }
 
@@ -619,6 +796,15 @@ qlc_status qlc_encode(const uint8_t* d_in, size_t n, const qlc_lut* d_lut, uint3
   }
   const size_t ws_need = qlc_encode_workspace_size(n, chunk_symbols);
   if (ws_bytes < ws_need) return QLC_ERR_CAPACITY;
+  if (n_chunks <= kPartMaxChunks) {
+    const int sms = sm_count(), parts = (int)(n_groups_of(n_chunks) * kParts);
+    const int want = (int)((n_chunks + kEncWarps - 1) / kEncWarps);
+    lengths_kernel<<<want < 6 * sms ? want : 6 * sms, kEncThreads, 0, st>>>(d_in, n, d_lut, chunk_symbols, d_out,
+                                                                            d_status);
+    pack_kernel<<<parts < kEncCtasPerSm * sms ? parts : kEncCtasPerSm * sms, kEncThreads, 0, st>>>(
+        d_in, n, d_lut, chunk_symbols, d_out, out_cap, reinterpret_cast<unsigned long long*>(d_out_bytes), d_status);
+    return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  }
   if (cudaMemsetAsync(d_ws, 0, ws_need, st) != cudaSuccess) return QLC_ERR_CUDA;
   EncArgs A = {};
   A.in = d_in;
