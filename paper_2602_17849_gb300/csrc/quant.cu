@@ -42,35 +42,44 @@ __device__ __forceinline__ uint32_t e4m3_rne(float v) {
   return min(code, 0x7Fu) | ((u >> 24) & 0x80u);
 }
 
-// Codes of two products q = x * y, y within 2 ulp of 1 / scale, from the
-// hardware conversion to e4m3 (round to nearest even).  Below 448 its grid is
-// this format's grid (subnormals m 2^-9, normals (1 + m/8) 2^(e-7), sign bit
-// 7), so the codes agree there; it saturates at 448 (0x7E), and this format
-// goes on to 480 (0x7F), the code of every magnitude above the midpoint 464.
-// The rule rounds the quotient x / scale once; q is within 2^-21.6 |q| of it
-// (y's error and the product's rounding).  Each value is converted twice,
-// moved up and down by 2^-20 of itself, which brackets the quotient: both
-// codes equal (the code is monotone in the value) means the quotient has
-// that code too.  Above 464 the code's low bit is set by a flag computed on
-// the FMA pipe: (|v| - 464) 2^20 clamped to [0, 1] is 1.0 above 464 (the
-// fp32 neighbours of 464 are 2^-15 away) and 0.0 up to it, and
-// f0 + 256 f1 + 2^23 holds the two flags in its low bits, one per byte.
-// Gives both sides' codes (qa | qb << 8): where a byte differs the caller
-// takes the exact division for that element.
+// x / scale rounded to nearest, from y = 1 / scale rounded to nearest: the
+// product q0 = x y and one correction by its fused-multiply-add residual
+// (Markstein's correction step).  It equals the fp32 division for every scale
+// mantissa with every x whose quotient lies within three floats of a value or
+// a rounding midpoint of the format (checked exhaustively on the host with
+// IEEE fmaf), and elsewhere lies on the same side of every midpoint; so the
+// code taken from it is the rule's.  Scales from 2^-80 on: below, the residual
+// of an element that matters could be subnormal.  The residual is formed as
+// q0 scale - x and multiplied by -y, which keeps -0.
+// Three FMA-pipe operations per element (bf16, 61 Mi elements with the
+// histogram: 38 us; fp32, 256 Mi: 220 us) replaced a bracket (two conversions of
+// the product moved up and down by 2^-20, an exact division where they
+// differed): bf16 elements, whose quotients often lie on midpoints, sent
+// nearly every warp step to that division (59 us; fp32 234 us).
+__device__ __forceinline__ float quotient(float x, float scale, float y) {
+  const float q0 = x * y;
+  return fmaf(fmaf(q0, scale, -x), -y, q0);
+}
+// Codes of four quotients, the first lowest, from the hardware conversion to
+// e4m3 (round to nearest even).  Below 448 its grid is this format's grid
+// (subnormals m 2^-9, normals (1 + m/8) 2^(e-7), sign bit 7), so the codes
+// agree there; it saturates at 448 (0x7E), and this format goes on to 480
+// (0x7F), the code of every magnitude above the midpoint 464.  So the code's
+// low bit is set by a flag computed on the FMA pipe: (|v| - 464) 2^20 clamped
+// to [0, 1] is 1.0 above 464 (the fp32 neighbours of 464 are 2^-15 away) and
+// 0.0 up to it, and f0 + 256 f1 + 2^23 holds two flags in its low bits, one
+// per byte.
 __device__ __forceinline__ uint32_t sat_flags(float a, float b) {
   const float fa = __saturatef(fmaf(fabsf(a), 0x1p20f, -464.0f * 0x1p20f));
   const float fb = __saturatef(fmaf(fabsf(b), 0x1p20f, -464.0f * 0x1p20f));
   return __float_as_uint(fmaf(fb, 256.0f, fa + 0x1p23f));
 }
-__device__ __forceinline__ void e4m3x2_bracket(float qa, float qb, uint32_t* up, uint32_t* lo) {
-  constexpr float d = 0x1p-20f;
-  const float ua = fmaf(qa, d, qa), ub = fmaf(qb, d, qb);  // the larger magnitudes
-  const float la = fmaf(qa, -d, qa), lb = fmaf(qb, -d, qb);
-  uint16_t cu, cl;
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(cu) : "f"(ub), "f"(ua));
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(cl) : "f"(lb), "f"(la));
-  *up = (uint32_t)cu | (sat_flags(ua, ub) & 0x0101u);  // 0x7E -> 0x7F above 464
-  *lo = (uint32_t)cl | (sat_flags(la, lb) & 0x0101u);
+__device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
+  uint16_t lo, hi;
+  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(lo) : "f"(b), "f"(a));
+  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(hi) : "f"(d), "f"(c));
+  const uint32_t flags = __byte_perm(sat_flags(a, b), sat_flags(c, d), 0x5410) & 0x01010101u;
+  return __byte_perm(lo, hi, 0x5410) | flags;  // 0x7E -> 0x7F above 464
 }
 
 // amax / 480 rounded to nearest.  For amax in [2^-100, FLT_MAX] a product
@@ -158,36 +167,17 @@ __device__ __forceinline__ float lane_codes(const float (&v)[E], uint32_t (&w)[E
 #pragma unroll
   for (int o = 1; o < kLanesPerBlock; o <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   const float scale = scale_of(amax);
-  // one reciprocal per lane and block, within 2 ulp for scale in
-  // [2^-126, 2^126]; a scale below 2^-125 takes the exact division for
-  // every element
-  const float y = __fdividef(1.0f, scale);
-  // dw: nonzero bytes mark the elements whose code the bracket leaves open
-  // (all of them for a scale below 2^-125)
-  uint32_t dw[kWords], open = 0u;
-  const uint32_t all = scale >= 0x1p-125f ? 0u : ~0u;
+  const float y = __frcp_rn(scale);
 #pragma unroll
-  for (int t = 0; t < kWords; t++) {
-    uint32_t u0, l0, u1, l1;
-    e4m3x2_bracket(v[4 * t] * y, v[4 * t + 1] * y, &u0, &l0);
-    e4m3x2_bracket(v[4 * t + 2] * y, v[4 * t + 3] * y, &u1, &l1);
-    w[t] = __byte_perm(u0, u1, 0x5410);
-    dw[t] = (w[t] ^ __byte_perm(l0, l1, 0x5410)) | all;
-    open |= dw[t];
-  }
-  if (!(scale > 0.0f)) {
-#pragma unroll
-    for (int t = 0; t < kWords; t++) w[t] = 0u;
-  } else if (open != 0u) {  // rare: the open elements alone take the exact division
+  for (int t = 0; t < kWords; t++)
+    w[t] = e4m3x4(quotient(v[4 * t], scale, y), quotient(v[4 * t + 1], scale, y), quotient(v[4 * t + 2], scale, y),
+                  quotient(v[4 * t + 3], scale, y));
+  if (!(scale >= 0x1p-80f)) {  // rare: exact division, or codes 0x00 for a scale of 0
 #pragma unroll
     for (int t = 0; t < kWords; t++) {
-      while (dw[t] != 0u) {
-        const uint32_t sh = (uint32_t)(__ffs(dw[t]) - 1) & ~7u;  // bit 0 of the byte
-        const uint32_t jb = sh >> 3;
-        const float vj = jb == 0 ? v[4 * t] : jb == 1 ? v[4 * t + 1] : jb == 2 ? v[4 * t + 2] : v[4 * t + 3];
-        w[t] = (w[t] & ~(0xFFu << sh)) | (e4m3_rne(vj / scale) << sh);
-        dw[t] &= ~(0xFFu << sh);
-      }
+      w[t] = 0u;
+      if (scale > 0.0f)
+        for (int j = 0; j < 4; j++) w[t] |= e4m3_rne(v[4 * t + j] / scale) << (8 * j);
     }
   }
   return scale;
