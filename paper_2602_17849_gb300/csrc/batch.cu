@@ -25,91 +25,6 @@ __device__ __forceinline__ bool al16(const void* p) {
   return (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
 }
 
-// Work items of one shard; 0 (and a status) for a shard that cannot be run.
-__device__ uint64_t item_count(int kind, const qlc_desc& d, uint32_t cs, uint32_t* status) {
-  if (kind == kPlanEncode) {
-    const uint64_t n = d.in_bytes;
-    const uint64_t n_chunks = (n + cs - 1) / cs;
-    if (!d.out || !d.lut || !al16(d.out) || !al16(d.lut) || !aligned(d.out_bytes, 8) ||
-        (n > 0 && (!d.in || !al16(d.in))) || n_chunks > 0xFFFFFFFFull) {
-      set_status(status, QLC_ERR_ARG);
-      return 0;
-    }
-    if (d.out_cap < encoded_bound(n, cs)) {
-      set_status(status, QLC_ERR_CAPACITY);
-      return 0;
-    }
-    return n == 0 ? 1 : n_groups_of(n_chunks);
-  }
-  // decode: the container's groups, from a header that at least parses
-  if (!d.in || !al16(d.in) || !aligned(d.out_bytes, 8) || (d.out_cap > 0 && (!d.out || !al16(d.out)))) {
-    set_status(status, QLC_ERR_ARG);
-    return 0;
-  }
-  const uint8_t* c = static_cast<const uint8_t*>(d.in);
-  if (d.in_bytes < kIndexOff || *reinterpret_cast<const uint32_t*>(c) != 0x31434C51u) {
-    set_status(status, QLC_ERR_CORRUPT);
-    return 0;
-  }
-  const uint64_t groups = n_groups_of(*reinterpret_cast<const uint32_t*>(c + 20));
-  if (groups > d.in_bytes / 16) {  // every group takes at least 16 payload bytes
-    set_status(status, QLC_ERR_CORRUPT);
-    return 0;
-  }
-  return groups ? groups : 1;  // an empty container still gets its header checked
-}
-
-__global__ void __launch_bounds__(kPlanThreads)
-plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w, uint32_t* status) {
-  __shared__ unsigned long long s_warp[kPlanThreads / 32];
-  __shared__ unsigned long long s_carry;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < 16) w.ticket[tid] = 0;  // the 64 bytes of counters
-  if (tid == 0) s_carry = 0;
-  __syncthreads();
-  for (int base = 0; base < n_shards; base += kPlanThreads) {
-    const int s = base + tid;
-    const unsigned long long cnt = s < n_shards ? item_count(kind, descs[s], cs, status) : 0ull;
-    unsigned long long incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    unsigned long long wpre = 0, total = 0;
-    for (int i = 0; i < kPlanThreads / 32; i++) {
-      wpre += i < warp ? s_warp[i] : 0ull;
-      total += s_warp[i];
-    }
-    if (s < n_shards) w.item_base[s] = s_carry + wpre + incl - cnt;
-    __syncthreads();
-    if (tid == 0) s_carry += total;
-    __syncthreads();
-  }
-  unsigned long long total = s_carry;
-  if (kind == kPlanEncode && total > w.gstat_cap) {
-    if (tid == 0) set_status(status, QLC_ERR_CAPACITY);
-    total = 0;
-  }
-  if (tid == 0) w.item_base[n_shards] = total;
-  if (kind == kPlanEncode)
-    for (unsigned long long i = tid; i < total; i += kPlanThreads) w.gstat[i] = 0;
-}
-
-// ------------------------------------------------------------- histograms
-
-// Histogram work items of shard s: its 64 KiB pieces, and one more without
-// bytes that stands for the flush after it (about as long as a piece), so that
-// a run of small shards is not all one CTA's.  0 for a shard that is empty or
-// cannot be read (its encode reports it: histograms have no status word).
-__device__ __forceinline__ unsigned long long hist_items(const qlc_desc* descs, int n_shards, int s) {
-  if (s >= n_shards) return 0;
-  const qlc_desc* d = descs + s;
-  return d->in && al16(d->in) && d->in_bytes ? (d->in_bytes + kHistItem - 1) / kHistItem + 1 : 0;
-}
-
 // Inclusive prefix sums of the CTA's kHcThreads values v (thread t's at
 // s_incl[t]); returns their total.  Called by every thread; s_warp holds a
 // value per warp.
@@ -134,6 +49,108 @@ __device__ __forceinline__ unsigned long long cta_scan(unsigned long long v, uns
   const unsigned long long total = __shfl_sync(0xffffffffu, w, 31);
   __syncthreads();
   return total;
+}
+
+// A shard's work: its groups (a shard that cannot be run has none and sets a
+// status), and for decoding its symbols and the spans per group (0: the items
+// are the groups in any case).
+struct ShardWork {
+  uint64_t groups, symbols;
+  uint32_t per_group;
+};
+__device__ ShardWork shard_work(int kind, const qlc_desc& d, uint32_t cs, uint32_t* status) {
+  ShardWork w = {0, 0, 0};
+  if (kind == kPlanEncode) {
+    const uint64_t n = d.in_bytes;
+    const uint64_t n_chunks = (n + cs - 1) / cs;
+    if (!d.out || !d.lut || !al16(d.out) || !al16(d.lut) || !aligned(d.out_bytes, 8) ||
+        (n > 0 && (!d.in || !al16(d.in))) || n_chunks > 0xFFFFFFFFull) {
+      set_status(status, QLC_ERR_ARG);
+    } else if (d.out_cap < encoded_bound(n, cs)) {
+      set_status(status, QLC_ERR_CAPACITY);
+    } else {
+      w.groups = n == 0 ? 1 : n_groups_of(n_chunks);
+    }
+    return w;
+  }
+  // decode: the container's groups, from a header that at least parses
+  if (!d.in || !al16(d.in) || !aligned(d.out_bytes, 8) || (d.out_cap > 0 && (!d.out || !al16(d.out)))) {
+    set_status(status, QLC_ERR_ARG);
+    return w;
+  }
+  if (d.in_bytes < kIndexOff) {
+    set_status(status, QLC_ERR_CORRUPT);
+    return w;
+  }
+  const uint4 h0 = *static_cast<const uint4*>(d.in);                    // magic .. n
+  const uint2 h1 = *reinterpret_cast<const uint2*>(static_cast<const uint8_t*>(d.in) + 16);  // chunk_symbols, n_chunks
+  const uint64_t groups = n_groups_of(h1.y);
+  if (h0.x != 0x31434C51u || groups > d.in_bytes / 16) {  // every group takes at least 16 payload bytes
+    set_status(status, QLC_ERR_CORRUPT);
+    return w;
+  }
+  w.groups = groups ? groups : 1;  // an empty container still gets its header checked
+  w.symbols = min((uint64_t)h0.z | (uint64_t)h0.w << 32, (uint64_t)d.out_cap);
+  if (groups && chunk_symbols_ok(h1.x)) w.per_group = SpanShape(h1.x).per_group;  // the decoder refuses another chunk size
+  return w;
+}
+
+__global__ void __launch_bounds__(kPlanThreads)
+plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w, uint32_t* status) {
+  static_assert(kPlanThreads == kHcThreads, "cta_scan");
+  __shared__ unsigned long long s_incl[kPlanThreads], s_warp[kPlanThreads / 32];
+  const int tid = threadIdx.x;
+  dependents_may_start();
+  // every thread keeps its shards' groups and spans per group in item_base
+  // until the number of symbols has settled which of them are the items
+  unsigned long long symbols = 0;
+  for (int s = tid; s < n_shards; s += kPlanThreads) {
+    const ShardWork sw = shard_work(kind, descs[s], cs, status);
+    symbols += sw.symbols;
+    w.item_base[s] = sw.groups | (unsigned long long)sw.per_group << 40;
+  }
+  bool split = false;
+  if (kind == kPlanDecode) {
+    split = cta_scan(symbols, s_incl, s_warp, tid) <= kSplitMax;
+  }
+  if (tid < 16) w.ticket[tid] = 0;  // the 64 bytes of counters
+  unsigned long long total = 0;
+  for (int base = 0; base < n_shards; base += kPlanThreads) {
+    const int s = base + tid;
+    unsigned long long cnt = 0;
+    if (s < n_shards) {
+      const unsigned long long v = w.item_base[s];
+      const uint32_t per_group = (uint32_t)(v >> 40);
+      cnt = v & ((1ull << 40) - 1);
+      if (split && per_group) cnt = (cnt * per_group + kSpanWarps - 1) / kSpanWarps;
+    }
+    const unsigned long long part = cta_scan(cnt, s_incl, s_warp, tid);
+    if (s < n_shards) w.item_base[s] = total + s_incl[tid] - cnt;
+    total += part;
+  }
+  if (kind == kPlanEncode && total > w.gstat_cap) {
+    if (tid == 0) set_status(status, QLC_ERR_CAPACITY);
+    total = 0;
+  }
+  if (tid == 0) {
+    w.item_base[n_shards] = total;
+    if (kind == kPlanDecode)
+      w.ticket[kTicketWay] = split ? kWaySplit : total <= (unsigned long long)kFewWarpsPerSm * cs ? kWayEven : kWayGroups;
+  }
+  if (kind == kPlanEncode)
+    for (unsigned long long i = tid; i < total; i += kPlanThreads) w.gstat[i] = 0;
+}
+
+// ------------------------------------------------------------- histograms
+
+// Histogram work items of shard s: its 64 KiB pieces, and one more without
+// bytes that stands for the flush after it (about as long as a piece), so that
+// a run of small shards is not all one CTA's.  0 for a shard that is empty or
+// cannot be read (its encode reports it: histograms have no status word).
+__device__ __forceinline__ unsigned long long hist_items(const qlc_desc* descs, int n_shards, int s) {
+  if (s >= n_shards) return 0;
+  const qlc_desc* d = descs + s;
+  return d->in && al16(d->in) && d->in_bytes ? (d->in_bytes + kHistItem - 1) / kHistItem + 1 : 0;
 }
 
 // Each CTA (32 warps, hist_cols.cuh; one per SM) takes a contiguous run of

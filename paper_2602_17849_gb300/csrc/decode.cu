@@ -20,6 +20,8 @@
 // of its use so that no memory access lies on the round-to-round chain.
 // Output: each lane writes its 32 symbols of a block with one 32-byte
 // streaming store.
+#include <atomic>
+
 #define QLC_FILE_ID 1
 #include "decode_common.cuh"
 #include "decode_span.cuh"
@@ -48,7 +50,7 @@ struct LaneShared {
   uint32_t col[kColRows][32];  // word k of lane l at col[k % 16][l]
   uint4 stage[kStageVec][32];  // vector v of lane l at stage[v % 8][l]
 };
-// ... of a CTA of one such warp: with its code table and header.
+// ... and of a CTA of one such warp: with its code table and header.
 struct DecShared {
   LaneShared lanes;
   uint8_t T[2048];                // code -> symbol
@@ -365,7 +367,8 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
     decode_group<kOut>(h, in, out, scales, g, sm.lanes, sm.T, d, status, lane, aligned32, sc_vec);
 }
 
-// Shared memory of a split-decoding CTA; its warps decode spans, or groups.
+// Shared memory of a CTA of kSpanWarps warps that decode spans, or groups, of
+// one container.
 struct SpanShared {
   union {
     SpanWarp span;
@@ -428,13 +431,44 @@ decode_span_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __re
   }
 }
 
-// A batch: warps take (shard, group) items from a device counter; a warp
-// re-reads the header and rebuilds its table when its shard changes.
+// ---------------------------------------------------------------- batches
+//
+// Three ways, by the batch's size (plan_kernel decides, on the device): split
+// up to kSplitMax symbols; a lane per chunk with the first items dealt out
+// evenly while there are no more groups than warps; and, above, a lane per
+// chunk with all items from a counter.
+
+// The shard an item belongs to changed: reads its header and builds its table.
+// Reports a bad one and returns its status.
+__device__ __forceinline__ uint32_t enter_shard(const qlc_desc& dd, DecHeader* h, uint8_t* hdr, uint8_t* T,
+                                                uint32_t* seen, uint32_t* status, int lane) {
+  __syncwarp();  // every lane is done with the previous shard's header
+  load_header(static_cast<const uint8_t*>(dd.in), dd.in_bytes, hdr, lane, 32);
+  __syncwarp();
+  const uint32_t err = parse_header(hdr, dd.in_bytes, dd.out_cap, h, seen, lane);
+  if (err) {
+    if (lane == 0) {
+      if (err == QLC_ERR_CAPACITY && dd.out_bytes) *dd.out_bytes = h->n;
+      set_status(status, err);
+    }
+    return err;
+  }
+  build_table(hdr, T, lane, 32);
+  __syncwarp();
+  return 0;
+}
+
+// Many groups: warps take (shard, group) items from a device counter.  A CTA is
+// one warp, so that the table's address is a constant (an add less for every
+// lookup than with several tables per CTA: 1152 shards 1764 us, not 1790-1830).
 __global__ void __launch_bounds__(32, kDecCtasPerSm)
 decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
                     const unsigned long long* __restrict__ item_base, unsigned int* __restrict__ ticket,
                     uint32_t* __restrict__ status) {
   __shared__ DecShared sm;
+  __shared__ void* volatile s_out;  // the current item's output
+  dependency_wait();
+  if (ticket[kTicketWay] != kWayGroups) return;
   const int lane = threadIdx.x;
   LaneDec d;
   if (!lane_init(sm.lanes, d, lane)) {
@@ -444,7 +478,6 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
   const unsigned long long total = item_base[n_shards];
   int cur = -1, bad = -1;
   DecHeader h;
-  __shared__ void* volatile s_out;  // the current item's output
   while (true) {
     unsigned long long t = 0;
     if (lane == 0) t = atomicAdd(ticket, 1u);
@@ -453,24 +486,13 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
     const int sh = shard_of_warp(item_base, n_shards, t, lane);
     if (sh == bad) continue;
     const qlc_desc dd = descs[sh];
-    const uint8_t* in = static_cast<const uint8_t*>(dd.in);
     const uint64_t g = t - item_base[sh];
     if (sh != cur) {
-      __syncwarp();  // every lane is done with the previous shard's header
-      load_header(in, dd.in_bytes, sm.hdr, lane, 32);
-      __syncwarp();
-      const uint32_t err = parse_header(sm.hdr, dd.in_bytes, dd.out_cap, &h, sm.seen, lane);
-      if (err) {
-        if (lane == 0) {
-          if (err == QLC_ERR_CAPACITY && dd.out_bytes) *dd.out_bytes = h.n;
-          set_status(status, err);
-        }
+      if (enter_shard(dd, &h, sm.hdr, sm.T, sm.seen, status, lane)) {
         bad = sh;
         cur = -1;
         continue;
       }
-      build_table(sm.hdr, sm.T, lane, 32);
-      __syncwarp();
       cur = sh;
     }
     if (g == 0 && lane == 0 && dd.out_bytes) *dd.out_bytes = h.n;
@@ -479,7 +501,112 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
     if (lane == 0) s_out = dd.out;
     __syncwarp();
     if (g < h.n_groups)
-      decode_group<kOutCodes>(h, in, nullptr, nullptr, g, sm.lanes, sm.T, d, status, lane, aligned32, false, &s_out);
+      decode_group<kOutCodes>(h, static_cast<const uint8_t*>(dd.in), nullptr, nullptr, g, sm.lanes, sm.T, d, status, lane,
+                              aligned32, false, &s_out);
+  }
+}
+
+// The barrier of a team of kSpanWarps warps within its CTA.
+__device__ __forceinline__ void team_sync(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(32 * kSpanWarps) : "memory");
+}
+
+// Few groups: one CTA per SM, of kSpanCtasPerSm teams of kSpanWarps warps.
+struct FewShared {
+  union {
+    SpanShared span[kSpanCtasPerSm];                // a team's
+    DecShared own[kSpanWarps * kSpanCtasPerSm];     // a warp's
+  };
+};
+constexpr int kFewWarps = kSpanWarps * kSpanCtasPerSm;
+static_assert(kFewWarps == kFewWarpsPerSm, "plan_kernel compares the groups with these warps");
+__global__ void __launch_bounds__(32 * kFewWarps, 1)
+decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsigned long long* __restrict__ item_base,
+                  unsigned int* __restrict__ ticket, uint32_t* __restrict__ status) {
+  extern __shared__ __align__(16) uint8_t few_sm[];
+  __shared__ void* volatile s_out[kFewWarps];  // the warps' current outputs
+  __shared__ volatile unsigned long long s_item[kSpanCtasPerSm];
+  FewShared& all = *reinterpret_cast<FewShared*>(few_sm);
+  dependents_may_start();
+  dependency_wait();
+  const uint32_t way = ticket[kTicketWay];
+  if (way == kWayGroups) return;
+  const int lane = threadIdx.x % 32;
+  const int wid = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0);  // so known to be the same in all lanes
+  const unsigned long long total = item_base[n_shards];
+  DecHeader h;
+  if (way == kWayEven) {
+    // A group for every warp at most: item t goes to warp t / SMs of SM t mod
+    // SMs, so every SM, and every quarter of an SM, has the same number, give
+    // or take one.  From the counter, the CTAs that an SM got first took items
+    // that others lacked: 24 shards of 4 KiB - 64 MiB (1814 groups) 256 us,
+    // now 165.
+    const unsigned long long t = (unsigned long long)wid * gridDim.x + blockIdx.x;
+    if (t >= total) return;
+    DecShared& sm = all.own[wid];
+    LaneDec d;
+    if (!lane_init(sm.lanes, d, lane)) {
+      if (lane == 0) set_status(status, QLC_ERR_CUDA);
+      return;
+    }
+    const int sh = shard_of_warp(item_base, n_shards, t, lane);
+    const qlc_desc dd = descs[sh];
+    const uint64_t g = t - item_base[sh];
+    if (enter_shard(dd, &h, sm.hdr, sm.T, sm.seen, status, lane)) return;
+    if (g == 0 && lane == 0 && dd.out_bytes) *dd.out_bytes = h.n;
+    if (lane == 0) s_out[wid] = dd.out;
+    __syncwarp();
+    if (g < h.n_groups)
+      decode_group<kOutCodes>(h, static_cast<const uint8_t*>(dd.in), nullptr, nullptr, g, sm.lanes, sm.T, d, status, lane,
+                              (reinterpret_cast<uintptr_t>(dd.out) & 31u) == 0, false, &s_out[wid]);
+    return;
+  }
+  // Split: items are kSpanWarps spans of one shard, which a team decodes with a
+  // table that its warps share.
+  const int team = wid / kSpanWarps, warp = wid % kSpanWarps, tid = 32 * warp + lane;
+  SpanShared& sm = all.span[team];
+  int cur = -1;
+  uint32_t err = 0;
+  for (unsigned long long t = (unsigned long long)team * gridDim.x + blockIdx.x; t < total;) {
+    const int sh = shard_of_warp(item_base, n_shards, t, lane);  // the same in every warp of the team
+    const qlc_desc dd = descs[sh];
+    const uint8_t* in = static_cast<const uint8_t*>(dd.in);
+    const uint32_t q = (uint32_t)(t - item_base[sh]);
+    if (sh != cur) {
+      load_header(in, dd.in_bytes, sm.hdr, tid, 32 * kSpanWarps);
+      team_sync(team);
+      err = parse_header(sm.hdr, dd.in_bytes, dd.out_cap, &h, sm.seen[warp], lane);
+      if (!err) build_table(sm.hdr, sm.T, tid, 32 * kSpanWarps);
+      team_sync(team);
+      cur = sh;
+    }
+    if (q == 0 && tid == 0) {
+      if ((!err || err == QLC_ERR_CAPACITY) && dd.out_bytes) *dd.out_bytes = h.n;
+      if (err) set_status(status, err);
+    }
+    if (!err) {
+      const uint64_t s = (uint64_t)q * kSpanWarps + warp;
+      if (split_pays(h, h.n)) {
+        const SpanShape shape(h.cs);
+        const uint32_t k = (uint32_t)lane / shape.lanes, seg = (uint32_t)lane - k * shape.lanes;
+        const uint64_t g = s / shape.per_group;
+        const uint32_t r = (uint32_t)(s - g * shape.per_group);
+        if (g < h.n_groups)
+          decode_span<kOutCodes>(h, shape, in, dd.out, nullptr, g, r * shape.chunks, k, seg, sm.w[warp].span, sm.T,
+                                 warm_bits(h.len_lo, h.len_hi), status, lane);
+      } else if (s < h.n_groups) {  // a shard has at least as many spans as groups
+        LaneDec d;
+        if (lane_init(sm.w[warp].lanes, d, lane))
+          decode_group<kOutCodes>(h, in, dd.out, nullptr, s, sm.w[warp].lanes, sm.T, d, status, lane,
+                                  (reinterpret_cast<uintptr_t>(dd.out) & 31u) == 0);
+        else if (lane == 0)
+          set_status(status, QLC_ERR_CUDA);
+      }
+    }
+    if (tid == 0) s_item[team] = kSpanCtasPerSm * gridDim.x + (unsigned long long)atomicAdd(ticket, 1u);
+    team_sync(team);  // ... and every warp is done with the header and the table
+    t = s_item[team];
+    team_sync(team);
   }
 }
 
@@ -550,6 +677,20 @@ extern "C" qlc_status qlc_decode_dequantize(const uint8_t* d_in, size_t in_bytes
   return launch_decode<QLC_DTYPE_BF16>(d_in, in_bytes, d_out, d_scales, out_cap, d_n_out, d_status, st);
 }
 
+// Raises decode_few_kernel's shared-memory limit, once per device (a function
+// attribute, allowed inside stream capture).
+static bool decode_few_smem_ok() {
+  static std::atomic<bool> done[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
+  if (dev < 64 && done[dev].load(std::memory_order_relaxed)) return true;
+  if (cudaFuncSetAttribute(decode_few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FewShared)) !=
+      cudaSuccess)
+    return false;
+  if (dev < 64) done[dev].store(true, std::memory_order_relaxed);
+  return true;
+}
+
 extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, void* d_ws, size_t ws_bytes,
                                        uint32_t* d_status, const qlc_launch* h_launch, qlc_stream_t stream) {
   NvtxRange nvtx_range("qlc_decode_batch");
@@ -558,12 +699,17 @@ extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, vo
   BatchWs w;
   if (!batch_ws_layout(d_ws, ws_bytes, n_shards, &w)) return QLC_ERR_CAPACITY;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  plan_kernel<<<1, kPlanThreads, 0, st>>>(kPlanDecode, d_descs, n_shards, 0, w, d_status);
+  plan_kernel<<<1, kPlanThreads, 0, st>>>(kPlanDecode, d_descs, n_shards, (uint32_t)sm_count(), w, d_status);
   if (cudaGetLastError() != cudaSuccess) return QLC_ERR_CUDA;
   int per_sm = kDecCtasPerSm;
   if (h_launch && h_launch->decode_ctas_per_sm > 0 && h_launch->decode_ctas_per_sm < kDecCtasPerSm)
     per_sm = h_launch->decode_ctas_per_sm;
-  decode_batch_kernel<<<sm_count() * per_sm, 32, 0, st>>>(d_descs, n_shards, w.item_base, w.ticket, d_status);
+  if (!decode_few_smem_ok()) return QLC_ERR_CUDA;
+  // which of the two has the work is decided on the device; the other returns at once
+  const int sms = sm_count();
+  launch_after(decode_few_kernel, sms, 32 * kFewWarps, sizeof(FewShared), st, d_descs, n_shards, w.item_base, w.ticket,
+               d_status);
+  launch_after(decode_batch_kernel, sms * per_sm, 32, 0, st, d_descs, n_shards, w.item_base, w.ticket, d_status);
   return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
 }
 

@@ -32,9 +32,7 @@
 
 namespace qlc {
 
-constexpr int kSpanWarps = 4;                         // warps per CTA; they share the code table
 constexpr int kSpanCtasPerSm = 5;                     // resident: bounded by shared memory
-constexpr uint32_t kPiece = 128;                      // symbols per lane, about
 constexpr uint32_t kSpanSyms = 32 * kPiece;           // symbols per warp at most
 constexpr uint32_t kSpanVecs = (127 + kSpanSyms * kMaxCode + 127) / 128;  // 16-byte vectors that hold a span's bits
 constexpr uint32_t kSpanWords = 4 * kSpanVecs + 4;    // and words read past the end (never consumed)
@@ -96,17 +94,6 @@ __device__ __forceinline__ uint32_t four_symbols(const uint32_t* bits, uint32_t&
   return __byte_perm(ab, cd, 0x5410);
 }
 
-// Geometry of a container's spans: a chunk takes `lanes` lanes, a warp
-// `chunks` chunks (of one group), a group `per_group` spans.
-struct SpanShape {
-  uint32_t lanes, chunks, per_group;
-  __device__ __forceinline__ explicit SpanShape(uint32_t cs) {
-    lanes = (cs + kPiece - 1) / kPiece;
-    chunks = 32 / lanes;
-    per_group = (kGroupChunks + chunks - 1) / chunks;
-  }
-};
-
 // Bits of warm-up before a piece.  Under Table 1 a reader is on the true
 // boundaries after 37 codewords (264 bits) in 99.7 % of cases.  A scheme whose
 // lengths are all even but the last area's keeps a wrong parity until such a
@@ -129,7 +116,6 @@ __device__ __forceinline__ uint32_t warm_bits(uint32_t len_lo, uint32_t len_hi) 
 // anything but the shortest codeword never find the boundaries from a wrong
 // phase, and their pieces are corrected one after the other: they keep a lane
 // per chunk at every size.
-constexpr uint64_t kSplitMax = 64ull << 20;       // symbols: streams that resynchronise fast
 constexpr uint64_t kSplitMaxSlow = 40ull << 20;   // ... slowly
 __device__ __forceinline__ bool split_pays(const DecHeader& h, uint64_t total) {
   const uint64_t bits = 8 * h.payload_bytes, least = h.n * (h.len_lo & 0xFFu);

@@ -447,9 +447,10 @@ encode_kernel(EncArgs A) {
   const uint64_t group_syms = (uint64_t)kGroupChunks * cs;
   const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(&s_stage[warp][0][0]);
   const uint32_t* tab = &s_enc[lane];
-  const uint64_t n_items = A.descs ? A.item_base[A.n_shards] : A.n_items;
   const qlc_lut* cur_lut = nullptr;
   for (int i = tid; i < kEncWarps * 2 * kWStage; i += kEncThreads) (&s_stage[0][0][0])[i] = 0;
+  dependency_wait();
+  const uint64_t n_items = A.descs ? A.item_base[A.n_shards] : A.n_items;
 
   while (true) {
     __syncthreads();
@@ -613,6 +614,7 @@ lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __rest
   __shared__ __align__(16) uint32_t s_enc[256 * 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t n_chunks = (n + cs - 1) / cs;
+  dependents_may_start();
   const uint32_t e = table_entry(lut->enc[tid]);
   stage_entry(s_enc, tid, e);
   if (__syncthreads_or(e == 0)) {  // not a LUT of this library: refused
@@ -639,9 +641,10 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __restric
   __shared__ unsigned long long s_sum[kEncWarps];
   __shared__ uint32_t s_more[4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < kEncWarps * 2 * kWStage; i += kEncThreads) (&s_stage[0][0][0])[i] = 0;
+  dependency_wait();
   const uint32_t e = table_entry(lut->enc[tid]);
   stage_entry(s_enc, tid, e);
-  for (int i = tid; i < kEncWarps * 2 * kWStage; i += kEncThreads) (&s_stage[0][0][0])[i] = 0;
   if (__syncthreads_or(e == 0)) return;  // lengths_kernel has set the status
   const uint32_t* tab = &s_enc[lane];
   const uint32_t n_chunks = (uint32_t)((n + cs - 1) / cs);  // <= kPartMaxChunks
@@ -801,8 +804,9 @@ qlc_status qlc_encode(const uint8_t* d_in, size_t n, const qlc_lut* d_lut, uint3
     const int want = (int)((n_chunks + kEncWarps - 1) / kEncWarps);
     lengths_kernel<<<want < 6 * sms ? want : 6 * sms, kEncThreads, 0, st>>>(d_in, n, d_lut, chunk_symbols, d_out,
                                                                             d_status);
-    pack_kernel<<<parts < kEncCtasPerSm * sms ? parts : kEncCtasPerSm * sms, kEncThreads, 0, st>>>(
-        d_in, n, d_lut, chunk_symbols, d_out, out_cap, reinterpret_cast<unsigned long long*>(d_out_bytes), d_status);
+    if (cudaGetLastError() != cudaSuccess) return QLC_ERR_CUDA;
+    launch_after(pack_kernel, parts < kEncCtasPerSm * sms ? parts : kEncCtasPerSm * sms, kEncThreads, 0, st, d_in, n, d_lut,
+                 chunk_symbols, d_out, out_cap, reinterpret_cast<unsigned long long*>(d_out_bytes), d_status);
     return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
   }
   if (cudaMemsetAsync(d_ws, 0, ws_need, st) != cudaSuccess) return QLC_ERR_CUDA;
@@ -878,7 +882,7 @@ qlc_status qlc_encode_batch(const qlc_desc* d_descs, int n_shards, uint32_t chun
   A.status = d_status;
   A.gstat_cap = w.gstat_cap;
   // the item count is only known on the device: launch the full resident grid
-  encode_kernel<<<enc_grid(~0ull, h_launch), kEncThreads, 0, st>>>(A);
+  launch_after(encode_kernel, enc_grid(~0ull, h_launch), kEncThreads, 0, st, A);
   return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
 }
 

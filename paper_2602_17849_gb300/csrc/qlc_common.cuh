@@ -172,6 +172,31 @@ __device__ __forceinline__ int shard_of_warp(const unsigned long long* __restric
 // Number of SMs of the current device (cached per device).
 int sm_count();
 
+// Programmatic dependent launch, between kernels of one call.  A kernel started
+// with launch_after, directly behind another kernel of the same call, may have
+// its CTAs resident, and the launch itself behind it, while that kernel still
+// runs: that one calls dependents_may_start(), and this one touches no memory
+// before dependency_wait(), which returns when that kernel is complete.  The
+// first kernel of a call is launched as usual: what comes before it in the
+// stream is not known (behind a memset node of a captured graph, the wait does
+// not hold).
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+template <typename... P, typename... A>
+inline bool launch_after(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess;
+}
+
 // A named NVTX range around a host entry point: profilers (nsys, ncu with
 // --nvtx) show the kernels a call launches under the call's name.  Without a
 // profiler attached a push or pop is a call through an empty slot.
@@ -182,12 +207,32 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
+// --------------------------------------------- the split decoder's geometry
+constexpr int kSpanWarps = 4;                    // warps per CTA; they share the code table
+constexpr uint32_t kPiece = 128;                 // symbols per lane, about
+constexpr uint64_t kSplitMax = 64ull << 20;      // symbols in a launch: see split_pays
+
+// Geometry of a container's spans: a chunk takes `lanes` lanes, a warp
+// `chunks` chunks (of one group), a group `per_group` spans.
+struct SpanShape {
+  uint32_t lanes, chunks, per_group;
+  __device__ __forceinline__ explicit SpanShape(uint32_t cs) {
+    lanes = (cs + kPiece - 1) / kPiece;
+    chunks = 32 / lanes;
+    per_group = (kGroupChunks + chunks - 1) / chunks;
+  }
+};
+
 // ----------------------------------------------------------------- batches
 // Batch workspace: 64 bytes of counters, item_base[n_shards + 1] (first work
 // item of each shard; the last entry is the total), then one look-back word
 // per encode work item.
+// Counter word that says how a batch is decoded (decode.cu).
+constexpr int kTicketWay = 1;
+enum DecodeWay : uint32_t { kWayGroups = 0, kWaySplit = 1, kWayEven = 2 };
+constexpr uint32_t kFewWarpsPerSm = 20;  // kWayEven: a warp per group
 struct BatchWs {
-  unsigned int* ticket;                // shared by encode / decode
+  unsigned int* ticket;                // [0] shared by encode / decode
   unsigned long long* item_base;
   unsigned long long* gstat;
   unsigned long long gstat_cap;        // look-back words available
@@ -208,9 +253,11 @@ constexpr int kPlanThreads = 1024;
 constexpr uint64_t kHistItem = 64 * 1024;  // symbols per histogram work item
 
 // One CTA: the number of work items of every shard (encode: groups of 32
-// chunks; decode: the container's groups),
+// chunks; decode: the container's groups, or in a batch of up to kSplitMax
+// symbols sets of kSpanWarps spans),
 // their exclusive prefix in item_base, and zeroed counters / look-back words.
-// Shards that cannot be processed get no items and set *status.
+// Shards that cannot be processed get no items and set *status.  cs: the chunk
+// size (encode), or the number of SMs (decode).
 __global__ void plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w,
                             uint32_t* status);
 

@@ -94,3 +94,29 @@ def test_checked_build():
                        capture_output=True, text=True, timeout=900)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
     assert "no index check failed" in r.stdout
+
+
+@pytest.mark.parametrize("total", [60 << 20, 70 << 20, 500 << 20])
+def test_batches_decoded_in_each_of_three_ways(qlc, total):
+    """Split up to 64 Mi symbols, a warp per group up to 20 per SM, and above;
+    with an empty, a nearly constant and a corrupt shard among them."""
+    sizes = [0, 5, 4096 * 33 + 1, 3 << 20, 40_000]
+    sizes += [(total - sum(sizes)) // 4 // 16 * 16] * 4
+    kinds = ["t4", "gauss", "laplace", "constant", "t4", "t4", "relu_t4", "gauss", "laplace"]
+    _, shards = inputs.make_shards(sizes, kinds, list(range(len(sizes))), "cuda")
+    b = qlc.Batch(shards, 4096 if total > 100 << 20 else 2048)
+    b.encode()
+    b.decode()
+    torch.cuda.synchronize()
+    b.check()
+    assert b.n_out.tolist() == sizes
+    for i, x in enumerate(shards):
+        assert torch.equal(b.output(i), x), i
+    b.container(4)[330] ^= 0x11  # its index
+    b.decoded.zero_()
+    b.decode()
+    assert int(b.status.item()) == qlc.ERR_CORRUPT
+    b.status.zero_()
+    for i, x in enumerate(shards):
+        if i != 4:
+            assert torch.equal(b.output(i), x), i
