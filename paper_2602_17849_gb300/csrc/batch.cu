@@ -111,9 +111,10 @@ plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs 
   }
   bool split = false;
   if (kind == kPlanDecode) {
-    split = cta_scan(symbols, s_incl, s_warp, tid) <= kSplitMax;
+    symbols = cta_scan(symbols, s_incl, s_warp, tid);
+    split = symbols <= kSplitMax;
   }
-  if (tid < 16) w.ticket[tid] = 0;  // the 64 bytes of counters
+  if (tid < 16) w.ticket[tid] = tid == kTicketSymbols && split ? (uint32_t)symbols : 0u;  // the 64 bytes of counters
   unsigned long long total = 0;
   for (int base = 0; base < n_shards; base += kPlanThreads) {
     const int s = base + tid;

@@ -29,7 +29,6 @@
 namespace qlc {
 
 constexpr int kDecCtasPerSm = 20;  // 20 x (8.3 KB + 1 KB reserved); at 24 the register cap (80) spills
-
 // cp.async (global -> shared, 16 bytes, bypassing L1) and its groups.
 __device__ __forceinline__ void cp_async16(uint32_t smem, const void* g) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem), "l"(g) : "memory");
@@ -43,6 +42,12 @@ __device__ __forceinline__ void cp_async_wait() {
 constexpr uint32_t kBlk = 32;       // symbols per lane per block
 constexpr uint32_t kStageVec = 8;   // 16-byte vectors staged per lane (128 B of its stream)
 constexpr uint32_t kColRows = 16;   // words in each lane's column ring
+
+// How a lane reads its column ring: in shared memory at a constant address, or
+// at an address in registers, which costs no add when the ring is aligned to
+// its 2 KB (kRingMany, kRingFew; the latter for few warps per SM, see step_to).
+enum Ring { kRingStatic, kRingMany, kRingFew };
+constexpr uint32_t kRingBytes = kColRows * 128;
 
 // Shared memory of one warp decoding a group: the lanes' staging ring and
 // column ring.
@@ -115,13 +120,21 @@ struct LaneDec {
           : "memory");
     tv += q;
   }
+  template <Ring kRing>
   __device__ __forceinline__ uint32_t ring(const LaneShared& sm, uint32_t k) const {
-    return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint8_t*>(sm.col) + (((k << 7) & 0x780u) | lane4));
+    if constexpr (kRing == kRingStatic) {
+      return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint8_t*>(sm.col) + (((k << 7) & 0x780u) | lane4));
+    } else {
+      uint32_t v;
+      asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(((k << 7) & 0x780u) | col_s) : "memory");
+      return v;
+    }
   }
   // Set-up at bit S of the group: fill the staging ring, wait for it, move
   // the words the first block can read, load the buffer, refill.  Words
   // j .. j + 2 (at most two vectors) go to the buffer before the rest is
   // moved: the ring holds 16 words, and word j + 16 shares word j's row.
+  template <Ring kRing>
   __device__ __forceinline__ void start(const LaneShared& sm, uint32_t S) {
     p = S;
     tv = fv = min(S >> 7, vend);
@@ -131,9 +144,9 @@ struct LaneDec {
     const uint32_t j = S >> 5;
     move(j + 2);
     move(j + 2);
-    hi = ring(sm, j);
-    lo = ring(sm, j + 1);
-    nxt = ring(sm, j + 2);
+    hi = ring<kRing>(sm, j);
+    lo = ring<kRing>(sm, j + 1);
+    nxt = ring<kRing>(sm, j + 2);
 #pragma unroll
     for (int i = 0; i < 3; i++) move(j + 13);
     fetch<5>(min(tv + kStageVec, vend));
@@ -154,15 +167,34 @@ struct LaneDec {
   }
   // Advances the position to pn (less than 32 bits on): when it crosses into
   // the next word the buffer moves up a word and the word after nxt is read.
+  // With kRingFew as predicated instructions, which shortens the chain of a
+  // warp that has a quarter of an SM nearly to itself (16 Mi equal symbols 85
+  // -> 79 us, 1814 groups of a batch 167 -> 161 us); the compiler's form issues
+  // less, which counts with many warps (256 Mi symbols 181 us, not 188).
+  template <Ring kRing>
   __device__ __forceinline__ void step_to(const LaneShared& sm, uint32_t pn) {
-    if ((pn ^ p) & 32u) {
+    if constexpr (kRing == kRingFew) {
+      asm volatile(
+          "{\n\t.reg .pred q;\n\t.reg .b32 t;\n\t"
+          "xor.b32 t, %3, %4;\n\t"
+          "and.b32 t, t, 32;\n\t"
+          "setp.ne.u32 q, t, 0;\n\t"
+          "@q mov.b32 %0, %1;\n\t"
+          "@q mov.b32 %1, %2;\n\t"
+          "@q ld.shared.u32 %2, [%5];\n\t"
+          "}"
+          : "+r"(hi), "+r"(lo), "+r"(nxt)
+          : "r"(pn), "r"(p), "r"((((pn << 2) + 256u) & 0x780u) | col_s)  // row (pn / 32 + 2) % 16
+          : "memory");
+    } else if ((pn ^ p) & 32u) {
       hi = lo;
       lo = nxt;
-      nxt = ring(sm, (pn >> 5) + 2);
+      nxt = ring<kRing>(sm, (pn >> 5) + 2);
     }
     p = pn;
   }
   // Two symbols (at most 22 bits) from the window, packed as s0 | s1 << 8.
+  template <Ring kRing>
   __device__ __forceinline__ uint32_t round2(const LaneShared& sm, const uint8_t* T, uint32_t len_lo, uint32_t len_hi) {
     const uint32_t x = __funnelshift_l(lo, hi, p);
     const uint32_t la = code_len(x, len_lo, len_hi);
@@ -172,16 +204,17 @@ struct LaneDec {
     const uint32_t lb = code_len(x2, len_lo, len_hi);
     const uint32_t ib = __funnelshift_l(x2, 0u, lb);
     const uint32_t b = QLC_GUARD(ib < 2048u, nullptr) ? (uint32_t)T[ib] : 0u;
-    step_to(sm, p + la + lb);
+    step_to<kRing>(sm, p + la + lb);
     return mad_lo(b, 256u, a);
   }
   // One symbol (ragged chunk ends only).
+  template <Ring kRing>
   __device__ __forceinline__ uint32_t round1(const LaneShared& sm, const uint8_t* T, uint32_t len_lo, uint32_t len_hi) {
     const uint32_t x = __funnelshift_l(lo, hi, p);
     const uint32_t la = code_len(x, len_lo, len_hi);
     const uint32_t ia = __funnelshift_l(x, 0u, la);
     const uint32_t a = QLC_GUARD(ia < 2048u, nullptr) ? (uint32_t)T[ia] : 0u;
-    step_to(sm, p + la);
+    step_to<kRing>(sm, p + la);
     return a;
   }
 };
@@ -201,34 +234,34 @@ __device__ __forceinline__ void st_cs_32(uint8_t* dst, const uint32_t w[8], bool
   }
 }
 
-// Thirty-two decoded symbols w of one chunk, starting at symbol index i of
-// the tensor (a multiple of 32), to their destination; sc is their block's
-// scale (dequantising outputs).
+// One block of 32 symbols of each of the group's 32 chunks (all of them whole)
+// as values: the lanes' words pass through a tile (at shared address
+// tile_s, a multiple of 1 KB; word k of lane l is word 32 k + (l ^ 4 k): no two
+// lanes of a write or a read share a bank), so that
+// eight lanes write the 128 (or 64) bytes of a chunk's block and a store covers
+// 4 lines.  With each lane writing its own block in pieces of 32 bytes a store
+// touched 32 lines, and those stores were half of the L1 data pipe's work (256
+// Mi fp32 values 328 us).  first: index of the first chunk's block in the
+// tensor; sc: the scale of this lane's block.
 template <int kOut>
-__device__ __forceinline__ void put32(void* out, float sc, uint64_t i, const uint32_t w[8], bool aligned32) {
-  if (kOut == kOutCodes) {
-    st_cs_32(static_cast<uint8_t*>(out) + i, w, aligned32);
-  } else {
-    // the block's 32 values share one scale (i is a multiple of 32); they go
-    // out in whole 32-byte sectors: 4 stores of 8 fp32, or 2 of 16 bf16
-    uint32_t v[kOut == QLC_DTYPE_F32 ? 32 : 16];
+__device__ __forceinline__ void put_tile(void* out, uint32_t tile_s, float sc, uint64_t first, uint32_t cs,
+                                         const uint32_t w[8], int lane) {
+  const uint32_t at = tile_s | 4u * lane;
 #pragma unroll
-    for (int j = 0; j < 32; j++) {
-      const float y = __uint_as_float(e4m3_scaled_bits(w[j >> 2], j & 3)) * 0x1p120f * sc;
-      if (kOut == QLC_DTYPE_F32) {
-        v[j] = __float_as_uint(y);
-      } else if (j & 1) {
-        const __nv_bfloat162 hb = __floats2bfloat162_rn(__uint_as_float(v[j >> 1]), y);
-        v[j >> 1] = *reinterpret_cast<const uint32_t*>(&hb);
-      } else {
-        v[j >> 1] = __float_as_uint(y);
-      }
-    }
-    constexpr int kVec = kOut == QLC_DTYPE_F32 ? 4 : 2;  // 32-byte pieces
-    uint8_t* dst = static_cast<uint8_t*>(out) + i * (kOut == QLC_DTYPE_F32 ? 4 : 2);
+  for (int k = 0; k < 8; k++)
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"((at ^ 16u * k) + 128u * k), "r"(w[k]) : "memory");
+  __syncwarp();
+  const uint32_t j = (uint32_t)lane >> 3, k = (uint32_t)lane & 7u;  // chunk 4 q + j, symbols 4 k ..
+  const uint32_t from = tile_s | 128u * k | 16u * k | 4u * j;
+  uint32_t v[8];
 #pragma unroll
-    for (int k = 0; k < kVec; k++) st_cs_32(dst + 32 * k, v + 8 * k, aligned32);
-  }
+  for (uint32_t q = 0; q < 8; q++) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v[q]) : "r"(from ^ 16u * q) : "memory");
+  constexpr uint32_t kElem = kOut == QLC_DTYPE_F32 ? 4 : 2;
+  uint8_t* dst = static_cast<uint8_t*>(out) + (first + j * cs + 4 * k) * kElem;
+#pragma unroll
+  for (uint32_t q = 0; q < 8; q++)
+    put4_values<kOut>(dst + (size_t)(4 * q * cs * kElem), __shfl_sync(0xffffffffu, sc, 4 * q + j), v[q]);
+  __syncwarp();
 }
 
 // Decodes group g of a validated container (one warp; lane = chunk).  With
@@ -236,11 +269,11 @@ __device__ __forceinline__ void put32(void* out, float sc, uint64_t i, const uin
 // instead of out: a pointer that is not a kernel parameter would otherwise
 // hold two registers across the decoding loop, which then issued about 10 %
 // more instructions (the batch decoder, 124.3 M against 112.8 M on 256 MiB).
-template <int kOut>
+template <int kOut, Ring kRing>
 __device__ __forceinline__ void decode_group(const DecHeader& h, const uint8_t* __restrict__ in, void* __restrict__ out,
                              const float* __restrict__ scales, uint64_t g, LaneShared& sm, const uint8_t* T, LaneDec& d,
                              uint32_t* status, int lane, bool aligned32, bool sc_vec = false,
-                             void* const volatile* out_slot = nullptr) {
+                             uint32_t tile_s = 0, void* const volatile* out_slot = nullptr) {
   const unsigned long long* group_off = reinterpret_cast<const unsigned long long*>(in + kIndexOff);
   const uint16_t* chunk_bits = reinterpret_cast<const uint16_t*>(in + kIndexOff + 8 * h.n_groups);
   const uint4* vbase = reinterpret_cast<const uint4*>(in + h.P);
@@ -273,7 +306,7 @@ __device__ __forceinline__ void decode_group(const DecHeader& h, const uint8_t* 
   d.gp = vbase + goff / 16;
   d.vend = (uint32_t)((gnext - goff) / 16);
   d.vlim = (h.in_bytes - h.P - goff) / 16;  // goff <= payload_bytes <= in_bytes - P (validated)
-  d.start(sm, S);
+  d.template start<kRing>(sm, S);
   const uint64_t i_chunk = c * cs;  // the chunk's first symbol
   const uint32_t nmax = __reduce_max_sync(0xffffffffu, nsym);
   // dequantising outputs: the scales of the chunk's whole blocks, four per
@@ -303,18 +336,29 @@ __device__ __forceinline__ void decode_group(const DecHeader& h, const uint8_t* 
     const float sc = (b & 3u) == 0 ? sc_cur.x : (b & 3u) == 1 ? sc_cur.y : (b & 3u) == 2 ? sc_cur.z : sc_cur.w;
     const uint32_t cnt = nsym > i0 ? min(kBlk, nsym - i0) : 0u;
     void* o = out_slot ? *out_slot : out;
+    const bool whole = kOut != kOutCodes && __all_sync(0xffffffffu, cnt == kBlk);
     if (cnt == kBlk) {
       uint32_t w[8];
 #pragma unroll
       for (int j = 0; j < 8; j++) {
-        const uint32_t p0 = d.round2(sm, T, len_lo, len_hi);
-        const uint32_t p1 = d.round2(sm, T, len_lo, len_hi);
+        const uint32_t p0 = d.template round2<kRing>(sm, T, len_lo, len_hi);
+        const uint32_t p1 = d.template round2<kRing>(sm, T, len_lo, len_hi);
         w[j] = __byte_perm(p0, p1, 0x5410);
       }
-      if (QLC_GUARD(i_chunk + i0 + kBlk <= h.out_cap, status)) put32<kOut>(o, sc, i_chunk + i0, w, aligned32);
+      if constexpr (kOut == kOutCodes) {
+        if (QLC_GUARD(i_chunk + i0 + kBlk <= h.out_cap, status)) st_cs_32(static_cast<uint8_t*>(o) + i_chunk + i0, w, aligned32);
+      } else if (whole) {
+        if (QLC_GUARD(g * kGroupChunks * cs + 31ull * cs + i0 + kBlk <= h.out_cap, status))
+          put_tile<kOut>(o, tile_s, sc, g * kGroupChunks * cs + i0, cs, w, lane);
+      } else if (QLC_GUARD(i_chunk + i0 + kBlk <= h.out_cap, status)) {  // a tensor's last group
+        constexpr uint32_t kElem = kOut == QLC_DTYPE_F32 ? 4 : 2;
+#pragma unroll
+        for (uint32_t j = 0; j < 8; j++)
+          put4_values<kOut>(static_cast<uint8_t*>(o) + (i_chunk + i0 + 4 * j) * kElem, sc, w[j]);
+      }
     } else {
       for (uint32_t k = 0; k < cnt; k++) {
-        const uint32_t sym = d.round1(sm, T, len_lo, len_hi);
+        const uint32_t sym = d.template round1<kRing>(sm, T, len_lo, len_hi);
         if (QLC_GUARD(i_chunk + i0 + k < h.out_cap, status)) put1<kOut>(o, scales, i_chunk + i0 + k, sym);
       }
     }
@@ -332,43 +376,100 @@ __device__ __forceinline__ bool lane_init(LaneShared& sm, LaneDec& d, int lane) 
   return (__cvta_generic_to_shared(sm.stage) & 15u) == 0;
 }
 
-// One container: every CTA (one warp) validates the header, builds its table
-// and decodes groups blockIdx.x, blockIdx.x + gridDim.x, ...
+// One container: one CTA per SM of up to dec_warps warps, which validate the header and
+// build the code table once, then decode spans (decode_span.cuh) where that
+// pays and else groups, a lane per chunk.  Spans and groups are dealt out warp
+// by warp over the SMs, so that every SM, and every quarter of an SM, has the
+// same number of them, give or take one.  (With a CTA per warp or per four, the
+// block scheduler puts up to 16 of 2048 working warps on some SMs, unless the
+// grid is as large as the groups; the host, which does not know the chunk,
+// could then be four times off: 50 Mi symbols in chunks of 1024 took 85 us.)
+constexpr int dec_warps(int out) { return out == kOutCodes ? 20 : 16; }  // 96 or 128 registers: values spill at 96
+struct LaneWarp {  // a warp that decodes groups
+  LaneShared lanes;
+  uint32_t tile[256];
+  uint8_t pad[1024];
+};
+static_assert(sizeof(LaneWarp) % kRingBytes == 0 && sizeof(LaneWarp) <= sizeof(SpanWarp), "");
+constexpr size_t one_bytes(int warps) { return warps * sizeof(SpanWarp) + kRingBytes; }
+// The first address at or after p that a column ring can have.
+__device__ __forceinline__ uint8_t* ring_aligned(uint8_t* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  return p + ((kRingBytes - a % kRingBytes) % kRingBytes);
+}
 template <int kOut>
-__global__ void __launch_bounds__(32, kDecCtasPerSm)
+__global__ void __launch_bounds__(32 * dec_warps(kOut), 1)
 decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restrict__ out,
               const float* __restrict__ scales, uint64_t out_cap, unsigned long long* __restrict__ n_out,
               uint32_t* __restrict__ status) {
-  __shared__ DecShared sm;
-  const int lane = threadIdx.x;
+  constexpr int kWarps = dec_warps(kOut);
+  extern __shared__ __align__(16) uint8_t one_sm[];
+  __shared__ uint8_t T[2048];                       // code -> symbol
+  __shared__ __align__(16) uint8_t hdr[kIndexOff];  // the container's header and dec
+  __shared__ uint32_t seen[kWarps][8];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // so known to be the same in all lanes
+  const uint32_t warps = blockDim.x / 32;
+  load_header(in, in_bytes, hdr, tid, blockDim.x);
+  __syncthreads();
   DecHeader h;
-  load_header(in, in_bytes, sm.hdr, lane, 32);
-  __syncwarp();
-  const uint32_t err = parse_header(sm.hdr, in_bytes, out_cap, &h, sm.seen, lane);
-  if (err) {
-    if (blockIdx.x == 0 && lane == 0) {
-      if (err == QLC_ERR_CAPACITY) *n_out = h.n;
-      set_status(status, err);
+  const uint32_t err = parse_header(hdr, in_bytes, out_cap, &h, seen[warp], lane);
+  if (blockIdx.x == 0 && tid == 0) {
+    if (!err || err == QLC_ERR_CAPACITY) *n_out = h.n;
+    if (err) set_status(status, err);
+  }
+  if (err) return;
+  build_table(hdr, T, tid, blockDim.x);
+  __syncthreads();
+  const uint32_t first = (uint32_t)warp * gridDim.x + blockIdx.x;
+  if (split_pays<kOut>(h, h.n)) {
+    const uint32_t stride = warps * gridDim.x;
+    const SpanShape shape(h.cs);
+    const uint32_t warm = warm_bits(h.len_lo, h.len_hi);
+    const uint32_t k = (uint32_t)lane / shape.lanes, seg = (uint32_t)lane - k * shape.lanes;
+    // span s is span r of group g; the step to the warp's next span is made in both
+    const uint32_t dg = stride / shape.per_group, dr = stride % shape.per_group;
+    uint64_t g = first / shape.per_group;
+    uint32_t r = first % shape.per_group;
+    while (g < h.n_groups) {
+      decode_span<kOut>(h, shape, in, out, scales, g, r * shape.chunks, k, seg, reinterpret_cast<SpanWarp*>(one_sm)[warp], T,
+                        warm, status, lane);
+      g += dg;
+      r += dr;
+      if (r >= shape.per_group) {
+        r -= shape.per_group;
+        g++;
+      }
     }
     return;
   }
-  if (blockIdx.x == 0 && lane == 0) *n_out = h.n;
-  if (blockIdx.x >= h.n_groups) return;
+  LaneWarp& sm = reinterpret_cast<LaneWarp*>(ring_aligned(one_sm))[warp];
   LaneDec d;
   if (!lane_init(sm.lanes, d, lane)) {
     if (lane == 0) set_status(status, QLC_ERR_CUDA);
     return;
   }
-  build_table(sm.hdr, sm.T, lane, 32);
-  __syncwarp();
   const bool aligned32 = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
   const bool sc_vec = (reinterpret_cast<uintptr_t>(scales) & 15u) == 0;  // scales read four at a time
-  for (uint64_t g = blockIdx.x; g < h.n_groups; g += gridDim.x)
-    decode_group<kOut>(h, in, out, scales, g, sm.lanes, sm.T, d, status, lane, aligned32, sc_vec);
+  const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(sm.tile);
+  // as many rounds of groups as the warps need, and no more warps than these
+  // rounds need: a last round that is nearly empty costs as much as a full one
+  // (200 Mi symbols in chunks of 2048, 3200 groups on 3040 warps: 158 us)
+  const uint64_t rounds = (h.n_groups + (uint64_t)warps * gridDim.x - 1) / ((uint64_t)warps * gridDim.x);
+  const uint32_t used = (uint32_t)((h.n_groups + rounds * gridDim.x - 1) / (rounds * gridDim.x));
+  if ((uint32_t)warp >= used) return;
+  const uint32_t stride = used * gridDim.x;
+  if (used <= (kOut == kOutCodes ? 8 : 4)) {
+    for (uint64_t g = first; g < h.n_groups; g += stride)
+      decode_group<kOut, kRingFew>(h, in, out, scales, g, sm.lanes, T, d, status, lane, aligned32, sc_vec, tile_s);
+  } else {
+    for (uint64_t g = first; g < h.n_groups; g += stride)
+      decode_group<kOut, kRingMany>(h, in, out, scales, g, sm.lanes, T, d, status, lane, aligned32, sc_vec, tile_s);
+  }
 }
 
-// Shared memory of a CTA of kSpanWarps warps that decode spans, or groups, of
-// one container.
+// Shared memory of a team of kSpanWarps warps that decode spans, or groups, of
+// one shard.
 struct SpanShared {
   union {
     SpanWarp span;
@@ -378,58 +479,6 @@ struct SpanShared {
   __align__(16) uint8_t hdr[kIndexOff];     // the container's header and dec
   uint32_t seen[kSpanWarps][8];
 };
-
-// One container, split: CTAs of kSpanWarps warps validate the header, build
-// the code table once and decode spans (decode_span.cuh), or whole groups
-// with a lane per chunk where that is faster (split_pays).
-template <int kOut>
-__global__ void __launch_bounds__(32 * kSpanWarps, kSpanCtasPerSm)
-decode_span_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restrict__ out,
-                   const float* __restrict__ scales, uint64_t out_cap, unsigned long long* __restrict__ n_out,
-                   uint32_t* __restrict__ status) {
-  __shared__ SpanShared sm;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  load_header(in, in_bytes, sm.hdr, tid, 32 * kSpanWarps);
-  __syncthreads();
-  DecHeader h;
-  const uint32_t err = parse_header(sm.hdr, in_bytes, out_cap, &h, sm.seen[warp], lane);
-  if (blockIdx.x == 0 && tid == 0) {
-    if (!err || err == QLC_ERR_CAPACITY) *n_out = h.n;
-    if (err) set_status(status, err);
-  }
-  if (err) return;
-  build_table(sm.hdr, sm.T, tid, 32 * kSpanWarps);
-  __syncthreads();
-  if (!split_pays(h, h.n)) {
-    LaneDec d;
-    if (!lane_init(sm.w[warp].lanes, d, lane)) {
-      if (lane == 0) set_status(status, QLC_ERR_CUDA);
-      return;
-    }
-    const bool aligned32 = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
-    const bool sc_vec = (reinterpret_cast<uintptr_t>(scales) & 15u) == 0;
-    for (uint64_t g = blockIdx.x + (uint64_t)warp * gridDim.x; g < h.n_groups; g += (uint64_t)gridDim.x * kSpanWarps)
-      decode_group<kOut>(h, in, out, scales, g, sm.w[warp].lanes, sm.T, d, status, lane, aligned32, sc_vec);
-    return;
-  }
-  const SpanShape shape(h.cs);
-  const uint32_t warm = warm_bits(h.len_lo, h.len_hi);
-  const uint32_t k = (uint32_t)lane / shape.lanes, seg = (uint32_t)lane - k * shape.lanes;
-  // span s is span r of group g; the step to the warp's next span is made in both
-  const uint32_t stride = gridDim.x * kSpanWarps, dg = stride / shape.per_group, dr = stride % shape.per_group;
-  const uint32_t s0 = blockIdx.x * kSpanWarps + warp;
-  uint64_t g = s0 / shape.per_group;
-  uint32_t r = s0 % shape.per_group;
-  while (g < h.n_groups) {
-    decode_span<kOut>(h, shape, in, out, scales, g, r * shape.chunks, k, seg, sm.w[warp].span, sm.T, warm, status, lane);
-    g += dg;
-    r += dr;
-    if (r >= shape.per_group) {
-      r -= shape.per_group;
-      g++;
-    }
-  }
-}
 
 // ---------------------------------------------------------------- batches
 //
@@ -501,8 +550,8 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
     if (lane == 0) s_out = dd.out;
     __syncwarp();
     if (g < h.n_groups)
-      decode_group<kOutCodes>(h, static_cast<const uint8_t*>(dd.in), nullptr, nullptr, g, sm.lanes, sm.T, d, status, lane,
-                              aligned32, false, &s_out);
+      decode_group<kOutCodes, kRingStatic>(h, static_cast<const uint8_t*>(dd.in), nullptr, nullptr, g, sm.lanes, sm.T, d, status, lane,
+                              aligned32, false, 0u, &s_out);
   }
 }
 
@@ -512,11 +561,19 @@ __device__ __forceinline__ void team_sync(int team) {
 }
 
 // Few groups: one CTA per SM, of kSpanCtasPerSm teams of kSpanWarps warps.
+struct FewOwn {
+  LaneShared lanes;
+  uint8_t T[2048];
+  __align__(16) uint8_t hdr[kRingBytes - 64];  // kIndexOff bytes of it
+  uint32_t seen[16];
+};
+static_assert(sizeof(FewOwn) % kRingBytes == 0, "");
 struct FewShared {
   union {
-    SpanShared span[kSpanCtasPerSm];                // a team's
-    DecShared own[kSpanWarps * kSpanCtasPerSm];     // a warp's
+    SpanShared span[kSpanCtasPerSm];            // a team's
+    FewOwn own[kSpanWarps * kSpanCtasPerSm];    // a warp's
   };
+  uint8_t align[kRingBytes];
 };
 constexpr int kFewWarps = kSpanWarps * kSpanCtasPerSm;
 static_assert(kFewWarps == kFewWarpsPerSm, "plan_kernel compares the groups with these warps");
@@ -530,6 +587,7 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
   dependents_may_start();
   dependency_wait();
   const uint32_t way = ticket[kTicketWay];
+  const uint64_t batch_symbols = ticket[kTicketSymbols];
   if (way == kWayGroups) return;
   const int lane = threadIdx.x % 32;
   const int wid = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0);  // so known to be the same in all lanes
@@ -543,7 +601,7 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
     // now 165.
     const unsigned long long t = (unsigned long long)wid * gridDim.x + blockIdx.x;
     if (t >= total) return;
-    DecShared& sm = all.own[wid];
+    FewOwn& sm = reinterpret_cast<FewOwn*>(ring_aligned(few_sm))[wid];
     LaneDec d;
     if (!lane_init(sm.lanes, d, lane)) {
       if (lane == 0) set_status(status, QLC_ERR_CUDA);
@@ -557,8 +615,8 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
     if (lane == 0) s_out[wid] = dd.out;
     __syncwarp();
     if (g < h.n_groups)
-      decode_group<kOutCodes>(h, static_cast<const uint8_t*>(dd.in), nullptr, nullptr, g, sm.lanes, sm.T, d, status, lane,
-                              (reinterpret_cast<uintptr_t>(dd.out) & 31u) == 0, false, &s_out[wid]);
+      decode_group<kOutCodes, kRingFew>(h, static_cast<const uint8_t*>(dd.in), nullptr, nullptr, g, sm.lanes, sm.T, d, status, lane,
+                              (reinterpret_cast<uintptr_t>(dd.out) & 31u) == 0, false, 0u, &s_out[wid]);
     return;
   }
   // Split: items are kSpanWarps spans of one shard, which a team decodes with a
@@ -586,7 +644,7 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
     }
     if (!err) {
       const uint64_t s = (uint64_t)q * kSpanWarps + warp;
-      if (split_pays(h, h.n)) {
+      if (split_pays<kOutCodes>(h, batch_symbols)) {
         const SpanShape shape(h.cs);
         const uint32_t k = (uint32_t)lane / shape.lanes, seg = (uint32_t)lane - k * shape.lanes;
         const uint64_t g = s / shape.per_group;
@@ -597,7 +655,7 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
       } else if (s < h.n_groups) {  // a shard has at least as many spans as groups
         LaneDec d;
         if (lane_init(sm.w[warp].lanes, d, lane))
-          decode_group<kOutCodes>(h, in, dd.out, nullptr, s, sm.w[warp].lanes, sm.T, d, status, lane,
+          decode_group<kOutCodes, kRingStatic>(h, in, dd.out, nullptr, s, sm.w[warp].lanes, sm.T, d, status, lane,
                                   (reinterpret_cast<uintptr_t>(dd.out) & 31u) == 0);
         else if (lane == 0)
           set_status(status, QLC_ERR_CUDA);
@@ -614,41 +672,30 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
 
 using namespace qlc;
 
-// One CTA (warp) per group where the container's groups are few enough, up
-// to kDecCtasPerSm per SM.  The host knows out_cap, not the chunk size: a
-// container of out_cap symbols has between min_groups (chunks of
-// QLC_MAX_CHUNK) and max_groups (chunks of QLC_MIN_CHUNK) groups.  A grid
-// much larger than the groups lets the block scheduler put up to 16 of the
-// working CTAs on some SMs and 13 on others (measured with 2048 groups: a
-// grid of 2048 or 2128 CTAs gives every SM 13 or 14 working CTAs, grids of
-// 2432 or 3040 up to 16, and decode runs 4 % slower).  So a container large
-// enough to fill the GPU at the largest chunk gets min_groups CTAs: every CTA
-// works at that chunk, and at smaller chunks each CTA takes several groups.
-static int decode_grid(uint64_t out_cap) {
-  const uint64_t per_group_min = (uint64_t)kGroupChunks * QLC_MIN_CHUNK;
-  const uint64_t per_group_max = (uint64_t)kGroupChunks * QLC_MAX_CHUNK;
-  const uint64_t max_groups = (out_cap + per_group_min - 1) / per_group_min;
-  const uint64_t min_groups = (out_cap + per_group_max - 1) / per_group_max;
-  const uint64_t sms = (uint64_t)sm_count(), cap = sms * kDecCtasPerSm;
-  const uint64_t want = min_groups >= 2 * sms ? min_groups : max_groups;
-  return (int)(want < 1 ? 1 : (want < cap ? want : cap));
-}
-
-// CTAs of the split decoder: a warp per span.
-static int span_grid(uint64_t out_cap) {
-  const uint64_t want = (out_cap / kSpanSyms + kSpanWarps) / kSpanWarps, cap = (uint64_t)sm_count() * kSpanCtasPerSm;
-  return (int)(want < cap ? want : cap);
+// Raises a kernel's shared-memory limit, once per device (a function
+// attribute, allowed inside stream capture).
+template <typename K>
+static bool smem_ok(K kernel, size_t bytes, std::atomic<bool> (&done)[64]) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
+  if (dev < 64 && done[dev].load(std::memory_order_relaxed)) return true;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
+  if (dev < 64) done[dev].store(true, std::memory_order_relaxed);
+  return true;
 }
 
 template <int kOut>
 static qlc_status launch_decode(const uint8_t* d_in, size_t in_bytes, void* d_out, const float* d_scales,
                                 size_t out_cap, uint64_t* d_n_out, uint32_t* d_status, cudaStream_t st) {
-  unsigned long long* no = reinterpret_cast<unsigned long long*>(d_n_out);
-  if (out_cap <= kSplitMax)
-    decode_span_kernel<kOut><<<span_grid(out_cap), 32 * kSpanWarps, 0, st>>>(d_in, in_bytes, d_out, d_scales, out_cap,
-                                                                             no, d_status);
-  else
-    decode_kernel<kOut><<<decode_grid(out_cap), 32, 0, st>>>(d_in, in_bytes, d_out, d_scales, out_cap, no, d_status);
+  static std::atomic<bool> done[64];
+  if (!smem_ok(decode_kernel<kOut>, one_bytes(dec_warps(kOut)), done)) return QLC_ERR_CUDA;
+  // a warp for every span there can be, four at least (a CTA of all warps and
+  // their shared memory starts 1 to 3 us later)
+  const uint64_t spans = out_cap / (kSpanSyms / 2) + 1, sms = (uint64_t)sm_count();
+  const uint64_t per_sm = (spans + sms - 1) / sms;
+  const int warps = per_sm >= dec_warps(kOut) ? dec_warps(kOut) : (int)((per_sm + 3) / 4 * 4);
+  decode_kernel<kOut><<<(int)(spans < sms ? spans : sms), 32 * warps, one_bytes(warps), st>>>(
+      d_in, in_bytes, d_out, d_scales, out_cap, reinterpret_cast<unsigned long long*>(d_n_out), d_status);
   return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
 }
 
@@ -677,20 +724,6 @@ extern "C" qlc_status qlc_decode_dequantize(const uint8_t* d_in, size_t in_bytes
   return launch_decode<QLC_DTYPE_BF16>(d_in, in_bytes, d_out, d_scales, out_cap, d_n_out, d_status, st);
 }
 
-// Raises decode_few_kernel's shared-memory limit, once per device (a function
-// attribute, allowed inside stream capture).
-static bool decode_few_smem_ok() {
-  static std::atomic<bool> done[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
-  if (dev < 64 && done[dev].load(std::memory_order_relaxed)) return true;
-  if (cudaFuncSetAttribute(decode_few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FewShared)) !=
-      cudaSuccess)
-    return false;
-  if (dev < 64) done[dev].store(true, std::memory_order_relaxed);
-  return true;
-}
-
 extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, void* d_ws, size_t ws_bytes,
                                        uint32_t* d_status, const qlc_launch* h_launch, qlc_stream_t stream) {
   NvtxRange nvtx_range("qlc_decode_batch");
@@ -704,7 +737,8 @@ extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, vo
   int per_sm = kDecCtasPerSm;
   if (h_launch && h_launch->decode_ctas_per_sm > 0 && h_launch->decode_ctas_per_sm < kDecCtasPerSm)
     per_sm = h_launch->decode_ctas_per_sm;
-  if (!decode_few_smem_ok()) return QLC_ERR_CUDA;
+  static std::atomic<bool> done[64];
+  if (!smem_ok(decode_few_kernel, sizeof(FewShared), done)) return QLC_ERR_CUDA;
   // which of the two has the work is decided on the device; the other returns at once
   const int sms = sm_count();
   launch_after(decode_few_kernel, sms, 32 * kFewWarps, sizeof(FewShared), st, d_descs, n_shards, w.item_base, w.ticket,

@@ -139,25 +139,28 @@ __device__ __forceinline__ void put1(void* out, const float* scales, uint64_t i,
   }
 }
 
-// Four decoded symbols w starting at index i of the tensor (a multiple of 4),
-// one streaming store; a warp's 32 calls cover contiguous bytes.
+// Four symbols w of one block as values at dst, one streaming store; a warp's
+// 32 stores cover few lines.
 template <int kOut>
-__device__ __forceinline__ void put4(void* out, const float* __restrict__ scales, uint64_t i, uint32_t w) {
-  if (kOut == kOutCodes) {
-    __stcs(reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(out) + i), w);
-    return;
-  }
-  const float sc = __ldg(scales + i / 32);
+__device__ __forceinline__ void put4_values(uint8_t* dst, float sc, uint32_t w) {
   float y[4];
 #pragma unroll
   for (int j = 0; j < 4; j++) y[j] = __uint_as_float(e4m3_scaled_bits(w, j)) * 0x1p120f * sc;
   if (kOut == QLC_DTYPE_F32) {
-    __stcs(reinterpret_cast<float4*>(static_cast<float*>(out) + i), make_float4(y[0], y[1], y[2], y[3]));
+    __stcs(reinterpret_cast<float4*>(dst), make_float4(y[0], y[1], y[2], y[3]));
   } else {
     const __nv_bfloat162 a = __floats2bfloat162_rn(y[0], y[1]), b = __floats2bfloat162_rn(y[2], y[3]);
-    __stcs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + i),
+    __stcs(reinterpret_cast<uint2*>(dst),
            make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b)));
   }
+}
+// Four decoded symbols w starting at index i of the tensor (a multiple of 4).
+template <int kOut>
+__device__ __forceinline__ void put4(void* out, const float* __restrict__ scales, uint64_t i, uint32_t w) {
+  if (kOut == kOutCodes)
+    __stcs(reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(out) + i), w);
+  else
+    put4_values<kOut>(static_cast<uint8_t*>(out) + i * (kOut == QLC_DTYPE_F32 ? 4 : 2), __ldg(scales + i / 32), w);
 }
 
 }  // namespace qlc

@@ -107,22 +107,31 @@ __device__ __forceinline__ uint32_t warm_bits(uint32_t len_lo, uint32_t len_hi) 
 }
 
 // Whether to decode a container split, where `total` symbols are decoded in
-// this launch.  A lane per chunk takes at least the 79 us of its longest
-// chain, however little there is; split, the time goes with the size, and
-// faster or slower with how fast readers find the true boundaries.  Measured
-// (us, split / lane per chunk, chunk 4096): 1 Mi symbols 15 / 79; 16 Mi
-// 27 / 80; 64 Mi Student-t 72 / 85, Gaussian 69 / 85, 18 % zeros under Table 2
-// 84 / 85, half zeros 93 / 85; 128 Mi Student-t 136 / 104.  Streams of hardly
-// anything but the shortest codeword never find the boundaries from a wrong
-// phase, and their pieces are corrected one after the other: they keep a lane
-// per chunk at every size.
-constexpr uint64_t kSplitMaxSlow = 40ull << 20;   // ... slowly
+// this launch.  A lane per chunk takes at least the time of its chain, about 19
+// us per 1024 symbols of chunk, and hardly more up to 40 Mi symbols; split, the
+// time goes with the size, and is longer where readers are slow to find the
+// true boundaries: in schemes of one parity, and in streams of mostly the
+// shortest codeword.  Measured (us, split / lane per chunk): chunk 4096,
+// Student-t 1 Mi 15 / 79, 16 Mi 27 / 80, 64 Mi 72 / 85, half zeros under Table 2
+// 43 Mi 77 / 81; chunk 2048, Student-t 32 Mi 43 / 53, half zeros under Table 2
+// 16 Mi 40 / 45, 32 Mi 58 / 53; chunk 1024, Student-t 8 Mi 19 / 27, 16 Mi 29 /
+// 31, 32 Mi 44 / 33, half zeros 8 Mi 25 / 27, 16 Mi 39 / 31; chunk 512,
+// Student-t 2 Mi 15 / 17, 8 Mi 19.1 / 18.4, half zeros 2 Mi 19 / 17.  Values:
+// chunk 4096, fp32, half zeros 29 Mi 70 / 109; chunk 1024, bf16, Student-t 8 Mi
+// 25 / 31, 16 Mi 40 / 36, half zeros 8 Mi 29 / 31, 16 Mi 46 / 36; chunk 4096,
+// bf16, Student-t 47 Mi 83 / 105, 60 Mi 121 / 109.
+// Hence the lines, proportional to the chunk; and streams of hardly anything
+// but the shortest codeword (fewer than 1/32 bit per symbol above it) never,
+// since they do not find the boundaries from a wrong phase, and their pieces
+// are corrected one after the other (64 Mi equal symbols 1216 us).
+template <int kOut>
 __device__ __forceinline__ bool split_pays(const DecHeader& h, uint64_t total) {
   const uint64_t bits = 8 * h.payload_bytes, least = h.n * (h.len_lo & 0xFFu);
-  const uint64_t excess = bits > least ? bits - least : 0;  // over the shortest code's bits
-  if (excess < h.n / 8) return false;
+  const uint64_t excess = bits > least ? bits - least : 0;
   const bool fast = mixed_parity(h.len_lo, h.len_hi) && excess >= h.n / 16 * 7;
-  return total <= (fast ? kSplitMax : kSplitMaxSlow);
+  const uint64_t cs = h.cs, line = (cs << 13) + (cs << 12);
+  const uint64_t most = fast ? (cs < 512 ? 0 : kOut == kOutCodes ? cs << 14 : line) : cs < 1024 ? 0 : line - (3ull << 20);
+  return excess >= h.n / 32 && total <= most;
 }
 
 // Decodes a span of a validated container: chunks c0 .. c0 + shape.chunks - 1

@@ -210,7 +210,7 @@ struct NvtxRange {
 // --------------------------------------------- the split decoder's geometry
 constexpr int kSpanWarps = 4;                    // warps per CTA; they share the code table
 constexpr uint32_t kPiece = 128;                 // symbols per lane, about
-constexpr uint64_t kSplitMax = 64ull << 20;      // symbols in a launch: see split_pays
+constexpr uint64_t kSplitMax = 64ull << 20;      // symbols of a batch decoded split: see split_pays
 
 // Geometry of a container's spans: a chunk takes `lanes` lanes, a warp
 // `chunks` chunks (of one group), a group `per_group` spans.
@@ -229,6 +229,7 @@ struct SpanShape {
 // per encode work item.
 // Counter word that says how a batch is decoded (decode.cu).
 constexpr int kTicketWay = 1;
+constexpr int kTicketSymbols = 2;  // the batch's symbols, in kWaySplit
 enum DecodeWay : uint32_t { kWayGroups = 0, kWaySplit = 1, kWayEven = 2 };
 constexpr uint32_t kFewWarpsPerSm = 20;  // kWayEven: a warp per group
 struct BatchWs {
