@@ -163,6 +163,17 @@ qlc_status qlc_encode(const uint8_t *d_in, size_t n, const qlc_lut *d_lut,
                       void *d_ws, size_t ws_bytes, uint64_t *d_out_bytes,
                       uint32_t *d_status, qlc_stream_t stream);
 
+/* qlc_histogram, qlc_build_lut_best (over h_schemes[0..n_schemes), 1..8) and
+ * qlc_encode of one tensor in one call (Sections 4 to 7), which the stream
+ * runs with fewer and closer launches: the same histogram in d_hist, the same
+ * LUT in d_lut and the same container.  Arguments, alignment and errors as of
+ * those three; everything is checked before anything is launched. */
+qlc_status qlc_encode_tensor(const uint8_t *d_in, size_t n, const qlc_scheme *h_schemes,
+                             int n_schemes, uint32_t chunk_symbols, uint64_t *d_hist,
+                             qlc_lut *d_lut, uint8_t *d_out, size_t out_cap, void *d_ws,
+                             size_t ws_bytes, uint64_t *d_out_bytes, uint32_t *d_status,
+                             qlc_stream_t stream);
+
 /* Same result as qlc_encode, for callers that cannot allocate device memory
  * (for example a plugin whose host framework's allocator owns the GPU's
  * memory, or a request path that must not call cudaMalloc).  The paper has no

@@ -512,7 +512,7 @@ __device__ __forceinline__ uint32_t enter_shard(const qlc_desc& dd, DecHeader* h
 // lookup than with several tables per CTA: 1152 shards 1764 us, not 1790-1830).
 __global__ void __launch_bounds__(32, kDecCtasPerSm)
 decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
-                    const unsigned long long* __restrict__ item_base, unsigned int* __restrict__ ticket,
+                    const unsigned long long* item_base, unsigned int* ticket,
                     uint32_t* __restrict__ status) {
   __shared__ DecShared sm;
   __shared__ void* volatile s_out;  // the current item's output
@@ -578,8 +578,8 @@ struct FewShared {
 constexpr int kFewWarps = kSpanWarps * kSpanCtasPerSm;
 static_assert(kFewWarps == kFewWarpsPerSm, "plan_kernel compares the groups with these warps");
 __global__ void __launch_bounds__(32 * kFewWarps, 1)
-decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsigned long long* __restrict__ item_base,
-                  unsigned int* __restrict__ ticket, uint32_t* __restrict__ status) {
+decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsigned long long* item_base,
+                  unsigned int* ticket, uint32_t* __restrict__ status) {
   extern __shared__ __align__(16) uint8_t few_sm[];
   __shared__ void* volatile s_out[kFewWarps];  // the warps' current outputs
   __shared__ volatile unsigned long long s_item[kSpanCtasPerSm];

@@ -23,7 +23,7 @@
 #include <utility>
 
 #define QLC_FILE_ID 2
-#include "qlc_common.cuh"
+#include "lut.cuh"
 #include "../../include/qlc_testing.h"
 
 namespace qlc {
@@ -608,14 +608,27 @@ encode_kernel(EncArgs A) {
 //            block that two parts share belongs to the part it starts in, whose
 //            CTA also encodes the up to 43 symbols after the part that reach
 //            into it.
+// With kBuild every CTA ranks the histogram itself (about 1 us), and the first
+// writes the LUT: no kernel of its own between the histogram and this one.
+template <bool kBuild>
 __global__ void __launch_bounds__(kEncThreads)
-lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __restrict__ lut, uint32_t cs, uint8_t* out,
-               uint32_t* status) {
+lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const unsigned long long* __restrict__ hist, SchemeSet set,
+               qlc_lut* lut, uint32_t cs, uint8_t* out, uint32_t* status) {
+  static_assert(kEncThreads == kLutThreads, "a thread per symbol");
   __shared__ __align__(16) uint32_t s_enc[256 * 32];
+  __shared__ unsigned long long s_key[kBuild ? 256 : 1], s_bits[8][kLutThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t n_chunks = (n + cs - 1) / cs;
   dependents_may_start();
-  const uint32_t e = table_entry(lut->enc[tid]);
+  uint32_t e;
+  if constexpr (kBuild) {
+    dependency_wait();
+    const LutRow row = rank_and_choose(hist, set, s_key, s_bits, tid);
+    if (blockIdx.x == 0) write_lut(lut, row, set, tid);
+    e = table_entry(row.entry);
+  } else {
+    e = table_entry(lut->enc[tid]);
+  }
   stage_entry(s_enc, tid, e);
   if (__syncthreads_or(e == 0)) {  // not a LUT of this library: refused
     if (blockIdx.x == 0 && tid == 0) set_status(status, QLC_ERR_ARG);
@@ -633,7 +646,7 @@ lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __rest
 constexpr uint32_t kParts = kGroupChunks / kEncWarps;  // parts per group
 
 __global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm)
-pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __restrict__ lut, uint32_t cs, uint8_t* out,
+pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* lut, uint32_t cs, uint8_t* out,
             uint64_t out_cap, unsigned long long* out_bytes, uint32_t* status) {
   __shared__ __align__(16) uint32_t s_enc[256 * 32];
   __shared__ __align__(16) uint32_t s_stage[kEncWarps][2][kWStage];
@@ -643,7 +656,7 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __restric
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < kEncWarps * 2 * kWStage; i += kEncThreads) (&s_stage[0][0][0])[i] = 0;
   dependency_wait();
-  const uint32_t e = table_entry(lut->enc[tid]);
+  const uint32_t e = table_entry(__ldcg(&lut->enc[tid]));
   stage_entry(s_enc, tid, e);
   if (__syncthreads_or(e == 0)) return;  // lengths_kernel has set the status
   const uint32_t* tab = &s_enc[lane];
@@ -661,7 +674,7 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __restric
     for (uint32_t b = 8 * g_at + 32 * warp; b < 8 * g; b += 32 * kEncWarps) {
       uint32_t bits = 0;
       if (b + lane < 8 * g) {
-        const uint2 q = *reinterpret_cast<const uint2*>(chunk_bits + 4 * (b + lane));
+        const uint2 q = __ldcg(reinterpret_cast<const uint2*>(chunk_bits + 4 * (b + lane)));
         bits = (q.x & 0xFFFFu) + (q.x >> 16) + (q.y & 0xFFFFu) + (q.y >> 16);
       }
 #pragma unroll
@@ -671,7 +684,7 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* __restric
     sum = warp_sum_u64(sum);
     // the group's chunks: bit offsets, in every warp
     const uint32_t cg = g * kGroupChunks + lane;
-    const uint32_t cb = cg < n_chunks ? chunk_bits[cg] : 0u;
+    const uint32_t cb = cg < n_chunks ? __ldcg(&chunk_bits[cg]) : 0u;
     uint32_t incl = cb;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -779,52 +792,105 @@ static int enc_grid(uint64_t items, const qlc_launch* launch) {
   return (int)(items < 1 ? 1 : (items < cap ? items : cap));
 }
 
-qlc_status qlc_encode(const uint8_t* d_in, size_t n, const qlc_lut* d_lut, uint32_t chunk_symbols,
-                      uint8_t* d_out, size_t out_cap, void* d_ws, size_t ws_bytes,
-                      uint64_t* d_out_bytes, uint32_t* d_status, qlc_stream_t stream) {
-  NvtxRange nvtx_range("qlc_encode");
+// Argument checks of the single-tensor encoders.
+static qlc_status check_encode(const uint8_t* d_in, size_t n, const qlc_lut* d_lut, uint32_t chunk_symbols,
+                               const uint8_t* d_out, size_t out_cap, const void* d_ws, size_t ws_bytes,
+                               const uint64_t* d_out_bytes, const uint32_t* d_status) {
   if (!d_lut || !d_out || !d_out_bytes || (n > 0 && (!d_in || !d_ws))) return QLC_ERR_ARG;
   if (!chunk_symbols_ok(chunk_symbols)) return QLC_ERR_ARG;
   if (!aligned(d_in, 16) || !aligned(d_out, 16) || !aligned(d_lut, 16) || !aligned(d_ws, 16) ||
       !aligned(d_out_bytes, 8) || !aligned(d_status, 4))
     return QLC_ERR_ARG;
-  const uint64_t n_chunks = (n + chunk_symbols - 1) / chunk_symbols;
-  if (n_chunks > 0xFFFFFFFFull) return QLC_ERR_ARG;
+  if ((n + chunk_symbols - 1) / chunk_symbols > 0xFFFFFFFFull) return QLC_ERR_ARG;
   if (out_cap < qlc_encoded_size(n, chunk_symbols)) return QLC_ERR_CAPACITY;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (n == 0) {
-    header_only_kernel<<<1, 256, 0, st>>>(d_out, chunk_symbols, d_lut,
-                                          reinterpret_cast<unsigned long long*>(d_out_bytes));
-    return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
-  }
-  const size_t ws_need = qlc_encode_workspace_size(n, chunk_symbols);
-  if (ws_bytes < ws_need) return QLC_ERR_CAPACITY;
-  if (n_chunks <= kPartMaxChunks) {
+  if (n > 0 && ws_bytes < qlc_encode_workspace_size(n, chunk_symbols)) return QLC_ERR_CAPACITY;
+  return QLC_OK;
+}
+
+// Launches the encoder behind the histogram of the same call, building the LUT
+// from it (hist), or with the caller's LUT (hist NULL).  Look-back words are
+// cleared by the caller where clear_lookback says so.
+static bool looks_back(size_t n, uint32_t cs) { return (n + cs - 1) / cs > kPartMaxChunks; }
+static qlc_status clear_lookback(size_t n, uint32_t cs, void* d_ws, cudaStream_t st) {
+  if (!looks_back(n, cs)) return QLC_OK;
+  return cudaMemsetAsync(d_ws, 0, qlc_encode_workspace_size(n, cs), st) == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+}
+static qlc_status launch_encode(const uint8_t* d_in, size_t n, const uint64_t* d_hist, const SchemeSet& set, qlc_lut* d_lut,
+                                uint32_t cs, uint8_t* d_out, size_t out_cap, void* d_ws, size_t ws_bytes,
+                                uint64_t* d_out_bytes, uint32_t* d_status, cudaStream_t st) {
+  unsigned long long* ob = reinterpret_cast<unsigned long long*>(d_out_bytes);
+  const unsigned long long* hist = reinterpret_cast<const unsigned long long*>(d_hist);
+  const uint64_t n_chunks = (n + cs - 1) / cs;
+  if (n > 0 && !looks_back(n, cs)) {
     const int sms = sm_count(), parts = (int)(n_groups_of(n_chunks) * kParts);
-    const int want = (int)((n_chunks + kEncWarps - 1) / kEncWarps);
-    lengths_kernel<<<want < 6 * sms ? want : 6 * sms, kEncThreads, 0, st>>>(d_in, n, d_lut, chunk_symbols, d_out,
-                                                                            d_status);
+    const int want = (int)((n_chunks + kEncWarps - 1) / kEncWarps), grid = want < 6 * sms ? want : 6 * sms;
+    if (hist)
+      launch_after(lengths_kernel<true>, grid, kEncThreads, 0, st, d_in, n, hist, set, d_lut, cs, d_out, d_status);
+    else
+      lengths_kernel<false><<<grid, kEncThreads, 0, st>>>(d_in, n, nullptr, set, d_lut, cs, d_out, d_status);
     if (cudaGetLastError() != cudaSuccess) return QLC_ERR_CUDA;
     launch_after(pack_kernel, parts < kEncCtasPerSm * sms ? parts : kEncCtasPerSm * sms, kEncThreads, 0, st, d_in, n, d_lut,
-                 chunk_symbols, d_out, out_cap, reinterpret_cast<unsigned long long*>(d_out_bytes), d_status);
+                 cs, d_out, out_cap, ob, d_status);
     return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
   }
-  if (cudaMemsetAsync(d_ws, 0, ws_need, st) != cudaSuccess) return QLC_ERR_CUDA;
+  if (hist) {
+    const qlc_status s = launch_luts(d_hist, 1, set, d_lut, n > 0, st);
+    if (s != QLC_OK) return s;
+  }
+  if (n == 0) {
+    header_only_kernel<<<1, 256, 0, st>>>(d_out, cs, d_lut, ob);
+    return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  }
   EncArgs A = {};
   A.in = d_in;
   A.n = n;
   A.lut = d_lut;
   A.out = d_out;
-  A.out_bytes = reinterpret_cast<unsigned long long*>(d_out_bytes);
+  A.out_bytes = ob;
   A.n_items = n_groups_of(n_chunks);
-  A.cs = chunk_symbols;
+  A.cs = cs;
   A.ticket = static_cast<unsigned int*>(d_ws);
   A.gstat = reinterpret_cast<unsigned long long*>(static_cast<uint8_t*>(d_ws) + 16);
   A.status = d_status;
   A.out_cap = out_cap;
   A.gstat_cap = (ws_bytes - 16) / 8;
-  encode_kernel<<<enc_grid(A.n_items, nullptr), kEncThreads, 0, st>>>(A);
+  if (hist)
+    launch_after(encode_kernel, enc_grid(A.n_items, nullptr), kEncThreads, 0, st, A);
+  else
+    encode_kernel<<<enc_grid(A.n_items, nullptr), kEncThreads, 0, st>>>(A);
   return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+}
+
+qlc_status qlc_encode(const uint8_t* d_in, size_t n, const qlc_lut* d_lut, uint32_t chunk_symbols,
+                      uint8_t* d_out, size_t out_cap, void* d_ws, size_t ws_bytes,
+                      uint64_t* d_out_bytes, uint32_t* d_status, qlc_stream_t stream) {
+  NvtxRange nvtx_range("qlc_encode");
+  qlc_status s = check_encode(d_in, n, d_lut, chunk_symbols, d_out, out_cap, d_ws, ws_bytes, d_out_bytes, d_status);
+  if (s != QLC_OK) return s;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  s = clear_lookback(n, chunk_symbols, d_ws, st);
+  if (s != QLC_OK) return s;
+  SchemeSet none;
+  none.count = 0;
+  return launch_encode(d_in, n, nullptr, none, const_cast<qlc_lut*>(d_lut), chunk_symbols, d_out, out_cap, d_ws, ws_bytes,
+                       d_out_bytes, d_status, st);
+}
+
+qlc_status qlc_encode_tensor(const uint8_t* d_in, size_t n, const qlc_scheme* h_schemes, int n_schemes,
+                             uint32_t chunk_symbols, uint64_t* d_hist, qlc_lut* d_lut, uint8_t* d_out, size_t out_cap,
+                             void* d_ws, size_t ws_bytes, uint64_t* d_out_bytes, uint32_t* d_status,
+                             qlc_stream_t stream) {
+  NvtxRange nvtx_range("qlc_encode_tensor");
+  SchemeSet set;
+  if (!d_hist || !aligned(d_hist, 8) || !scheme_set(h_schemes, n_schemes, &set)) return QLC_ERR_ARG;
+  qlc_status s = check_encode(d_in, n, d_lut, chunk_symbols, d_out, out_cap, d_ws, ws_bytes, d_out_bytes, d_status);
+  if (s != QLC_OK) return s;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  s = clear_lookback(n, chunk_symbols, d_ws, st);  // before the kernels, which then follow one another directly
+  if (s == QLC_OK) s = launch_histogram(d_in, n, d_hist, 0, st);
+  if (s != QLC_OK) return s;
+  return launch_encode(d_in, n, d_hist, set, d_lut, chunk_symbols, d_out, out_cap, d_ws, ws_bytes, d_out_bytes, d_status,
+                       st);
 }
 
 qlc_status qlc_test_encode_stalled_lookback(const uint8_t* d_in, size_t n, const qlc_lut* d_lut,

@@ -2,6 +2,7 @@
 // kernels of libqlc, plus their C-ABI entry points.
 #define QLC_FILE_ID 3
 #include "hist_cols.cuh"
+#include "lut.cuh"
 #include "../../include/qlc_testing.h"
 
 #include <algorithm>
@@ -18,6 +19,7 @@ __global__ void __launch_bounds__(kHcThreads, 1)
 hist_kernel(const uint8_t* __restrict__ in, uint64_t n, unsigned long long* __restrict__ hist, bool overwrite) {
   __shared__ __align__(16) uint32_t cols[kHcColWords];
   const int tid = threadIdx.x, lane = tid & 31;
+  dependents_may_start();
   zero_cols(cols, tid);
   __syncthreads();
   const uint32_t col = lane_col(cols, lane);
@@ -40,102 +42,16 @@ hist_kernel(const uint8_t* __restrict__ in, uint64_t n, unsigned long long* __re
 // and no memset precedes it.
 constexpr uint64_t kHistCtaVecs = 4096;
 
-// Rank of a symbol (Section 7): symbols with a larger count, or the same
-// count and a smaller value, come first.  With key(t) = count(t) * 256 +
-// (255 - t), which is unique and orders exactly that way (counts stay below
-// 2^56), the rank of s is the number of keys above key(s): no sort, one
-// comparison per key.  One thread per symbol; all threads read the same key
-// at a time (a broadcast).
-constexpr int kLutThreads = 256;
-
-__device__ __forceinline__ void load_keys(const unsigned long long* __restrict__ hist, unsigned long long* key,
-                                          int tid) {
-  key[tid] = (hist[tid] << 8) | (unsigned long long)(255 - tid);
-}
-
-// The rank of symbol s.
-__device__ __forceinline__ int rank_of(const unsigned long long* key, int s) {
-  const unsigned long long k = key[s];
-  int r = 0;
-#pragma unroll 16
-  for (int t = 0; t < 256; t++) r += key[t] > k;
-  return r;
-}
-
-// Codeword of a rank under a scheme (Section 5): area code i, then the
-// rank's position in area i in area_bits[i] bits; 8-bit areas store the rank.
-__host__ __device__ inline uint32_t lut_entry(const qlc_scheme& sc, int r) {
-  uint32_t base = 0;
-  for (int i = 0; i < 8; i++) {
-    const uint32_t n = sc.area_n[i];
-    if ((uint32_t)r < base + n) {
-      const uint32_t b = sc.area_bits[i];
-      const uint32_t suffix = b == 8 ? (uint32_t)r : (uint32_t)r - base;
-      const uint32_t code = ((uint32_t)i << b) | suffix;
-      return (code << 4) | (3 + b);
-    }
-    base += n;
-  }
-  return 0;
-}
-
-__global__ void __launch_bounds__(kLutThreads)
-lut_kernel(const unsigned long long* __restrict__ hist, qlc_scheme sc, qlc_lut* __restrict__ lut) {
-  __shared__ unsigned long long key[256];
-  const int tid = threadIdx.x;
-  load_keys(hist, key, tid);
-  __syncthreads();
-  const int s = tid;
-  const int r = rank_of(key, s);
-  lut->enc[s] = (uint16_t)lut_entry(sc, r);
-  lut->dec[r] = (uint8_t)s;
-  if (tid < (int)(sizeof(qlc_scheme) / 4))
-    reinterpret_cast<uint32_t*>(&lut->scheme)[tid] = reinterpret_cast<const uint32_t*>(&sc)[tid];
-}
-
-struct SchemeSet {
-  qlc_scheme s[8];
-  int count;
-};
-
-// Section 6: the scheme can be adapted to the distribution.  Each candidate
-// is scored by its payload bits sum_s count[s] * len(rank[s]) and the
-// smallest wins (ties: the earlier candidate).
 // One CTA per histogram: CTA b builds luts[b] from hists[b * 256 ...].
 __global__ void __launch_bounds__(kLutThreads)
 lut_best_kernel(const unsigned long long* __restrict__ hists, SchemeSet set, qlc_lut* __restrict__ luts) {
-  constexpr int kWarps = kLutThreads / 32;
   __shared__ unsigned long long key[256];
-  __shared__ unsigned long long bits[8][kWarps];
-  const unsigned long long* hist = hists + (size_t)blockIdx.x * 256;
-  qlc_lut* lut = luts + blockIdx.x;
+  __shared__ unsigned long long bits[8][kLutThreads / 32];
   const int tid = threadIdx.x;
-  load_keys(hist, key, tid);
-  __syncthreads();
-  const int s = tid, warp = tid >> 5, lane = tid & 31;
-  const int r = rank_of(key, s);
-  const unsigned long long count = key[s] >> 8;
-  for (int k = 0; k < set.count; k++) {
-    unsigned long long v = count * (unsigned long long)(lut_entry(set.s[k], r) & 15u);
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) bits[k][warp] = v;
-  }
-  __syncthreads();
-  int best = 0;
-  unsigned long long best_bits = ~0ull;
-  for (int k = 0; k < set.count; k++) {
-    unsigned long long t = 0;
-    for (int w = 0; w < kWarps; w++) t += bits[k][w];
-    if (t < best_bits) {
-      best_bits = t;
-      best = k;
-    }
-  }
-  const qlc_scheme& sc = set.s[best];
-  lut->enc[s] = (uint16_t)lut_entry(sc, r);
-  lut->dec[r] = (uint8_t)s;
-  if (tid < (int)(sizeof(qlc_scheme) / 4))
-    reinterpret_cast<uint32_t*>(&lut->scheme)[tid] = reinterpret_cast<const uint32_t*>(&sc)[tid];
+  dependents_may_start();
+  dependency_wait();
+  const LutRow row = rank_and_choose(hists + (size_t)blockIdx.x * 256, set, key, bits, tid);
+  write_lut(luts + blockIdx.x, row, set, tid);
 }
 
 int sm_count() {
@@ -179,6 +95,48 @@ static qlc_scheme clean_scheme(const qlc_scheme* s) {
   return c;
 }
 
+namespace qlc {
+
+bool scheme_set(const qlc_scheme* h_schemes, int n_schemes, SchemeSet* set) {
+  if (!h_schemes || n_schemes < 1 || n_schemes > 8) return false;
+  set->count = n_schemes;
+  for (int k = 0; k < n_schemes; k++) {
+    if (!scheme_valid(&h_schemes[k])) return false;
+    set->s[k] = clean_scheme(&h_schemes[k]);
+  }
+  return true;
+}
+
+qlc_status launch_histogram(const uint8_t* d_in, size_t n, uint64_t* d_hist, int accumulate, cudaStream_t st) {
+  // One CTA per SM, at least kHistCtaVecs vectors each; a CTA counts under
+  // 2^31 bytes.
+  const uint64_t nvec = n / 16;
+  uint64_t grid = (nvec + kHistCtaVecs - 1) / kHistCtaVecs;
+  const uint64_t cap = (uint64_t)sm_count();
+  if (grid > cap) grid = cap;
+  const uint64_t floor_grid = (nvec >> 27) + 1;
+  if (grid < floor_grid) grid = floor_grid;
+  if (grid > 0x7fffffffu) return QLC_ERR_ARG;
+  const bool overwrite = !accumulate && n > 0 && grid == 1;
+  if (!accumulate && !overwrite && cudaMemsetAsync(d_hist, 0, 256 * sizeof(uint64_t), st) != cudaSuccess)
+    return QLC_ERR_CUDA;
+  if (n == 0) return QLC_OK;
+  hist_kernel<<<(int)grid, kHcThreads, 0, st>>>(d_in, n, reinterpret_cast<unsigned long long*>(d_hist), overwrite);
+  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+}
+
+qlc_status launch_luts(const uint64_t* d_hists, int n_luts, const SchemeSet& set, qlc_lut* d_luts, bool after,
+                       cudaStream_t st) {
+  const unsigned long long* h = reinterpret_cast<const unsigned long long*>(d_hists);
+  if (after)
+    launch_after(lut_best_kernel, n_luts, kLutThreads, 0, st, h, set, d_luts);
+  else
+    lut_best_kernel<<<n_luts, kLutThreads, 0, st>>>(h, set, d_luts);
+  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+}
+
+}  // namespace qlc
+
 extern "C" {
 
 int qlc_version(void) { return QLC_VERSION; }
@@ -209,22 +167,7 @@ qlc_status qlc_histogram(const uint8_t* d_in, size_t n, uint64_t* d_hist, int ac
   NvtxRange nvtx_range("qlc_histogram");
   if (!d_hist || (n > 0 && !d_in)) return QLC_ERR_ARG;
   if (!aligned(d_in, 16) || !aligned(d_hist, 8)) return QLC_ERR_ARG;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  // One CTA per SM, at least kHistCtaVecs vectors each; a CTA counts under
-  // 2^31 bytes.
-  const uint64_t nvec = n / 16;
-  uint64_t grid = (nvec + kHistCtaVecs - 1) / kHistCtaVecs;
-  const uint64_t cap = (uint64_t)sm_count();
-  if (grid > cap) grid = cap;
-  const uint64_t floor_grid = (nvec >> 27) + 1;
-  if (grid < floor_grid) grid = floor_grid;
-  if (grid > 0x7fffffffu) return QLC_ERR_ARG;
-  const bool overwrite = !accumulate && n > 0 && grid == 1;
-  if (!accumulate && !overwrite && cudaMemsetAsync(d_hist, 0, 256 * sizeof(uint64_t), st) != cudaSuccess)
-    return QLC_ERR_CUDA;
-  if (n == 0) return QLC_OK;
-  hist_kernel<<<(int)grid, kHcThreads, 0, st>>>(d_in, n, reinterpret_cast<unsigned long long*>(d_hist), overwrite);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  return launch_histogram(d_in, n, d_hist, accumulate, reinterpret_cast<cudaStream_t>(stream));
 }
 
 qlc_status qlc_build_lut(const uint64_t* d_hist, const qlc_scheme* h_scheme, qlc_lut* d_lut,
@@ -232,9 +175,10 @@ qlc_status qlc_build_lut(const uint64_t* d_hist, const qlc_scheme* h_scheme, qlc
   NvtxRange nvtx_range("qlc_build_lut");
   if (!d_hist || !d_lut || !scheme_valid(h_scheme)) return QLC_ERR_ARG;
   if (!aligned(d_hist, 8) || !aligned(d_lut, 16)) return QLC_ERR_ARG;
-  lut_kernel<<<1, kLutThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      reinterpret_cast<const unsigned long long*>(d_hist), clean_scheme(h_scheme), d_lut);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  SchemeSet set;
+  set.count = 1;
+  set.s[0] = clean_scheme(h_scheme);
+  return launch_luts(d_hist, 1, set, d_lut, false, reinterpret_cast<cudaStream_t>(stream));
 }
 
 qlc_status qlc_build_lut_best(const uint64_t* d_hist, const qlc_scheme* h_schemes, int n_schemes,
@@ -243,14 +187,8 @@ qlc_status qlc_build_lut_best(const uint64_t* d_hist, const qlc_scheme* h_scheme
   if (!d_hist || !d_lut || !h_schemes || n_schemes < 1 || n_schemes > 8) return QLC_ERR_ARG;
   if (!aligned(d_hist, 8) || !aligned(d_lut, 16)) return QLC_ERR_ARG;
   SchemeSet set;
-  set.count = n_schemes;
-  for (int k = 0; k < n_schemes; k++) {
-    if (!scheme_valid(&h_schemes[k])) return QLC_ERR_ARG;
-    set.s[k] = clean_scheme(&h_schemes[k]);
-  }
-  lut_best_kernel<<<1, kLutThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      reinterpret_cast<const unsigned long long*>(d_hist), set, d_lut);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  if (!scheme_set(h_schemes, n_schemes, &set)) return QLC_ERR_ARG;
+  return launch_luts(d_hist, 1, set, d_lut, false, reinterpret_cast<cudaStream_t>(stream));
 }
 
 qlc_status qlc_build_lut_batch(const uint64_t* d_hists, int n_luts, const qlc_scheme* h_schemes,
@@ -260,14 +198,8 @@ qlc_status qlc_build_lut_batch(const uint64_t* d_hists, int n_luts, const qlc_sc
     return QLC_ERR_ARG;
   if (!aligned(d_hists, 8) || !aligned(d_luts, 16)) return QLC_ERR_ARG;
   SchemeSet set;
-  set.count = n_schemes;
-  for (int k = 0; k < n_schemes; k++) {
-    if (!scheme_valid(&h_schemes[k])) return QLC_ERR_ARG;
-    set.s[k] = clean_scheme(&h_schemes[k]);
-  }
-  lut_best_kernel<<<n_luts, kLutThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      reinterpret_cast<const unsigned long long*>(d_hists), set, d_luts);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  if (!scheme_set(h_schemes, n_schemes, &set)) return QLC_ERR_ARG;
+  return launch_luts(d_hists, n_luts, set, d_luts, false, reinterpret_cast<cudaStream_t>(stream));
 }
 
 qlc_status qlc_build_lut_host(const uint64_t* h_hist, const qlc_scheme* h_scheme, qlc_lut* h_lut) {

@@ -156,7 +156,7 @@ __device__ __forceinline__ uint32_t e4m3_scaled_bits(uint32_t w, int j) {
 // whose entry is <= t narrows it, so 1152 shards take 3 rounds of loads
 // instead of the 11 dependent loads of a binary search.  Every lane returns
 // the same shard.
-__device__ __forceinline__ int shard_of_warp(const unsigned long long* __restrict__ item_base, int n_shards,
+__device__ __forceinline__ int shard_of_warp(const unsigned long long* item_base, int n_shards,
                                              unsigned long long t, int lane) {
   int lo = 0, hi = n_shards;  // item_base[lo] <= t; the shard lies in [lo, hi)
   while (hi - lo > 1) {
@@ -176,7 +176,9 @@ int sm_count();
 // with launch_after, directly behind another kernel of the same call, may have
 // its CTAs resident, and the launch itself behind it, while that kernel still
 // runs: that one calls dependents_may_start(), and this one touches no memory
-// before dependency_wait(), which returns when that kernel is complete.  The
+// before dependency_wait(), which returns when that kernel is complete, and
+// reads what that kernel wrote without the read-only cache (no __restrict__ on
+// such pointers, or __ldcg).  The
 // first kernel of a call is launched as usual: what comes before it in the
 // stream is not known (behind a memset node of a captured graph, the wait does
 // not hold).

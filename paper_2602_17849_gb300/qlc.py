@@ -72,6 +72,7 @@ def _load() -> ctypes.CDLL:
     L.qlc_encode_workspace_size.argtypes = [sz, u32]
     L.qlc_encode_workspace_size.restype = sz
     L.qlc_encode.argtypes = [P, sz, P, u32, P, sz, P, sz, P, P, P]
+    L.qlc_encode_tensor.argtypes = [P, sz, P, i32, u32, P, P, P, sz, P, sz, P, P, P]
     L.qlc_decode.argtypes = [P, sz, P, sz, P, P, P]
     L.qlc_peek_header.argtypes = [P, sz, P, P]
     L.qlc_scheme_search.argtypes = [P, P, P]
@@ -88,7 +89,7 @@ def _load() -> ctypes.CDLL:
     L.qlc_dequantize_e4m3.argtypes = [P, P, sz, P, i32, P]
     L.qlc_decode_dequantize.argtypes = [P, sz, P, P, i32, sz, P, P, P]
     for f in ("qlc_scheme_table", "qlc_histogram", "qlc_build_lut", "qlc_build_lut_host",
-              "qlc_build_lut_best", "qlc_encode", "qlc_decode", "qlc_peek_header", "qlc_encode_noalloc",
+              "qlc_build_lut_best", "qlc_encode", "qlc_encode_tensor", "qlc_decode", "qlc_peek_header", "qlc_encode_noalloc",
               "qlc_histogram_batch", "qlc_build_lut_batch", "qlc_encode_batch", "qlc_decode_batch",
               "qlc_quantize_e4m3", "qlc_dequantize_e4m3", "qlc_decode_dequantize"):
         getattr(L, f).restype = i32
@@ -96,10 +97,13 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:  # what current_stream() returns, without building a Stream object
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -156,6 +160,22 @@ def as_scheme(scheme) -> qlc_scheme:
         return qlc_scheme_table(scheme)
     n, b = scheme[0], scheme[1]
     return make_scheme(n, b, scheme[2] if len(scheme) > 2 else 0)
+
+
+_scheme_arrays = {}  # (1,), (2,), (1, 2), (2, 1): the paper's tables never change
+
+
+def _scheme_array(schemes):
+    """(ctypes array, count) of a scheme or a list of candidates."""
+    schemes = schemes if isinstance(schemes, list) else [schemes]
+    if len(schemes) <= 2 and all(type(s) is int for s in schemes):
+        key = tuple(schemes)
+        arr = _scheme_arrays.get(key)
+        if arr is None:
+            arr = (qlc_scheme * len(key))(*[qlc_scheme_table(s) for s in key])
+            _scheme_arrays[key] = arr
+        return arr, len(key)
+    return (qlc_scheme * len(schemes))(*[as_scheme(s) for s in schemes]), len(schemes)
 
 
 def qlc_scheme_check(scheme) -> bool:
@@ -219,6 +239,17 @@ def qlc_encode(d_in: torch.Tensor, d_lut: torch.Tensor, chunk_symbols: int, d_ou
     _check(lib.qlc_encode(_ptr(d_in), n, _ptr(d_lut), int(chunk_symbols), _ptr(d_out), _nbytes(d_out),
                           _ptr(d_ws), _nbytes(d_ws) if d_ws is not None else 0, _ptr(d_out_bytes),
                           _ptr(d_status), _stream(stream)), "qlc_encode")
+
+
+def qlc_encode_tensor(d_in: torch.Tensor, schemes, chunk_symbols: int, d_hist: torch.Tensor, d_lut: torch.Tensor,
+                      d_out: torch.Tensor, d_ws: torch.Tensor, d_out_bytes: torch.Tensor, d_status: torch.Tensor,
+                      n: int | None = None, stream=None) -> None:
+    """Histogram, LUT (a scheme, or the best of a list) and container in one call."""
+    arr, count = _scheme_array(schemes)
+    n = _nbytes(d_in) if n is None else n
+    _check(lib.qlc_encode_tensor(_ptr(d_in), n, arr, count, int(chunk_symbols), _ptr(d_hist), _ptr(d_lut),
+                                 _ptr(d_out), _nbytes(d_out), _ptr(d_ws), _nbytes(d_ws) if d_ws is not None else 0,
+                                 _ptr(d_out_bytes), _ptr(d_status), _stream(stream)), "qlc_encode_tensor")
 
 
 def qlc_decode(d_in: torch.Tensor, d_out: torch.Tensor, d_n_out: torch.Tensor, d_status: torch.Tensor,
@@ -338,6 +369,10 @@ def _align16(v: int) -> int:
 
 # ------------------------------------------------------------ conveniences
 
+_CODEC_RESULTS = 2048 + 1024           # after the histogram and the LUT (800 bytes)
+_CODEC_WS = _CODEC_RESULTS + 3 * 8     # after out_bytes, n_out and status ...
+_CODEC_WS += -_CODEC_WS % 16           # ... 16-byte aligned
+
 class Codec:
     """Device buffers for encoding/decoding tensors of up to `max_n` symbols.
 
@@ -353,15 +388,18 @@ class Codec:
         cap = qlc_encoded_size(self.max_n, self.chunk_symbols)
         if cap == 0:
             raise QlcError(ERR_ARG, "chunk_symbols")
-        z = dict(device=self.device)
         self.cap = cap
-        self.hist = torch.zeros(256, dtype=torch.int64, **z)
-        self.lut = torch.zeros(LUT_BYTES, dtype=torch.uint8, **z)
-        self.ws = torch.zeros(max(16, qlc_encode_workspace_size(self.max_n, self.chunk_symbols)),
-                              dtype=torch.uint8, **z)
-        self.out_bytes = torch.zeros(1, dtype=torch.int64, **z)
-        self.n_out = torch.zeros(1, dtype=torch.int64, **z)
-        self.status = torch.zeros(1, dtype=torch.int32, **z)
+        # one zeroed allocation: histogram, LUT, results, workspace
+        ws = max(16, qlc_encode_workspace_size(self.max_n, self.chunk_symbols))
+        buf = torch.zeros(_CODEC_WS + ws, dtype=torch.uint8, device=self.device)
+        words = buf[_CODEC_RESULTS:_CODEC_RESULTS + 24].view(torch.int64)
+        self.hist = buf[:2048].view(torch.int64)
+        self.lut = buf[2048:2048 + LUT_BYTES]
+        self.out_bytes = words[0:1]
+        self.n_out = words[1:2]
+        self.status = words[2:3].view(torch.int32)[:1]
+        self.ws = buf[_CODEC_WS:]
+        self._results = words  # out_bytes, n_out, status: read back together
 
     def new_container(self) -> torch.Tensor:
         return torch.empty(self.cap, dtype=torch.uint8, device=self.device)
@@ -370,11 +408,9 @@ class Codec:
         """Histogram -> LUT (self.scheme, or the best of a list) -> container."""
         n = x.numel()
         if build_lut:
-            qlc_histogram(x, self.hist, n=n, stream=stream)
-            if isinstance(self.scheme, list):  # several candidates: the best for this histogram
-                qlc_build_lut_best(self.hist, self.scheme, self.lut, stream=stream)
-            else:
-                qlc_build_lut(self.hist, self.scheme, self.lut, stream=stream)
+            qlc_encode_tensor(x, self.scheme, self.chunk_symbols, self.hist, self.lut, out, self.ws, self.out_bytes,
+                              self.status, n=n, stream=stream)
+            return
         qlc_encode(x, self.lut, self.chunk_symbols, out, self.ws, self.out_bytes, self.status,
                    n=n, stream=stream)
 
@@ -394,18 +430,19 @@ def encode(x: torch.Tensor, scheme=1, chunk_symbols: int = 4096) -> torch.Tensor
     codec = Codec(max(x.numel(), 1), chunk_symbols, scheme, x.device)
     out = codec.new_container()
     codec.encode_into(x.reshape(-1), out)
-    codec.check()
-    return out[: int(codec.out_bytes.item())]
+    nbytes, _, status = codec._results.tolist()  # one read-back, which waits for the encoder
+    if status != OK:
+        raise QlcError(status, "device")
+    return out[:nbytes]
 
 
 def decode(container: torch.Tensor) -> torch.Tensor:
     """Decoded bytes of a CUDA container (synchronises to size the output)."""
     n, total = qlc_peek_header(container[:HEADER_BYTES].cpu().numpy().tobytes())
     out = torch.empty(max(n, 1), dtype=torch.uint8, device=container.device)
-    n_out = torch.zeros(1, dtype=torch.int64, device=container.device)
-    status = torch.zeros(1, dtype=torch.int32, device=container.device)
-    qlc_decode(container, out, n_out, status, out_cap=n)
-    st = int(status.item())
+    words = torch.zeros(2, dtype=torch.int64, device=container.device)  # n_out, status
+    qlc_decode(container, out, words[:1], words[1:].view(torch.int32)[:1], out_cap=n)
+    st = words.tolist()[1]
     if st != OK:
         raise QlcError(st, "qlc_decode")
     return out[:n]
