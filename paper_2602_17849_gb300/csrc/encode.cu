@@ -146,12 +146,13 @@ __device__ unsigned long long lookback(unsigned long long* gstat, uint64_t g, ui
   return excl;
 }
 
-__device__ void write_header(uint8_t* out, uint64_t n, uint32_t cs, uint64_t n_chunks,
-                             const qlc_lut* lut, int tid) {
+// The header but its dec; every thread of a CTA of 256 calls it.
+__device__ void write_header_of(uint8_t* out, uint64_t n, uint32_t cs, uint64_t n_chunks, const qlc_scheme* scheme,
+                                int tid) {
   if (tid == 0) {
     *reinterpret_cast<uint32_t*>(out + 0) = 0x31434C51u;  // "QLC1"
     *reinterpret_cast<uint16_t*>(out + 4) = QLC_VERSION;
-    out[6] = lut->scheme.id;
+    out[6] = scheme->id;
     out[7] = 0;
     *reinterpret_cast<unsigned long long*>(out + 8) = n;
     *reinterpret_cast<uint32_t*>(out + 16) = cs;
@@ -159,13 +160,16 @@ __device__ void write_header(uint8_t* out, uint64_t n, uint32_t cs, uint64_t n_c
     *reinterpret_cast<unsigned long long*>(out + 56) = 0;
   }
   if (tid < 8) {
-    *reinterpret_cast<uint16_t*>(out + 24 + 2 * tid) = lut->scheme.area_n[tid];
-    out[40 + tid] = lut->scheme.area_bits[tid];
+    *reinterpret_cast<uint16_t*>(out + 24 + 2 * tid) = scheme->area_n[tid];
+    out[40 + tid] = scheme->area_bits[tid];
   }
-  if (tid < 256) out[64 + tid] = lut->dec[tid];
   const uint64_t idx_end = kIndexOff + 8 * n_groups_of(n_chunks) + 2 * n_chunks;
   const uint64_t P = payload_start(n_chunks);
   if (idx_end + tid < P) out[idx_end + tid] = 0;
+}
+__device__ void write_header(uint8_t* out, uint64_t n, uint32_t cs, uint64_t n_chunks, const qlc_lut* lut, int tid) {
+  write_header_of(out, n, cs, n_chunks, &lut->scheme, tid);
+  if (tid < 256) out[64 + tid] = lut->dec[tid];
 }
 
 // Work source of the encode kernel: one tensor (descs == nullptr), or the
@@ -616,7 +620,8 @@ lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const unsigned long l
                qlc_lut* lut, uint32_t cs, uint8_t* out, uint32_t* status) {
   static_assert(kEncThreads == kLutThreads, "a thread per symbol");
   __shared__ __align__(16) uint32_t s_enc[256 * 32];
-  __shared__ unsigned long long s_key[kBuild ? 256 : 1], s_bits[8][kLutThreads / 32];
+  __shared__ __align__(16) unsigned long long s_key[kBuild ? 256 : 2];
+  __shared__ unsigned long long s_bits[8][kLutThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t n_chunks = (n + cs - 1) / cs;
   dependents_may_start();
@@ -624,7 +629,11 @@ lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const unsigned long l
   if constexpr (kBuild) {
     dependency_wait();
     const LutRow row = rank_and_choose(hist, set, s_key, s_bits, tid);
-    if (blockIdx.x == 0) write_lut(lut, row, set, tid);
+    if (blockIdx.x == 0) {
+      write_lut(lut, row, set, tid);
+      write_header_of(out, n, cs, n_chunks, &set.s[row.scheme], tid);
+      out[64 + row.rank] = (uint8_t)tid;
+    }
     e = table_entry(row.entry);
   } else {
     e = table_entry(lut->enc[tid]);
@@ -634,7 +643,7 @@ lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const unsigned long l
     if (blockIdx.x == 0 && tid == 0) set_status(status, QLC_ERR_ARG);
     return;
   }
-  if (blockIdx.x == 0) write_header(out, n, cs, n_chunks, lut, tid);
+  if (!kBuild && blockIdx.x == 0) write_header(out, n, cs, n_chunks, lut, tid);
   uint16_t* chunk_bits = reinterpret_cast<uint16_t*>(out + kIndexOff + 8 * n_groups_of(n_chunks));
   for (uint64_t c = (uint64_t)blockIdx.x * kEncWarps + warp; c < n_chunks; c += (uint64_t)gridDim.x * kEncWarps) {
     const uint64_t beg = c * cs;

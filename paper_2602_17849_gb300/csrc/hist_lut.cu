@@ -45,7 +45,7 @@ constexpr uint64_t kHistCtaVecs = 4096;
 // One CTA per histogram: CTA b builds luts[b] from hists[b * 256 ...].
 __global__ void __launch_bounds__(kLutThreads)
 lut_best_kernel(const unsigned long long* __restrict__ hists, SchemeSet set, qlc_lut* __restrict__ luts) {
-  __shared__ unsigned long long key[256];
+  __shared__ __align__(16) unsigned long long key[256];
   __shared__ unsigned long long bits[8][kLutThreads / 32];
   const int tid = threadIdx.x;
   dependents_may_start();

@@ -14,17 +14,29 @@ namespace qlc {
 // at a time (a broadcast).
 constexpr int kLutThreads = 256;
 
-__device__ __forceinline__ void load_keys(const unsigned long long* __restrict__ hist, unsigned long long* key,
-                                          int tid) {
-  key[tid] = (__ldcg(hist + tid) << 8) | (unsigned long long)(255 - tid);  // from L2: the kernel before may have just written it
+// From L2: the kernel before may have just written the counts.
+__device__ __forceinline__ unsigned long long load_key(const unsigned long long* __restrict__ hist, int s) {
+  return (__ldcg(hist + s) << 8) | (unsigned long long)(255 - s);
 }
 
-// The rank of symbol s.
+// The rank of symbol s.  Keys of a tensor below 2^24 symbols fit in 32 bits
+// (small): a comparison and an add per key, where 64 bits take three operations
+// and twice the loads.
 __device__ __forceinline__ int rank_of(const unsigned long long* key, int s) {
   const unsigned long long k = key[s];
   int r = 0;
 #pragma unroll 16
   for (int t = 0; t < 256; t++) r += key[t] > k;
+  return r;
+}
+__device__ __forceinline__ int rank_of_small(const uint32_t* key, int s) {
+  const uint32_t k = key[s];
+  int r = 0;
+#pragma unroll 8
+  for (int t = 0; t < 64; t++) {
+    const uint4 q = reinterpret_cast<const uint4*>(key)[t];
+    r += (q.x > k) + (q.y > k) + (q.z > k) + (q.w > k);
+  }
   return r;
 }
 
@@ -61,18 +73,24 @@ struct LutRow {
 // Ranks the symbols of a histogram and picks the scheme (Section 6: the scheme
 // can be adapted to the distribution): each candidate is scored by its payload
 // bits sum_s count[s] * len(rank[s]) and the smallest wins (ties: the earlier
-// candidate).  Thread s is symbol s.  key and bits are scratch.
+// candidate).  Thread s is symbol s.  key (256 entries, 16-byte aligned) and bits are scratch.
 __device__ __forceinline__ LutRow rank_and_choose(const unsigned long long* __restrict__ hist, const SchemeSet& set,
-                                                  unsigned long long (&key)[256],
+                                                  unsigned long long* key,
                                                   unsigned long long (&bits)[8][kLutThreads / 32], int tid) {
-  load_keys(hist, key, tid);
+  // (the counts are bounded by their sum, but the caller's histogram may be any)
+  const unsigned long long own = load_key(hist, tid);
+  const bool small = !__syncthreads_or(own >> 32 != 0);
+  if (small)
+    reinterpret_cast<uint32_t*>(key)[tid] = (uint32_t)own;
+  else
+    key[tid] = own;
   __syncthreads();
   LutRow row;
-  row.rank = rank_of(key, tid);
+  row.rank = small ? rank_of_small(reinterpret_cast<const uint32_t*>(key), tid) : rank_of(key, tid);
   row.scheme = 0;
   if (set.count > 1) {
     const int warp = tid >> 5, lane = tid & 31;
-    const unsigned long long count = key[tid] >> 8;
+    const unsigned long long count = own >> 8;
     for (int k = 0; k < set.count; k++) {
       unsigned long long v = count * (unsigned long long)(lut_entry(set.s[k], row.rank) & 15u);
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

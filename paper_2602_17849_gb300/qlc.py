@@ -427,10 +427,20 @@ class Codec:
 
 def encode(x: torch.Tensor, scheme=1, chunk_symbols: int = 4096) -> torch.Tensor:
     """Container of a CUDA uint8 tensor, trimmed to its size (synchronises)."""
-    codec = Codec(max(x.numel(), 1), chunk_symbols, scheme, x.device)
-    out = codec.new_container()
-    codec.encode_into(x.reshape(-1), out)
-    nbytes, _, status = codec._results.tolist()  # one read-back, which waits for the encoder
+    x = x.reshape(-1)
+    n, chunk_symbols = x.numel(), int(chunk_symbols)
+    cap = qlc_encoded_size(n, chunk_symbols)
+    if cap == 0:
+        raise QlcError(ERR_ARG, "chunk_symbols")
+    ws = max(16, qlc_encode_workspace_size(n, chunk_symbols))
+    # laid out as a Codec's buffers, and zeroed for the status word
+    buf = torch.zeros((_CODEC_WS + ws + 7) // 8, dtype=torch.int64, device=x.device)
+    out = torch.empty(cap, dtype=torch.uint8, device=x.device)
+    arr, count = _scheme_array(scheme)
+    p, r = buf.data_ptr(), buf.data_ptr() + _CODEC_RESULTS
+    _check(lib.qlc_encode_tensor(x.data_ptr(), n, arr, count, chunk_symbols, p, p + 2048, out.data_ptr(), cap,
+                                 p + _CODEC_WS, ws, r, r + 16, _stream(None)), "qlc_encode_tensor")
+    nbytes, _, status = buf[_CODEC_RESULTS // 8:_CODEC_RESULTS // 8 + 3].tolist()  # waits for the encoder
     if status != OK:
         raise QlcError(status, "device")
     return out[:nbytes]
@@ -441,7 +451,9 @@ def decode(container: torch.Tensor) -> torch.Tensor:
     n, total = qlc_peek_header(container[:HEADER_BYTES].cpu().numpy().tobytes())
     out = torch.empty(max(n, 1), dtype=torch.uint8, device=container.device)
     words = torch.zeros(2, dtype=torch.int64, device=container.device)  # n_out, status
-    qlc_decode(container, out, words[:1], words[1:].view(torch.int32)[:1], out_cap=n)
+    p = words.data_ptr()
+    _check(lib.qlc_decode(container.data_ptr(), _nbytes(container), out.data_ptr(), n, p, p + 8, _stream(None)),
+           "qlc_decode")
     st = words.tolist()[1]
     if st != OK:
         raise QlcError(st, "qlc_decode")
