@@ -672,18 +672,6 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
 
 using namespace qlc;
 
-// Raises a kernel's shared-memory limit, once per device (a function
-// attribute, allowed inside stream capture).
-template <typename K>
-static bool smem_ok(K kernel, size_t bytes, std::atomic<bool> (&done)[64]) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
-  if (dev < 64 && done[dev].load(std::memory_order_relaxed)) return true;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
-  if (dev < 64) done[dev].store(true, std::memory_order_relaxed);
-  return true;
-}
-
 template <int kOut>
 static qlc_status launch_decode(const uint8_t* d_in, size_t in_bytes, void* d_out, const float* d_scales,
                                 size_t out_cap, uint64_t* d_n_out, uint32_t* d_status, cudaStream_t st) {

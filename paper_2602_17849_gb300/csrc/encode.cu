@@ -1,21 +1,30 @@
 // encode.cu -- QLC encoder (Sections 5 and 7) writing container v1.
 //
-// One persistent kernel.  CTAs take groups (32 chunks) in ticket order; the
-// LUT is staged in shared memory once per tensor, one copy per lane, so every
-// lookup is free of bank conflicts.
-//   pass 1  each warp sums the code lengths of its chunks (w, w+8, ...) ->
-//           chunk_bits;
-//   look-back  warp 0 scans the 32 chunk sizes, publishes the group's padded
-//           byte size and finds the sum of all earlier groups' sizes
-//           (decoupled look-back, bounded waits);
-//   pass 2  each warp re-reads its chunks (from L2: at most three groups per
-//           SM are in flight) and packs them, 512 symbols per step: codeword
-//           pairs, a warp scan of the lanes' bit counts, per-lane word
-//           accumulation into a per-warp staging window (completed words are
-//           plain stores, a lane's partial last word one shared OR), and
-//           16-byte streaming stores of every completed 16-byte block; blocks
-//           shared by neighbouring chunks are merged once per group.
-// HBM traffic is one read of the input and one write of the container.
+// encode_kernel, one persistent kernel: teams of eight warps, two to a CTA, take
+// groups (32 chunks) in ticket order; the LUT is staged in shared memory once per
+// team and tensor, one copy per lane, so every lookup is free of bank conflicts.
+//   pass 1  each warp sums the code lengths of four chunks in a row -> chunk_bits;
+//   look-back  warp 0 publishes the group's padded byte size and finds the sum of
+//           all earlier groups' sizes (decoupled look-back, bounded waits), while
+//           the other warps pack their first step;
+//   pass 2  each warp re-reads its four chunks (about two thirds from L2) and
+//           packs them as one run of the group's bit stream, 1024 symbols per
+//           step: codeword pairs, a warp scan of the lanes' bit counts, per-lane
+//           word accumulation into a per-warp staging window (completed words
+//           are plain stores, a lane's partial last word one shared OR), and
+//           16-byte streaming stores of every completed 16-byte block.
+// Small tensors take lengths_kernel and pack_kernel instead.
+//
+// 256 Mi symbols, t4 data: 184 us (217 with three CTAs of 8 warps, 512 symbols a
+// step, a chunk at a time with blocks merged by the CTA).  16.3 instructions per
+// symbol (22 before): 4 for a length, 12 for packing.  It is bound by the shared-
+// memory pipe (42.7 M wavefronts, 73 % busy: two lookups per symbol, and word
+// stores at 1.7 wavefronts) and the integer pipe (65 %), and loses about a fifth
+// of its warps' time to the look-back and its barriers.  Measured and left out:
+// teams of 16 warps 201 us; the next group's pass 1 before this group's pass 2
+// 223 us (the re-reads then miss L2); pass 1 and pass 2 as two kernels 78 + 140
+// us; shift and OR by one wide multiply-add 193 us (fewer integer instructions,
+// more in all).
 #include <cuda.h>
 
 #include <mutex>
@@ -28,15 +37,23 @@
 
 namespace qlc {
 
-constexpr int kEncThreads = 256;
-constexpr int kEncWarps = kEncThreads / 32;
-constexpr int kEncCtasPerSm = 3;
-constexpr int kSub = 32 * 16;  // symbols a warp packs per step (16 per lane)
-// per-warp staging buffer: 4 guard words, 4 carry words, one step's words, 4 spare
-constexpr int kWStage = 4 + 4 + (kSub * kMaxCode + 31) / 32 + 4;
+constexpr int kPartThreads = 256;  // of lengths_kernel and pack_kernel
+constexpr int kPartWarps = kPartThreads / 32;
+constexpr int kPackCtasPerSm = 3;
+constexpr int kTeams = 2;  // of a CTA of encode_kernel
+constexpr int kTeamThreads = 256;
+constexpr int kTeamWarps = kTeamThreads / 32;
+constexpr int kRun = kGroupChunks / kTeamWarps;  // chunks of a group that a warp takes
+constexpr int kEncCtasPerSm = 2;
+constexpr uint32_t kBatch = 2048;  // symbols whose lengths a warp sums while it fetches the next ones
+// Shared address of encode_kernel's tables; dynamic shared memory starts at or below it.
+constexpr uint32_t kTableAddr = 2048;
+constexpr int kHalf = 32 * 16;  // symbols of half a step, 16 per lane
+// words of a warp's staging window: a block carried over, one step's bits, one spare block
+constexpr int kWStage = 4 + (2 * kHalf * kMaxCode + 31) / 32 + 4;
 constexpr int kPass1Unroll = 8;
 // Tensors of up to this many chunks are encoded in parts (lengths_kernel, pack_kernel).
-constexpr uint64_t kPartMaxChunks = 1 << 14;
+constexpr uint64_t kPartMaxChunks = 4096;
 
 constexpr unsigned long long kFlagAgg = 1ull << 62;
 constexpr unsigned long long kFlagPrefix = 2ull << 62;
@@ -49,26 +66,48 @@ __device__ __forceinline__ void red_or(uint32_t saddr, uint32_t v) {
   asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(saddr), "r"(v) : "memory");
 }
 
-// When the accumulator's first word is complete (nb >= 32): store it to the
-// shared word at wa, move the spill word lo up, advance wa and nb by one word.
-// One predicate drives all of it, with no branch.
-__device__ __forceinline__ void emit_if_full(uint32_t& hi, uint32_t& wa, uint32_t& nb, uint32_t lo) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\t"
-      "setp.ge.u32 q, %2, 32;\n\t"
-      "@q st.shared.u32 [%1], %0;\n\t"
-      "selp.b32 %0, %3, %0, q;\n\t"
-      "@q add.u32 %1, %1, 4;\n\t"
-      "@q sub.u32 %2, %2, 32;\n\t"
-      "}"
-      : "+r"(hi), "+r"(wa), "+r"(nb)
-      : "r"(lo)
-      : "memory");
-}
-
 __device__ __forceinline__ uint32_t ld_shared_u32(uint32_t saddr) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(saddr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_shared_u32(uint32_t saddr, uint32_t v) {
+  asm volatile("st.shared.u32 [%0], %1;" ::"r"(saddr), "r"(v) : "memory");
+}
+
+// Appends the MSB-aligned bits P (at most 22) to the accumulator: hi holds the
+// bits of the current word, at shared address wa.  at is the stream position
+// before P and next the one after it; only their low six bits count.  When the
+// word is complete it is stored and hi gets what spills over: one predicate,
+// no branch.
+__device__ __forceinline__ void append(uint32_t& hi, uint32_t& wa, uint32_t P, uint32_t at, uint32_t next) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      ".reg .b32 t, lo;\n\t"
+      "shf.r.wrap.b32 t, %2, 0, %3;\n\t"   // P >> (at & 31)
+      "shf.r.wrap.b32 lo, 0, %2, %3;\n\t"  // P << (32 - (at & 31)), 0 when that is 32
+      "or.b32 %0, %0, t;\n\t"
+      "xor.b32 t, %3, %4;\n\t"
+      "and.b32 t, t, 32;\n\t"
+      "setp.ne.u32 q, t, 0;\n\t"
+      "@q st.shared.u32 [%1], %0;\n\t"
+      "selp.b32 %0, lo, %0, q;\n\t"
+      "@q add.u32 %1, %1, 4;\n\t"
+      "}"
+      : "+r"(hi), "+r"(wa)
+      : "r"(P), "r"(at), "r"(next)
+      : "memory");
+}
+
+// Inclusive sum over the warp's lanes.
+__device__ __forceinline__ uint32_t warp_scan(uint32_t v) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1)
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
+        "shfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t"
+        "@p add.u32 %0, %0, t;\n\t}"
+        : "+r"(v)
+        : "r"(o));
   return v;
 }
 
@@ -83,22 +122,44 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
   return v;
 }
 
-// The encoder table holds one copy per lane (entry s of lane l at word
-// 32 s + l), so the 32 lanes of a lookup always hit 32 different banks.
-// tab points at this lane's copy.
-__device__ __forceinline__ uint32_t enc_entry(const uint32_t* tab, uint32_t s) { return tab[s << 5]; }
+// The encoder table holds one copy per lane, so the 32 lanes of a lookup always
+// hit 32 different banks.
+struct PartTable {  // rows of 128 bytes
+  const uint8_t* col;  // this lane's word of row 0
+  __device__ __forceinline__ uint32_t at(uint32_t s) const {
+    return *reinterpret_cast<const uint32_t*>(col + (s << 7));
+  }
+  // entry of byte j of w
+  __device__ __forceinline__ uint32_t of(uint32_t w, int j) const { return at(__byte_perm(w, 0, 0x4440 + j)); }
+};
+// Two teams' tables side by side in rows of 256 bytes, at a constant address: one
+// byte permute makes the whole offset (symbol << 8 | col), where rows of 128
+// bytes take two instructions.
+struct WideTable {
+  uint32_t col;  // 128 * team + 4 * lane
+  __device__ __forceinline__ uint32_t load(uint32_t offset) const {
+    uint32_t e;
+    asm volatile("ld.shared.u32 %0, [%1 + %2];" : "=r"(e) : "r"(offset), "n"(kTableAddr));
+    return e;
+  }
+  __device__ __forceinline__ uint32_t at(uint32_t s) const { return load((s << 8) | col); }
+  __device__ __forceinline__ uint32_t of(uint32_t w, int j) const {
+    return load(__byte_perm(w, col, 0x5504 | (j << 4)));
+  }
+};
 
 // Sum of the encoder entries of 16 symbols.  An entry is
 // codeword << (32 - len) | len with len <= 11, so its bits below 21 are the
 // length alone, and the low 21 bits of a sum of entries are the sum of the
 // lengths as long as that stays below 2^21.
-__device__ __forceinline__ uint32_t entry_sum16(const uint32_t* tab, uint4 q) {
+template <class Table>
+__device__ __forceinline__ uint32_t entry_sum16(const Table& tab, uint4 q) {
   const uint32_t w[4] = {q.x, q.y, q.z, q.w};
   uint32_t s = 0;
 #pragma unroll
   for (int k = 0; k < 4; k++)
 #pragma unroll
-    for (int j = 0; j < 4; j++) s += enc_entry(tab, __byte_perm(w[k], 0, 0x4440 + j));
+    for (int j = 0; j < 4; j++) s += tab.of(w[k], j);
   return s;
 }
 
@@ -146,7 +207,7 @@ __device__ unsigned long long lookback(unsigned long long* gstat, uint64_t g, ui
   return excl;
 }
 
-// The header but its dec; every thread of a CTA of 256 calls it.
+// The header but its dec; 256 threads call it.
 __device__ void write_header_of(uint8_t* out, uint64_t n, uint32_t cs, uint64_t n_chunks, const qlc_scheme* scheme,
                                 int tid) {
   if (tid == 0) {
@@ -193,120 +254,134 @@ struct EncArgs {
   uint64_t gstat_cap;  // look-back words at gstat
 };
 
-// Packing state of one warp within one chunk.  The warp appends 512
-// symbols per step (16 per lane, in lane order) to the chunk's bit stream in a
-// per-warp staging window; completed 16-byte blocks go to the payload, except
-// the chunk's first block when it is shared with the previous chunk, which
-// goes to the chunk's seam slot.
+// Packing state of one warp within a run of chunks.  A step appends 512 or 1024
+// symbols, 16 per lane and half, to the bit stream in the warp's staging
+// window; completed 16-byte blocks go to the payload, and the block in work
+// moves to the window's front.
+// Where a run goes: its group's payload (null: nowhere, the group is given up) and
+// the 16-byte blocks there (for the checked build).
+struct Place {
+  uint4* dst;
+  uint32_t blk_lim;
+};
+
+template <class Table, class Find>
 struct Packer {
-  const uint32_t* tab;   // this lane's copy of the encoder table
-  uint32_t* stage;       // the warp's two staging buffers
-  uint32_t stage_s;      // their shared address
-  uint4* dst;            // the group's payload
-  uint32_t seam_s;       // shared address of the chunk's seam slot [0]
-  uint32_t seam_idx_s;   // and of its block index
-  uint32_t seam_blk;     // block shared with the previous chunk, ~0u if none
-  uint32_t blk_lim;      // 16-byte blocks available at dst (checked build)
-  uint32_t base_bit;     // group-relative bit of the step's first symbol
-  uint32_t win;          // group-relative word held at stage word 4 (a multiple of 4)
-  uint32_t cur;          // staging buffer in use
+  Table tab;
+  const Find& find;  // the place, asked for when the first step's blocks are there
+  uint32_t* stage;   // the warp's window
+  uint32_t stage_s;  // its shared address
+  uint4* dst;        // the window's block `lane` in the payload
+  uint32_t off;      // bits in the window, below 128 between steps
+  uint32_t blk;      // the window's first block within the payload
+  uint32_t blk_lim;  // 16-byte blocks of the payload (checked build)
+  bool shared;       // the run's first block starts before it
   int lane;
 
-  // Moves block b (< nblk) of the current buffer out and zeroes it; branch-free.
-  __device__ __forceinline__ void put_block(uint32_t b, uint32_t nblk, const uint32_t* sb) const {
-    const uint32_t blk = win / 4 + b;
-    if (!QLC_GUARD(b >= nblk || blk < blk_lim, nullptr)) nblk = 0;
-    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sb) + 16u * b;
-    asm volatile(
-        "{\n\t"
-        ".reg .pred p, s, g;\n\t"
-        ".reg .b32 a0, a1, a2, a3, z;\n\t"
-        "mov.b32 z, 0;\n\t"
-        "setp.lt.u32 p, %0, %1;\n\t"
-        "setp.eq.and.u32 s, %2, %3, p;\n\t"
-        "setp.ne.and.u32 g, %2, %3, p;\n\t"
-        "@p ld.shared.v4.u32 {a0, a1, a2, a3}, [%4];\n\t"
-        "@p st.shared.v4.u32 [%4], {z, z, z, z};\n\t"
-        "prmt.b32 a0, a0, 0, 0x0123;\n\t"
-        "prmt.b32 a1, a1, 0, 0x0123;\n\t"
-        "prmt.b32 a2, a2, 0, 0x0123;\n\t"
-        "prmt.b32 a3, a3, 0, 0x0123;\n\t"
-        "@g st.global.cs.v4.u32 [%5], {a0, a1, a2, a3};\n\t"
-        "@s st.shared.v4.u32 [%6], {a0, a1, a2, a3};\n\t"
-        "@s st.shared.u32 [%7], %2;\n\t"
-        "}" ::"r"(b),
-        "r"(nblk), "r"(blk), "r"(seam_blk), "r"(sa), "l"(dst + blk), "r"(seam_s), "r"(seam_idx_s)
-        : "memory");
+  __device__ __forceinline__ void put_block(uint32_t b, uint32_t nblk, bool skip) const {
+    if (b < nblk && !skip && QLC_GUARD(blk + b < blk_lim, nullptr)) {
+      const uint4 v = reinterpret_cast<const uint4*>(stage)[b];
+      st_cs_v4(dst + (b - lane), make_uint4(bswap32(v.x), bswap32(v.y), bswap32(v.z), bswap32(v.w)));
+    }
   }
 
-  template <bool kRagged>
-  __device__ __forceinline__ void step(uint4 q, int cnt) {
-    // 16 codewords -> 8 pairs: MSB-aligned (at most 22 bits), lengths in L8.
-    // An entry is codeword << (32 - len) | len, so e & 31 == len.
-    const uint32_t qw[4] = {q.x, q.y, q.z, q.w};
-    uint32_t e[16];
+  // kHalves 1 or 2: symbols in q[0 .. kHalves).  kRagged: the lane's first cnt
+  // symbols of q[0] alone (total_cnt over all lanes), and no block from blk_end
+  // on.  first: the run's first step.  False when the group is given up.
+  template <int kHalves, bool kRagged>
+  __device__ __forceinline__ bool step(const uint4 (&q)[kHalves], int cnt, bool first, uint32_t total_cnt,
+                                       uint32_t blk_end) {
+    // codeword pairs: P MSB-aligned (at most 22 bits); c the running sum of the
+    // entries, whose low 21 bits are the bits so far
+    uint32_t P[kHalves][8], c[kHalves][8];
 #pragma unroll
-    for (int j = 0; j < 16; j++) {
-      e[j] = enc_entry(tab, __byte_perm(qw[j >> 2], 0, 0x4440 + (j & 3)));
-      if (kRagged) e[j] = j < cnt ? e[j] : 0u;
-    }
-    uint32_t P[8], L8[8];
-    uint32_t L = 0;
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-      const uint32_t e0 = e[2 * k], e1 = e[2 * k + 1];
-      // second code right after the first: e1 >> len0 also moves e1's length
-      // field down to bits 0..3-len0, which the mask clears with e0's (the pair
-      // itself, at most 22 bits, sits at bits 31..10)
-      P[k] = (e0 | __funnelshift_r(e1, 0u, e0)) & ~31u;
-      L8[k] = (e0 + e1) & 31u;  // the two lengths; code bits sit above bit 20
-      L += L8[k];
-    }
-    uint32_t incl = L;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-    // Each lane packs its pairs into a two-word accumulator (hi:lo, hi
-    // first) that starts at the lane's bit offset within its first word,
-    // preloaded with that word (the bits carried from the previous step, in
-    // lane 0; zero elsewhere).  Every completed word is stored whole: a lane's
-    // first word also holds the previous lane's last bits, which that lane
-    // ORs in afterwards with its partial last word.  Stores precede the ORs
-    // in program order, and no two lanes store the same word.
-    const uint32_t p = base_bit + incl - L + 32u * (4u - win);  // bit relative to stage word 0
-    if (QLC_GUARD(((p + L) >> 5) < (uint32_t)kWStage, nullptr)) {
-      uint32_t wa = stage_s + cur * kWStage * 4 + (p >> 5) * 4;
-      uint32_t nb = p & 31u;  // bits in hi
-      uint32_t hi = ld_shared_u32(wa);
+    for (int h = 0; h < kHalves; h++) {
+      const uint32_t w[4] = {q[h].x, q[h].y, q[h].z, q[h].w};
+      uint32_t sum = 0;
 #pragma unroll
       for (int k = 0; k < 8; k++) {
-        hi |= P[k] >> nb;
-        const uint32_t lo = __funnelshift_rc(0u, P[k], nb);  // P << (32 - nb), 0 when nb == 0
-        nb += L8[k];                                         // at most 31 + 22
-        emit_if_full(hi, wa, nb, lo);
+        uint32_t e0 = tab.of(w[k / 2], 2 * k & 3), e1 = tab.of(w[k / 2], (2 * k & 3) + 1);
+        if (kRagged) {
+          e0 = 2 * k < cnt ? e0 : 0u;
+          e1 = 2 * k + 1 < cnt ? e1 : 0u;
+        }
+        // the second code right after the first: e1 >> len0 (a shift takes the
+        // low five bits of e0) also moves e1's length down to bits 0..3, which
+        // the mask clears with e0's
+        P[h][k] = (e0 | __funnelshift_r(e1, 0u, e0)) & ~31u;
+        sum += e0 + e1;
+        c[h][k] = sum;
       }
-      red_or(wa, hi);  // the partial last word (0 adds nothing)
+    }
+    // one scan for both halves, of at most 32 * 176 bits each
+    const uint32_t len = kHalves == 2 ? __byte_perm(c[0][7], c[kHalves - 1][7], 0x5410) : c[0][7] & 0xFFFFu;
+    const uint32_t incl = warp_scan(len);
+    const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+    const uint32_t excl = incl - len;
+    const uint32_t end = off + (tot & 0xFFFFu) + (tot >> 16);
+    // Each lane packs its pairs from its bit of the stream on; lane 0 goes on
+    // with the word in work.  A completed word is stored whole: a lane's first
+    // one lacks the previous lane's last bits, which that lane ORs in when all
+    // words are stored.  16 codes have at least 48 bits, so each lane completes
+    // a word, no two lanes store the same one and nothing has to be zero
+    // before; only the last lane's last word is still to be written.  In a
+    // ragged step a lane may have few bits or none, so there the words it can
+    // reach are zeroed and every last word is OR-ed.
+    if (kRagged) {
+      const uint32_t words = ((off + total_cnt * kMaxCode) >> 5) + 1;
+      for (uint32_t i = (off >> 5) + 1 + lane; i <= words; i += 32)
+        if (QLC_GUARD(i < (uint32_t)kWStage, nullptr)) stage[i] = 0;
+      __syncwarp();
+    }
+    uint32_t hi[kHalves], wa[kHalves];
+#pragma unroll
+    for (int h = 0; h < kHalves; h++) {
+      uint32_t p = off + (excl & 0xFFFFu);
+      if (h == 1) p = off + (tot & 0xFFFFu) + (excl >> 16);
+      wa[h] = stage_s + (p >> 5) * 4;
+      hi[h] = 0;
+      if (h == 0 && lane == 0) hi[0] = ld_shared_u32(wa[0]);
+      if (QLC_GUARD(((p + (c[h][7] & 0xFFFFu)) >> 5) < (uint32_t)kWStage, nullptr)) {
+        uint32_t at = p;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+          const uint32_t next = p + c[h][k];
+          append(hi[h], wa[h], P[h][k], at, next);
+          at = next;
+        }
+      }
     }
     __syncwarp();
-    // completed 16-byte blocks go out (at most 45 per step: 128 carried +
-    // 512 * 11 new bits); the partial last block moves to the other buffer
-    const uint32_t end_bit = base_bit + total;
-    const uint32_t nblk = ((end_bit >> 5) - win) / 4;
-    uint32_t* sb = stage + cur * kWStage + 4;
-    put_block(lane, nblk, sb);
-    if (nblk > 32) put_block(lane + 32, nblk, sb);
-    if (lane < 4) {
-      stage[(cur ^ 1) * kWStage + 4 + lane] = sb[4 * nblk + lane];
-      sb[4 * nblk + lane] = 0;
+#pragma unroll
+    for (int h = 0; h < kHalves; h++) {
+      if (!kRagged && h == kHalves - 1 && lane == 31)
+        st_shared_u32(wa[h], hi[h]);
+      else
+        red_or(wa[h], hi[h]);
     }
-    seam_blk = ~0u;  // only a chunk's first step can complete its first block
-    win += 4 * nblk;
-    base_bit = end_bit;
-    cur ^= 1;
     __syncwarp();
+    uint32_t nblk = end >> 7;
+    if (kRagged) nblk = min(nblk, blk_end - blk);
+    bool skip = false;
+    if (first) {
+      const Place p = find();
+      if (!p.dst) return false;
+      dst = p.dst + blk + lane;
+      blk_lim = p.blk_lim;
+      skip = lane == 0 && shared;
+    }
+    put_block(lane, nblk, skip);
+    if (kHalves == 2 || nblk > 32) put_block(lane + 32, nblk, false);
+    if (kHalves == 2 && nblk > 64) put_block(lane + 64, nblk, false);
+    uint32_t carry = 0;
+    if (lane < 4) carry = stage[4 * nblk + lane];
+    __syncwarp();
+    if (lane < 4) stage[lane] = carry;
+    dst += nblk;
+    blk += nblk;
+    off = end & 127u;
+    __syncwarp();
+    return true;
   }
 };
 
@@ -317,16 +392,17 @@ __device__ __forceinline__ uint32_t table_entry(uint32_t e) {
   const uint32_t len = e & 15u, code = e >> 4;
   return len < 3 || len > kMaxCode || (code >> len) != 0 ? 0u : (code << (32 - len)) | len;
 }
-// Stages entry v of symbol s, one copy per lane.
-__device__ __forceinline__ void stage_entry(uint32_t* s_enc, int s, uint32_t v) {
-  uint4* row = reinterpret_cast<uint4*>(&s_enc[32 * s]);
+// Stages entry v of symbol s at its row, one copy per lane; pieces in an order
+// that spreads the threads' stores over the banks.
+__device__ __forceinline__ void stage_entry(uint8_t* row, int s, uint32_t v) {
 #pragma unroll
-  for (int k = 0; k < 8; k++) row[k] = make_uint4(v, v, v, v);
+  for (int k = 0; k < 8; k++) reinterpret_cast<uint4*>(row)[(k + s) & 7] = make_uint4(v, v, v, v);
 }
 
 // Bits of m symbols at p (16-byte aligned; m <= 4096, so that a lane's sum
 // stays below 2^21), the same in every lane.
-__device__ __forceinline__ uint32_t chunk_length(const uint32_t* tab, const uint8_t* p, uint32_t m, int lane) {
+template <class Table>
+__device__ __forceinline__ uint32_t chunk_length(const Table& tab, const uint8_t* p, uint32_t m, int lane) {
   uint32_t bits = 0;
   const uint32_t nv = m / 16;
   const uint4* v = reinterpret_cast<const uint4*>(p);
@@ -339,287 +415,345 @@ __device__ __forceinline__ uint32_t chunk_length(const uint32_t* tab, const uint
     for (int u = 0; u < kPass1Unroll; u++) bits += entry_sum16(tab, q[u]);
   }
   for (; k < nv; k += 32) bits += entry_sum16(tab, ldg_nc_v4(v + k));
-  for (uint32_t t = nv * 16 + lane; t < m; t += 32) bits += enc_entry(tab, p[t]);
+  for (uint32_t t = nv * 16 + lane; t < m; t += 32) bits += tab.at(p[t]);
   return warp_sum_u32(bits & ((1u << 21) - 1));
 }
 
-// The 16-byte blocks that chunks share with their neighbours: a chunk's first
-// / last one, and their block index within the group (~0u if none).
-struct Seams {
-  __align__(16) uint4 blk[kGroupChunks][2];
-  uint32_t idx[kGroupChunks][2];
-};
-
-// Packs chunk c of a group (m symbols at src, group-relative bits [S, E)) to
-// the group's payload dst; the blocks it shares with its neighbours wait in
-// seam slot c.
-__device__ __forceinline__ void pack_chunk(const uint32_t* tab, uint32_t* stage, uint32_t stage_s, const uint8_t* p,
-                                           uint32_t m, uint32_t S, uint32_t E, uint4* dst, uint32_t blk_lim,
-                                           Seams& seam, uint32_t c, int lane) {
-  Packer pk;
-  pk.tab = tab;
-  pk.stage = stage;
-  pk.stage_s = stage_s;
-  pk.dst = dst;
-  pk.blk_lim = blk_lim;
-  pk.seam_s = (uint32_t)__cvta_generic_to_shared(&seam.blk[c][0]);
-  pk.seam_idx_s = (uint32_t)__cvta_generic_to_shared(&seam.idx[c][0]);
-  pk.seam_blk = (S & 127u) ? (S >> 7) : ~0u;
-  pk.base_bit = S;
-  pk.win = (S >> 5) & ~3u;
-  pk.cur = 0;
-  pk.lane = lane;
-  // full steps, with the input of the next two steps in flight
-  const uint32_t n_full = m / kSub;
-  const uint4* src = reinterpret_cast<const uint4*>(p) + lane;
-  uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
-  if (n_full > 0) q0 = ldg_nc_v4(src);
-  if (n_full > 1) q1 = ldg_nc_v4(src + 32);
-  for (uint32_t i = 0; i < n_full; i++) {
-    const uint4 q = q0;
-    q0 = q1;
-    if (i + 2 < n_full) q1 = ldg_nc_v4(src + 32 * (i + 2));
-    pk.step<false>(q, 16);
-  }
-  // a ragged end (chunks of a size that kSub does not divide, or a tensor's
-  // last chunk): lane l takes symbols 16 l ...
-  if (m % kSub) {
-    const uint32_t off = n_full * kSub + 16u * lane;
-    const int cnt = off < m ? (int)min(16u, m - off) : 0;
-    uint32_t w[4] = {0, 0, 0, 0};
+// The first step's symbols of a run of m at p.
+__device__ __forceinline__ void load_first(uint4 (&q)[2], const uint8_t* p, uint32_t m, int lane) {
 #pragma unroll
-    for (int j = 0; j < 16; j++)
-      if (j < cnt) w[j >> 2] |= (uint32_t)p[off + j] << (8 * (j & 3));
-    pk.step<true>(make_uint4(w[0], w[1], w[2], w[3]), cnt);
+  for (uint32_t h = 0; h < 2; h++)
+    q[h] = h < m / kHalf ? ldg_nc_v4(reinterpret_cast<const uint4*>(p) + lane + 32 * h) : make_uint4(0, 0, 0, 0);
+}
+
+// Packs a run of a group's chunks: m symbols at p (next: load_first of them),
+// group-relative bits [S, E), rest more symbols of the group behind them, to the
+// place that find() tells, which every run calls once.  A 16-byte block belongs
+// to the run that its first bit falls in: the run also encodes the symbols after
+// it that reach into its last block (48 have 144 bits or more; a run ends on a
+// multiple of 128 symbols or with its tensor, so they never fill a step), and
+// leaves its first block out when that starts before the run.  Runs need nothing
+// from one another, and no barrier.
+template <class Table, class Find>
+__device__ __forceinline__ void pack_run(const Table& tab, uint32_t* stage, const uint8_t* p, uint32_t m, uint64_t rest,
+                                         uint32_t S, uint32_t E, uint4 (&next)[2], const Find& find, int lane) {
+  const uint32_t blk_end = (E + 127u) >> 7;
+  if ((S + 127u) >> 7 >= blk_end) {  // the last symbols of a tensor, in another run's block
+    find();
+    return;
   }
-  // the chunk's partial last block (shared with the next chunk, or the
-  // group's zero-padded end) goes to the seam; the buffer is left zeroed
-  if (lane == 0) {
-    uint32_t* cb = pk.stage + pk.cur * kWStage + 4;
-    if (E & 127u) {
-      seam.blk[c][1] = make_uint4(bswap32(cb[0]), bswap32(cb[1]), bswap32(cb[2]), bswap32(cb[3]));
-      seam.idx[c][1] = E >> 7;
+  if (E & 127u) m += (uint32_t)min(rest, (uint64_t)48);
+  Packer<Table, Find> pk = {tab, find, stage};
+  pk.stage_s = (uint32_t)__cvta_generic_to_shared(stage);
+  pk.off = S & 127u;
+  pk.blk = S >> 7;
+  pk.shared = pk.off != 0;
+  pk.lane = lane;
+  bool first = true;
+  if (lane < 4) stage[lane] = 0;
+  __syncwarp();
+  // full steps, with the input of the next one in flight
+  const uint32_t n_half = m / kHalf;
+  const uint4* src = reinterpret_cast<const uint4*>(p) + lane;
+  uint32_t i = 0;
+  for (; i + 2 <= n_half; i += 2) {
+    const uint4 q[2] = {next[0], next[1]};
+#pragma unroll
+    for (uint32_t h = 0; h < 2; h++)
+      if (i + 2 + h < n_half) next[h] = ldg_nc_v4(src + 32 * (i + 2 + h));
+    if (!pk.template step<2, false>(q, 16, first, 0, 0)) return;
+    first = false;
+  }
+  if (i < n_half) {
+    const uint4 q[1] = {next[0]};
+    if (!pk.template step<1, false>(q, 16, first, 0, 0)) return;
+    first = false;
+  }
+  // what is left, 16 symbols a lane
+  if (m % kHalf) {
+    const uint32_t at = n_half * kHalf + 16u * lane;
+    const int cnt = at < m ? (int)min(16u, m - at) : 0;
+    uint4 q[1] = {make_uint4(0, 0, 0, 0)};
+    if (cnt == 16) {
+      q[0] = ldg_nc_v4(reinterpret_cast<const uint4*>(p + at));
+    } else {
+      uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int j = 0; j < 16; j++)
+        if (j < cnt) w[j >> 2] |= (uint32_t)p[at + j] << (8 * (j & 3));
+      q[0] = make_uint4(w[0], w[1], w[2], w[3]);
     }
-    cb[0] = cb[1] = cb[2] = cb[3] = 0;
+    if (!pk.template step<1, true>(q, cnt, first, m % kHalf, blk_end)) return;
+  }
+  // the group's zero-padded end
+  if (pk.blk < blk_end && lane == 0 && QLC_GUARD(pk.blk < pk.blk_lim, nullptr)) {
+    uint32_t v[4];
+#pragma unroll
+    for (uint32_t k = 0; k < 4; k++) v[k] = k <= pk.off >> 5 ? bswap32(stage[k]) : 0u;
+    st_cs_v4(pk.dst, make_uint4(v[0], v[1], v[2], v[3]));
   }
   __syncwarp();
 }
 
-// Seams of a group's chunks [first, first + 32) that were packed together
-// (warp-wide): the lane of chunk l writes the block holding the chunk's end,
-// OR-ed with the blocks of chunk l + 1 that fall in the same 16 bytes and with
-// more (the bits that follow the last of these chunks).  A chunk shorter than
-// a block (only the last chunk of a tensor) is merged by the lane of the chunk
-// before it.
-__device__ __forceinline__ void merge_seams(const Seams& seam, uint4* dst, uint32_t blk_lim, uint32_t more_idx,
-                                            uint4 more, uint32_t* status, int lane) {
-  const uint32_t i1 = seam.idx[lane][1];
-  const bool mine = i1 != ~0u && !(lane > 0 && seam.idx[lane - 1][1] == i1);
-  if (!mine) return;
-  uint4 v = seam.blk[lane][1];
-  auto merge = [&](uint4 u) {
-    v.x |= u.x;
-    v.y |= u.y;
-    v.z |= u.z;
-    v.w |= u.w;
-  };
-  if (lane + 1 < kGroupChunks)
-    for (int k = 0; k < 2; k++)
-      if (seam.idx[lane + 1][k] == i1) merge(seam.blk[lane + 1][k]);
-  if (i1 == more_idx) merge(more);
-  if (QLC_GUARD(i1 < blk_lim, status)) st_cs_v4(&dst[i1], v);
+struct TeamShared {
+  unsigned long long item, first, excl;
+  const uint8_t* in;
+  uint64_t n;
+  const qlc_lut* lut;
+  uint8_t* out;
+  uint64_t cap;
+  unsigned long long* ob;
+  int err;
+  uint32_t chunk_bits[kGroupChunks];
+};
+struct EncShared {
+  uint8_t table[256 << 8];  // codeword << (32 - len) | len, one copy per team and lane
+  __align__(16) uint32_t stage[kTeams * kTeamWarps][kWStage];
+  TeamShared team[kTeams];
+};
+// dynamic shared memory starts at 1024
+constexpr size_t kEncSharedBytes = sizeof(EncShared) + kTableAddr - 1024;
+
+// Barriers of a team's threads.  The second one is for a group's offset, which
+// warp 0 tells the others.
+__device__ __forceinline__ void team_sync(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeamThreads) : "memory");
+}
+__device__ __forceinline__ void offset_tell(int team) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(team + 1 + kTeams), "n"(kTeamThreads) : "memory");
+}
+__device__ __forceinline__ void offset_wait(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(team + 1 + kTeams), "n"(kTeamThreads) : "memory");
+}
+__device__ __forceinline__ bool team_or(int team, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, %2, %3, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)v), "r"(team + 1), "n"(kTeamThreads)
+      : "memory");
+  return r != 0;
 }
 
-__global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm)
-encode_kernel(EncArgs A) {
-  __shared__ __align__(16) uint32_t s_enc[256 * 32];  // codeword << (32 - len) | len, one copy per lane
-  __shared__ __align__(16) uint32_t s_stage[kEncWarps][2][kWStage];  // per-warp ping-pong
-  __shared__ uint32_t s_chunk_bits[kGroupChunks];
-  __shared__ uint32_t s_chunk_start[kGroupChunks + 1];  // group-relative bit of each chunk
-  __shared__ Seams s_seam;
-  __shared__ unsigned long long s_item, s_first, s_excl;
-  __shared__ const uint8_t* s_in;
-  __shared__ uint64_t s_n;
-  __shared__ const qlc_lut* s_lut;
-  __shared__ uint8_t* s_out;
-  __shared__ uint64_t s_cap;
-  __shared__ unsigned long long* s_ob;
-  __shared__ int s_err;
+// The next group and, in a batch, its tensor (warp-wide).
+__device__ __forceinline__ void take_item(const EncArgs& A, uint64_t n_items, TeamShared& ts, int lane) {
+  unsigned long long t = 0;
+  if (lane == 0) t = atomicAdd(A.ticket, 1u);
+  t = __shfl_sync(0xffffffffu, t, 0);
+  const int shard = A.descs && t < n_items ? shard_of_warp(A.item_base, A.n_shards, t, lane) : 0;
+  if (lane != 0) return;
+  ts.item = t;
+  if (t >= n_items) return;
+  if (A.descs) {
+    const qlc_desc d = A.descs[shard];
+    ts.first = A.item_base[shard];
+    ts.in = static_cast<const uint8_t*>(d.in);
+    ts.n = d.in_bytes;
+    ts.lut = d.lut;
+    ts.out = static_cast<uint8_t*>(d.out);
+    ts.cap = d.out_cap;
+    ts.ob = reinterpret_cast<unsigned long long*>(d.out_bytes);
+  } else {
+    ts.first = 0;
+    ts.in = A.in;
+    ts.n = A.n;
+    ts.lut = A.lut;
+    ts.out = A.out;
+    ts.cap = A.out_cap;
+    ts.ob = A.out_bytes;
+  }
+}
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// Lengths of a warp's kRun full chunks, cs symbols each from p on (cs a multiple
+// of kBatch), to put(chunk of the run, bits): the next symbols are on their way
+// while a batch is summed.
+template <class Put>
+__device__ __forceinline__ void run_lengths(const WideTable& tab, const uint8_t* p, uint32_t cs, int lane, Put put) {
+  constexpr int kV = kBatch / 512;
+  const uint4* src = reinterpret_cast<const uint4*>(p) + lane;
+  const uint32_t per = cs / kBatch, total = per * kRun;
+  uint4 q[2][kV];
+  uint32_t bits = 0, left = per, c = 0;
+  auto fetch = [&](uint4 (&d)[kV]) {
+#pragma unroll
+    for (int u = 0; u < kV; u++) d[u] = ldg_nc_v4(src + 32 * u);
+    src += 32 * kV;
+  };
+  auto add = [&](const uint4 (&d)[kV]) {
+#pragma unroll
+    for (int u = 0; u < kV; u++) bits += entry_sum16(tab, d[u]);
+    if (--left == 0) {
+      put(c++, warp_sum_u32(bits & ((1u << 21) - 1)));
+      bits = 0;
+      left = per;
+    }
+  };
+  fetch(q[0]);
+  for (uint32_t j = 0; j < total; j += 2) {  // total is even: kRun is
+    fetch(q[1]);
+    add(q[0]);
+    if (j + 2 < total) fetch(q[0]);
+    add(q[1]);
+  }
+}
+
+// A team's work on one group.
+__device__ __forceinline__ void encode_group(const EncArgs& A, EncShared& sh, TeamShared& ts, int team,
+                                             const qlc_lut*& cur_lut) {
+  const int tid = threadIdx.x % kTeamThreads, lane = tid & 31, warp = tid >> 5;
   const uint32_t cs = A.cs;
   const uint64_t group_syms = (uint64_t)kGroupChunks * cs;
-  const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(&s_stage[warp][0][0]);
-  const uint32_t* tab = &s_enc[lane];
+  const WideTable tab = {128u * team + 4u * lane};
+  const uint64_t n = ts.n, item = ts.item, g = item - ts.first;  // g: the group within its tensor
+  uint8_t* out = ts.out;
+  const qlc_lut* lut = ts.lut;
+  if (lut != cur_lut) {
+    const uint32_t e = tid < 256 ? table_entry(lut->enc[tid]) : 1u;
+    if (team_or(team, e == 0)) {  // the tensor is refused
+      if (tid == 0) {
+        set_status(A.status, QLC_ERR_ARG);
+        st_release_u64(&A.gstat[item], kFlagError);
+      }
+      cur_lut = nullptr;
+      return;
+    }
+    if (tid < 256) stage_entry(sh.table + 256 * tid + 128 * team, tid, e);
+    cur_lut = lut;
+    team_sync(team);
+  }
+  const uint64_t n_chunks = (n + cs - 1) / cs;
+  const uint64_t n_groups = n_groups_of(n_chunks);
+  if (g == 0) write_header(out, n, cs, n_chunks, lut, tid);
+  if (n == 0) {  // an empty shard of a batch: header-only container
+    if (tid == 0) {
+      *reinterpret_cast<unsigned long long*>(out + 48) = 0;
+      if (ts.ob) *ts.ob = payload_start(n_chunks);
+    }
+    return;
+  }
+  const uint64_t gbeg = g * group_syms;
+  const uint64_t gend = min(gbeg + group_syms, n);
+  const uint32_t c0 = warp * kRun;  // the warp's chunks
+  const uint64_t beg = gbeg + (uint64_t)c0 * cs, end = min(beg + (uint64_t)kRun * cs, gend);
+  const uint8_t* p = ts.in + beg;
+
+  // ---- pass 1: bits of each chunk
+  {
+    uint16_t* chunk_bits = reinterpret_cast<uint16_t*>(out + kIndexOff + 8 * n_groups);
+    auto put = [&](uint32_t i, uint32_t bits) {
+      const uint32_t c = c0 + i;
+      if (lane != 0) return;
+      ts.chunk_bits[c] = bits;
+      if (QLC_GUARD(g * kGroupChunks + c < n_chunks, A.status)) chunk_bits[g * kGroupChunks + c] = (uint16_t)bits;
+    };
+    if (gend - gbeg == group_syms && cs % kBatch == 0) {
+      run_lengths(tab, p, cs, lane, put);
+    } else {
+      for (uint32_t i = 0; i < kRun; i++) {
+        const uint64_t cbeg = beg + (uint64_t)i * cs;
+        if (cbeg < gend)
+          put(i, chunk_length(tab, ts.in + cbeg, (uint32_t)(min(cbeg + cs, gend) - cbeg), lane));
+        else if (lane == 0)
+          ts.chunk_bits[c0 + i] = 0;
+      }
+    }
+  }
+  uint4 next[2] = {};
+  if (beg < gend) load_first(next, p, (uint32_t)(end - beg), lane);
+  team_sync(team);
+
+  const uint32_t cb = ts.chunk_bits[lane];
+  const uint32_t incl = warp_scan(cb);  // group-relative bit of each chunk's end
+  // ---- look-back, by warp 0: this group's byte offset in the payload.  The other
+  // warps pack their first step meanwhile.
+  if (warp == 0) {
+    const uint64_t gbytes = align16((__shfl_sync(0xffffffffu, incl, 31) + 7) / 8);
+    bool err = !QLC_GUARD(item < A.gstat_cap, A.status);
+    const unsigned long long excl = err ? 0ull : lookback(A.gstat, item, ts.first, gbytes, lane, &err);
+    if (lane == 0) {
+      ts.excl = excl;
+      ts.err = err;
+      if (err) {
+        set_status(A.status, QLC_ERR_TIMEOUT);
+      } else {
+        if (QLC_GUARD(g < n_groups, A.status)) reinterpret_cast<unsigned long long*>(out + kIndexOff)[g] = excl;
+        if (g == n_groups - 1) {
+          *reinterpret_cast<unsigned long long*>(out + 48) = excl + gbytes;
+          if (ts.ob) *ts.ob = payload_start(n_chunks) + excl + gbytes;
+        }
+      }
+    }
+    __syncwarp();
+    offset_tell(team);
+  }
+  const auto find = [&]() -> Place {
+    if (warp != 0) offset_wait(team);
+    if (ts.err) return {nullptr, 0};
+    const uint64_t start = payload_start((ts.n + cs - 1) / cs) + ts.excl;
+    return {reinterpret_cast<uint4*>(ts.out + start), (uint32_t)min((ts.cap - start) / 16, (uint64_t)0xFFFFFFFEu)};
+  };
+
+  // ---- pass 2: the warp's chunks, one run of the group's bit stream
+  if (beg >= gend || !QLC_GUARD(end <= n, A.status)) {
+    find();
+    return;
+  }
+  const uint32_t S = __shfl_sync(0xffffffffu, incl - cb, c0), E = __shfl_sync(0xffffffffu, incl, c0 + kRun - 1);
+  pack_run(tab, sh.stage[threadIdx.x >> 5], p, (uint32_t)(end - beg), gend - end, S, E, next, find, lane);
+}
+
+__global__ void __launch_bounds__(kTeams* kTeamThreads, kEncCtasPerSm)
+encode_kernel(EncArgs A) {
+  extern __shared__ __align__(16) uint8_t enc_smem[];
+  const uint32_t smem_s = (uint32_t)__cvta_generic_to_shared(enc_smem);
+  if (smem_s > kTableAddr) {  // does not happen; the host's size counts on it too
+    if (threadIdx.x == 0) set_status(A.status, QLC_ERR_CUDA);
+    return;
+  }
+  EncShared& sh = *reinterpret_cast<EncShared*>(enc_smem + (kTableAddr - smem_s));
+  const int team = threadIdx.x / kTeamThreads, lane = threadIdx.x & 31, warp = threadIdx.x % kTeamThreads / 32;
   const qlc_lut* cur_lut = nullptr;
-  for (int i = tid; i < kEncWarps * 2 * kWStage; i += kEncThreads) (&s_stage[0][0][0])[i] = 0;
   dependency_wait();
   const uint64_t n_items = A.descs ? A.item_base[A.n_shards] : A.n_items;
-
+  if (team > 0 && n_items <= gridDim.x) return;  // a CTA per group
+  TeamShared& ts = sh.team[team];
   while (true) {
-    __syncthreads();
-    if (warp == 0) {  // the next group and, in a batch, its shard
-      unsigned long long t = 0;
-      if (lane == 0) t = atomicAdd(A.ticket, 1u);
-      t = __shfl_sync(0xffffffffu, t, 0);
-      const int sh = A.descs && t < n_items ? shard_of_warp(A.item_base, A.n_shards, t, lane) : 0;
-      if (lane == 0) {
-        s_item = t;
-        if (t < n_items) {
-          if (A.descs) {
-            const qlc_desc d = A.descs[sh];
-            s_first = A.item_base[sh];
-            s_in = static_cast<const uint8_t*>(d.in);
-            s_n = d.in_bytes;
-            s_lut = d.lut;
-            s_out = static_cast<uint8_t*>(d.out);
-            s_cap = d.out_cap;
-            s_ob = reinterpret_cast<unsigned long long*>(d.out_bytes);
-          } else {
-            s_first = 0;
-            s_in = A.in;
-            s_n = A.n;
-            s_lut = A.lut;
-            s_out = A.out;
-            s_cap = A.out_cap;
-            s_ob = A.out_bytes;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    const unsigned long long item = s_item;
-    if (item >= n_items) break;
-    const uint64_t g = item - s_first;  // group within its tensor
-    const uint8_t* in = s_in;
-    const uint64_t n = s_n;
-    uint8_t* out = s_out;
-    const qlc_lut* lut = s_lut;
-    if (lut != cur_lut) {
-      const uint32_t e = table_entry(lut->enc[tid]);
-      const bool bad = e == 0;  // the tensor is refused
-      if (__syncthreads_or(bad)) {
-        if (tid == 0) {
-          set_status(A.status, QLC_ERR_ARG);
-          st_release_u64(&A.gstat[item], kFlagError);
-        }
-        cur_lut = nullptr;
-        continue;
-      }
-      stage_entry(s_enc, tid, e);
-      cur_lut = lut;
-      __syncthreads();
-    }
-    const uint64_t n_chunks = (n + cs - 1) / cs;
-    const uint64_t n_groups = n_groups_of(n_chunks);
-    const uint64_t P = payload_start(n_chunks);
-    if (n == 0) {  // an empty shard of a batch: header-only container
-      write_header(out, 0, cs, 0, lut, tid);
-      if (tid == 0) {
-        *reinterpret_cast<unsigned long long*>(out + 48) = 0;
-        if (s_ob) *s_ob = P;
-      }
-      continue;
-    }
-    uint8_t* payload = out + P;
-    unsigned long long* group_off = reinterpret_cast<unsigned long long*>(out + kIndexOff);
-    uint16_t* chunk_bits = reinterpret_cast<uint16_t*>(out + kIndexOff + 8 * n_groups);
-    const uint64_t gbeg = g * group_syms;
-    const uint64_t gend = min(gbeg + group_syms, n);
-    if (g == 0) write_header(out, n, cs, n_chunks, lut, tid);
-
-    // ---- pass 1: bits of each chunk; warp w takes chunks w, w+8, ...
-    for (uint32_t c = warp; c < kGroupChunks; c += kEncWarps) {
-      const uint64_t cbeg = gbeg + (uint64_t)c * cs;
-      uint32_t bits = 0;
-      if (cbeg < gend) {
-        const uint32_t m = (uint32_t)(min(cbeg + cs, gend) - cbeg);
-        bits = chunk_length(tab, in + cbeg, m, lane);
-        if (lane == 0 && QLC_GUARD(g * kGroupChunks + c < n_chunks, A.status))
-          chunk_bits[g * kGroupChunks + c] = (uint16_t)bits;
-      }
-      if (lane == 0) s_chunk_bits[c] = bits;
-    }
-    __syncthreads();
-
-    // ---- look-back: this group's byte offset in the payload
-    if (warp == 0) {
-      const uint32_t cb = s_chunk_bits[lane];
-      uint32_t incl = cb;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      s_chunk_start[lane] = incl - cb;
-      if (lane == 31) s_chunk_start[32] = incl;
-      s_seam.idx[lane][0] = s_seam.idx[lane][1] = ~0u;
-      const uint32_t gbits = __shfl_sync(0xffffffffu, incl, 31);
-      const uint64_t gbytes = align16((gbits + 7) / 8);
-      bool err = !QLC_GUARD(item < A.gstat_cap, A.status);
-      const unsigned long long excl = err ? 0ull : lookback(A.gstat, item, s_first, gbytes, lane, &err);
-      if (lane == 0) {
-        s_excl = excl;
-        s_err = err;
-        if (err) {
-          set_status(A.status, QLC_ERR_TIMEOUT);
-        } else {
-          if (QLC_GUARD(g < n_groups, A.status)) group_off[g] = excl;
-          if (g == n_groups - 1) {
-            *reinterpret_cast<unsigned long long*>(out + 48) = excl + gbytes;
-            if (s_ob) *s_ob = P + excl + gbytes;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    if (s_err) continue;
-    uint4* dst = reinterpret_cast<uint4*>(payload + s_excl);
-    const uint32_t blk_lim = (uint32_t)min((uint64_t)((s_cap - P - s_excl) / 16), (uint64_t)0xFFFFFFFEu);
-
-    // ---- pass 2: each warp packs its own chunks (w, w+8, w+16, w+24), 512
-    // symbols per step, with warp scans only: a chunk's start bit is known
-    // from pass 1.  Completed 16-byte blocks go straight out, except the 16-
-    // byte blocks a chunk shares with its neighbours, which wait in s_seam.
-    for (uint32_t c = warp; c < kGroupChunks; c += kEncWarps) {
-      const uint64_t cbeg = gbeg + (uint64_t)c * cs;
-      if (cbeg >= gend) break;
-      const uint32_t m = (uint32_t)(min(cbeg + cs, gend) - cbeg);
-      if (!QLC_GUARD(cbeg + m <= n, A.status)) break;
-      pack_chunk(tab, &s_stage[warp][0][0], stage_s, in + cbeg, m, s_chunk_start[c], s_chunk_start[c + 1], dst, blk_lim,
-                 s_seam, c, lane);
-    }
-    __syncthreads();
-    if (warp == 0) merge_seams(s_seam, dst, blk_lim, ~0u, make_uint4(0, 0, 0, 0), A.status, lane);
+    team_sync(team);
+    // taken early (by a warp that is done before the others) a group would be
+    // waited for longer by those after it: 1152 tensors 2680 us instead of 2570
+    if (warp == 0) take_item(A, n_items, ts, lane);
+    team_sync(team);
+    if (ts.item >= n_items) break;
+    encode_group(A, sh, ts, team, cur_lut);
   }
 }
 
 // ------------------------------------------------------- tensors of few groups
 //
-// A CTA per group leaves most of the GPU idle below a few hundred groups, and
-// a CTA takes about 30 us for a group of 32 x 4096 symbols.  Up to
+// A team per group leaves most of the GPU idle below a few hundred groups, and
+// a team takes about 20 us for a group of 32 x 4096 symbols.  Up to
 // kPartMaxChunks chunks the work is cut finer, in two kernels without
 // look-back (and without the memset of its words).  Histogram, LUT and encode
-// of Student-t symbols, us, a CTA per group / parts: 256 Ki symbols in chunks
-// of 4096 48.5 / 31, 1 Mi 48 / 31.8, 4 Mi 49 / 33, 16 Mi 52.6 / 44, 64 Mi
-// 113.6 / 97, 96 Mi 145 / 141, 256 Mi 296 / 320; in chunks of 1024 16 Mi 61 /
-// 54, 64 Mi 131 / 134; in chunks of 128 2 Mi 54 / 49, 8 Mi 102.5 / 105: the
-// line lies at 16384 chunks.
+// of Student-t symbols, us, by groups / in parts: in chunks of 4096 4 Mi symbols
+// 34 / 23.3, 12 Mi 37.6 / 35, 16 Mi 40 / 37.6, 24 Mi 48.2 / 46.5, 32 Mi 49.3 /
+// 54.7, 40 Mi 73.5 / 64.9, 64 Mi 80.8 / 91.6, 256 Mi 245 / 309; in chunks of 1024
+// 4 Mi 28.7 / 29.4, 8 Mi 29.1 / 33.9, 64 Mi 99.8 / 142; in chunks of 128 0.5 Mi
+// 23.6 / 21.8, 1 Mi 23.9 / 27.8, 8 Mi 67 / 93: the line lies at 4096 chunks.
 //   lengths  a warp per chunk: chunk_bits (and the container's header);
-//   pack     a CTA per part of kEncWarps chunks, a chunk per warp. The sizes of
+//   pack     a CTA per part of kPartWarps chunks, a chunk per warp. The sizes of
 //            the groups before a part's are summed from chunk_bits (2 bytes per
-//            chunk, from L2), so a CTA needs nothing from the others. A 16-byte
-//            block that two parts share belongs to the part it starts in, whose
-//            CTA also encodes the up to 43 symbols after the part that reach
-//            into it.
+//            chunk, from L2), so a CTA needs nothing from the others.
 // With kBuild every CTA ranks the histogram itself (about 1 us), and the first
 // writes the LUT: no kernel of its own between the histogram and this one.
 template <bool kBuild>
-__global__ void __launch_bounds__(kEncThreads)
+__global__ void __launch_bounds__(kPartThreads)
 lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const unsigned long long* __restrict__ hist, SchemeSet set,
                qlc_lut* lut, uint32_t cs, uint8_t* out, uint32_t* status) {
-  static_assert(kEncThreads == kLutThreads, "a thread per symbol");
-  __shared__ __align__(16) uint32_t s_enc[256 * 32];
+  static_assert(kPartThreads == kLutThreads, "a thread per symbol");
+  __shared__ __align__(16) uint8_t s_enc[256 << 7];
   __shared__ __align__(16) unsigned long long s_key[kBuild ? 256 : 2];
   __shared__ unsigned long long s_bits[8][kLutThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -638,37 +772,34 @@ lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const unsigned long l
   } else {
     e = table_entry(lut->enc[tid]);
   }
-  stage_entry(s_enc, tid, e);
+  stage_entry(s_enc + 128 * tid, tid, e);
   if (__syncthreads_or(e == 0)) {  // not a LUT of this library: refused
     if (blockIdx.x == 0 && tid == 0) set_status(status, QLC_ERR_ARG);
     return;
   }
   if (!kBuild && blockIdx.x == 0) write_header(out, n, cs, n_chunks, lut, tid);
   uint16_t* chunk_bits = reinterpret_cast<uint16_t*>(out + kIndexOff + 8 * n_groups_of(n_chunks));
-  for (uint64_t c = (uint64_t)blockIdx.x * kEncWarps + warp; c < n_chunks; c += (uint64_t)gridDim.x * kEncWarps) {
+  for (uint64_t c = (uint64_t)blockIdx.x * kPartWarps + warp; c < n_chunks; c += (uint64_t)gridDim.x * kPartWarps) {
     const uint64_t beg = c * cs;
-    const uint32_t bits = chunk_length(&s_enc[lane], in + beg, (uint32_t)min((uint64_t)cs, n - beg), lane);
+    const uint32_t bits = chunk_length(PartTable{s_enc + 4 * lane}, in + beg, (uint32_t)min((uint64_t)cs, n - beg), lane);
     if (lane == 0) chunk_bits[c] = (uint16_t)bits;
   }
 }
 
-constexpr uint32_t kParts = kGroupChunks / kEncWarps;  // parts per group
+constexpr uint32_t kParts = kGroupChunks / kPartWarps;  // parts per group
 
-__global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm)
+__global__ void __launch_bounds__(kPartThreads, kPackCtasPerSm)
 pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* lut, uint32_t cs, uint8_t* out,
             uint64_t out_cap, unsigned long long* out_bytes, uint32_t* status) {
-  __shared__ __align__(16) uint32_t s_enc[256 * 32];
-  __shared__ __align__(16) uint32_t s_stage[kEncWarps][2][kWStage];
-  __shared__ Seams s_seam;
-  __shared__ unsigned long long s_sum[kEncWarps];
-  __shared__ uint32_t s_more[4];
+  __shared__ __align__(16) uint8_t s_enc[256 << 7];
+  __shared__ __align__(16) uint32_t s_stage[kPartWarps][kWStage];
+  __shared__ unsigned long long s_sum[kPartWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < kEncWarps * 2 * kWStage; i += kEncThreads) (&s_stage[0][0][0])[i] = 0;
   dependency_wait();
   const uint32_t e = table_entry(__ldcg(&lut->enc[tid]));
-  stage_entry(s_enc, tid, e);
+  stage_entry(s_enc + 128 * tid, tid, e);
   if (__syncthreads_or(e == 0)) return;  // lengths_kernel has set the status
-  const uint32_t* tab = &s_enc[lane];
+  const PartTable tab = {s_enc + 4 * lane};
   const uint32_t n_chunks = (uint32_t)((n + cs - 1) / cs);  // <= kPartMaxChunks
   const uint32_t n_groups = (uint32_t)n_groups_of(n_chunks);
   const uint64_t P = payload_start(n_chunks);
@@ -677,10 +808,16 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* lut, uint
   unsigned long long excl = 0;  // payload offset of group g_at
   uint32_t g_at = 0;
   for (uint32_t item = blockIdx.x; item < n_groups * kParts; item += gridDim.x) {
-    const uint32_t g = item / kParts, first = (item % kParts) * kEncWarps;  // the part's first chunk in the group
+    const uint32_t g = item / kParts, first = (item % kParts) * kPartWarps;  // the part's first chunk in the group
+    const uint32_t c = first + warp;
+    const uint64_t gbeg = (uint64_t)g * kGroupChunks * cs;
+    const uint64_t gend = min(gbeg + (uint64_t)kGroupChunks * cs, n);
+    const uint64_t beg = gbeg + (uint64_t)c * cs, end = min(beg + cs, gend);
+    uint4 next[2] = {};
+    if (beg < gend) load_first(next, in + beg, (uint32_t)(end - beg), lane);
     // the sizes of groups g_at .. g - 1 (all of 32 chunks): 8 lanes per group, 4 chunks each
     unsigned long long sum = 0;
-    for (uint32_t b = 8 * g_at + 32 * warp; b < 8 * g; b += 32 * kEncWarps) {
+    for (uint32_t b = 8 * g_at + 32 * warp; b < 8 * g; b += 32 * kPartWarps) {
       uint32_t bits = 0;
       if (b + lane < 8 * g) {
         const uint2 q = __ldcg(reinterpret_cast<const uint2*>(chunk_bits + 4 * (b + lane)));
@@ -701,13 +838,11 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* lut, uint
       if (lane >= o) incl += t;
     }
     const uint32_t gbits = __shfl_sync(0xffffffffu, incl, 31);
-    __syncthreads();  // the previous part's seams and sums are done with
+    __syncthreads();  // the previous part's sums are done with
     if (lane == 0) s_sum[warp] = sum;
-    if (warp == 0) s_seam.idx[lane][0] = s_seam.idx[lane][1] = ~0u;
-    if (tid < 4) s_more[tid] = 0;
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < kEncWarps; w++) excl += s_sum[w];
+    for (int w = 0; w < kPartWarps; w++) excl += s_sum[w];
     g_at = g;
     if (first == 0 && tid == 0) {
       const unsigned long long gbytes = align16((gbits + 7) / 8);
@@ -717,45 +852,14 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* lut, uint
         *out_bytes = P + excl + gbytes;
       }
     }
-    uint4* dst = reinterpret_cast<uint4*>(out + P + excl);
-    const uint32_t blk_lim = (uint32_t)min((uint64_t)((out_cap - P - excl) / 16), (uint64_t)0xFFFFFFFEu);
-    const uint64_t gbeg = (uint64_t)g * kGroupChunks * cs;
-    const uint64_t gend = min(gbeg + (uint64_t)kGroupChunks * cs, n);
-    const uint32_t c = first + warp;
     const uint32_t E = __shfl_sync(0xffffffffu, incl, c), S = E - __shfl_sync(0xffffffffu, cb, c);
-    const uint64_t cbeg = gbeg + (uint64_t)c * cs;
-    if (cbeg < gend) {
-      pack_chunk(tab, &s_stage[warp][0][0], (uint32_t)__cvta_generic_to_shared(&s_stage[warp][0][0]), in + cbeg,
-                 (uint32_t)min((uint64_t)cs, gend - cbeg), S, E, dst, blk_lim, s_seam, c, lane);
-      // a tensor's last chunk may lie within one block: the part before has it
-      if (c == first && (S & 127u) && (S >> 7) == (E >> 7) && lane == 0) s_seam.idx[c][1] = ~0u;
-    }
-    // the symbols after the part that fall in its last block, two per lane
-    const uint64_t after = gbeg + (uint64_t)(first + kEncWarps) * cs;
-    const uint32_t end = __shfl_sync(0xffffffffu, incl, first + kEncWarps - 1);
-    const bool shared_end = (end & 127u) != 0 && after < gend;
-    if (warp == 0 && shared_end) {
-      const uint64_t i = after + 2 * lane;
-      const uint32_t e0 = i < gend ? enc_entry(tab, in[i]) : 0u, e1 = i + 1 < gend ? enc_entry(tab, in[i + 1]) : 0u;
-      const uint32_t l0 = e0 & 31u, len = l0 + (e1 & 31u);
-      uint32_t pos = len;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, pos, o);
-        if (lane >= o) pos += t;
-      }
-      pos += (end & 127u) - len;
-      auto put = [&](uint32_t code, uint32_t at) {  // an MSB-aligned codeword at bit `at` of the block
-        if (at < 128) atomicOr(&s_more[at >> 5], code >> (at & 31u));
-        if (at < 96 && (at & 31u)) atomicOr(&s_more[(at >> 5) + 1], code << (32u - (at & 31u)));
-      };
-      put(e0 & ~31u, pos);
-      put(e1 & ~31u, pos + l0);
-    }
-    __syncthreads();
-    if (warp == 0)
-      merge_seams(s_seam, dst, blk_lim, shared_end ? end >> 7 : ~0u,
-                  make_uint4(bswap32(s_more[0]), bswap32(s_more[1]), bswap32(s_more[2]), bswap32(s_more[3])), status, lane);
+    if (beg < gend)
+      pack_run(tab, s_stage[warp], in + beg, (uint32_t)(end - beg), gend - end, S, E, next,
+               [&]() -> Place {
+                 return {reinterpret_cast<uint4*>(out + P + excl),
+                         (uint32_t)min((uint64_t)((out_cap - P - excl) / 16), (uint64_t)0xFFFFFFFEu)};
+               },
+               lane);
   }
 }
 
@@ -793,12 +897,20 @@ size_t qlc_encode_workspace_size(size_t n, uint32_t chunk_symbols) {
   return (size_t)(16 + 8 * n_groups_of(n_chunks));
 }
 
-static int enc_grid(uint64_t items, const qlc_launch* launch) {
+// Launches encode_kernel for up to `items` groups, after the previous kernel of
+// the same call (pdl) or by itself.
+static qlc_status launch_groups(const EncArgs& A, uint64_t items, const qlc_launch* launch, bool pdl, cudaStream_t st) {
+  static std::atomic<bool> done[64];
+  if (!smem_ok(encode_kernel, kEncSharedBytes, done)) return QLC_ERR_CUDA;
   int per_sm = kEncCtasPerSm;
-  if (launch && launch->encode_ctas_per_sm > 0 && launch->encode_ctas_per_sm < kEncCtasPerSm)
-    per_sm = launch->encode_ctas_per_sm;
+  if (launch && launch->encode_ctas_per_sm > 0 && launch->encode_ctas_per_sm < per_sm) per_sm = launch->encode_ctas_per_sm;
   const uint64_t cap = (uint64_t)sm_count() * per_sm;
-  return (int)(items < 1 ? 1 : (items < cap ? items : cap));
+  const int grid = (int)(items < 1 ? 1 : (items < cap ? items : cap));
+  if (pdl)
+    launch_after(encode_kernel, grid, kTeams * kTeamThreads, kEncSharedBytes, st, A);
+  else
+    encode_kernel<<<grid, kTeams * kTeamThreads, kEncSharedBytes, st>>>(A);
+  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
 }
 
 // Argument checks of the single-tensor encoders.
@@ -832,13 +944,13 @@ static qlc_status launch_encode(const uint8_t* d_in, size_t n, const uint64_t* d
   const uint64_t n_chunks = (n + cs - 1) / cs;
   if (n > 0 && !looks_back(n, cs)) {
     const int sms = sm_count(), parts = (int)(n_groups_of(n_chunks) * kParts);
-    const int want = (int)((n_chunks + kEncWarps - 1) / kEncWarps), grid = want < 6 * sms ? want : 6 * sms;
+    const int want = (int)((n_chunks + kPartWarps - 1) / kPartWarps), grid = want < 6 * sms ? want : 6 * sms;
     if (hist)
-      launch_after(lengths_kernel<true>, grid, kEncThreads, 0, st, d_in, n, hist, set, d_lut, cs, d_out, d_status);
+      launch_after(lengths_kernel<true>, grid, kPartThreads, 0, st, d_in, n, hist, set, d_lut, cs, d_out, d_status);
     else
-      lengths_kernel<false><<<grid, kEncThreads, 0, st>>>(d_in, n, nullptr, set, d_lut, cs, d_out, d_status);
+      lengths_kernel<false><<<grid, kPartThreads, 0, st>>>(d_in, n, nullptr, set, d_lut, cs, d_out, d_status);
     if (cudaGetLastError() != cudaSuccess) return QLC_ERR_CUDA;
-    launch_after(pack_kernel, parts < kEncCtasPerSm * sms ? parts : kEncCtasPerSm * sms, kEncThreads, 0, st, d_in, n, d_lut,
+    launch_after(pack_kernel, parts < kPackCtasPerSm * sms ? parts : kPackCtasPerSm * sms, kPartThreads, 0, st, d_in, n, d_lut,
                  cs, d_out, out_cap, ob, d_status);
     return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
   }
@@ -863,11 +975,7 @@ static qlc_status launch_encode(const uint8_t* d_in, size_t n, const uint64_t* d
   A.status = d_status;
   A.out_cap = out_cap;
   A.gstat_cap = (ws_bytes - 16) / 8;
-  if (hist)
-    launch_after(encode_kernel, enc_grid(A.n_items, nullptr), kEncThreads, 0, st, A);
-  else
-    encode_kernel<<<enc_grid(A.n_items, nullptr), kEncThreads, 0, st>>>(A);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  return launch_groups(A, A.n_items, nullptr, hist != nullptr, st);
 }
 
 qlc_status qlc_encode(const uint8_t* d_in, size_t n, const qlc_lut* d_lut, uint32_t chunk_symbols,
@@ -932,8 +1040,7 @@ qlc_status qlc_test_encode_stalled_lookback(const uint8_t* d_in, size_t n, const
   A.status = d_status;
   A.out_cap = out_cap;
   A.gstat_cap = (ws_bytes - 16) / 8;
-  encode_kernel<<<enc_grid(A.n_items, nullptr), kEncThreads, 0, st>>>(A);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  return launch_groups(A, A.n_items, nullptr, false, st);
 }
 
 qlc_status qlc_encode_batch(const qlc_desc* d_descs, int n_shards, uint32_t chunk_symbols, void* d_ws,
@@ -957,8 +1064,7 @@ qlc_status qlc_encode_batch(const qlc_desc* d_descs, int n_shards, uint32_t chun
   A.status = d_status;
   A.gstat_cap = w.gstat_cap;
   // the item count is only known on the device: launch the full resident grid
-  launch_after(encode_kernel, enc_grid(~0ull, h_launch), kEncThreads, 0, st, A);
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  return launch_groups(A, ~0ull, h_launch, true, st);
 }
 
 }  // extern "C"

@@ -5,6 +5,8 @@
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/qlc.h"
 
 namespace qlc {
@@ -52,6 +54,18 @@ __host__ __device__ __forceinline__ bool aligned(const void* p, uintptr_t a) {
 // First error wins.
 __device__ __forceinline__ void set_status(uint32_t* st, uint32_t code) {
   if (st) atomicCAS(st, 0u, code);
+}
+
+// Raises a kernel's shared-memory limit, once per device (a function
+// attribute, allowed inside stream capture).
+template <typename K>
+static bool smem_ok(K kernel, size_t bytes, std::atomic<bool> (&done)[64]) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
+  if (dev < 64 && done[dev].load(std::memory_order_relaxed)) return true;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
+  if (dev < 64) done[dev].store(true, std::memory_order_relaxed);
+  return true;
 }
 
 // Checked build (-DQLC_CHECKED): QLC_GUARD(cond, status) is false when an
