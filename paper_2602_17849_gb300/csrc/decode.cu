@@ -527,10 +527,20 @@ decode_batch_kernel(const qlc_desc* __restrict__ descs, int n_shards,
   const unsigned long long total = item_base[n_shards];
   int cur = -1, bad = -1;
   DecHeader h;
+  // Items t + 1 .. t_end - 1 are taken.  While more than eight per warp are left
+  // a warp takes several in a row, mostly of one shard, whose table it then
+  // builds once: 48000 groups 3379 -> 3357 us, 25600 in 400 shards 1855 -> 1848;
+  // with twice as many at a time the last ones take too long (1897).
+  unsigned long long t = 0, t_end = 0;
   while (true) {
-    unsigned long long t = 0;
-    if (lane == 0) t = atomicAdd(ticket, 1u);
-    t = __shfl_sync(0xffffffffu, t, 0);
+    if (++t >= t_end) {
+      const uint32_t left = t < total ? (uint32_t)min(total - t, 0xFFFFFFFFull) : 0u;
+      const uint32_t k = min(max(left / (4 * gridDim.x), 1u), 4u);
+      uint32_t first = 0;
+      if (lane == 0) first = atomicAdd(ticket, k);
+      t = __shfl_sync(0xffffffffu, first, 0);
+      t_end = t + k;
+    }
     if (t >= total) break;
     const int sh = shard_of_warp(item_base, n_shards, t, lane);
     if (sh == bad) continue;
