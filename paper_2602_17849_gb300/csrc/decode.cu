@@ -269,7 +269,7 @@ __device__ __forceinline__ void put_tile(void* out, uint32_t tile_s, float sc, u
 // instead of out: a pointer that is not a kernel parameter would otherwise
 // hold two registers across the decoding loop, which then issued about 10 %
 // more instructions (the batch decoder, 124.3 M against 112.8 M on 256 MiB).
-template <int kOut, Ring kRing>
+template <int kOut, Ring kRing, bool kTile = true>
 __device__ __forceinline__ void decode_group(const DecHeader& h, const uint8_t* __restrict__ in, void* __restrict__ out,
                              const float* __restrict__ scales, uint64_t g, LaneShared& sm, const uint8_t* T, LaneDec& d,
                              uint32_t* status, int lane, bool aligned32, bool sc_vec = false,
@@ -336,7 +336,7 @@ __device__ __forceinline__ void decode_group(const DecHeader& h, const uint8_t* 
     const float sc = (b & 3u) == 0 ? sc_cur.x : (b & 3u) == 1 ? sc_cur.y : (b & 3u) == 2 ? sc_cur.z : sc_cur.w;
     const uint32_t cnt = nsym > i0 ? min(kBlk, nsym - i0) : 0u;
     void* o = out_slot ? *out_slot : out;
-    const bool whole = kOut != kOutCodes && __all_sync(0xffffffffu, cnt == kBlk);
+    const bool whole = kOut != kOutCodes && kTile && __all_sync(0xffffffffu, cnt == kBlk);
     if (cnt == kBlk) {
       uint32_t w[8];
 #pragma unroll
@@ -451,7 +451,6 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
   }
   const bool aligned32 = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
   const bool sc_vec = (reinterpret_cast<uintptr_t>(scales) & 15u) == 0;  // scales read four at a time
-  const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(sm.tile);
   // as many rounds of groups as the warps need, and no more warps than these
   // rounds need: a last round that is nearly empty costs as much as a full one
   // (200 Mi symbols in chunks of 2048, 3200 groups on 3040 warps: 158 us)
@@ -459,7 +458,14 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
   const uint32_t used = (uint32_t)((h.n_groups + rounds * gridDim.x - 1) / (rounds * gridDim.x));
   if ((uint32_t)warp >= used) return;
   const uint32_t stride = used * gridDim.x;
-  if (used <= (kOut == kOutCodes ? 8 : 4)) {
+  const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(sm.tile);
+  if (kOut != kOutCodes && kOut != QLC_DTYPE_F32 && used <= 3) {
+    // with so few warps what counts is a warp's own chain, which is shorter
+    // without the tile for 2-byte values (26 Mi in chunks of 2048 60.6 -> 56 us;
+    // at four warps 111 us with it, 126 without)
+    for (uint64_t g = first; g < h.n_groups; g += stride)
+      decode_group<kOut, kRingFew, false>(h, in, out, scales, g, sm.lanes, T, d, status, lane, aligned32, sc_vec);
+  } else if (used <= (kOut == kOutCodes ? 8 : 4)) {
     for (uint64_t g = first; g < h.n_groups; g += stride)
       decode_group<kOut, kRingFew>(h, in, out, scales, g, sm.lanes, T, d, status, lane, aligned32, sc_vec, tile_s);
   } else {

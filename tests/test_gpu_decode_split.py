@@ -68,6 +68,36 @@ def test_values_on_both_sides_of_the_choice(qlc, dtype):
         assert torch.equal(y.view(torch.int16), want.view(torch.int16)), n
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n", [8 << 20, (8 << 20) + 32, 400 * 32768 + 45, 540 * 32768, 700 * 32768 + 77])
+def test_values_by_groups_per_sm(qlc, dtype, n):
+    """Chunks of 1024: both sides of the choice, then up to 3, 4 and 5 groups per SM."""
+    codes = inputs.make_e4m3("t4", n, seed=n % 97, device="cuda")
+    scales = torch.rand((n + 31) // 32, device="cuda") + 0.01
+    codec = qlc.Codec(n, 1024)
+    cont = codec.new_container()
+    codec.encode_into(codes, cont)
+    y, want = torch.zeros(n, dtype=dtype, device="cuda"), torch.zeros(n, dtype=dtype, device="cuda")
+    qlc.qlc_decode_dequantize(cont, scales, y, codec.n_out, codec.status)
+    qlc.qlc_dequantize_e4m3(codes, scales, want)
+    codec.check()
+    assert torch.equal(y.view(torch.int16), want.view(torch.int16))
+
+
+def test_batch_warps_that_take_several_groups(qlc):
+    """4900 groups on one warp per SM: four at a time, across shards, then fewer."""
+    sizes = [(1 << 16) * i + 16 * i for i in range(50)]
+    xs = [inputs.make_e4m3("t4", n, seed=i, device="cuda") for i, n in enumerate(sizes)]
+    assert sum(sizes) > 64 << 20
+    b = qlc.Batch(xs, 512, launch=(0, 1))
+    b.encode()
+    b.decode()
+    torch.cuda.synchronize()
+    b.check()
+    for i, x in enumerate(xs):
+        assert torch.equal(b.output(i), x), i
+
+
 def test_corrupt_payload_and_index_statuses(qlc):
     rng = np.random.default_rng(3)
     for sid, cs in ((1, 4096), (2, 1024), (1, 1280)):
