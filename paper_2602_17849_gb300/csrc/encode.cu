@@ -567,14 +567,16 @@ __device__ __forceinline__ void take_item(const EncArgs& A, uint64_t n_items, Te
   }
 }
 
-// Lengths of a warp's kRun full chunks, cs symbols each from p on (cs a multiple
-// of kBatch), to put(chunk of the run, bits): the next symbols are on their way
-// while a batch is summed.
-template <class Put>
+// Lengths of a warp's kRun full chunks, cs symbols each from p on, to put(chunk
+// of the run, bits): the next kBatch symbols are on their way while a batch is
+// summed.  kPer 1: cs is a multiple of kBatch; 2: half of it (200 Mi symbols 275
+// -> 248 us, a chunk at a time before; the end of a chunk looked for after every
+// 512 symbols, for all sizes alike, costs 9 % at 4096).
+template <int kPer, class Put>
 __device__ __forceinline__ void run_lengths(const WideTable& tab, const uint8_t* p, uint32_t cs, int lane, Put put) {
   constexpr int kV = kBatch / 512;
   const uint4* src = reinterpret_cast<const uint4*>(p) + lane;
-  const uint32_t per = cs / kBatch, total = per * kRun;
+  const uint32_t per = cs / kBatch, total = kPer == 2 ? kRun / 2 : per * kRun;
   uint4 q[2][kV];
   uint32_t bits = 0, left = per, c = 0;
   auto fetch = [&](uint4 (&d)[kV]) {
@@ -584,8 +586,14 @@ __device__ __forceinline__ void run_lengths(const WideTable& tab, const uint8_t*
   };
   auto add = [&](const uint4 (&d)[kV]) {
 #pragma unroll
-    for (int u = 0; u < kV; u++) bits += entry_sum16(tab, d[u]);
-    if (--left == 0) {
+    for (int u = 0; u < kV; u++) {
+      bits += entry_sum16(tab, d[u]);
+      if (kPer == 2 && u % 2 == 1) {
+        put(c++, warp_sum_u32(bits & ((1u << 21) - 1)));
+        bits = 0;
+      }
+    }
+    if (kPer == 1 && --left == 0) {
       put(c++, warp_sum_u32(bits & ((1u << 21) - 1)));
       bits = 0;
       left = per;
@@ -650,7 +658,9 @@ __device__ __forceinline__ void encode_group(const EncArgs& A, EncShared& sh, Te
       if (QLC_GUARD(g * kGroupChunks + c < n_chunks, A.status)) chunk_bits[g * kGroupChunks + c] = (uint16_t)bits;
     };
     if (gend - gbeg == group_syms && cs % kBatch == 0) {
-      run_lengths(tab, p, cs, lane, put);
+      run_lengths<1>(tab, p, cs, lane, put);
+    } else if (gend - gbeg == group_syms && cs == kBatch / 2) {
+      run_lengths<2>(tab, p, cs, lane, put);
     } else {
       for (uint32_t i = 0; i < kRun; i++) {
         const uint64_t cbeg = beg + (uint64_t)i * cs;
