@@ -14,6 +14,15 @@
 // fp32 (or 16 bf16) elements, so one block of 32 is 4 (or 2) lanes and its
 // absmax is a 2 (or 1) step butterfly.  Codes leave as one 8- (or 16-) byte
 // store per lane.
+//
+// One CTA of up to 32 warps per SM, which count into one table of a column per
+// lane (word of code c and lane l at 256 c + 4 l: the 32 lanes of a warp update 32
+// different banks, whatever the codes, and a byte permute makes the address).
+// With a histogram per warp of 8 an update took 2.9 wavefronts of the shared-
+// memory pipe, which was 81 % busy with 16-bit input.  Quantise, LUT and encode,
+// us, before / now: fp32, 256 Mi elements 428 / 405, bf16, 61 Mi 112 / 109.5; 4 Mi
+// fp32 32.4 / 30.5.  Input in flight: three slots per warp (two 413 / 112, four
+// 418 / 110).  fp32 is bound by HBM, bf16 by instruction issue (16 an element).
 #include <cuda_bf16.h>
 
 #include <atomic>
@@ -23,10 +32,15 @@
 
 namespace qlc {
 
-constexpr int kQuantWarps = 8;
+constexpr int kQuantWarps = 32;  // at most, of the one CTA per SM
 constexpr int kQuantThreads = kQuantWarps * 32;
-constexpr int kQuantDepth = 4;  // input ring slots (warp steps) per warp
+constexpr int kQuantDepth = 3;  // input ring slots (warp steps) per warp
 constexpr int kQuantVec = 2;    // 16-byte input vectors per lane and step
+// Shared address of the histogram; dynamic shared memory starts (at 1024) below it.
+constexpr uint32_t kColAddr = 2048;
+constexpr size_t quant_smem(int warps) {
+  return kColAddr - 1024 + (256u << 8) + (size_t)warps * kQuantDepth * kQuantVec * 512;
+}
 
 // The e4m3 byte nearest to v, ties to the even code, saturating (|v| finite).
 // With k = max(exponent of |v|, -6), the grid of e4m3 values around |v| is
@@ -204,18 +218,25 @@ quantize_kernel(const void* __restrict__ x, uint64_t n, uint8_t* __restrict__ co
   constexpr int kLanesPerBlock = 32 / E;
   constexpr uint32_t kStep = 32 * E;             // elements per warp step
   constexpr uint32_t kWords = E / 4;             // code words per lane
-  constexpr uint32_t kSlot = kQuantWarps * kQuantVec * 512u;  // bytes of a ring slot
-  __shared__ uint32_t sh[kQuantWarps][256];  // per-warp histograms
-  __shared__ uint4 ring[kQuantDepth][kQuantWarps][kQuantVec * 32];
-  if (hist) {
-    for (int i = threadIdx.x; i < kQuantWarps * 256; i += kQuantThreads) (&sh[0][0])[i] = 0;
+  constexpr uint32_t kSlot = kQuantVec * 512u;  // bytes of a ring slot
+  extern __shared__ __align__(16) uint8_t quant_sm[];
+  const uint32_t smem_s = (uint32_t)__cvta_generic_to_shared(quant_sm);
+  if (smem_s > kColAddr) {  // does not happen; the host's size counts on it too
+    if (threadIdx.x == 0) set_status(status, QLC_ERR_CUDA);
+    return;
+  }
+  uint8_t* cols = quant_sm + (kColAddr - smem_s);
+  if (hist) {  // the half of each row that is counted in
+    for (uint32_t i = threadIdx.x; i < 256 * 8; i += blockDim.x)
+      reinterpret_cast<uint4*>(cols)[i / 8 * 16 + i % 8] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t* my = sh[warp];
+  const uint32_t cta_warps = blockDim.x / 32;
+  uint4* ring = reinterpret_cast<uint4*>(cols + (256 << 8)) + warp * kQuantDepth * kQuantVec * 32;
   const uint32_t n_steps = (uint32_t)((n + kStep - 1) / kStep);  // <= kQuantMaxSteps
-  const uint32_t warps = gridDim.x * kQuantWarps;
-  const uint32_t first = blockIdx.x * kQuantWarps + warp;
+  const uint32_t warps = gridDim.x * cta_warps;
+  const uint32_t first = blockIdx.x * cta_warps + warp;
   const uint32_t cnt = first < n_steps ? (n_steps - first + warps - 1) / warps : 0;  // this warp's steps
   // this warp's steps whose whole 1 KiB lies inside: all but a ragged last
   const uint32_t nfw = cnt > 0 && first + (cnt - 1) * warps == n_steps - 1 && (uint64_t)n_steps * kStep > n
@@ -226,9 +247,9 @@ quantize_kernel(const void* __restrict__ x, uint64_t n, uint8_t* __restrict__ co
   const bool scale_lane = lane % kLanesPerBlock == 0;
   // copy instruction u of lane l: bytes [512 u + 16 l, + 16) of the step
   const uint8_t* x_copy = static_cast<const uint8_t*>(x) + lane * 16;
-  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(&ring[0][warp][lane]);
-  auto fetch = [&](uint32_t k) {  // step k of this warp into slot k mod kQuantDepth
-    const uint32_t d = ring_s + (k % kQuantDepth) * kSlot;
+  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring + lane);
+  auto fetch = [&](uint32_t k, uint32_t slot) {  // step k of this warp into slot k mod kQuantDepth
+    const uint32_t d = ring_s + slot * kSlot;
     const uint64_t b = (uint64_t)(first + k * warps) * (512u * kQuantVec);
     if (k < nfw) {
 #pragma unroll
@@ -248,25 +269,26 @@ quantize_kernel(const void* __restrict__ x, uint64_t n, uint8_t* __restrict__ co
 #pragma unroll
     for (int j = 0; j < E; j++) {
       if (j < m) {
-        const uint32_t c = __byte_perm(w[j / 4], 0, 0x4440 + (j % 4));
-        atomicAdd(&my[c], 1u);
+        const uint32_t at = __byte_perm(w[j / 4], 4u * lane, 0x5504 | (j % 4) << 4);  // code << 8 | 4 lane
+        asm volatile("red.shared.add.u32 [%0 + %1], %2;" ::"r"(at), "n"(kColAddr), "r"(1u) : "memory");
       }
     }
   };
 #pragma unroll
-  for (uint32_t d = 0; d + 1 < kQuantDepth; d++) fetch(d);
+  for (uint32_t d = 0; d + 1 < kQuantDepth; d++) fetch(d, d);
   bool bad = false;
-  uint32_t s = first, k = 0;
+  uint32_t s = first, k = 0, slot = 0;  // slot: k mod kQuantDepth
   for (; k < nfw; k++, s += warps) {
     // groups committed so far: kQuantDepth - 1 + k; step k's is complete
     // when at most kQuantDepth - 2 are pending
     q_cp_async_wait<kQuantDepth - 2>();
     __syncwarp();
-    fetch(k + kQuantDepth - 1);  // into the slot step k - 1 was read from
+    fetch(k + kQuantDepth - 1, slot == 0 ? kQuantDepth - 1 : slot - 1);  // the slot step k - 1 was read from
     float v[E];
-    const uint4* r = &ring[k % kQuantDepth][warp][lane * kQuantVec];
+    const uint4* r = ring + slot * kQuantVec * 32 + lane * kQuantVec;
 #pragma unroll
     for (int u = 0; u < kQuantVec; u++) QuantIo<kDtype>::unpack(r[u], v + u * QuantIo<kDtype>::kPerVec);
+    slot = slot + 1 == kQuantDepth ? 0 : slot + 1;
     uint32_t w[kWords];
     const float scale = lane_codes<E>(v, w, bad);
     if (scale_lane && QLC_GUARD((uint64_t)s * kStep + lane * E < n, status)) s_lane[(uint64_t)s * (kStep / 32)] = scale;
@@ -284,7 +306,7 @@ quantize_kernel(const void* __restrict__ x, uint64_t n, uint8_t* __restrict__ co
     const uint64_t i = (uint64_t)s * kStep + (uint64_t)lane * E;
     float v[E];
     if (i + E <= n) {
-      const uint4* r = &ring[k % kQuantDepth][warp][lane * kQuantVec];
+      const uint4* r = ring + slot * kQuantVec * 32 + lane * kQuantVec;
 #pragma unroll
       for (int u = 0; u < kQuantVec; u++) QuantIo<kDtype>::unpack(r[u], v + u * QuantIo<kDtype>::kPerVec);
     } else {
@@ -300,10 +322,10 @@ quantize_kernel(const void* __restrict__ x, uint64_t n, uint8_t* __restrict__ co
   q_cp_async_wait<0>();
   if (__syncthreads_or(bad) && threadIdx.x == 0) set_status(status, QLC_ERR_ARG);
   if (hist) {
-    for (int b = threadIdx.x; b < 256; b += kQuantThreads) {
+    for (uint32_t b = threadIdx.x; b < 256; b += blockDim.x) {
       uint32_t t = 0;
-#pragma unroll
-      for (int w = 0; w < kQuantWarps; w++) t += sh[w][b];
+#pragma unroll 8
+      for (uint32_t l = 0; l < 32; l++) t += reinterpret_cast<const uint32_t*>(cols + 256 * b)[(l + b) & 31];
       if (t) atomicAdd(&hist[b], (unsigned long long)t);
     }
   }
@@ -362,24 +384,19 @@ dequantize_kernel(const uint8_t* __restrict__ codes, const float* __restrict__ s
 }  // namespace qlc
 
 namespace qlc {
-// Resident quantiser CTAs per SM (the occupancy calculator's figure, cached
-// per device below 64 and dtype; at least 1).
-static int quant_ctas_per_sm(qlc_dtype dtype) {
-  static std::atomic<int> cached[64][2];
-  const int k = dtype == QLC_DTYPE_F32 ? 0 : 1;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) dev = 64;
-  if (dev < 64) {
-    const int c = cached[dev][k].load(std::memory_order_relaxed);
-    if (c > 0) return c;
-  }
-  int v = 0;
-  const cudaError_t e =
-      k == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, quantize_kernel<QLC_DTYPE_F32>, kQuantThreads, 0)
-             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, quantize_kernel<QLC_DTYPE_BF16>, kQuantThreads, 0);
-  if (e != cudaSuccess || v <= 0) v = 1;
-  if (dev < 64) cached[dev][k].store(v, std::memory_order_relaxed);
-  return v;
+template <int kDtype>
+static qlc_status launch_quantize(const void* x, uint64_t n, uint64_t steps, uint8_t* codes, float* scales,
+                                  unsigned long long* hist, uint32_t* status, cudaStream_t st) {
+  static std::atomic<bool> done[64];
+  if (!smem_ok(quantize_kernel<kDtype>, quant_smem(kQuantWarps), done)) return QLC_ERR_CUDA;
+  // one CTA per SM, each warp looping over its steps with its copies in flight;
+  // small inputs over all SMs, in CTAs of four warps at least
+  const uint64_t sms = sm_count(), per_sm = (steps + sms - 1) / sms;
+  const int warps = per_sm >= kQuantWarps ? kQuantWarps : (int)((per_sm + 3) / 4 * 4);
+  const uint64_t want = (steps + warps - 1) / warps;
+  quantize_kernel<kDtype><<<(int)(want < sms ? want : sms), 32 * warps, quant_smem(warps), st>>>(x, n, codes, scales, hist,
+                                                                                            status);
+  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
 }
 }  // namespace qlc
 
@@ -398,27 +415,23 @@ extern "C" qlc_status qlc_quantize_e4m3(const void* d_x, qlc_dtype dtype, size_t
   if (d_hist && !accumulate && cudaMemsetAsync(d_hist, 0, 256 * sizeof(uint64_t), st) != cudaSuccess)
     return QLC_ERR_CUDA;
   if (n == 0) return QLC_OK;
-  // one resident wave: each CTA loops over its steps with its copies in
-  // flight; inputs above kQuantMaxSteps steps go in several launches (slices
-  // of whole blocks, the histogram accumulating)
+  // inputs above kQuantMaxSteps steps go in several launches (slices of whole
+  // blocks, the histogram accumulating)
   const uint64_t step = (uint64_t)32 * kQuantVec * (dtype == QLC_DTYPE_F32 ? 4 : 8);  // elements per warp step
   const uint64_t elem = dtype == QLC_DTYPE_F32 ? 4 : 2;
   const uint64_t slice = kQuantMaxSteps * step;
-  const uint64_t cap = (uint64_t)sm_count() * quant_ctas_per_sm(dtype);
   unsigned long long* h = reinterpret_cast<unsigned long long*>(d_hist);
   for (uint64_t off = 0; off < n; off += slice) {
     const uint64_t m = n - off < slice ? n - off : slice;
-    const uint64_t want = (m + step * kQuantWarps - 1) / (step * kQuantWarps);
-    const int grid = (int)(want < cap ? want : cap);
     const void* xs = static_cast<const uint8_t*>(d_x) + off * elem;
-    if (dtype == QLC_DTYPE_F32)
-      quantize_kernel<QLC_DTYPE_F32><<<grid, kQuantThreads, 0, st>>>(xs, m, d_codes + off, d_scales + off / 32, h,
-                                                                     d_status);
-    else
-      quantize_kernel<QLC_DTYPE_BF16><<<grid, kQuantThreads, 0, st>>>(xs, m, d_codes + off, d_scales + off / 32, h,
-                                                                      d_status);
+    const uint64_t steps = (m + step - 1) / step;
+    const qlc_status s =
+        dtype == QLC_DTYPE_F32
+            ? launch_quantize<QLC_DTYPE_F32>(xs, m, steps, d_codes + off, d_scales + off / 32, h, d_status, st)
+            : launch_quantize<QLC_DTYPE_BF16>(xs, m, steps, d_codes + off, d_scales + off / 32, h, d_status, st);
+    if (s != QLC_OK) return s;
   }
-  return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  return QLC_OK;
 }
 
 extern "C" qlc_status qlc_dequantize_e4m3(const uint8_t* d_codes, const float* d_scales, size_t n, void* d_out,

@@ -38,3 +38,28 @@ def test_scales_around_the_line(dtype, e):
     assert np.array_equal(scales.cpu().numpy().view(np.uint32), osc.view(np.uint32))
     assert np.array_equal(codes.cpu().numpy(), oc)
     assert torch.equal(hist, torch.bincount(codes.long(), minlength=256))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("per_sm", [1, 4, 5, 31, 32, 33, 65])
+def test_warps_per_cta(dtype, per_sm):
+    """Around the numbers of warp steps where the CTAs grow and where a warp takes
+    a second and third one; the histogram adds to what is there."""
+    from paper_2602_17849_gb300 import _build
+    _build.build()
+    from paper_2602_17849_gb300 import qlc
+    step = 256 if dtype == torch.float32 else 512
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for n in (per_sm * sms * step, per_sm * sms * step + 1, per_sm * sms * step - 37):
+        x = torch.randn(n, generator=torch.Generator().manual_seed(n)).to(dtype)
+        xd = x.cuda()
+        codes = torch.empty(n, dtype=torch.uint8, device="cuda")
+        scales = torch.empty((n + 31) // 32, dtype=torch.float32, device="cuda")
+        hist = torch.ones(256, dtype=torch.int64, device="cuda")
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        qlc.qlc_quantize_e4m3(xd, codes, scales, hist, st, accumulate=True)
+        ost, oc, osc = oracle.quantize_block32(x.float().numpy())
+        assert int(st.item()) == ost == 0
+        assert np.array_equal(scales.cpu().numpy().view(np.uint32), osc.view(np.uint32))
+        assert np.array_equal(codes.cpu().numpy(), oc)
+        assert torch.equal(hist, torch.bincount(codes.long(), minlength=256) + 1)
