@@ -32,6 +32,7 @@
 #include <utility>
 
 #define QLC_FILE_ID 2
+#include "hist_cols.cuh"
 #include "lut.cuh"
 #include "../../include/qlc_testing.h"
 
@@ -873,6 +874,123 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* lut, uint
   }
 }
 
+// ------------------------------------------------------- one CTA
+//
+// Histogram, LUT and encode of a tensor of up to 16 chunks (64 KiB) in one CTA, a
+// warp per chunk: up to this size the three kernels that a larger tensor takes
+// are little but their own latency.  Back to back, us, three kernels / this one:
+// chunks of 4096, 4 KiB 13.7 / 9.4, 16 KiB 14.7 / 10.6, 64 KiB 16.8 / 14.8, 92 KiB
+// 18.6 / 17.9, 128 KiB 18.1 / 21.1; 32 chunks of 1024 12.1 / 12.4, of 2048 15.2 /
+// 17: one SM packs longer than the rest saves, hence 16 chunks.
+constexpr uint32_t kOneChunks = 16;
+struct OneShared {
+  union {
+    uint32_t cols[kHcColWords];     // the histogram's counters, then
+    uint8_t table[256 << 7];        // the encoder table
+  };
+  __align__(16) uint32_t key[256];
+  __align__(16) uint32_t stage[kOneChunks][kWStage];
+  uint32_t chunk_bits[kGroupChunks];
+  unsigned long long bits[8][kHcWarps];
+};
+static_assert(kHcWarps == (int)kGroupChunks && kOneChunks <= kGroupChunks, "a warp for every chunk of a group");
+
+__global__ void __launch_bounds__(kHcThreads)
+encode_one_kernel(const uint8_t* __restrict__ in, uint32_t n, SchemeSet set, uint32_t cs, unsigned long long* hist,
+                  qlc_lut* lut, uint8_t* out, uint64_t out_cap, unsigned long long* out_bytes) {
+  extern __shared__ __align__(16) uint8_t one_smem[];
+  OneShared& sh = *reinterpret_cast<OneShared*>(one_smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t n_chunks = (n + cs - 1) / cs;
+  const uint32_t beg = warp * cs, end = min(beg + cs, n);
+  uint4 next[2] = {};
+  if (beg < n) load_first(next, in + beg, end - beg, lane);
+  // ---- counts: thread tid has that of symbol tid / 4
+  zero_cols(sh.cols, tid);
+  __syncthreads();
+  const uint32_t col = lane_col(sh.cols, lane);
+  count_span(reinterpret_cast<const uint4*>(in), n / 16, col, tid);
+  count_bytes(in + n / 16 * 16, n % 16, col, tid);
+  __syncthreads();
+  const uint32_t count = sum_cols(sh.cols, tid), sym = tid >> 2, part = tid & 3;
+  const uint32_t key = count << 8 | (255u - sym);  // fits: n < 2^24
+  if (part == 0) {
+    hist[sym] = count;
+    sh.key[sym] = key;
+  }
+  __syncthreads();
+  // ---- rank (see rank_of): four threads per symbol, 64 keys each
+  int rank = 0;
+#pragma unroll
+  for (int t = 0; t < 16; t++) {
+    const uint4 q = reinterpret_cast<const uint4*>(sh.key)[4 * t + part];
+    rank += (q.x > key) + (q.y > key) + (q.z > key) + (q.w > key);
+  }
+  rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+  rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+  // ---- scheme (see rank_and_choose)
+  int scheme = 0;
+  if (set.count > 1) {
+    for (int k = 0; k < set.count; k++) {
+      const uint32_t len = lut_entry(set.s[k], rank) & 15u;
+      const uint32_t v = warp_sum_u32(part == 0 ? count * len : 0u);  // at most 11 * 2^17
+      if (lane == 0) sh.bits[k][warp] = v;
+    }
+    __syncthreads();
+    unsigned long long best = ~0ull;
+    for (int k = 0; k < set.count; k++) {
+      unsigned long long t = 0;
+      for (int w = 0; w < kHcWarps; w++) t += sh.bits[k][w];
+      if (t < best) {
+        best = t;
+        scheme = k;
+      }
+    }
+  }
+  const uint32_t entry = lut_entry(set.s[scheme], rank);
+  if (part == 0) {
+    lut->enc[sym] = (uint16_t)entry;
+    lut->dec[rank] = (uint8_t)sym;
+    out[64 + rank] = (uint8_t)sym;
+  }
+  if (tid < (int)(sizeof(qlc_scheme) / 4))
+    reinterpret_cast<uint32_t*>(&lut->scheme)[tid] = reinterpret_cast<const uint32_t*>(&set.s[scheme])[tid];
+  write_header_of(out, n, cs, n_chunks, &set.s[scheme], tid);
+  {
+    const uint32_t e = table_entry(entry);
+    uint4* row = reinterpret_cast<uint4*>(sh.table + 128 * sym);
+#pragma unroll
+    for (uint32_t k = 0; k < 2; k++) row[(2 * part + k + sym) & 7] = make_uint4(e, e, e, e);
+  }
+  __syncthreads();
+  // ---- chunk lengths
+  const PartTable tab = {sh.table + 4 * lane};
+  uint16_t* chunk_bits = reinterpret_cast<uint16_t*>(out + kIndexOff + 8);
+  uint32_t bits = 0;
+  if (beg < n) {
+    bits = chunk_length(tab, in + beg, end - beg, lane);
+    if (lane == 0) chunk_bits[warp] = (uint16_t)bits;
+  }
+  if (lane == 0) sh.chunk_bits[warp] = bits;
+  __syncthreads();
+  // ---- packing
+  const uint32_t cb = sh.chunk_bits[lane], incl = warp_scan(cb);
+  const uint64_t P = payload_start(n_chunks);
+  if (tid == 31) {  // the last lane of the scan
+    const unsigned long long bytes = align16((incl + 7) / 8);
+    *reinterpret_cast<unsigned long long*>(out + kIndexOff) = 0;
+    *reinterpret_cast<unsigned long long*>(out + 48) = bytes;
+    *out_bytes = P + bytes;
+  }
+  const uint32_t E = __shfl_sync(0xffffffffu, incl, warp), S = E - __shfl_sync(0xffffffffu, cb, warp);
+  if (beg < n)
+    pack_run(tab, sh.stage[warp], in + beg, end - beg, n - end, S, E, next,
+             [&]() -> Place {
+               return {reinterpret_cast<uint4*>(out + P), (uint32_t)min((out_cap - P) / 16, (uint64_t)0xFFFFFFFEu)};
+             },
+             lane);
+}
+
 // n = 0: a header-only container.
 __global__ void header_only_kernel(uint8_t* out, uint32_t cs, const qlc_lut* lut,
                                    unsigned long long* out_bytes) {
@@ -1013,6 +1131,14 @@ qlc_status qlc_encode_tensor(const uint8_t* d_in, size_t n, const qlc_scheme* h_
   qlc_status s = check_encode(d_in, n, d_lut, chunk_symbols, d_out, out_cap, d_ws, ws_bytes, d_out_bytes, d_status);
   if (s != QLC_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (n > 0 && n <= (size_t)kOneChunks * chunk_symbols) {
+    static std::atomic<bool> done[64];
+    if (!smem_ok(encode_one_kernel, sizeof(OneShared), done)) return QLC_ERR_CUDA;
+    encode_one_kernel<<<1, kHcThreads, sizeof(OneShared), st>>>(
+        d_in, (uint32_t)n, set, chunk_symbols, reinterpret_cast<unsigned long long*>(d_hist), d_lut, d_out, out_cap,
+        reinterpret_cast<unsigned long long*>(d_out_bytes));
+    return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
+  }
   s = clear_lookback(n, chunk_symbols, d_ws, st);  // before the kernels, which then follow one another directly
   if (s == QLC_OK) s = launch_histogram(d_in, n, d_hist, 0, st);
   if (s != QLC_OK) return s;

@@ -5,6 +5,7 @@ import pytest
 import torch
 
 from paper_2602_17849_gb300 import inputs
+from tests import _split_cases as S
 
 pytestmark = pytest.mark.gpu
 
@@ -31,8 +32,11 @@ def _separate(qlc, x, scheme, cs):
     return c, out
 
 
-# one histogram CTA and several; parts and look-back; no symbols at all
-@pytest.mark.parametrize("n,cs", [(0, 4096), (1, 128), (65536, 1024), (65537, 4096), (300_077, 1024),
+# one CTA for up to 16 chunks; one histogram CTA and several; parts and look-back; no symbols at all
+@pytest.mark.parametrize("n,cs", [(0, 4096), (1, 128), (15, 4096), (127, 128), (129, 128), (4096, 4096), (4097, 4096),
+                                  (16 * 128 - 1, 128), (16 * 128, 128), (16 * 128 + 1, 128), (15 * 640 + 3, 640),
+                                  (16 * 1024 - 1023, 1024), (16 * 4096 - 17, 4096), (16 * 4096, 4096),
+                                  (16 * 4096 + 1, 4096), (32 * 4096, 4096), (4096 * 128, 128), (4096 * 128 + 1, 128), (65536, 1024), (65537, 4096), (300_077, 1024),
                                   (16384 * 128, 128), (16384 * 128 + 1, 128), (5_000_011, 256)])
 @pytest.mark.parametrize("scheme", [1, [1, 2], [2]])
 def test_equals_the_three_calls(qlc, n, cs, scheme):
@@ -48,7 +52,23 @@ def test_equals_the_three_calls(qlc, n, cs, scheme):
     assert torch.equal(c.out_bytes, want.out_bytes) and torch.equal(out, want_out)
 
 
-@pytest.mark.parametrize("n,cs", [(40_000, 1024), (700_001, 4096), (3 << 20, 128)])
+@pytest.mark.parametrize("kind", ["uniform_bytes", "constant", "two"])
+def test_one_cta_of_other_bytes(qlc, kind):
+    """Counts with many ties, one symbol alone and two, against the three calls."""
+    for n, cs in ((777, 128), (16 * 512 - 5, 512), (60_003, 4096)):
+        x = torch.from_numpy(S.data(kind, n, n)).cuda()
+        for scheme in (1, [1, 2]):
+            want, want_out = _separate(qlc, x, scheme, cs)
+            c = qlc.Codec(n, cs, scheme)
+            out = torch.full((c.cap,), 0x5A, dtype=torch.uint8, device="cuda")
+            c.encode_into(x, out)
+            torch.cuda.synchronize()
+            c.check()
+            assert torch.equal(c.hist, want.hist) and torch.equal(c.lut, want.lut), (n, scheme)
+            assert torch.equal(c.out_bytes, want.out_bytes) and torch.equal(out, want_out), (n, scheme)
+
+
+@pytest.mark.parametrize("n,cs", [(9_000, 1024), (40_000, 1024), (700_001, 4096), (3 << 20, 128)])
 def test_captured_in_a_graph(qlc, n, cs):
     c = qlc.Codec(n, cs, [1, 2])
     out = c.new_container()
