@@ -54,7 +54,9 @@ __device__ uint32_t parse_header(const uint8_t* in, uint64_t in_bytes, uint64_t 
   h->n = *reinterpret_cast<const unsigned long long*>(in + 8);
   h->cs = *reinterpret_cast<const uint32_t*>(in + 16);
   h->n_chunks = *reinterpret_cast<const uint32_t*>(in + 20);
-  ok = ok && chunk_symbols_ok(h->cs) && h->n_chunks == (h->n + h->cs - 1) / h->cs;
+  // n_chunks == (n + cs - 1) / cs, without the division
+  const uint64_t up = h->n + h->cs - 1;
+  ok = ok && chunk_symbols_ok(h->cs) && (uint64_t)h->n_chunks * h->cs <= up && up < ((uint64_t)h->n_chunks + 1) * h->cs;
   // dec must be a permutation of 0..255
   if (lane < 8) s_seen[lane] = 0;
   __syncwarp();

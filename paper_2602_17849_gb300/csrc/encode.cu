@@ -768,7 +768,7 @@ lengths_kernel(const uint8_t* __restrict__ in, uint64_t n, const unsigned long l
   __shared__ __align__(16) unsigned long long s_key[kBuild ? 256 : 2];
   __shared__ unsigned long long s_bits[8][kLutThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint64_t n_chunks = (n + cs - 1) / cs;
+  const uint32_t n_chunks = ((uint32_t)n + cs - 1) / cs;  // <= kPartMaxChunks
   dependents_may_start();
   uint32_t e;
   if constexpr (kBuild) {
@@ -811,7 +811,7 @@ pack_kernel(const uint8_t* __restrict__ in, uint64_t n, const qlc_lut* lut, uint
   stage_entry(s_enc + 128 * tid, tid, e);
   if (__syncthreads_or(e == 0)) return;  // lengths_kernel has set the status
   const PartTable tab = {s_enc + 4 * lane};
-  const uint32_t n_chunks = (uint32_t)((n + cs - 1) / cs);  // <= kPartMaxChunks
+  const uint32_t n_chunks = ((uint32_t)n + cs - 1) / cs;  // <= kPartMaxChunks
   const uint32_t n_groups = (uint32_t)n_groups_of(n_chunks);
   const uint64_t P = payload_start(n_chunks);
   unsigned long long* group_off = reinterpret_cast<unsigned long long*>(out + kIndexOff);
