@@ -21,8 +21,8 @@
 // With a histogram per warp of 8 an update took 2.9 wavefronts of the shared-
 // memory pipe, which was 81 % busy with 16-bit input.  Quantise, LUT and encode,
 // us, before / now: fp32, 256 Mi elements 428 / 405, bf16, 61 Mi 112 / 109.5; 4 Mi
-// fp32 32.4 / 30.5.  Input in flight: three slots per warp (two 413 / 112, four
-// 418 / 110).  fp32 is bound by HBM, bf16 by instruction issue (16 an element).
+// fp32 32.4 / 30.5; the kernel alone 220 / 193 and 38 / 33.  Input in flight: three
+// slots per warp (two 413 / 112, four 418 / 110).  fp32 is bound by HBM, bf16 by instruction issue (16 an element).
 #include <cuda_bf16.h>
 
 #include <atomic>
@@ -65,8 +65,9 @@ __device__ __forceinline__ uint32_t e4m3_rne(float v) {
 // code taken from it is the rule's.  Scales from 2^-80 on: below, the residual
 // of an element that matters could be subnormal.  The residual is formed as
 // q0 scale - x and multiplied by -y, which keeps -0.
-// Three FMA-pipe operations per element (bf16, 61 Mi elements with the
-// histogram: 38 us; fp32, 256 Mi: 220 us) replaced a bracket (two conversions of
+// Three FMA-pipe operations per element (bf16, 61 M elements with the
+// histogram: 38 us, 33 with the table of columns; fp32, 256 Mi: 220 and 193 us)
+// replaced a bracket (two conversions of
 // the product moved up and down by 2^-20, an exact division where they
 // differed): bf16 elements, whose quotients often lie on midpoints, sent
 // nearly every warp step to that division (59 us; fp32 234 us).
