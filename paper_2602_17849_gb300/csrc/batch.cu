@@ -57,9 +57,10 @@ __device__ __forceinline__ unsigned long long cta_scan(unsigned long long v, uns
 struct ShardWork {
   uint64_t groups, symbols;
   uint32_t per_group;
+  uint64_t limit;  // symbols of a batch up to which its chunks are decoded split (see split_pays)
 };
 __device__ ShardWork shard_work(int kind, const qlc_desc& d, uint32_t cs, uint32_t* status) {
-  ShardWork w = {0, 0, 0};
+  ShardWork w = {0, 0, 0, 0};
   if (kind == kPlanEncode) {
     const uint64_t n = d.in_bytes;
     const uint64_t n_chunks = (n + cs - 1) / cs;
@@ -91,7 +92,14 @@ __device__ ShardWork shard_work(int kind, const qlc_desc& d, uint32_t cs, uint32
   }
   w.groups = groups ? groups : 1;  // an empty container still gets its header checked
   w.symbols = min((uint64_t)h0.z | (uint64_t)h0.w << 32, (uint64_t)d.out_cap);
-  if (groups && chunk_symbols_ok(h1.x)) w.per_group = SpanShape(h1.x).per_group;  // the decoder refuses another chunk size
+  if (groups && chunk_symbols_ok(h1.x)) {  // the decoder refuses another chunk size
+    w.per_group = SpanShape(h1.x).per_group;
+    const uint64_t c = h1.x;
+    if ((h0.y >> 16 & 0xFFu) == 2)  // codes of one parity
+      w.limit = c < 1024 ? 0 : (c << 13) + (c << 12) - (3u << 20);
+    else
+      w.limit = c < 512 ? 0 : c << 14;
+  }
   return w;
 }
 
@@ -103,16 +111,22 @@ plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs 
   dependents_may_start();
   // every thread keeps its shards' groups and spans per group in item_base
   // until the number of symbols has settled which of them are the items
-  unsigned long long symbols = 0;
+  unsigned long long symbols = 0, limits = 0;
   for (int s = tid; s < n_shards; s += kPlanThreads) {
     const ShardWork sw = shard_work(kind, descs[s], cs, status);
     symbols += sw.symbols;
+    limits += sw.symbols * sw.limit;
     w.item_base[s] = sw.groups | (unsigned long long)sw.per_group << 40;
   }
   bool split = false;
   if (kind == kPlanDecode) {
     symbols = cta_scan(symbols, s_incl, s_warp, tid);
+    // split where that pays for the average symbol: a shard that it does not pay
+    // for is decoded a lane per chunk there, but badly dealt out (135 shards, 18 Mi
+    // symbols in chunks of 1024: 94 us, 37 dealt out evenly; 300 shards, 49 Mi in
+    // chunks of 4096 under Table 2: 368 and 84)
     split = symbols <= kSplitMax;
+    if (split) split = symbols * symbols <= cta_scan(limits, s_incl, s_warp, tid);
   }
   if (tid < 16) w.ticket[tid] = tid == kTicketSymbols && split ? (uint32_t)symbols : 0u;  // the 64 bytes of counters
   unsigned long long total = 0;

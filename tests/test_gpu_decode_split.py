@@ -167,3 +167,19 @@ def test_batches_decoded_in_each_of_three_ways(qlc, total):
     for i, x in enumerate(shards):
         if i != 4:
             assert torch.equal(b.output(i), x), i
+
+
+@pytest.mark.parametrize("scheme", [1, 2, [1, 2]])
+@pytest.mark.parametrize("cs,total", [(256, 6), (512, 7), (512, 9), (1024, 9), (1024, 10), (1024, 15), (1024, 18), (2048, 34)])
+def test_batches_on_both_sides_of_the_choice(qlc, cs, total, scheme):
+    """Mebisymbols around the sizes up to which a batch of such chunks is split."""
+    m, kinds = 40, ("t4", "relu_t4", "gauss", "ffn2")
+    sizes = [(total << 20) * (i + 1) // (m * (m + 1) // 2) // 16 * 16 for i in range(m)]
+    xs = [inputs.make_e4m3(kinds[i % 4], n, seed=i, device="cuda") for i, n in enumerate(sizes)]
+    b = qlc.Batch(xs, cs, schemes=scheme)
+    b.encode()
+    b.decode()
+    torch.cuda.synchronize()
+    b.check()
+    for i, x in enumerate(xs):
+        assert torch.equal(b.output(i), x), i
