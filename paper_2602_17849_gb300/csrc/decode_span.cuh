@@ -119,7 +119,7 @@ __device__ __forceinline__ uint32_t warm_bits(uint32_t len_lo, uint32_t len_hi) 
 // Student-t 2 Mi 15 / 17, 8 Mi 19.1 / 18.4, half zeros 2 Mi 19 / 17.  Values:
 // chunk 4096, fp32, half zeros 29 Mi 70 / 109; chunk 1024, bf16, Student-t 8 Mi
 // 25 / 31, 12 Mi 37 / 33, 16 Mi 40 / 36, half zeros 8 Mi 29 / 31, 16 Mi 46 / 36;
-// chunk 2048, bf16, Student-t 24 Mi 52 / 58; chunk 4096, bf16, Student-t 47 Mi 83
+// chunk 2048, bf16, Student-t 24 Mi 52 / 58, fp32, half zeros 19 Mi 63 / 58; chunk 4096, bf16, Student-t 47 Mi 83
 // / 105, 48 Mi 98 / 105, 60 Mi 121 / 109.
 // Hence the lines, proportional to the chunk; and streams of hardly anything
 // but the shortest codeword (fewer than 1/32 bit per symbol above it) never,
@@ -132,7 +132,8 @@ __device__ __forceinline__ bool split_pays(const DecHeader& h, uint64_t total) {
   const bool fast = mixed_parity(h.len_lo, h.len_hi) && excess >= h.n / 16 * 7;
   const uint64_t cs = h.cs, line = (cs << 13) + (cs << 12);
   const uint64_t values = cs < 1024 ? cs << 12 : min(line, (cs << 14) + (cs << 12) - (12u << 20));
-  const uint64_t most = fast ? (cs < 512 ? 0 : kOut == kOutCodes ? cs << 14 : values) : cs < 1024 ? 0 : line - (3ull << 20);
+  const uint64_t slow = (kOut == kOutCodes ? line : (cs << 13) + (cs << 11)) - (3ull << 20);
+  const uint64_t most = fast ? (cs < 512 ? 0 : kOut == kOutCodes ? cs << 14 : values) : cs < 1024 ? 0 : slow;
   return excess >= h.n / 32 && total <= most;
 }
 
