@@ -498,7 +498,7 @@ struct SpanShared {
 // ---------------------------------------------------------------- batches
 //
 // Three ways, by the batch's size (plan_kernel decides, on the device): split
-// up to kSplitMax symbols; a lane per chunk with the first items dealt out
+// where that pays for its chunks and schemes; a lane per chunk with the first items dealt out
 // evenly while there are no more groups than warps; and, above, a lane per
 // chunk with all items from a counter.
 

@@ -226,7 +226,7 @@ struct NvtxRange {
 // --------------------------------------------- the split decoder's geometry
 constexpr int kSpanWarps = 4;                    // warps per CTA; they share the code table
 constexpr uint32_t kPiece = 128;                 // symbols per lane, about
-constexpr uint64_t kSplitMax = 64ull << 20;      // symbols of a batch decoded split: see split_pays
+constexpr uint64_t kSplitMax = 64ull << 20;      // symbols of a batch decoded split, at most: see split_pays
 
 // Geometry of a container's spans: a chunk takes `lanes` lanes, a warp
 // `chunks` chunks (of one group), a group `per_group` spans.
@@ -270,8 +270,8 @@ constexpr int kPlanThreads = 1024;
 constexpr uint64_t kHistItem = 64 * 1024;  // symbols per histogram work item
 
 // One CTA: the number of work items of every shard (encode: groups of 32
-// chunks; decode: the container's groups, or in a batch of up to kSplitMax
-// symbols sets of kSpanWarps spans),
+// chunks; decode: the container's groups, or in a batch that is decoded split
+// sets of kSpanWarps spans),
 // their exclusive prefix in item_base, and zeroed counters / look-back words.
 // Shards that cannot be processed get no items and set *status.  cs: the chunk
 // size (encode), or the number of SMs (decode).
