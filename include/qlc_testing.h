@@ -34,6 +34,13 @@ qlc_status qlc_test_encode_stalled_lookback(const uint8_t *d_in, size_t n, const
  * Synchronises the device.  In a normal build it returns 0xFFFFFFFF. */
 uint32_t qlc_test_check_take(void);
 
+/* Shared-memory use of the encode kernel, and of the quantise kernel with
+ * `warps` warps: `size` bytes from the fixed shared address `addr` on, out of
+ * `requested` bytes of dynamic shared memory, whose start may be any address up
+ * to addr.  Host only. */
+void qlc_test_encode_smem(uint32_t *addr, uint32_t *size, uint32_t *requested);
+void qlc_test_quantize_smem(int warps, uint32_t *addr, uint32_t *size, uint32_t *requested);
+
 #ifdef __cplusplus
 }
 #endif

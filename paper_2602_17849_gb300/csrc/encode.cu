@@ -512,8 +512,7 @@ struct EncShared {
   __align__(16) uint32_t stage[kTeams * kTeamWarps][kWStage];
   TeamShared team[kTeams];
 };
-// dynamic shared memory starts at 1024
-constexpr size_t kEncSharedBytes = sizeof(EncShared) + kTableAddr - 1024;
+constexpr size_t kEncSharedBytes = fixed_smem_bytes(kTableAddr, sizeof(EncShared));
 
 // Barriers of a team's threads.  The second one is for a group's offset, which
 // warp 0 tells the others.
@@ -720,7 +719,7 @@ __global__ void __launch_bounds__(kTeams* kTeamThreads, kEncCtasPerSm)
 encode_kernel(EncArgs A) {
   extern __shared__ __align__(16) uint8_t enc_smem[];
   const uint32_t smem_s = (uint32_t)__cvta_generic_to_shared(enc_smem);
-  if (smem_s > kTableAddr) {  // does not happen; the host's size counts on it too
+  if (smem_s > kTableAddr) {  // does not happen
     if (threadIdx.x == 0) set_status(A.status, QLC_ERR_CUDA);
     return;
   }
@@ -1144,6 +1143,12 @@ qlc_status qlc_encode_tensor(const uint8_t* d_in, size_t n, const qlc_scheme* h_
   if (s != QLC_OK) return s;
   return launch_encode(d_in, n, d_hist, set, d_lut, chunk_symbols, d_out, out_cap, d_ws, ws_bytes, d_out_bytes, d_status,
                        st);
+}
+
+void qlc_test_encode_smem(uint32_t* addr, uint32_t* size, uint32_t* requested) {
+  *addr = kTableAddr;
+  *size = (uint32_t)sizeof(EncShared);
+  *requested = (uint32_t)kEncSharedBytes;
 }
 
 qlc_status qlc_test_encode_stalled_lookback(const uint8_t* d_in, size_t n, const qlc_lut* d_lut,

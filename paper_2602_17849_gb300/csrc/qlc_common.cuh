@@ -68,6 +68,13 @@ static bool smem_ok(K kernel, size_t bytes, std::atomic<bool> (&done)[64]) {
   return true;
 }
 
+// Dynamic shared memory to ask for when `size` bytes are used from the shared
+// address `addr` on.  Where dynamic shared memory starts is up to the driver
+// (at 1024 on GB300, behind its own kilobyte), so the bytes below addr are asked
+// for too: the end is inside whatever the start, and the kernel itself refuses
+// a start above addr.
+constexpr size_t fixed_smem_bytes(uint32_t addr, size_t size) { return addr + size; }
+
 // Checked build (-DQLC_CHECKED): QLC_GUARD(cond, status) is false when an
 // index check fails; the caller then skips the access.  The first failure of
 // each .cu file is recorded in that file's g_check_site (file number << 16 |

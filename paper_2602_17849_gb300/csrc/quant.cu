@@ -29,6 +29,7 @@
 
 #define QLC_FILE_ID 5
 #include "qlc_common.cuh"
+#include "../../include/qlc_testing.h"
 
 namespace qlc {
 
@@ -36,11 +37,10 @@ constexpr int kQuantWarps = 32;  // at most, of the one CTA per SM
 constexpr int kQuantThreads = kQuantWarps * 32;
 constexpr int kQuantDepth = 3;  // input ring slots (warp steps) per warp
 constexpr int kQuantVec = 2;    // 16-byte input vectors per lane and step
-// Shared address of the histogram; dynamic shared memory starts (at 1024) below it.
+// Shared address of the histogram; dynamic shared memory starts at or below it.
 constexpr uint32_t kColAddr = 2048;
-constexpr size_t quant_smem(int warps) {
-  return kColAddr - 1024 + (256u << 8) + (size_t)warps * kQuantDepth * kQuantVec * 512;
-}
+constexpr size_t quant_used(int warps) { return (256u << 8) + (size_t)warps * kQuantDepth * kQuantVec * 512; }
+constexpr size_t quant_smem(int warps) { return fixed_smem_bytes(kColAddr, quant_used(warps)); }
 
 // The e4m3 byte nearest to v, ties to the even code, saturating (|v| finite).
 // With k = max(exponent of |v|, -6), the grid of e4m3 values around |v| is
@@ -222,7 +222,7 @@ quantize_kernel(const void* __restrict__ x, uint64_t n, uint8_t* __restrict__ co
   constexpr uint32_t kSlot = kQuantVec * 512u;  // bytes of a ring slot
   extern __shared__ __align__(16) uint8_t quant_sm[];
   const uint32_t smem_s = (uint32_t)__cvta_generic_to_shared(quant_sm);
-  if (smem_s > kColAddr) {  // does not happen; the host's size counts on it too
+  if (smem_s > kColAddr) {  // does not happen
     if (threadIdx.x == 0) set_status(status, QLC_ERR_CUDA);
     return;
   }
@@ -402,6 +402,12 @@ static qlc_status launch_quantize(const void* x, uint64_t n, uint64_t steps, uin
 }  // namespace qlc
 
 using namespace qlc;
+
+extern "C" void qlc_test_quantize_smem(int warps, uint32_t* addr, uint32_t* size, uint32_t* requested) {
+  *addr = kColAddr;
+  *size = (uint32_t)quant_used(warps);
+  *requested = (uint32_t)quant_smem(warps);
+}
 
 extern "C" qlc_status qlc_quantize_e4m3(const void* d_x, qlc_dtype dtype, size_t n, uint8_t* d_codes,
                                         float* d_scales, uint64_t* d_hist, int accumulate, uint32_t* d_status,
