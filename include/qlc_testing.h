@@ -34,6 +34,11 @@ qlc_status qlc_test_encode_stalled_lookback(const uint8_t *d_in, size_t n, const
  * Synchronises the device.  In a normal build it returns 0xFFFFFFFF. */
 uint32_t qlc_test_check_take(void);
 
+/* How often the library would raise a kernel's shared-memory limit over a
+ * sequence of calls, call i on device dev[i] in the context with the id id[i] (0:
+ * none), which is id_after[i] once the runtime has been called.  Host only. */
+int qlc_test_once_per_context(const int *dev, const uint64_t *id, const uint64_t *id_after, int calls);
+
 /* Shared-memory use of the encode kernel, and of the quantise kernel with
  * `warps` warps: `size` bytes from the fixed shared address `addr` on, out of
  * `requested` bytes of dynamic shared memory, whose start may be any address up

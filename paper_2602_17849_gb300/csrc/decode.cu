@@ -29,8 +29,6 @@
 // pipe, the shared-memory pipe (table lookups by random codes) and, with 13.5
 // groups per SM, by the chain of a lane's own rounds.  1152 tensors (3.4 GB)
 // 1757 us.
-#include <atomic>
-
 #define QLC_FILE_ID 1
 #include "decode_common.cuh"
 #include "decode_span.cuh"
@@ -700,7 +698,7 @@ using namespace qlc;
 template <int kOut>
 static qlc_status launch_decode(const uint8_t* d_in, size_t in_bytes, void* d_out, const float* d_scales,
                                 size_t out_cap, uint64_t* d_n_out, uint32_t* d_status, cudaStream_t st) {
-  static std::atomic<bool> done[64];
+  static OncePerContext done;
   if (!smem_ok(decode_kernel<kOut>, one_bytes(dec_warps(kOut)), done)) return QLC_ERR_CUDA;
   // a warp for every span there can be, four at least (a CTA of all warps and
   // their shared memory starts 1 to 3 us later)
@@ -750,7 +748,7 @@ extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, vo
   int per_sm = kDecCtasPerSm;
   if (h_launch && h_launch->decode_ctas_per_sm > 0 && h_launch->decode_ctas_per_sm < kDecCtasPerSm)
     per_sm = h_launch->decode_ctas_per_sm;
-  static std::atomic<bool> done[64];
+  static OncePerContext done;
   if (!smem_ok(decode_few_kernel, sizeof(FewShared), done)) return QLC_ERR_CUDA;
   // which of the two has the work is decided on the device; the other returns at once
   const int sms = sm_count();

@@ -25,8 +25,6 @@
 // 223 us (the re-reads then miss L2); pass 1 and pass 2 as two kernels 78 + 140
 // us; shift and OR by one wide multiply-add 193 us (fewer integer instructions,
 // more in all).
-#include <cuda.h>
-
 #include <mutex>
 #include <unordered_map>
 #include <utility>
@@ -1027,7 +1025,7 @@ size_t qlc_encode_workspace_size(size_t n, uint32_t chunk_symbols) {
 // Launches encode_kernel for up to `items` groups, after the previous kernel of
 // the same call (pdl) or by itself.
 static qlc_status launch_groups(const EncArgs& A, uint64_t items, const qlc_launch* launch, bool pdl, cudaStream_t st) {
-  static std::atomic<bool> done[64];
+  static OncePerContext done;
   if (!smem_ok(encode_kernel, kEncSharedBytes, done)) return QLC_ERR_CUDA;
   int per_sm = kEncCtasPerSm;
   if (launch && launch->encode_ctas_per_sm > 0 && launch->encode_ctas_per_sm < per_sm) per_sm = launch->encode_ctas_per_sm;
@@ -1131,7 +1129,7 @@ qlc_status qlc_encode_tensor(const uint8_t* d_in, size_t n, const qlc_scheme* h_
   if (s != QLC_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (n > 0 && n <= (size_t)kOneChunks * chunk_symbols) {
-    static std::atomic<bool> done[64];
+    static OncePerContext done;
     if (!smem_ok(encode_one_kernel, sizeof(OneShared), done)) return QLC_ERR_CUDA;
     encode_one_kernel<<<1, kHcThreads, sizeof(OneShared), st>>>(
         d_in, (uint32_t)n, set, chunk_symbols, reinterpret_cast<unsigned long long*>(d_hist), d_lut, d_out, out_cap,
@@ -1224,32 +1222,6 @@ namespace qlc {
 constexpr uint64_t kNoAllocMaxGroups = 65536;
 constexpr size_t kNoAllocScratchBytes = 16 + 8 * kNoAllocMaxGroups;  // 512 KiB + 16 B
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
-
-// Unique id of the calling thread's current CUDA context, 0 if there is none
-// or the driver cannot report it.  The driver entry points come through the
-// runtime, so the library needs no link to the driver library.
-static unsigned long long current_context_id() {
-  using GetCurrent = CUresult (*)(CUcontext*);
-  using GetId = CUresult (*)(CUcontext, unsigned long long*);
-  static GetCurrent get_current = nullptr;
-  static GetId get_id = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      get_current = reinterpret_cast<GetCurrent>(f);
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      get_id = reinterpret_cast<GetId>(f);
-  });
-  CUcontext ctx = nullptr;
-  unsigned long long id = 0;
-  if (!get_current || !get_id || get_current(&ctx) != CUDA_SUCCESS || !ctx || get_id(ctx, &id) != CUDA_SUCCESS)
-    return 0;
-  return id;
-}
 
 // Device address of g_noalloc_scratch in the current device's context (the
 // host-side symbol is not a device address).  It is looked up with the

@@ -5,9 +5,12 @@
 #include "lut.cuh"
 #include "../../include/qlc_testing.h"
 
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 #include <functional>
+#include <mutex>
 
 namespace qlc {
 
@@ -52,6 +55,31 @@ lut_best_kernel(const unsigned long long* __restrict__ hists, SchemeSet set, qlc
   dependency_wait();
   const LutRow row = rank_and_choose(hists + (size_t)blockIdx.x * 256, set, key, bits, tid);
   write_lut(luts + blockIdx.x, row, set, tid);
+}
+
+// The driver entry points come through the runtime, so the library needs no
+// link to the driver library.
+unsigned long long current_context_id() {
+  using GetCurrent = CUresult (*)(CUcontext*);
+  using GetId = CUresult (*)(CUcontext, unsigned long long*);
+  static GetCurrent get_current = nullptr;
+  static GetId get_id = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      get_current = reinterpret_cast<GetCurrent>(f);
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      get_id = reinterpret_cast<GetId>(f);
+  });
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+  if (!get_current || !get_id || get_current(&ctx) != CUDA_SUCCESS || !ctx || get_id(ctx, &id) != CUDA_SUCCESS)
+    return 0;
+  return id;
 }
 
 int sm_count() {
@@ -315,4 +343,16 @@ extern "C" uint32_t qlc_test_check_take(void) {
 #else
   return 0xFFFFFFFFu;
 #endif
+}
+
+extern "C" int qlc_test_once_per_context(const int* dev, const uint64_t* id, const uint64_t* id_after, int calls) {
+  qlc::OncePerContext once;
+  int done = 0;
+  for (int i = 0; i < calls; i++) {
+    bool acted = false;
+    once.ensure(dev[i], [&] { return acted ? (unsigned long long)id_after[i] : (unsigned long long)id[i]; },
+                [&] { return acted = true; });
+    done += acted;
+  }
+  return done;
 }

@@ -56,16 +56,41 @@ __device__ __forceinline__ void set_status(uint32_t* st, uint32_t code) {
   if (st) atomicCAS(st, 0u, code);
 }
 
-// Raises a kernel's shared-memory limit, once per device (a function
-// attribute, allowed inside stream capture).
+// Unique id of the calling thread's current CUDA context, 0 if there is none
+// or the driver cannot report it (hist_lut.cu).
+unsigned long long current_context_id();
+
+// Something that has to be done once in every context, by device: the id of
+// the context it was last done in.  A context's id is never given out again, so
+// a device reset or another context on the device is seen; without an id it is
+// done every time.  Any number of threads may call at once.
+class OncePerContext {
+ public:
+  template <class Id, class Do>
+  bool ensure(int dev, Id id_of, Do act) {
+    const unsigned long long id = id_of();
+    const bool kept = dev >= 0 && dev < kDevices;
+    if (kept && id != 0 && at_[dev].load(std::memory_order_relaxed) == id) return true;
+    if (!act()) return false;
+    // act makes the device's primary context current if none was
+    if (kept) at_[dev].store(id_of(), std::memory_order_relaxed);
+    return true;
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::atomic<unsigned long long> at_[kDevices] = {};
+};
+
+// Raises a kernel's shared-memory limit (a function attribute of the context,
+// allowed inside stream capture).
 template <typename K>
-static bool smem_ok(K kernel, size_t bytes, std::atomic<bool> (&done)[64]) {
+static bool smem_ok(K kernel, size_t bytes, OncePerContext& done) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
-  if (dev < 64 && done[dev].load(std::memory_order_relaxed)) return true;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
-  if (dev < 64) done[dev].store(true, std::memory_order_relaxed);
-  return true;
+  return done.ensure(dev, current_context_id, [&] {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  });
 }
 
 // Dynamic shared memory to ask for when `size` bytes are used from the shared

@@ -25,8 +25,6 @@
 // slots per warp (two 413 / 112, four 418 / 110).  fp32 is bound by HBM, bf16 by instruction issue (16 an element).
 #include <cuda_bf16.h>
 
-#include <atomic>
-
 #define QLC_FILE_ID 5
 #include "qlc_common.cuh"
 #include "../../include/qlc_testing.h"
@@ -388,7 +386,7 @@ namespace qlc {
 template <int kDtype>
 static qlc_status launch_quantize(const void* x, uint64_t n, uint64_t steps, uint8_t* codes, float* scales,
                                   unsigned long long* hist, uint32_t* status, cudaStream_t st) {
-  static std::atomic<bool> done[64];
+  static OncePerContext done;
   if (!smem_ok(quantize_kernel<kDtype>, quant_smem(kQuantWarps), done)) return QLC_ERR_CUDA;
   // one CTA per SM, each warp looping over its steps with its copies in flight;
   // small inputs over all SMs, in CTAs of four warps at least
