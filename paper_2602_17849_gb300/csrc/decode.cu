@@ -413,7 +413,7 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
   extern __shared__ __align__(16) uint8_t one_sm[];
   __shared__ uint8_t T[2048];                       // code -> symbol
   __shared__ __align__(16) uint8_t hdr[kIndexOff];  // the container's header and dec
-  __shared__ uint32_t seen[kWarps][8];
+  __shared__ uint32_t seen[kWarps][8], s_slow;
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // so known to be the same in all lanes
   const uint32_t warps = blockDim.x / 32;
@@ -426,10 +426,18 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
     if (err) set_status(status, err);
   }
   if (err) return;
+  const SplitData sd = {h.cs, h.len_lo, h.len_hi, h.n, h.payload_bytes};
+  const bool ask = split_samples(sd, kOut != kOutCodes, h.n);
+  if (ask && warp == 0) {  // every CTA looks at the same samples
+    static_assert(kSamples == 32 && 4 * 32 * kSampleWords <= sizeof(SpanWarp), "a sample per lane");
+    const bool slow = sample_is_slow(in, sd, h.n_chunks, lane, reinterpret_cast<uint32_t*>(one_sm) + lane * kSampleWords);
+    const unsigned all = __ballot_sync(0xffffffffu, slow);
+    if (lane == 0) s_slow = __popc(all);
+  }
   build_table(hdr, T, tid, blockDim.x);
   __syncthreads();
   const uint32_t first = (uint32_t)warp * gridDim.x + blockIdx.x;
-  if (split_pays<kOut>(h, h.n)) {
+  if (h.n <= split_most(sd, kOut != kOutCodes, ask ? s_slow : 0)) {
     const uint32_t stride = warps * gridDim.x;
     const SpanShape shape(h.cs);
     const uint32_t warm = warm_bits(h.len_lo, h.len_hi);
@@ -667,7 +675,8 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
     }
     if (!err) {
       const uint64_t s = (uint64_t)q * kSpanWarps + warp;
-      if (split_pays<kOutCodes>(h, batch_symbols)) {
+      const SplitData sd = {h.cs, h.len_lo, h.len_hi, h.n, h.payload_bytes};
+      if (batch_symbols <= split_most(sd, false, 0)) {
         const SpanShape shape(h.cs);
         const uint32_t k = (uint32_t)lane / shape.lanes, seg = (uint32_t)lane - k * shape.lanes;
         const uint64_t g = s / shape.per_group;

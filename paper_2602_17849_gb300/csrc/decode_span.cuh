@@ -8,7 +8,8 @@
 //   load     the span's bits go to shared memory, byte-swapped;
 //   guess    each lane but a chunk's first starts kWarm bits before its piece
 //            and steps over codewords (the 3-bit area code fixes the length)
-//            until it enters its piece;
+//            until it enters its piece; in a chunk whose codewords all have
+//            one length, as in padding, the boundaries are known;
 //   decode   each lane decodes from there to the end of its piece into its
 //            column of a staging table, and notes where it left the piece
 //            (its exit) and how many symbols it found;
@@ -16,9 +17,18 @@
 //            whose guess was another one decode again from there, until
 //            entries and exits agree all along every chunk: then, from each
 //            chunk's first lane on, every entry is the true one.  At most as
-//            many rounds as a chunk has pieces; nearly always none or one;
+//            many rounds as a chunk has pieces; nearly always none or one.  In
+//            a run of one symbol nobody resynchronises: pieces that repeat
+//            one codeword take their boundaries from where the run begins,
+//            all at once, and need no decoding;
 //   flush    a prefix sum of the counts places the lanes' symbols, which meet
 //            in shared memory and leave in whole lines.
+// Half of a tensor zeros (Student-t, Table 1, chunks of 4096): 1 Mi 103 -> 15 us,
+// 16 Mi 156 -> 27; the second half of every chunk 56 -> 19 and 144 -> 45; one chunk
+// of zeros in 64 Mi 191 -> 74 (none: 74); 64 Mi equal symbols under ranks of other
+// data 899 -> 69, since runs are not corrected piece after piece.  What still does
+// not resynchronise (sparse data, repeated patterns) is found by samples, and
+// larger containers of it are decoded a lane per chunk (split_rule.cuh).
 // A chunk is valid when its last piece ends at its last bit and its counts
 // add up to its symbols, which is when decoding it serially ends at its last
 // bit after that many symbols.
@@ -29,6 +39,7 @@
 #pragma once
 
 #include "decode_common.cuh"
+#include "split_rule.cuh"
 
 namespace qlc {
 
@@ -99,43 +110,130 @@ __device__ __forceinline__ uint32_t four_symbols(const uint32_t* bits, uint32_t&
 // lengths are all even but the last area's keeps a wrong parity until such a
 // code comes by, and gets twice as much (Table 2: 99 %).
 constexpr uint32_t kWarm = 264;
-__device__ __forceinline__ bool mixed_parity(uint32_t len_lo, uint32_t len_hi) {
-  return ((len_lo | (len_hi & 0xFFFFFFu)) & 0x01010101u) != 0;
-}
+constexpr int kRounds = 64;  // of corrections, twice as many as there can be
 __device__ __forceinline__ uint32_t warm_bits(uint32_t len_lo, uint32_t len_hi) {
   return mixed_parity(len_lo, len_hi) ? kWarm : 2 * kWarm;
 }
 
-// Whether to decode a container split, where `total` symbols are decoded in
-// this launch.  A lane per chunk takes at least the time of its chain, about 19
-// us per 1024 symbols of chunk, and hardly more up to 40 Mi symbols; split, the
-// time goes with the size, and is longer where readers are slow to find the
-// true boundaries: in schemes of one parity, and in streams of mostly the
-// shortest codeword.  Measured (us, split / lane per chunk): chunk 4096,
-// Student-t 1 Mi 15 / 79, 16 Mi 27 / 80, 64 Mi 72 / 85, half zeros under Table 2
-// 43 Mi 77 / 81; chunk 2048, Student-t 32 Mi 43 / 53, half zeros under Table 2
-// 16 Mi 40 / 45, 32 Mi 58 / 53; chunk 1024, Student-t 8 Mi 19 / 27, 16 Mi 29 /
-// 31, 32 Mi 44 / 33, half zeros 8 Mi 25 / 27, 16 Mi 39 / 31; chunk 512,
-// Student-t 2 Mi 15 / 17, 8 Mi 19.1 / 18.4, half zeros 2 Mi 19 / 17.  Values:
-// chunk 4096, fp32, half zeros 29 Mi 70 / 109; chunk 1024, bf16, Student-t 8 Mi
-// 25 / 31, 12 Mi 37 / 33, 16 Mi 40 / 36, half zeros 8 Mi 29 / 31, 16 Mi 46 / 36;
-// chunk 2048, bf16, Student-t 24 Mi 52 / 58, fp32, half zeros 19 Mi 63 / 58; chunk 4096, bf16, Student-t 47 Mi 83
-// / 105, 48 Mi 98 / 105, 60 Mi 121 / 109.
-// Hence the lines, proportional to the chunk; and streams of hardly anything
-// but the shortest codeword (fewer than 1/32 bit per symbol above it) never,
-// since they do not find the boundaries from a wrong phase, and their pieces
-// are corrected one after the other (64 Mi equal symbols 1216 us).
-template <int kOut>
-__device__ __forceinline__ bool split_pays(const DecHeader& h, uint64_t total) {
-  const uint64_t bits = 8 * h.payload_bytes, least = h.n * (h.len_lo & 0xFFu);
-  const uint64_t excess = bits > least ? bits - least : 0;
-  const bool fast = mixed_parity(h.len_lo, h.len_hi) && excess >= h.n / 16 * 7;
-  const uint64_t cs = h.cs, line = (cs << 13) + (cs << 12);
-  const uint64_t values = cs < 1024 ? cs << 12 : min(line, (cs << 14) + (cs << 12) - (12u << 20));
-  const uint64_t slow = (kOut == kOutCodes ? line : (cs << 13) + (cs << 11)) - (3ull << 20);
-  const uint64_t most = fast ? (cs < 512 ? 0 : kOut == kOutCodes ? cs << 14 : values) : cs < 1024 ? 0 : slow;
-  return excess >= h.n / 32 && total <= most;
+// A lane's piece: bits [beg, end) of the chunk [cb, ce), positions in the span's
+// bits; piece number seg of the chunk.
+struct Piece {
+  uint32_t cb, ce, beg, end, seg;
+};
+
+// The first codeword boundary at or after `end`, from the boundary at.
+__device__ __forceinline__ uint32_t walk_to(const uint32_t* bits, uint32_t at, uint32_t end, uint32_t len_lo,
+                                            uint32_t len_hi) {
+  uint32_t p[4];
+  while (at < end) {
+    four_ends(bits, at, len_lo, len_hi, p);
+    at = p[0] >= end ? p[0] : p[1] >= end ? p[1] : p[2] >= end ? p[2] : p[3];
+  }
+  return at;
 }
+
+// Corrections (see decode_span).  A run of one symbol repeats its codeword: a
+// reader that starts at a wrong bit stays on the wrong boundaries as long as the
+// run lasts, and the true ones are known only from where the run begins.
+//
+// The period, up to kMaxCode, of the bits from the tenth bit of the piece to the
+// tenth behind it, or to the chunk's end; 0 if they have none.  The first 32 bits
+// rule nearly every piece out that is no run.
+__device__ __forceinline__ uint32_t run_period(const uint32_t* bits, const Piece& pc) {
+  const uint32_t from = pc.beg + kMaxCode - 1, to = min(pc.end + kMaxCode - 1, pc.ce);
+  if (from + 32 + kMaxCode > to) return 0;  // hardly longer than what it would save
+  const SpanBits w(bits, from);
+  uint32_t period = 0;
+#pragma unroll
+  for (uint32_t p = kMaxCode; p > 0; p--) period = w.x == __funnelshift_l(w.y, w.x, p) ? p : period;
+  if (period) {
+    // bit t against bit t + period, the last one below the chunk's end
+    const uint32_t stop = min(to, pc.ce - period);
+    for (uint32_t t = from + 32; t < stop; t += 32) {
+      const SpanBits v(bits, t);
+      uint32_t differ = v.x ^ __funnelshift_l(v.y, v.x, period);
+      if (stop - t < 32) differ >>= 32 - (stop - t);
+      if (differ) return 0;
+    }
+  }
+  return period;
+}
+
+// What a lane learns from a run that its piece goes on with from the piece
+// before: its entry, and the run's codeword length and symbol.
+struct Run {
+  uint32_t entry, len, sym;  // len 0: no run
+};
+
+// Called by all lanes, with the boundary x that the piece before leaves to this
+// one.  The boundaries of a run are those of its first piece.  A function of its
+// own, so that its registers and code are not the decoder's (inlined it cost 3 %).
+__device__ __noinline__ Run follow_run(const uint32_t* bits, const uint8_t* T, Piece pc, bool mine, uint32_t x,
+                                       uint32_t len_lo, uint32_t len_hi, int lane) {
+  const uint32_t period = mine ? run_period(bits, pc) : 0u;
+  if (!__any_sync(0xffffffffu, period != 0)) return {0u, 0u, 0u};
+  const uint32_t period_before = __shfl_up_sync(0xffffffffu, period, 1);
+  const bool goes_on = period != 0 && pc.seg != 0 && period_before == period;
+  const uint32_t heads = ~__ballot_sync(0xffffffffu, goes_on);
+  const int head = 31 - __clz(heads & (0xFFFFFFFFu >> (31 - lane)));
+  // a boundary within the run, the length there and the symbol (of use in heads)
+  uint32_t len = 0, sym = 0;
+  if (period) {
+    x = walk_to(bits, x, pc.beg + kMaxCode - 1, len_lo, len_hi);
+    const SpanBits w(bits, x);
+    len = code_len(w.x, len_lo, len_hi);
+    const uint32_t code = __funnelshift_l(w.x, 0u, len);
+    sym = QLC_GUARD(code < 2048u, nullptr) ? T[code] : 0u;
+  }
+  x = __shfl_sync(0xffffffffu, x, head);
+  len = __shfl_sync(0xffffffffu, len, head);
+  sym = __shfl_sync(0xffffffffu, sym, head);
+  if (!goes_on || len % period != 0 || x > pc.beg) return {0u, 0u, 0u};
+  return {x + (pc.beg - x + len - 1) / len * len, len, sym};
+}
+
+// Whether readers are slow to find the boundaries at sample i of a container: in
+// a group's first chunk, somewhere, readers from three bits in a row have not met
+// after `warm` bits.  A chunk of one codeword length has its boundaries known.
+// Nothing is taken for granted of the container but its n_chunks and payload
+// being inside it.  words: kSampleWords of shared memory.
+constexpr uint32_t kSampleVecs = 5, kSampleWords = 4 * kSampleVecs + 1;
+__device__ __forceinline__ bool sample_is_slow(const uint8_t* in, const SplitData& d, uint64_t n_chunks, uint32_t i,
+                                               uint32_t* words) {
+  const uint64_t n_groups = n_groups_of(n_chunks), g = i * n_groups / kSamples, first = g * kGroupChunks * d.cs;
+  if (n_groups == 0 || first >= d.n) return false;
+  const uint64_t goff = reinterpret_cast<const unsigned long long*>(in + kIndexOff)[g];
+  const uint32_t bits = reinterpret_cast<const uint16_t*>(in + kIndexOff + 8 * n_groups)[g * kGroupChunks];
+  const uint32_t nsym = (uint32_t)min((uint64_t)d.cs, d.n - first);
+  bool even = false;
+#pragma unroll
+  for (int k = 0; k < 4; k++)
+    even |= bits == nsym * (d.len_lo >> (8 * k) & 0xFFu) || bits == nsym * (d.len_hi >> (8 * k) & 0xFFu);
+  if (even || bits < 128 * kSampleVecs) return false;
+  const uint32_t v = (i * 0x9E3779B1u >> 16) % (bits / 128 - kSampleVecs + 1);
+  if ((goff & 15u) != 0 || goff > d.payload_bytes || d.payload_bytes - goff < 16 * (v + kSampleVecs)) return false;
+  const uint4* p = reinterpret_cast<const uint4*>(in + payload_start(n_chunks) + goff) + v;
+#pragma unroll
+  for (uint32_t k = 0; k < kSampleVecs; k++) {
+    const uint4 q = ldg_nc_v4(p + k);
+    words[4 * k] = bswap32(q.x);
+    words[4 * k + 1] = bswap32(q.y);
+    words[4 * k + 2] = bswap32(q.z);
+    words[4 * k + 3] = bswap32(q.w);
+  }
+  const uint32_t end = warm_bits(d.len_lo, d.len_hi);
+  uint32_t at[3] = {0, 1, 2}, e[4];  // side by side: a walk is a chain of latencies
+  while (min(at[0], min(at[1], at[2])) < end) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      four_ends(words, at[k], d.len_lo, d.len_hi, e);
+      const uint32_t to = e[0] >= end ? e[0] : e[1] >= end ? e[1] : e[2] >= end ? e[2] : e[3];
+      at[k] = at[k] < end ? to : at[k];
+    }
+  }
+  return at[0] != at[1] || at[0] != at[2];
+}
+static_assert((2 * kWarm + kMaxCode) / 32 + 2 < 4 * kSampleVecs, "readers stay within the sample");
 
 // Decodes a span of a validated container: chunks c0 .. c0 + shape.chunks - 1
 // of group g.  One warp; k and seg are the lane's chunk in the span and its
@@ -181,40 +279,50 @@ __device__ __forceinline__ void decode_span(const DecHeader& h, const SpanShape&
   const uint32_t S0 = __shfl_sync(0xffffffffu, E - B, 0);  // the span's first bit
   const uint32_t E0 = __reduce_max_sync(0xffffffffu, mine ? E : 0u);
   const uint32_t v0 = S0 >> 7, nv = (E0 + 127) / 128 - v0;
-  {
+  auto load_bits = [&]() {
     const uint4* gp = reinterpret_cast<const uint4*>(in + h.P + goff) + v0;
     for (uint32_t v = lane; v < nv; v += 32) {
       if (!QLC_GUARD(v < kSpanVecs && h.P + goff + 16 * (uint64_t)(v0 + v + 1) <= h.in_bytes, status)) continue;
       const uint4 q = ldg_nc_v4(gp + v);
       reinterpret_cast<uint4*>(sm.bits)[v] = make_uint4(bswap32(q.x), bswap32(q.y), bswap32(q.z), bswap32(q.w));
     }
-  }
+  };
+  load_bits();
   __syncwarp();
   const uint32_t cb = (mine ? E - B : S0) - 128u * v0;  // the chunk's first bit within sm.bits
   // Pieces of an odd number of words: lanes that have come equally far read 32
   // different banks (a stride of 27.4 words, for one, has four of them on one).
   const uint32_t B_max = __reduce_max_sync(0xffffffffu, B);
   const uint32_t piece = 32u * ((B_max + 32 * shape.lanes - 1) / (32 * shape.lanes) | 1u);
-  const uint32_t beg = cb + min(B, piece * seg), end = cb + min(B, piece * (seg + 1));
+  const Piece pc = {cb, cb + B, cb + min(B, piece * seg), cb + min(B, piece * (seg + 1)), seg};
+  const uint32_t beg = pc.beg, end = pc.end;
   const uint32_t len_lo = h.len_lo, len_hi = h.len_hi;
   uint32_t p[4];
   uint32_t entry = cb;
   if (mine && seg > 0) {
-    if (beg > cb + warm) entry = beg - warm;
-    while (entry < beg) {
-      four_ends(sm.bits, entry, len_lo, len_hi, p);
-      entry = p[0] >= beg ? p[0] : p[1] >= beg ? p[1] : p[2] >= beg ? p[2] : p[3];
+    const uint32_t len = code_len(SpanBits(sm.bits, cb).x, len_lo, len_hi);
+    if (B == nsym * len) {  // codewords of one length, as in a chunk of one symbol
+      entry = cb + (beg - cb + len - 1) / len * len;
+    } else {
+      if (beg > cb + warm) entry = beg - warm;
+      entry = walk_to(sm.bits, entry, beg, len_lo, len_hi);
     }
   }
   uint32_t exit = cb, count = 0;
-  bool again = mine;
-  while (true) {
+  bool again = mine, run = false;  // run: the piece is count times the symbol of run_word, and nothing is staged
+  uint32_t run_word = 0;
+  int round = 0;
+  for (; round <= kRounds; round++) {
     if (again) {
       uint32_t n4 = 0, at = entry, last = entry;
-      while (at < end) {
+      while (at < end && n4 < kStageWords) {
         last = at;
-        const uint32_t w = four_symbols(sm.bits, at, T, len_lo, len_hi);
-        if (n4 < kStageWords) sm.col[n4][lane] = w;
+        sm.col[n4][lane] = four_symbols(sm.bits, at, T, len_lo, len_hi);
+        n4++;
+      }
+      while (at < end) {  // more than the column holds: decoded again at the end
+        last = at;
+        four_symbols(sm.bits, at, T, len_lo, len_hi);
         n4++;
       }
       exit = at;
@@ -224,12 +332,23 @@ __device__ __forceinline__ void decode_span(const DecHeader& h, const SpanShape&
         exit = p[0] >= end ? p[0] : p[1] >= end ? p[1] : p[2] >= end ? p[2] : p[3];
         count -= (p[0] >= end) + (p[1] >= end) + (p[2] >= end);
       }
+      run = false;
     }
     __syncwarp();
     const uint32_t before = __shfl_up_sync(0xffffffffu, exit, 1);
     again = mine && seg > 0 && before != entry;
     if (!__any_sync(0xffffffffu, again)) break;
     if (again) entry = before;
+    if (round == 0) continue;  // nearly always all it takes
+    const Run r = follow_run(sm.bits, T, pc, mine, entry, len_lo, len_hi, lane);
+    if (r.len) {  // needs no decoding
+      entry = r.entry;
+      count = entry < end ? (end - entry + r.len - 1) / r.len : 0u;
+      exit = entry + count * r.len;
+      again = false;
+      run = true;
+      run_word = r.sym * 0x01010101u;
+    }
   }
   // positions of the lanes' symbols within the span
   uint32_t off = count;
@@ -242,28 +361,12 @@ __device__ __forceinline__ void decode_span(const DecHeader& h, const SpanShape&
   off -= count;
   const uint32_t chunk_off = __shfl_sync(0xffffffffu, off, lane - (int)seg);
   const bool bad = mine && seg == shape.lanes - 1 && (exit != cb + B || upto - chunk_off != nsym);
-  if (__any_sync(0xffffffffu, bad)) {
+  if (round > kRounds || __any_sync(0xffffffffu, bad)) {
     if (lane == 0) set_status(status, QLC_ERR_CORRUPT);
     return;
   }
   const uint64_t base = (g * kGroupChunks + c0) * h.cs;  // the span's first symbol
   const uint32_t total = __shfl_sync(0xffffffffu, upto, 31);
-  if (__any_sync(0xffffffffu, count > 4 * kStageWords)) {
-    // a piece with more symbols than its column holds (a run of short codes
-    // in a chunk of long ones): symbol by symbol, straight to the output
-    if (mine) {
-      uint32_t at = entry;
-      for (uint32_t i = 0; i < count; i++) {
-        const SpanBits w(sm.bits, at);
-        const uint32_t la = code_len(w.x, len_lo, len_hi), ia = __funnelshift_l(w.x, 0u, la);
-        const uint32_t sym = QLC_GUARD(ia < 2048u, nullptr) ? T[ia] : 0u;
-        at += la;
-        if (QLC_GUARD(base + off + i < h.out_cap, status)) put1<kOut>(out, scales, base + off + i, sym);
-      }
-    }
-    __syncwarp();
-    return;
-  }
   // The symbols, shifted to their place.  A lane's first and last words may
   // be shared with its neighbours: they start from zero and are OR-ed.
   uint32_t* ow = sm.bits;
@@ -273,27 +376,34 @@ __device__ __forceinline__ void decode_span(const DecHeader& h, const SpanShape&
   __syncwarp();  // every lane is done with the bits
   if (nout && fits) ow[slot(w0)] = ow[slot(w0 + nout - 1)] = 0u;
   __syncwarp();
-  if (nout && fits) {
-    const uint32_t sh = (off & 3u) * 8u, nin = (count + 3) >> 2;
-    uint32_t prev = sm.col[0][lane];
-    uint32_t tail = prev;  // the last staged word
+  const uint32_t nin = (count + 3) >> 2;
+  auto place = [&](auto word) {  // word(i): the lane's word i
+    const uint32_t sh = (off & 3u) * 8u;
+    uint32_t prev = word(0u);
+    const uint32_t head = prev << sh;
     uint32_t t = 1;
     for (; t + 1 < nout; t++) {
-      const uint32_t cur = sm.col[t][lane];
+      const uint32_t cur = word(t);
       ow[slot(w0 + t)] = __funnelshift_l(prev, cur, sh);
       prev = cur;
     }
     // prev is word t - 1; the last output word holds the rest of it and, when
     // there is one, of word t
-    tail = t < nin ? sm.col[t][lane] : 0u;
+    const uint32_t tail = t < nin ? word(t) : 0u;
     const uint32_t keep = 0xFFFFFFFFu >> ((32u - 8u * (off + count)) & 31u);  // the bytes of the last output word
-    const uint32_t head = sm.col[0][lane] << sh;
     if (nout == 1) {
       atomicOr(&ow[slot(w0)], head & keep);
     } else {
       atomicOr(&ow[slot(w0)], head);
       atomicOr(&ow[slot(w0 + nout - 1)], __funnelshift_l(prev, tail, sh) & keep);
     }
+  };
+  const uint32_t held = run ? 0u : kStageWords;  // words that are staged
+  const bool unstaged = __any_sync(0xffffffffu, nin > held);
+  if (unstaged) {
+    if (nout && fits) place([&](uint32_t i) { return i < held ? sm.col[i][lane] : run_word; });
+  } else if (nout && fits) {
+    place([&](uint32_t i) { return sm.col[i][lane]; });
   }
   __syncwarp();
   if (kOut == kOutCodes && total == kSpanSyms && QLC_GUARD(base + kSpanSyms <= h.out_cap, status)) {
@@ -316,6 +426,22 @@ __device__ __forceinline__ void decode_span(const DecHeader& h, const SpanShape&
     }
   }
   __syncwarp();
+  // A piece with more symbols than its column holds (short codewords in a chunk
+  // of long ones): the rest of them, byte by byte over what was written there.
+  if (unstaged) {
+    const bool rest = !run && count > 4 * kStageWords;
+    if (!__any_sync(0xffffffffu, rest)) return;
+    load_bits();
+    __syncwarp();
+    uint32_t at = entry;
+    for (uint32_t i = 0; rest && i < count; i += 4) {
+      const uint32_t w = four_symbols(sm.bits, at, T, len_lo, len_hi);
+      if (i < 4 * kStageWords) continue;
+      for (uint32_t b = 0; b < 4 && i + b < count; b++)
+        if (QLC_GUARD(base + off + i + b < h.out_cap, status)) put1<kOut>(out, scales, base + off + i + b, w >> (8 * b) & 0xFFu);
+    }
+    __syncwarp();
+  }
 }
 
 }  // namespace qlc

@@ -3,12 +3,14 @@
 #define QLC_FILE_ID 3
 #include "hist_cols.cuh"
 #include "lut.cuh"
+#include "split_rule.cuh"
 #include "../../include/qlc_testing.h"
 
 #include <cuda.h>
 
 #include <algorithm>
 #include <atomic>
+#include <cstring>
 #include <functional>
 #include <mutex>
 
@@ -355,4 +357,23 @@ extern "C" int qlc_test_once_per_context(const int* dev, const uint64_t* id, con
     done += acted;
   }
   return done;
+}
+
+static qlc::SplitData split_data_of(const void* h_hdr) {
+  const uint8_t* p = static_cast<const uint8_t*>(h_hdr);
+  qlc::SplitData d = {};
+  memcpy(&d.cs, p + 16, 4);
+  memcpy(&d.n, p + 8, 8);
+  memcpy(&d.payload_bytes, p + 48, 8);
+  memcpy(&d.len_lo, p + 40, 4);
+  memcpy(&d.len_hi, p + 44, 4);
+  d.len_lo += 0x03030303u;
+  d.len_hi += 0x03030303u;
+  return d;
+}
+extern "C" uint64_t qlc_test_split_most(const void* h_hdr, int values, uint32_t slow) {
+  return qlc::split_most(split_data_of(h_hdr), values != 0, slow);
+}
+extern "C" int qlc_test_split_samples(const void* h_hdr, int values, uint64_t total) {
+  return qlc::split_samples(split_data_of(h_hdr), values != 0, total);
 }
