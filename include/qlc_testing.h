@@ -46,13 +46,22 @@ int qlc_test_once_per_context(const int *dev, const uint64_t *id, const uint64_t
 void qlc_test_encode_smem(uint32_t *addr, uint32_t *size, uint32_t *requested);
 void qlc_test_quantize_smem(int warps, uint32_t *addr, uint32_t *size, uint32_t *requested);
 
-/* The rule by which containers are decoded split (into codes, or values != 0),
- * for a host copy of a container's first 64 bytes: the most symbols of one launch
- * for which it is, when `slow` of 32 samples are places where readers are slow to
- * find the codeword boundaries; and whether samples are taken when `total`
- * symbols are decoded in the launch (without them slow counts as 0).  Host only. */
-uint64_t qlc_test_split_most(const void *h_hdr, int values, uint32_t slow);
-int qlc_test_split_samples(const void *h_hdr, int values, uint64_t total);
+/* The rule by which containers are decoded split, for a host copy of a
+ * container's first 64 bytes, decoded to codes (into 0), to values (1) or as a
+ * shard of a batch (2): the most symbols of one launch for which it is, when `slow`
+ * of 32 samples are places where readers are slow to find the codeword
+ * boundaries; and whether samples are taken when `total` symbols are decoded in
+ * the launch (without them slow counts as 0).  Host only. */
+uint64_t qlc_test_split_most(const void *h_hdr, int into, uint32_t slow);
+int qlc_test_split_samples(const void *h_hdr, int into, uint64_t total);
+
+/* Counter words that qlc_decode_batch leaves at the start of its workspace: how
+ * the batch was decoded (0: a warp per group, from a counter; 1: split; 2: a warp
+ * per group, dealt out evenly), its symbols, and its slow samples (both 0 unless
+ * split). */
+#define QLC_TEST_WS_WAY 1
+#define QLC_TEST_WS_SYMBOLS 2
+#define QLC_TEST_WS_SLOW 3
 
 #ifdef __cplusplus
 }

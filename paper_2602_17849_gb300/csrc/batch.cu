@@ -7,6 +7,7 @@
 // counter, so shards of very different sizes share the GPU evenly and no host
 // round trip is needed.  The histogram kernel scans the sizes itself.
 #define QLC_FILE_ID 4
+#include "decode_span.cuh"
 #include "hist_cols.cuh"
 
 namespace qlc {
@@ -52,15 +53,12 @@ __device__ __forceinline__ unsigned long long cta_scan(unsigned long long v, uns
 }
 
 // A shard's work: its groups (a shard that cannot be run has none and sets a
-// status), and for decoding its symbols and the spans per group (0: the items
-// are the groups in any case).
+// status), and for decoding its symbols.
 struct ShardWork {
   uint64_t groups, symbols;
-  uint32_t per_group;
-  uint64_t limit;  // symbols of a batch up to which its chunks are decoded split (see split_pays)
 };
 __device__ ShardWork shard_work(int kind, const qlc_desc& d, uint32_t cs, uint32_t* status) {
-  ShardWork w = {0, 0, 0, 0};
+  ShardWork w = {0, 0};
   if (kind == kPlanEncode) {
     const uint64_t n = d.in_bytes;
     const uint64_t n_chunks = (n + cs - 1) / cs;
@@ -92,52 +90,97 @@ __device__ ShardWork shard_work(int kind, const qlc_desc& d, uint32_t cs, uint32
   }
   w.groups = groups ? groups : 1;  // an empty container still gets its header checked
   w.symbols = min((uint64_t)h0.z | (uint64_t)h0.w << 32, (uint64_t)d.out_cap);
-  if (groups && chunk_symbols_ok(h1.x)) {  // the decoder refuses another chunk size
-    w.per_group = SpanShape(h1.x).per_group;
-    const uint64_t c = h1.x;
-    if ((h0.y >> 16 & 0xFFu) == 2)  // codes of one parity
-      w.limit = c < 1024 ? 0 : (c << 13) + (c << 12) - (3u << 20);
-    else
-      w.limit = c < 512 ? 0 : c << 14;
-  }
   return w;
+}
+
+// What the split rule looks at of a shard that has groups.
+__device__ __forceinline__ bool shard_data(const qlc_desc& d, SplitData* sd, uint64_t* n_chunks) {
+  return split_data(static_cast<const uint8_t*>(d.in), d.in_bytes, sd, n_chunks) && *n_chunks > 0;
+}
+
+// Of kSamples samples of the batch's shards that are looked at (split_samples):
+// those that are slow.  Called by all threads; at most kSampleThreads samples, as
+// many of every shard.
+constexpr int kSampleThreads = 256;
+__device__ uint32_t slow_samples(const qlc_desc* descs, int n_shards, const unsigned long long* item_base, uint64_t total,
+                                 int tid) {
+  __shared__ uint32_t words[kSampleThreads * kSampleWords];
+  const int per = min(max(kSampleThreads / n_shards, 1), (int)kSamples);  // samples of a shard
+  bool asked = false, slow = false;
+  if (tid < kSampleThreads) {
+    const int s = n_shards <= kSampleThreads ? tid / per : (int)((int64_t)tid * n_shards / kSampleThreads);
+    SplitData sd;
+    uint64_t n_chunks;
+    if (s < n_shards && item_base[s] != 0 && shard_data(descs[s], &sd, &n_chunks) && split_samples(sd, kSplitBatch, total)) {
+      asked = true;
+      const uint32_t i = per > 1 ? tid % per * kSamples / per : tid % kSamples;
+      slow = sample_is_slow(static_cast<const uint8_t*>(descs[s].in), sd, n_chunks, i, words + tid * kSampleWords);
+    }
+  }
+  const uint32_t tries = __syncthreads_count(asked), found = __syncthreads_count(slow);
+  return tries ? (found * kSamples + tries - 1) / tries : 0;
 }
 
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w, uint32_t* status) {
   static_assert(kPlanThreads == kHcThreads, "cta_scan");
   __shared__ unsigned long long s_incl[kPlanThreads], s_warp[kPlanThreads / 32];
+  __shared__ uint32_t s_chunk[2];
   const int tid = threadIdx.x;
   dependents_may_start();
-  // every thread keeps its shards' groups and spans per group in item_base
-  // until the number of symbols has settled which of them are the items
-  unsigned long long symbols = 0, limits = 0;
+  // every thread keeps its shards' groups, and the items they make in a split
+  // batch, in item_base until the number of symbols has settled which it is
+  unsigned long long symbols = 0;
   for (int s = tid; s < n_shards; s += kPlanThreads) {
     const ShardWork sw = shard_work(kind, descs[s], cs, status);
     symbols += sw.symbols;
-    limits += sw.symbols * sw.limit;
-    w.item_base[s] = sw.groups | (unsigned long long)sw.per_group << 40;
+    w.item_base[s] = sw.groups;
   }
   bool split = false;
+  uint32_t slow = 0;
   if (kind == kPlanDecode) {
     symbols = cta_scan(symbols, s_incl, s_warp, tid);
-    // split where that pays for the average symbol: a shard that it does not pay
-    // for is decoded a lane per chunk there, but badly dealt out (135 shards, 18 Mi
-    // symbols in chunks of 1024: 94 us, 37 dealt out evenly; 300 shards, 49 Mi in
-    // chunks of 4096 under Table 2: 368 and 84)
     split = symbols <= kSplitMax;
-    if (split) split = symbols * symbols <= cta_scan(limits, s_incl, s_warp, tid);
+    if (split) {
+      // Split where that pays for every shard: one that it does not pay for is
+      // decoded a lane per chunk, which takes its chunk's chain, and that is what the
+      // whole batch takes when it is dealt out evenly.  Only shards of chunks less
+      // than half as long as the longest hold nothing up.
+      slow = slow_samples(descs, n_shards, w.item_base, symbols, tid);
+      uint32_t longest = 0, held = 0;  // chunks: of all shards, and of those that are not split
+      for (int s = tid; s < n_shards; s += kPlanThreads) {
+        SplitData sd;
+        uint64_t n_chunks;
+        const unsigned long long groups = w.item_base[s];
+        if (groups == 0 || !shard_data(descs[s], &sd, &n_chunks)) continue;  // (nothing or a refusal to decode)
+        longest = max(longest, sd.cs);
+        const bool pays = symbols <= split_most(sd, kSplitBatch, split_samples(sd, kSplitBatch, symbols) ? slow : 0);
+        if (!pays) held = max(held, sd.cs);
+        // items of kSpanWarps spans, or of as many groups
+        const uint64_t parts = pays ? groups * SpanShape(sd.cs).per_group : groups;
+        w.item_base[s] = groups | (parts + kSpanWarps - 1) / kSpanWarps << 32;
+      }
+      longest = __reduce_max_sync(0xffffffffu, longest);
+      held = __reduce_max_sync(0xffffffffu, held);
+      if (tid < 2) s_chunk[tid] = 0;
+      __syncthreads();
+      if (tid % 32 == 0) {
+        atomicMax(&s_chunk[0], longest);
+        atomicMax(&s_chunk[1], held);
+      }
+      __syncthreads();
+      split = 2 * s_chunk[1] <= s_chunk[0];
+    }
   }
-  if (tid < 16) w.ticket[tid] = tid == kTicketSymbols && split ? (uint32_t)symbols : 0u;  // the 64 bytes of counters
+  // the 64 bytes of counters
+  if (tid < 16) w.ticket[tid] = !split ? 0u : tid == kTicketSymbols ? (uint32_t)symbols : tid == kTicketSlow ? slow : 0u;
   unsigned long long total = 0;
   for (int base = 0; base < n_shards; base += kPlanThreads) {
     const int s = base + tid;
     unsigned long long cnt = 0;
     if (s < n_shards) {
-      const unsigned long long v = w.item_base[s];
-      const uint32_t per_group = (uint32_t)(v >> 40);
-      cnt = v & ((1ull << 40) - 1);
-      if (split && per_group) cnt = (cnt * per_group + kSpanWarps - 1) / kSpanWarps;
+      const unsigned long long v = w.item_base[s], groups = v & 0xFFFFFFFFu;
+      cnt = split && v >> 32 ? v >> 32 : groups;
     }
     const unsigned long long part = cta_scan(cnt, s_incl, s_warp, tid);
     if (s < n_shards) w.item_base[s] = total + s_incl[tid] - cnt;

@@ -427,7 +427,8 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
   }
   if (err) return;
   const SplitData sd = {h.cs, h.len_lo, h.len_hi, h.n, h.payload_bytes};
-  const bool ask = split_samples(sd, kOut != kOutCodes, h.n);
+  constexpr SplitInto kInto = kOut == kOutCodes ? kSplitCodes : kSplitValues;
+  const bool ask = split_samples(sd, kInto, h.n);
   if (ask && warp == 0) {  // every CTA looks at the same samples
     static_assert(kSamples == 32 && 4 * 32 * kSampleWords <= sizeof(SpanWarp), "a sample per lane");
     const bool slow = sample_is_slow(in, sd, h.n_chunks, lane, reinterpret_cast<uint32_t*>(one_sm) + lane * kSampleWords);
@@ -437,7 +438,7 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
   build_table(hdr, T, tid, blockDim.x);
   __syncthreads();
   const uint32_t first = (uint32_t)warp * gridDim.x + blockIdx.x;
-  if (h.n <= split_most(sd, kOut != kOutCodes, ask ? s_slow : 0)) {
+  if (h.n <= split_most(sd, kInto, ask ? s_slow : 0)) {
     const uint32_t stride = warps * gridDim.x;
     const SpanShape shape(h.cs);
     const uint32_t warm = warm_bits(h.len_lo, h.len_hi);
@@ -619,6 +620,7 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
   dependency_wait();
   const uint32_t way = ticket[kTicketWay];
   const uint64_t batch_symbols = ticket[kTicketSymbols];
+  const uint32_t batch_slow = ticket[kTicketSlow];
   if (way == kWayGroups) return;
   const int lane = threadIdx.x % 32;
   const int wid = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0);  // so known to be the same in all lanes
@@ -676,7 +678,7 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
     if (!err) {
       const uint64_t s = (uint64_t)q * kSpanWarps + warp;
       const SplitData sd = {h.cs, h.len_lo, h.len_hi, h.n, h.payload_bytes};
-      if (batch_symbols <= split_most(sd, false, 0)) {
+      if (batch_symbols <= split_most(sd, kSplitBatch, split_samples(sd, kSplitBatch, batch_symbols) ? batch_slow : 0)) {
         const SpanShape shape(h.cs);
         const uint32_t k = (uint32_t)lane / shape.lanes, seg = (uint32_t)lane - k * shape.lanes;
         const uint64_t g = s / shape.per_group;
@@ -684,7 +686,7 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
         if (g < h.n_groups)
           decode_span<kOutCodes>(h, shape, in, dd.out, nullptr, g, r * shape.chunks, k, seg, sm.w[warp].span, sm.T,
                                  warm_bits(h.len_lo, h.len_hi), status, lane);
-      } else if (s < h.n_groups) {  // a shard has at least as many spans as groups
+      } else if (s < h.n_groups) {
         LaneDec d;
         if (lane_init(sm.w[warp].lanes, d, lane))
           decode_group<kOutCodes, kRingStatic>(h, in, dd.out, nullptr, s, sm.w[warp].lanes, sm.T, d, status, lane,

@@ -31,7 +31,7 @@ __device__ __forceinline__ void load_header(const uint8_t* in, uint64_t in_bytes
 // Parses and validates the header (all lanes, redundantly) from its copy in
 // shared memory; same checks, in the same order of kinds, as the container
 // rules: 0 = ok, else a status.
-__device__ uint32_t parse_header(const uint8_t* in, uint64_t in_bytes, uint64_t out_cap,
+static __device__ uint32_t parse_header(const uint8_t* in, uint64_t in_bytes, uint64_t out_cap,
                                  DecHeader* h, uint32_t* s_seen, int lane) {
   if (in_bytes < kIndexOff) return QLC_ERR_CORRUPT;
   const uint32_t w0 = *reinterpret_cast<const uint32_t*>(in);

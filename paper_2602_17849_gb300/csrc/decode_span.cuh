@@ -168,7 +168,7 @@ struct Run {
 // Called by all lanes, with the boundary x that the piece before leaves to this
 // one.  The boundaries of a run are those of its first piece.  A function of its
 // own, so that its registers and code are not the decoder's (inlined it cost 3 %).
-__device__ __noinline__ Run follow_run(const uint32_t* bits, const uint8_t* T, Piece pc, bool mine, uint32_t x,
+static __device__ __noinline__ Run follow_run(const uint32_t* bits, const uint8_t* T, Piece pc, bool mine, uint32_t x,
                                        uint32_t len_lo, uint32_t len_hi, int lane) {
   const uint32_t period = mine ? run_period(bits, pc) : 0u;
   if (!__any_sync(0xffffffffu, period != 0)) return {0u, 0u, 0u};

@@ -371,9 +371,9 @@ static qlc::SplitData split_data_of(const void* h_hdr) {
   d.len_hi += 0x03030303u;
   return d;
 }
-extern "C" uint64_t qlc_test_split_most(const void* h_hdr, int values, uint32_t slow) {
-  return qlc::split_most(split_data_of(h_hdr), values != 0, slow);
+extern "C" uint64_t qlc_test_split_most(const void* h_hdr, int into, uint32_t slow) {
+  return qlc::split_most(split_data_of(h_hdr), (qlc::SplitInto)into, slow);
 }
-extern "C" int qlc_test_split_samples(const void* h_hdr, int values, uint64_t total) {
-  return qlc::split_samples(split_data_of(h_hdr), values != 0, total);
+extern "C" int qlc_test_split_samples(const void* h_hdr, int into, uint64_t total) {
+  return qlc::split_samples(split_data_of(h_hdr), (qlc::SplitInto)into, total);
 }

@@ -258,7 +258,7 @@ struct NvtxRange {
 // --------------------------------------------- the split decoder's geometry
 constexpr int kSpanWarps = 4;                    // warps per CTA; they share the code table
 constexpr uint32_t kPiece = 128;                 // symbols per lane, about
-constexpr uint64_t kSplitMax = 64ull << 20;      // symbols of a batch decoded split, at most: see split_pays
+constexpr uint64_t kSplitMax = 64ull << 20;      // symbols of a batch decoded split, at most: see split_most
 
 // Geometry of a container's spans: a chunk takes `lanes` lanes, a warp
 // `chunks` chunks (of one group), a group `per_group` spans.
@@ -278,6 +278,7 @@ struct SpanShape {
 // Counter word that says how a batch is decoded (decode.cu).
 constexpr int kTicketWay = 1;
 constexpr int kTicketSymbols = 2;  // the batch's symbols, in kWaySplit
+constexpr int kTicketSlow = 3;     // of kSamples samples of its unsure shards (split_rule.cuh), in kWaySplit
 enum DecodeWay : uint32_t { kWayGroups = 0, kWaySplit = 1, kWayEven = 2 };
 constexpr uint32_t kFewWarpsPerSm = 20;  // kWayEven: a warp per group
 struct BatchWs {
