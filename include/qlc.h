@@ -229,7 +229,8 @@ typedef struct qlc_desc {
   uint64_t *out_bytes; /* encode: container size; decode: n (device pointer or NULL) */
 } qlc_desc;            /* 48 bytes */
 
-/* Launch shape knobs (an autotuner picks them); 0 = library default. */
+/* Launch shape knobs (an autotuner picks them); 0 = library default.  They hold
+ * for every batch and change no result. */
 typedef struct qlc_launch {
   uint16_t encode_ctas_per_sm; /* resident encode CTAs (512 threads) per SM, 1 or 2 (larger: 2) */
   uint16_t decode_ctas_per_sm; /* resident decode warps per SM, 1..20 (larger: 20) */

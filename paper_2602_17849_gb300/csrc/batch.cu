@@ -138,9 +138,9 @@ plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs 
   }
   bool split = false;
   uint32_t slow = 0;
-  if (kind == kPlanDecode) {
+  if (kind != kPlanEncode) {
     symbols = cta_scan(symbols, s_incl, s_warp, tid);
-    split = symbols <= kSplitMax;
+    split = kind == kPlanDecode && symbols <= kSplitMax;
     if (split) {
       // Split where that pays for every shard: one that it does not pay for is
       // decoded a lane per chunk, which takes its chunk's chain, and that is what the
@@ -192,8 +192,7 @@ plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs 
   }
   if (tid == 0) {
     w.item_base[n_shards] = total;
-    if (kind == kPlanDecode)
-      w.ticket[kTicketWay] = split ? kWaySplit : total <= (unsigned long long)kFewWarpsPerSm * cs ? kWayEven : kWayGroups;
+    if (kind != kPlanEncode) w.ticket[kTicketWay] = split ? kWaySplit : total <= cs ? kWayEven : kWayGroups;
   }
   if (kind == kPlanEncode)
     for (unsigned long long i = tid; i < total; i += kPlanThreads) w.gstat[i] = 0;

@@ -592,7 +592,11 @@ __device__ __forceinline__ void team_sync(int team) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(32 * kSpanWarps) : "memory");
 }
 
-// Few groups: one CTA per SM, of kSpanCtasPerSm teams of kSpanWarps warps.
+// Few groups: one CTA per SM, of up to kFewWarps warps, in teams of kSpanWarps
+// where the batch is decoded split.
+constexpr int kFewTeams = 5;
+constexpr int kFewWarps = kSpanWarps * kFewTeams;
+static_assert(kFewWarps == kDecCtasPerSm, "both bounded by qlc_launch.decode_ctas_per_sm");
 struct FewOwn {
   LaneShared lanes;
   uint8_t T[2048];
@@ -600,22 +604,18 @@ struct FewOwn {
   uint32_t seen[16];
 };
 static_assert(sizeof(FewOwn) % kRingBytes == 0, "");
-struct FewShared {
-  union {
-    SpanShared span[kSpanCtasPerSm];            // a team's
-    FewOwn own[kSpanWarps * kSpanCtasPerSm];    // a warp's
-  };
-  uint8_t align[kRingBytes];
-};
-constexpr int kFewWarps = kSpanWarps * kSpanCtasPerSm;
-static_assert(kFewWarps == kFewWarpsPerSm, "plan_kernel compares the groups with these warps");
+// Shared memory: a SpanShared for every team, or a FewOwn for every warp, behind
+// what aligns it.
+constexpr size_t few_bytes(int warps) {
+  const size_t teams = (size_t)(warps / kSpanWarps) * sizeof(SpanShared), own = warps * sizeof(FewOwn);
+  return (teams > own ? teams : own) + kRingBytes;
+}
 __global__ void __launch_bounds__(32 * kFewWarps, 1)
 decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsigned long long* item_base,
                   unsigned int* ticket, uint32_t* __restrict__ status) {
   extern __shared__ __align__(16) uint8_t few_sm[];
   __shared__ void* volatile s_out[kFewWarps];  // the warps' current outputs
-  __shared__ volatile unsigned long long s_item[kSpanCtasPerSm];
-  FewShared& all = *reinterpret_cast<FewShared*>(few_sm);
+  __shared__ volatile unsigned long long s_item[kFewTeams];
   dependents_may_start();
   dependency_wait();
   const uint32_t way = ticket[kTicketWay];
@@ -655,7 +655,9 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
   // Split: items are kSpanWarps spans of one shard, which a team decodes with a
   // table that its warps share.
   const int team = wid / kSpanWarps, warp = wid % kSpanWarps, tid = 32 * warp + lane;
-  SpanShared& sm = all.span[team];
+  const uint32_t teams = blockDim.x / (32 * kSpanWarps);
+  if (team >= (int)teams) return;  // warps that make no team
+  SpanShared& sm = reinterpret_cast<SpanShared*>(few_sm)[team];
   int cur = -1;
   uint32_t err = 0;
   for (unsigned long long t = (unsigned long long)team * gridDim.x + blockIdx.x; t < total;) {
@@ -695,7 +697,7 @@ decode_few_kernel(const qlc_desc* __restrict__ descs, int n_shards, const unsign
           set_status(status, QLC_ERR_CUDA);
       }
     }
-    if (tid == 0) s_item[team] = kSpanCtasPerSm * gridDim.x + (unsigned long long)atomicAdd(ticket, 1u);
+    if (tid == 0) s_item[team] = teams * gridDim.x + (unsigned long long)atomicAdd(ticket, 1u);
     team_sync(team);  // ... and every warp is done with the header and the table
     t = s_item[team];
     team_sync(team);
@@ -746,6 +748,12 @@ extern "C" qlc_status qlc_decode_dequantize(const uint8_t* d_in, size_t in_bytes
   return launch_decode<QLC_DTYPE_BF16>(d_in, in_bytes, d_out, d_scales, out_cap, d_n_out, d_status, st);
 }
 
+// Resident decode warps per SM of a batch.
+static int decode_warps(const qlc_launch* launch) {
+  const int n = launch ? launch->decode_ctas_per_sm : 0;
+  return n > 0 && n < kDecCtasPerSm ? n : kDecCtasPerSm;
+}
+
 extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, void* d_ws, size_t ws_bytes,
                                        uint32_t* d_status, const qlc_launch* h_launch, qlc_stream_t stream) {
   NvtxRange nvtx_range("qlc_decode_batch");
@@ -754,17 +762,14 @@ extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, vo
   BatchWs w;
   if (!batch_ws_layout(d_ws, ws_bytes, n_shards, &w)) return QLC_ERR_CAPACITY;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  plan_kernel<<<1, kPlanThreads, 0, st>>>(kPlanDecode, d_descs, n_shards, (uint32_t)sm_count(), w, d_status);
-  if (cudaGetLastError() != cudaSuccess) return QLC_ERR_CUDA;
-  int per_sm = kDecCtasPerSm;
-  if (h_launch && h_launch->decode_ctas_per_sm > 0 && h_launch->decode_ctas_per_sm < kDecCtasPerSm)
-    per_sm = h_launch->decode_ctas_per_sm;
+  const int per_sm = decode_warps(h_launch), sms = sm_count();
   static OncePerContext done;
-  if (!smem_ok(decode_few_kernel, sizeof(FewShared), done)) return QLC_ERR_CUDA;
+  if (!smem_ok(decode_few_kernel, few_bytes(kFewWarps), done)) return QLC_ERR_CUDA;
+  plan_kernel<<<1, kPlanThreads, 0, st>>>(per_sm < kSpanWarps ? kPlanDecodeGroups : kPlanDecode, d_descs, n_shards,
+                                          (uint32_t)(per_sm * sms), w, d_status);
+  if (cudaGetLastError() != cudaSuccess) return QLC_ERR_CUDA;
   // which of the two has the work is decided on the device; the other returns at once
-  const int sms = sm_count();
-  launch_after(decode_few_kernel, sms, 32 * kFewWarps, sizeof(FewShared), st, d_descs, n_shards, w.item_base, w.ticket,
-               d_status);
+  launch_after(decode_few_kernel, sms, 32 * per_sm, few_bytes(per_sm), st, d_descs, n_shards, w.item_base, w.ticket, d_status);
   launch_after(decode_batch_kernel, sms * per_sm, 32, 0, st, d_descs, n_shards, w.item_base, w.ticket, d_status);
   return cudaGetLastError() == cudaSuccess ? QLC_OK : QLC_ERR_CUDA;
 }

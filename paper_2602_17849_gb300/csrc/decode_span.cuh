@@ -43,7 +43,6 @@
 
 namespace qlc {
 
-constexpr int kSpanCtasPerSm = 5;                     // resident: bounded by shared memory
 constexpr uint32_t kSpanSyms = 32 * kPiece;           // symbols per warp at most
 constexpr uint32_t kSpanVecs = (127 + kSpanSyms * kMaxCode + 127) / 128;  // 16-byte vectors that hold a span's bits
 constexpr uint32_t kSpanWords = 4 * kSpanVecs + 4;    // and words read past the end (never consumed)

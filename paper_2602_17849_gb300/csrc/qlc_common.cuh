@@ -280,7 +280,6 @@ constexpr int kTicketWay = 1;
 constexpr int kTicketSymbols = 2;  // the batch's symbols, in kWaySplit
 constexpr int kTicketSlow = 3;     // of kSamples samples of its unsure shards (split_rule.cuh), in kWaySplit
 enum DecodeWay : uint32_t { kWayGroups = 0, kWaySplit = 1, kWayEven = 2 };
-constexpr uint32_t kFewWarpsPerSm = 20;  // kWayEven: a warp per group
 struct BatchWs {
   unsigned int* ticket;                // [0] shared by encode / decode
   unsigned long long* item_base;
@@ -298,16 +297,17 @@ inline bool batch_ws_layout(void* ws, size_t bytes, int n_shards, BatchWs* w) {
   return true;
 }
 
-enum PlanKind { kPlanEncode = 1, kPlanDecode = 2 };
+// kPlanDecodeGroups: decoding by warps too few for the split way.
+enum PlanKind { kPlanEncode = 1, kPlanDecode = 2, kPlanDecodeGroups = 3 };
 constexpr int kPlanThreads = 1024;
 constexpr uint64_t kHistItem = 64 * 1024;  // symbols per histogram work item
 
 // One CTA: the number of work items of every shard (encode: groups of 32
 // chunks; decode: the container's groups, or in a batch that is decoded split
-// sets of kSpanWarps spans),
-// their exclusive prefix in item_base, and zeroed counters / look-back words.
-// Shards that cannot be processed get no items and set *status.  cs: the chunk
-// size (encode), or the number of SMs (decode).
+// sets of kSpanWarps spans or groups), their exclusive prefix in item_base, and
+// zeroed counters / look-back words.  Shards that cannot be processed get no items
+// and set *status.  cs: the chunk size (encode), or the warps of
+// decode_few_kernel (decode): up to as many groups are dealt out evenly.
 __global__ void plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w,
                             uint32_t* status);
 
