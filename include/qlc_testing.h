@@ -46,6 +46,11 @@ int qlc_test_once_per_context(const int *dev, const uint64_t *id, const uint64_t
 void qlc_test_encode_smem(uint32_t *addr, uint32_t *size, uint32_t *requested);
 void qlc_test_quantize_smem(int warps, uint32_t *addr, uint32_t *size, uint32_t *requested);
 
+/* What a batch is launched with for these knobs (NULL: the defaults): encode CTAs
+ * and decode warps per SM.  Host only. */
+int qlc_test_encode_ctas(const qlc_launch *h_launch);
+int qlc_test_decode_warps(const qlc_launch *h_launch);
+
 /* The rule by which containers are decoded split, for a host copy of a
  * container's first 64 bytes, decoded to codes (into 0), to values (1) or as a
  * shard of a batch (2): the most symbols of one launch for which it is, when `slow`

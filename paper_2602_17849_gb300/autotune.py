@@ -19,7 +19,7 @@ from . import qlc
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "autotune_cache.json")
 
 CHUNKS = (2048, 4096)
-ENC_CTAS = (2, 3)
+ENC_CTAS = (1, 2)
 DEC_CTAS = (12, 16, 20)
 
 

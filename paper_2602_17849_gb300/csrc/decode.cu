@@ -32,6 +32,7 @@
 #define QLC_FILE_ID 1
 #include "decode_common.cuh"
 #include "decode_span.cuh"
+#include "../../include/qlc_testing.h"
 
 namespace qlc {
 
@@ -753,6 +754,8 @@ static int decode_warps(const qlc_launch* launch) {
   const int n = launch ? launch->decode_ctas_per_sm : 0;
   return n > 0 && n < kDecCtasPerSm ? n : kDecCtasPerSm;
 }
+
+extern "C" int qlc_test_decode_warps(const qlc_launch* h_launch) { return decode_warps(h_launch); }
 
 extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, void* d_ws, size_t ws_bytes,
                                        uint32_t* d_status, const qlc_launch* h_launch, qlc_stream_t stream) {

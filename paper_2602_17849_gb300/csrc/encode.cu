@@ -1022,14 +1022,18 @@ size_t qlc_encode_workspace_size(size_t n, uint32_t chunk_symbols) {
   return (size_t)(16 + 8 * n_groups_of(n_chunks));
 }
 
+// Resident encode CTAs per SM.
+static int encode_ctas(const qlc_launch* launch) {
+  const int n = launch ? launch->encode_ctas_per_sm : 0;
+  return n > 0 && n < kEncCtasPerSm ? n : kEncCtasPerSm;
+}
+
 // Launches encode_kernel for up to `items` groups, after the previous kernel of
 // the same call (pdl) or by itself.
 static qlc_status launch_groups(const EncArgs& A, uint64_t items, const qlc_launch* launch, bool pdl, cudaStream_t st) {
   static OncePerContext done;
   if (!smem_ok(encode_kernel, kEncSharedBytes, done)) return QLC_ERR_CUDA;
-  int per_sm = kEncCtasPerSm;
-  if (launch && launch->encode_ctas_per_sm > 0 && launch->encode_ctas_per_sm < per_sm) per_sm = launch->encode_ctas_per_sm;
-  const uint64_t cap = (uint64_t)sm_count() * per_sm;
+  const uint64_t cap = (uint64_t)sm_count() * encode_ctas(launch);
   const int grid = (int)(items < 1 ? 1 : (items < cap ? items : cap));
   if (pdl)
     launch_after(encode_kernel, grid, kTeams * kTeamThreads, kEncSharedBytes, st, A);
@@ -1142,6 +1146,8 @@ qlc_status qlc_encode_tensor(const uint8_t* d_in, size_t n, const qlc_scheme* h_
   return launch_encode(d_in, n, d_hist, set, d_lut, chunk_symbols, d_out, out_cap, d_ws, ws_bytes, d_out_bytes, d_status,
                        st);
 }
+
+int qlc_test_encode_ctas(const qlc_launch* h_launch) { return encode_ctas(h_launch); }
 
 void qlc_test_encode_smem(uint32_t* addr, uint32_t* size, uint32_t* requested) {
   *addr = kTableAddr;
