@@ -114,13 +114,24 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def _traffic_for(kernel_file: str):
+CSRC = os.path.join(ROOT, "paper_2602_17849_gb300", "csrc")
+
+
+def source_digest(kernel_file: str, csrc: str = CSRC) -> str:
+    """Of a kernel's source file and of all headers beside it, in which much of
+    the kernels stands."""
+    h = hashlib.sha256()
+    for name in [kernel_file] + sorted(n for n in os.listdir(csrc) if n.endswith(".cuh")):
+        with open(os.path.join(csrc, name), "rb") as f:
+            h.update(name.encode() + b"\0" + f.read() + b"\0")
+    return h.hexdigest()[:16]
+
+
+def _traffic_for(kernel_file: str, path: str = os.path.join(ROOT, "profiles", "traffic.txt")):
     """DRAM bytes per launch from the committed ncu summary, if it was taken
     on the current source of the kernel (else None)."""
-    path = os.path.join(ROOT, "profiles", "traffic.txt")
-    src = os.path.join(ROOT, "paper_2602_17849_gb300", "csrc", kernel_file)
     try:
-        digest = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+        digest = source_digest(kernel_file)
         for line in open(path):
             f = line.split()
             if len(f) >= 4 and f[0] == kernel_file and f[1] == digest and f[2] == WORKLOAD:
