@@ -399,7 +399,6 @@ class Codec:
         self.n_out = words[1:2]
         self.status = words[2:3].view(torch.int32)[:1]
         self.ws = buf[_CODEC_WS:]
-        self._results = words  # out_bytes, n_out, status: read back together
 
     def new_container(self) -> torch.Tensor:
         return torch.empty(self.cap, dtype=torch.uint8, device=self.device)
