@@ -217,8 +217,9 @@ qlc_status qlc_decode(const uint8_t *d_in, size_t in_bytes, uint8_t *d_out,
  * Many tensors ("shards", e.g. the 18 layers x 64 devices = 1152 shards per
  * tensor type of Section 3) in one launch per step.  A batch is an array of
  * descriptors in device memory.  Work is split into items of one group of 32
- * chunks; persistent CTAs take items from a device-side counter, so shards of
- * very different sizes share the GPU evenly.  Per-shard errors go to
+ * chunks (decoding: or a few chunks), which are dealt out evenly over the SMs or
+ * taken from a device-side counter by persistent CTAs, so shards of very
+ * different sizes share the GPU evenly.  Per-shard errors go to
  * *d_status; other shards are unaffected. */
 typedef struct qlc_desc {
   const void *in;      /* encode / histogram: the shard's symbols; decode: its container */
@@ -245,7 +246,8 @@ size_t qlc_batch_workspace_size(int n_shards, uint64_t total_symbols, uint32_t c
 /* Histograms of the shards (Section 4).  shared = 0: d_hists holds
  * n_shards x 256 counts, one histogram per shard; shared = 1: one histogram
  * over all shards (an a-priori LUT per tensor type, Section 7).  Overwrites
- * d_hists.  Uses d_ws.  Async on stream. */
+ * d_hists.  d_ws and ws_bytes are checked as for the other batch calls and not
+ * used.  Async on stream. */
 qlc_status qlc_histogram_batch(const qlc_desc *d_descs, int n_shards, uint64_t *d_hists, int shared,
                                void *d_ws, size_t ws_bytes, qlc_stream_t stream);
 

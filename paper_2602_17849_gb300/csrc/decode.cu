@@ -508,10 +508,10 @@ struct SpanShared {
 
 // ---------------------------------------------------------------- batches
 //
-// Three ways, by the batch's size (plan_kernel decides, on the device): split
-// where that pays for its chunks and schemes; a lane per chunk with the first items dealt out
-// evenly while there are no more groups than warps; and, above, a lane per
-// chunk with all items from a counter.
+// Three ways (plan_kernel decides, on the device): split, where that pays for its
+// shards (split_rule.cuh); else a lane per chunk, with a group for every warp dealt
+// out evenly while there are no more groups than warps, and above with all groups
+// from a counter.
 
 // The shard an item belongs to changed: reads its header and builds its table.
 // Reports a bad one and returns its status.

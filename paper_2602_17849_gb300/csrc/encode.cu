@@ -16,10 +16,10 @@
 // Small tensors take lengths_kernel and pack_kernel instead.
 //
 // 256 Mi symbols, t4 data: 184 us (217 with three CTAs of 8 warps, 512 symbols a
-// step, a chunk at a time with blocks merged by the CTA).  16.3 instructions per
+// step, a chunk at a time with blocks merged by the CTA).  16.8 instructions per
 // symbol (22 before): 4 for a length, 12 for packing.  It is bound by the shared-
-// memory pipe (42.7 M wavefronts, 73 % busy: two lookups per symbol, and word
-// stores at 1.7 wavefronts) and the integer pipe (65 %), and loses about a fifth
+// memory pipe (34.7 M wavefronts, 72 % busy: two lookups per symbol, and word
+// stores at 1.7 wavefronts) and the integer pipe (71 %), and loses about a fifth
 // of its warps' time to the look-back and its barriers.  Measured and left out:
 // teams of 16 warps 201 us; the next group's pass 1 before this group's pass 2
 // 223 us (the re-reads then miss L2); pass 1 and pass 2 as two kernels 78 + 140

@@ -12,8 +12,9 @@
 // per warp (32 KB each) only 7 warps fit on an SM, and they could not keep the
 // pipe busy.  256 MiB of Student-t bytes, one CTA per SM: 7 warps with 7
 // tables 62-69 us, 28 warps with 7 tables 67 us, with 4 tables 48.5 us, 32
-// warps with 4 / 2 / 1 tables 48.5 / 46.4 / 44.9 us (5.98 TB/s, 89 % of a
-// device copy's rate); 16 and 8 warps with one table 50.7 and 77 us.
+// warps with 4 / 2 / 1 tables 48.5 / 46.4 / 44.9 us; 16 and 8 warps with one
+// table 50.7 and 77 us.  (Back to back; by itself, with a cold cache, the
+// kernel takes 47.7 us, 5.6 TB/s, 83 % of a device copy's rate.)
 #pragma once
 
 #include "qlc_common.cuh"

@@ -256,7 +256,7 @@ struct NvtxRange {
 };
 
 // --------------------------------------------- the split decoder's geometry
-constexpr int kSpanWarps = 4;                    // warps per CTA; they share the code table
+constexpr int kSpanWarps = 4;                    // warps of a team of the batch decoder; they share a code table
 constexpr uint32_t kPiece = 128;                 // symbols per lane, about
 constexpr uint64_t kSplitMax = 64ull << 20;      // symbols of a batch decoded split, at most: see split_most
 
