@@ -121,13 +121,14 @@ __device__ uint32_t slow_samples(const qlc_desc* descs, int n_shards, const unsi
   return tries ? (found * kSamples + tries - 1) / tries : 0;
 }
 
-__global__ void __launch_bounds__(kPlanThreads)
+__global__ void __launch_bounds__(kPlanThreads, 1)
 plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w, uint32_t* status) {
   static_assert(kPlanThreads == kHcThreads, "cta_scan");
   __shared__ unsigned long long s_incl[kPlanThreads], s_warp[kPlanThreads / 32];
   __shared__ uint32_t s_chunk[2];
   const int tid = threadIdx.x;
   dependents_may_start();
+  if (tid < 2) s_chunk[tid] = 0;  // published by the scan's barriers
   // every thread keeps its shards' groups, and the items they make in a split
   // batch, in item_base until the number of symbols has settled which it is
   unsigned long long symbols = 0;
@@ -146,24 +147,32 @@ plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs 
       // decoded a lane per chunk, which takes its chunk's chain, and that is what the
       // whole batch takes when it is dealt out evenly.  Only shards of chunks less
       // than half as long as the longest hold nothing up.
-      slow = slow_samples(descs, n_shards, w.item_base, symbols, tid);
       uint32_t longest = 0, held = 0;  // chunks: of all shards, and of those that are not split
-      for (int s = tid; s < n_shards; s += kPlanThreads) {
-        SplitData sd;
-        uint64_t n_chunks;
-        const unsigned long long groups = w.item_base[s];
-        if (groups == 0 || !shard_data(descs[s], &sd, &n_chunks)) continue;  // (nothing or a refusal to decode)
-        longest = max(longest, sd.cs);
-        const bool pays = symbols <= split_most(sd, kSplitBatch, split_samples(sd, kSplitBatch, symbols) ? slow : 0);
-        if (!pays) held = max(held, sd.cs);
-        // items of kSpanWarps spans, or of as many groups
-        const uint64_t parts = pays ? groups * SpanShape(sd.cs).per_group : groups;
-        w.item_base[s] = groups | (parts + kSpanWarps - 1) / kSpanWarps << 32;
+      bool asked = false;
+      auto settle = [&](bool look) {
+        for (int s = tid; s < n_shards; s += kPlanThreads) {
+          SplitData sd;
+          uint64_t n_chunks;
+          const unsigned long long groups = w.item_base[s] & 0xFFFFFFFFu;
+          if (groups == 0 || !shard_data(descs[s], &sd, &n_chunks)) continue;  // (nothing or a refusal to decode)
+          const bool ask = split_samples(sd, kSplitBatch, symbols);
+          asked = asked || ask;
+          longest = max(longest, sd.cs);
+          if (ask && look) continue;  // not yet known
+          const bool pays = symbols <= split_most(sd, kSplitBatch, ask ? slow : 0);
+          if (!pays) held = max(held, sd.cs);
+          // items of kSpanWarps spans, or of as many groups
+          const uint64_t parts = pays ? groups * SpanShape(sd.cs).per_group : groups;
+          w.item_base[s] = groups | (parts + kSpanWarps - 1) / kSpanWarps << 32;
+        }
+      };
+      settle(true);
+      if (__syncthreads_or(asked)) {
+        slow = slow_samples(descs, n_shards, w.item_base, symbols, tid);
+        settle(false);
       }
       longest = __reduce_max_sync(0xffffffffu, longest);
       held = __reduce_max_sync(0xffffffffu, held);
-      if (tid < 2) s_chunk[tid] = 0;
-      __syncthreads();
       if (tid % 32 == 0) {
         atomicMax(&s_chunk[0], longest);
         atomicMax(&s_chunk[1], held);
