@@ -68,7 +68,7 @@ struct DecShared {
   LaneShared lanes;
   uint8_t T[2048];                // code -> symbol
   __align__(16) uint8_t hdr[kIndexOff];  // the container's header and dec
-  __align__(8) uint32_t seen[64];
+  uint32_t seen[64];
 };
 
 // A lane's bit stream, positions group-relative.  The stream's words j and
@@ -416,8 +416,7 @@ decode_kernel(const uint8_t* __restrict__ in, uint64_t in_bytes, void* __restric
   extern __shared__ __align__(16) uint8_t one_sm[];
   __shared__ uint8_t T[2048];                       // code -> symbol
   __shared__ __align__(16) uint8_t hdr[kIndexOff];  // the container's header and dec
-  __shared__ __align__(8) uint32_t seen[kWarps][64];
-  __shared__ uint32_t s_slow;
+  __shared__ uint32_t seen[kWarps][64], s_slow;
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // so known to be the same in all lanes
   const uint32_t warps = blockDim.x / 32;
