@@ -57,7 +57,7 @@ __device__ __forceinline__ unsigned long long cta_scan(unsigned long long v, uns
 struct ShardWork {
   uint64_t groups, symbols;
 };
-__device__ ShardWork shard_work(int kind, const qlc_desc& d, uint32_t cs, uint32_t* status) {
+__device__ ShardWork shard_work(PlanKind kind, const qlc_desc& d, uint32_t cs, uint32_t* status) {
   ShardWork w = {0, 0};
   if (kind == kPlanEncode) {
     const uint64_t n = d.in_bytes;
@@ -121,8 +121,9 @@ __device__ uint32_t slow_samples(const qlc_desc* descs, int n_shards, const unsi
   return tries ? (found * kSamples + tries - 1) / tries : 0;
 }
 
+template <bool kDecode>
 __global__ void __launch_bounds__(kPlanThreads, 1)
-plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w, uint32_t* status) {
+plan_kernel(PlanKind kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w, uint32_t* status) {
   static_assert(kPlanThreads == kHcThreads, "cta_scan");
   __shared__ unsigned long long s_incl[kPlanThreads], s_warp[kPlanThreads / 32];
   __shared__ uint32_t s_chunk[2];
@@ -139,7 +140,7 @@ plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs 
   }
   bool split = false;
   uint32_t slow = 0;
-  if (kind != kPlanEncode) {
+  if constexpr (kDecode) {
     symbols = cta_scan(symbols, s_incl, s_warp, tid);
     split = kind == kPlanDecode && symbols <= kSplitMax;
     if (split) {
@@ -201,10 +202,19 @@ plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs 
   }
   if (tid == 0) {
     w.item_base[n_shards] = total;
-    if (kind != kPlanEncode) w.ticket[kTicketWay] = split ? kWaySplit : total <= cs ? kWayEven : kWayGroups;
+    if (kDecode) w.ticket[kTicketWay] = split ? kWaySplit : total <= cs ? kWayEven : kWayGroups;
   }
   if (kind == kPlanEncode)
     for (unsigned long long i = tid; i < total; i += kPlanThreads) w.gstat[i] = 0;
+}
+
+bool launch_plan(PlanKind kind, const qlc_desc* descs, int n_shards, uint32_t cs, const BatchWs& w, uint32_t* status,
+                 cudaStream_t st) {
+  if (kind == kPlanEncode)
+    plan_kernel<false><<<1, kPlanThreads, 0, st>>>(kind, descs, n_shards, cs, w, status);
+  else
+    plan_kernel<true><<<1, kPlanThreads, 0, st>>>(kind, descs, n_shards, cs, w, status);
+  return cudaGetLastError() == cudaSuccess;
 }
 
 // ------------------------------------------------------------- histograms

@@ -770,9 +770,9 @@ extern "C" qlc_status qlc_decode_batch(const qlc_desc* d_descs, int n_shards, vo
   const int per_sm = decode_warps(h_launch), sms = sm_count();
   static OncePerContext done;
   if (!smem_ok(decode_few_kernel, few_bytes(kFewWarps), done)) return QLC_ERR_CUDA;
-  plan_kernel<<<1, kPlanThreads, 0, st>>>(per_sm < kSpanWarps ? kPlanDecodeGroups : kPlanDecode, d_descs, n_shards,
-                                          (uint32_t)(per_sm * sms), w, d_status);
-  if (cudaGetLastError() != cudaSuccess) return QLC_ERR_CUDA;
+  if (!launch_plan(per_sm < kSpanWarps ? kPlanDecodeGroups : kPlanDecode, d_descs, n_shards, (uint32_t)(per_sm * sms), w,
+                   d_status, st))
+    return QLC_ERR_CUDA;
   // which of the two has the work is decided on the device; the other returns at once
   launch_after(decode_few_kernel, sms, 32 * per_sm, few_bytes(per_sm), st, d_descs, n_shards, w.item_base, w.ticket, d_status);
   launch_after(decode_batch_kernel, sms * per_sm, 32, 0, st, d_descs, n_shards, w.item_base, w.ticket, d_status);

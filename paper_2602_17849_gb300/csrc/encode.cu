@@ -1197,8 +1197,7 @@ qlc_status qlc_encode_batch(const qlc_desc* d_descs, int n_shards, uint32_t chun
   BatchWs w;
   if (!batch_ws_layout(d_ws, ws_bytes, n_shards, &w)) return QLC_ERR_CAPACITY;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  plan_kernel<<<1, kPlanThreads, 0, st>>>(kPlanEncode, d_descs, n_shards, chunk_symbols, w, d_status);
-  if (cudaGetLastError() != cudaSuccess) return QLC_ERR_CUDA;
+  if (!launch_plan(kPlanEncode, d_descs, n_shards, chunk_symbols, w, d_status, st)) return QLC_ERR_CUDA;
   EncArgs A = {};
   A.descs = d_descs;
   A.item_base = w.item_base;

@@ -302,13 +302,13 @@ enum PlanKind { kPlanEncode = 1, kPlanDecode = 2, kPlanDecodeGroups = 3 };
 constexpr int kPlanThreads = 1024;
 constexpr uint64_t kHistItem = 64 * 1024;  // symbols per histogram work item
 
-// One CTA: the number of work items of every shard (encode: groups of 32
-// chunks; decode: the container's groups, or in a batch that is decoded split
-// sets of kSpanWarps spans or groups), their exclusive prefix in item_base, and
-// zeroed counters / look-back words.  Shards that cannot be processed get no items
-// and set *status.  cs: the chunk size (encode), or the warps of
-// decode_few_kernel (decode): up to as many groups are dealt out evenly.
-__global__ void plan_kernel(int kind, const qlc_desc* descs, int n_shards, uint32_t cs, BatchWs w,
-                            uint32_t* status);
+// Launches plan_kernel (batch.cu), one CTA: the number of work items of every shard
+// (encode: groups of 32 chunks; decode: the container's groups, or in a batch that
+// is decoded split sets of kSpanWarps spans or groups), their exclusive prefix in
+// item_base, and zeroed counters / look-back words.  Shards that cannot be
+// processed get no items and set *status.  cs: the chunk size (encode), or the
+// warps of decode_few_kernel (decode): up to as many groups are dealt out evenly.
+bool launch_plan(PlanKind kind, const qlc_desc* descs, int n_shards, uint32_t cs, const BatchWs& w, uint32_t* status,
+                 cudaStream_t st);
 
 }  // namespace qlc
