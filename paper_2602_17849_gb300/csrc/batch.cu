@@ -240,7 +240,7 @@ __device__ __forceinline__ unsigned long long hist_items(const qlc_desc* descs, 
 // a load and two warp scans, where a planning kernel of its own and the search
 // in its prefix cost a launch and a chain of dependent loads.  24 shards of
 // 4 KiB - 64 MiB (139 MB): 30 us, from 4.5 us of planning and 43.5 us; 1152
-// shards (3.4 GB): 547 us (6.2 TB/s), from 600 us.
+// shards (3.4 GB): 541-547 us (6.2 TB/s), from 600 us.
 __global__ void __launch_bounds__(kHcThreads, 1)
 hist_batch_kernel(const qlc_desc* descs, int n_shards, unsigned long long* hists, int shared) {
   __shared__ __align__(16) uint32_t cols[kHcColWords];

@@ -24,11 +24,11 @@
 //   flush    a prefix sum of the counts places the lanes' symbols, which meet
 //            in shared memory and leave in whole lines.
 // Half of a tensor zeros (Student-t, Table 1, chunks of 4096): 1 Mi 103 -> 15 us,
-// 16 Mi 156 -> 27; the second half of every chunk 56 -> 19 and 144 -> 45; one chunk
-// of zeros in 64 Mi 191 -> 74 (none: 74); 64 Mi equal symbols under ranks of other
-// data 899 -> 69, since runs are not corrected piece after piece.  What still does
-// not resynchronise (sparse data, repeated patterns) is found by samples, and
-// larger containers of it are decoded a lane per chunk (split_rule.cuh).
+// 16 Mi 156 -> 27; the second half of every chunk 1 Mi 56 -> 19; one chunk of zeros
+// in 64 Mi 191 -> 74 (none: 74); 64 Mi equal symbols under ranks of other data 900
+// -> 68, since runs are not corrected piece after piece.  What still does not
+// resynchronise (sparse data, repeated patterns) is found by samples, and larger
+// containers of it are decoded a lane per chunk (split_rule.cuh).
 // A chunk is valid when its last piece ends at its last bit and its counts
 // add up to its symbols, which is when decoding it serially ends at its last
 // bit after that many symbols.
